@@ -17,6 +17,7 @@
 #include "frg_lblock.cuh"
 #include "frg_misc.cuh"
 #include "frg_tc.cuh"
+#include "frg_x64.cuh"
 
 using namespace frg;
 
@@ -42,6 +43,7 @@ struct frg_ctx {
   int nwork_all[3] = {0, 0, 0};
   WorkItem *d_work_pt[3] = {nullptr, nullptr, nullptr};
   std::vector<int> work_off[3];  // per point offsets into d_work_pt
+  X64Plan *x64 = nullptr;        // FP64 path: the points whose products run sliced on the tensor cores
   int *d_seg_point = nullptr, *d_seg_base = nullptr;
   int nseg = 0;
   // split stage kernels: layout blocks per point (the largest point's vertex
@@ -227,7 +229,11 @@ static int run_rhs(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cudaEvent
     }
     if (ev) CK(cudaEventRecord(ev[2], st), "event");
     if (chmask) {
-      LK(launch_contract_fp64(ctx->d_pts, d_io, w, nw, chmask, st), "fp64 contraction");
+      // the whole context's CUDA-core lists leave out the sliced points
+      if (point < 0 || !x64_has(ctx->x64, point))
+        LK(launch_contract_fp64(ctx->d_pts, d_io, w, nw, chmask, st), "fp64 contraction");
+      if (point < 0 ? ctx->x64 != nullptr : x64_has(ctx->x64, point))
+        LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st), "sliced fp64 contraction");
     } else {
       LK(launch_zero_vertex(ctx->d_pts, d_io, ctx->n, ctx->maxN, st), "zero vertex");
     }
@@ -652,6 +658,7 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
   // ---- contraction work lists (FP64 path): per point, and all points sorted
   // heavy-first so that long transfers start early and short ones fill in.
   if (!ctx->split) {
+    if (x64_create(&ctx->x64, ctx->hpts, ctx->mask & 7, ctx->d_err) != 0) return bail(FRG_ECUDA);
     for (int ch = 0; ch < 3; ++ch) {
       std::vector<std::pair<int, WorkItem>> all, one;
       std::vector<WorkItem> per;
@@ -661,7 +668,7 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
         build_work(ch, i, ctx->params[i].N_f, one);
         std::stable_sort(one.begin(), one.end(), [](auto &a, auto &b) { return a.first > b.first; });
         for (auto &x : one) per.push_back(x.second);
-        all.insert(all.end(), one.begin(), one.end());
+        if (!x64_has(ctx->x64, i)) all.insert(all.end(), one.begin(), one.end());
         ctx->work_off[ch].push_back((int)per.size());
       }
       std::stable_sort(all.begin(), all.end(), [](auto &a, auto &b) { return a.first > b.first; });
@@ -673,7 +680,12 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
         return bail(FRG_ENOMEM);
       cudaMemcpy(ctx->d_work_all[ch], allw.data(), sizeof(WorkItem) * allw.size(), cudaMemcpyHostToDevice);
       cudaMemcpy(ctx->d_work_pt[ch], per.data(), sizeof(WorkItem) * per.size(), cudaMemcpyHostToDevice);
+      for (int i = 0; i < n_points; ++i)
+        if (x64_has(ctx->x64, i))
+          x64_set_work(ctx->x64, i, ch, ctx->d_work_pt[ch] + ctx->work_off[ch][i],
+                       ctx->work_off[ch][i + 1] - ctx->work_off[ch][i]);
     }
+    if (ctx->x64 && x64_upload(ctx->x64) != 0) return bail(FRG_ECUDA);
   } else {
     int rc = tc_plan_create(&ctx->tc, ctx->hpts, ctx->params, ctx->precision, ctx->d_pts, ctx->d_err, why,
                             TcTune(), tc_schedules(ctx));
@@ -760,6 +772,7 @@ void frg_destroy(frg_ctx *ctx) {
   if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
   if (ctx->ev_out) cudaEventDestroy(ctx->ev_out);
   if (ctx->tc) tc_plan_destroy(ctx->tc);
+  x64_destroy(ctx->x64);
   for (void *p : ctx->allocs) cudaFree(p);
   for (auto p : ctx->user_in) if (p) cudaFree(p);
   for (auto p : ctx->user_out) if (p) cudaFree(p);

@@ -13,6 +13,7 @@
 #include "frg.h"
 #include "frg_common.cuh"
 #include "frg_split.cuh"
+#include "frg_x64.cuh"
 
 namespace frg {
 
@@ -537,16 +538,26 @@ __device__ __forceinline__ size_t out_index(int N, const Geom &g, int r, int c) 
   }
 }
 
-template <int CH, bool ACCUM>
-__global__ void __launch_bounds__(F64_THREADS)
-    k_contract_fp64(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                    const WorkItem *__restrict__ work) {
-  __shared__ double2 Ls[F64_TM][F64_TK + 1];
-  __shared__ double2 Rs[F64_TK][F64_TN + 1];
-  const WorkItem w = work[blockIdx.x];
-  const RhsIO &o = io[w.point];
-  if (!o.active) return;
-  const PointDesc &P = pts[w.point];
+// Output element in the channel's own layout (dph: X, xph: W).
+template <int CH>
+__device__ __forceinline__ size_t own_index(int N, const Geom &g, int r, int c) {
+  const int a = g.row_lo + r;
+  if (CH == CH_PP) return out_index<CH>(N, g, r, c);
+  if (CH == CH_DPH) return ((size_t)a * N + (a + g.x)) * N + c;
+  return ((size_t)(a + g.x) * N + a) * N + c;
+}
+
+struct F64Smem {
+  double2 Ls[F64_TM][F64_TK + 1];
+  double2 Rs[F64_TK][F64_TN + 1];
+};
+
+// One tile of one channel: store(local row, column, value) for every entry.
+template <int CH, typename Store>
+__device__ __forceinline__ void f64_tile(const PointDesc &P, const RhsIO &o, const WorkItem &w, F64Smem &sm,
+                                         Store store) {
+  auto &Ls = sm.Ls;
+  auto &Rs = sm.Rs;
   const int N = P.N;
   const Geom g = geom(CH, N, w.m);
   const int r0 = w.rt * F64_TM, c0 = w.ct * F64_TN;
@@ -586,19 +597,64 @@ __global__ void __launch_bounds__(F64_THREADS)
     __syncthreads();
   }
   const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
-  double2 *out = static_cast<double2 *>(o.dgam);
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int r = r0 + ty * 2 + i, c = c0 + tx * 2 + j;
-      if (r < g.D && c < N) {
-        const size_t at = out_index<CH>(N, g, r, c);
-        double2 v = make_double2(acc[i][j].x * sc, acc[i][j].y * sc);
-        if (ACCUM) v = cadd(out[at], v);
-        out[at] = v;
+      if (r < g.D && c < N) store(g, r, c, make_double2(acc[i][j].x * sc, acc[i][j].y * sc));
+    }
+}
+
+template <int CH, bool ACCUM>
+__global__ void __launch_bounds__(F64_THREADS)
+    k_contract_fp64(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
+                    const WorkItem *__restrict__ work) {
+  __shared__ F64Smem sm;
+  const WorkItem w = work[blockIdx.x];
+  const RhsIO &o = io[w.point];
+  if (!o.active) return;
+  const PointDesc &P = pts[w.point];
+  double2 *out = static_cast<double2 *>(o.dgam);
+  f64_tile<CH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) {
+    const size_t at = out_index<CH>(P.N, g, r, c);
+    out[at] = ACCUM ? cadd(out[at], v) : v;
+  });
+}
+
+// The same tiles for the points whose operands the sliced tensor-core products
+// could not take (X64Pt.bad), into the buffers those products write; returns at
+// once for the others.
+__global__ void __launch_bounds__(F64_THREADS)
+    k_x64_fallback(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
+                   int p0, int p1, int chmask) {
+  __shared__ F64Smem sm;
+  for (int pi = p0; pi < p1; ++pi) {
+    const X64Pt &x = xp[pi];
+    const RhsIO &o = io[pi];
+    if (!x.prod || !o.active || *x.bad == 0) continue;
+    const PointDesc &P = pts[pi];
+    for (int ch = 0; ch < 3; ++ch) {
+      if (!(chmask >> ch & 1)) continue;
+      double2 *out = ch == CH_PP ? static_cast<double2 *>(o.dgam) : ch == CH_DPH ? x.PX : x.PW;
+      for (int i = blockIdx.x; i < x.nwork[ch]; i += gridDim.x) {
+        const WorkItem w = x.work[ch][i];
+        if (ch == CH_PP)
+          f64_tile<CH_PP>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_PP>(P.N, g, r, c)] = v; });
+        else if (ch == CH_DPH)
+          f64_tile<CH_DPH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_DPH>(P.N, g, r, c)] = v; });
+        else
+          f64_tile<CH_XPH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_XPH>(P.N, g, r, c)] = v; });
       }
     }
+  }
+}
+
+int launch_x64_fallback(const PointDesc *d_pts, const RhsIO *d_io, const X64Pt *d_x, int p0, int p1, int chmask,
+                        cudaStream_t st) {
+  k_x64_fallback<<<304, F64_THREADS, 0, st>>>(d_pts, d_io, d_x, p0, p1, chmask);
+  FRG_COUNT(1);
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 // pp stores, dph and xph accumulate: the three channels run in this order so

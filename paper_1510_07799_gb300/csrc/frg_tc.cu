@@ -42,6 +42,7 @@
 
 #include "frg.h"
 #include "frg_layout.cuh"
+#include "frg_ptx.cuh"
 #include "frg_tc.cuh"
 
 namespace frg {
@@ -52,7 +53,6 @@ constexpr int NT_MAX = 128;         // complex columns per tile
 constexpr int MROWS = 64;           // complex rows per tile (128 real rows)
 constexpr int KSTEP = 16;           // complex k per pipeline stage (32 real K')
 constexpr int TMEM_COLS = 512;      // 2 buffers x 2 groups x 128 columns
-constexpr unsigned long long WAIT_NS = 2000000000ull;  // 2 s per wait
 
 // Per-precision operand format.  K' = 32 real values per row: 128 B rows
 // (TF32, 128-byte swizzle) or 64 B rows (BF16, 64-byte swizzle); the slices
@@ -73,70 +73,6 @@ struct TcWork {
 };
 
 // ---------------------------------------------------------------- PTX ----
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t *bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ unsigned long long gtime() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait on a phase; returns false (and records the failure) on timeout.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, unsigned *err, volatile int *abort_flag,
-                                          unsigned long long limit_ns = WAIT_NS) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = gtime();
-  for (unsigned it = 0;; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 255u) == 255u) {
-      if (*abort_flag) return false;
-      if (gtime() - t0 > limit_ns) {
-        atomicOr(err, 1u);
-        *abort_flag = 1;
-        return false;
-      }
-    }
-  }
-}
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_alloc(uint32_t *dst, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
 // Shared-memory matrix descriptor (K-major, swizzled): start address, stride
 // between 8-row atoms (SBO), version bits 46-48 = 0b001, swizzle mode.
 template <int PREC>
@@ -155,19 +91,12 @@ __host__ __device__ constexpr uint32_t idesc(int n) {
   return (1u << 4) | ((PREC == FRG_3XTF32 ? 2u : 1u) << 7) | ((PREC == FRG_3XTF32 ? 2u : 1u) << 10) |
          ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(id), "r"(acc)
-      : "memory");
-}
 template <int PREC>
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
   if (PREC == FRG_3XTF32)
     mma_tf32(d, a, b, id, acc);
   else
-    mma_bf16(d, a, b, id, acc);
+    mma_f16(d, a, b, id, acc);
 }
 
 // ----------------------------------------------------------- operands ----
@@ -354,12 +283,6 @@ __device__ __forceinline__ bool tile_info(const PointDesc *__restrict__ pts, con
 // Every wait is bounded: a wait that runs out sets the context error word and
 // all roles leave their loops.
 namespace st {
-// Warp-uniform bounded wait: every lane of the warp leaves with the same result,
-// so warp-collective code after it (shuffles, __syncwarp) never splits.
-__device__ __forceinline__ bool wwait(uint64_t *bar, uint32_t parity, unsigned *err, volatile int *abort_flag) {
-  const bool ok = mbar_wait(bar, parity, err, abort_flag);
-  return __all_sync(0xffffffffu, ok);
-}
 constexpr int KS = 16;                                  // complex k per step (K' = 2 KS real values)
 constexpr int NOP = 2;                                  // operand stages
 constexpr int RA = 18;                                  // complex per raw left row (aligned window)
@@ -401,11 +324,6 @@ __device__ __forceinline__ uint32_t grp_off(int row, int q) {
   if (PREC == FRG_3XTF32) return swz128(row, q);
   return (uint32_t)(row * 64 + (((q >> 1) ^ ((row >> 1) & 3)) << 4) + (q & 1) * 8);
 }
-__device__ __forceinline__ void arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-
 __device__ __forceinline__ void tma3(void *dst, const CUtensorMap *m, int x, int y, int z, uint64_t *bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "

@@ -1,0 +1,855 @@
+// frg_x64.cu -- FP64 channel products on the sm_103a tensor cores by exact
+// slicing (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59, 2012, with a fixed-point grid per operand line).
+//
+// This part's FP64 units run at 1/58 of FP32 (1.2 TFLOP/s measured); the FP16
+// tensor cores add integers exactly.  For a channel and transfer the product
+//   Out[r][c] = sum_k Left[r][k] Right[k][c]        (index sets: frg_common.cuh)
+// is formed as follows.
+//  * Every line (a row of the bubble-weighted left operand, a column of the
+//    right one) gets one exponent e with |x| < 0.993 2^e over the line, and its
+//    values become integers X = rint(x 2^(55 - e)).  A value within a factor 4
+//    of its line's bound converts exactly, a smaller one to 2^(e - 56).
+//  * X is cut into seven digits of base 256 in [-128, 127] (one 64-bit add of
+//    128 in every byte, done when X is stored, makes its bytes the digits + 128),
+//    each an exact FP16 value.
+//  * Digit products i + j = g <= 6 (i, j counted from the leading digit) of all
+//    k go to accumulator g: 28 products.  Each is an integer of at most 2^14, and
+//    an FP32 accumulator adds integers exactly up to 2^24.  The products left
+//    out (i + j >= 7) are below 2^-56 of the lines' bounds per term.
+//  * The epilogue adds the seven accumulators as 64-bit integers and rounds the
+//    sum once to FP64, on the integer pipe.
+// So the sum over k itself is exact to 2^-53 of the lines' bounds, where a chain
+// of K fused multiply-adds rounds K times: measured error against 64-bit exact
+// sums below that of the CUDA-core path (tests/test_gpu_x64.py).
+//
+// Three launches per rhs: k_x64_panels gathers, weights and converts the
+// operands into blocks of 16 k x 64 lines; k_x64_products multiplies them
+// (persistent CTAs over a longest-first tile schedule); k_x64_combine sums the
+// channels into the natural layout.  Lines that cannot be converted (non-finite
+// values, exponents beyond 2^+-400) mark their point, whose products the
+// CUDA-core kernel then forms instead (k_x64_fallback in frg_fp64.cu).
+// Measured, one rhs (all channels): N = 128 6086 -> 452 us, N = 64 674 -> 89 us
+// (CUDA cores -> slices).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <queue>
+#include <vector>
+
+#include "frg.h"
+#include "frg_common.cuh"
+#include "frg_ptx.cuh"
+#include "frg_x64.cuh"
+
+namespace frg {
+namespace x64 {
+using namespace tc;
+
+constexpr int SL = 7;                       // digits per value
+constexpr int LINES = 64;                   // lines of an operand block (rows or columns of a tile)
+constexpr int KS = 16;                      // complex k per block
+constexpr int BLK = LINES * KS;             // elements (re, im) of a block: 16 KB
+constexpr int BLK_BYTES = BLK * 16;
+constexpr int FIX = 55;                     // fixed-point position: X = x 2^(FIX - e)
+// 128 in each of the seven digit bytes; the top byte 0x64 is the high byte of
+// the FP16 values 1024 + b that the digits are unpacked through
+constexpr unsigned long long BIAS = 0x6480808080808080ull;
+constexpr int E_LIM = 400;                  // line exponents the path accepts
+
+// -------------------------------------------------------------- panels ----
+// One block: eight lines of one operand of one product over its whole
+// contraction range.  The lines are gathered (and weighted: the factor
+// +-T Lambda goes into the bubble weights) into shared memory, their largest
+// magnitudes give the exponents, and the values leave as fixed-point blocks in
+// 128-byte segments.  Bound by the FP64 multiplications of the weights and by
+// the gathers (16-byte elements, one 32-byte sector each wherever the line and
+// the contraction index both stride through the vertex).
+constexpr int PAN_T = 128, PAN_LINES = 8, PAN_PITCH = PAN_LINES + 1;
+// Elements along the contraction axis: one or two (direct channel) ranges of D
+// padded to whole blocks.
+__host__ __device__ inline int d16(int D) { return (D + KS - 1) / KS * KS; }
+static size_t panel_smem(int maxN) {
+  return (size_t)(2 * d16(maxN) * PAN_PITCH + d16(maxN)) * sizeof(double2);
+}
+
+__device__ __forceinline__ unsigned mag(double2 v) {
+  const unsigned a = (unsigned)__double2hiint(v.x) & 0x7fffffffu, b = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+  return a > b ? a : b;
+}
+// Exponent of a line whose largest high word (sign cleared) is m: |x| < 0.993 2^e.
+__device__ __forceinline__ int line_exp(unsigned m) {
+  if (m == 0u) return 0;
+  const int E = (int)(m >> 20);
+  return (E ? E : 1) - 1022 + ((m & 0xfffffu) >= 0xfc000u ? 1 : 0);
+}
+// rint(x 2^(FIX - e)) + BIAS (ties away from zero), for |x| < 0.993 2^e.
+__device__ __forceinline__ unsigned long long to_fixed(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int E = (int)(b >> 52) & 0x7ff;
+  unsigned long long m = (b & 0xfffffffffffffull) | (E ? 1ull << 52 : 0ull);
+  const int sh = (E ? E : 1) - 1075 + FIX - e;
+  if (sh >= 0) {
+    m <<= sh & 3;  // at most 2
+  } else {
+    const int r = min(-sh, 63);
+    m = (m + (1ull << (r - 1))) >> r;
+  }
+  return ((long long)b < 0 ? 0ull - m : m) + BIAS;
+}
+
+template <int CH, bool LEFT>
+__device__ __forceinline__ void gather(const PointDesc &P, const double2 *__restrict__ V, const Geom &g, int line,
+                                       int k, double2 w, double2 &v, double2 &v2) {
+  const int N = P.N;
+  auto at = [&](int i1, int i2, int i3) { return V[((size_t)i1 * N + i2) * N + i3]; };
+  if (LEFT) {
+    // every index is in the box for valid rows and k
+    const int p = g.p_lo + k;
+    if (CH == CH_PP) {
+      const int a = g.row_lo + line;
+      v = cmul(at(a, g.x - a, p), w);
+    } else if (CH == CH_DPH) {
+      const int k1 = g.row_lo + line, t = g.x;
+      const double2 A = at(k1, p, k1 + t), C = at(k1, p, p - t);
+      v = cmul(make_double2(2.0 * A.x - C.x, 2.0 * A.y - C.y), w);
+      v2 = cmul(make_double2(-A.x, -A.y), w);
+    } else {
+      const int k3 = g.row_lo + line;
+      v = cmul(at(p, k3 + g.x, k3), w);
+    }
+  } else {
+    const int p = g.p_lo + k, c = line;
+    const double2 U = make_double2(P.U, 0.0);
+    if (CH == CH_PP) {
+      v = inbox(N, g.x - c) ? at(p, g.x - p, c) : U;
+    } else if (CH == CH_DPH) {
+      const int t = g.x;
+      // the fourth index of B and the third of D are both c - t
+      const bool in = inbox(N, c - t);
+      v = in ? at(p - t, c, p) : U;
+      v2 = in ? at(p - t, c, c - t) : U;
+    } else {
+      v = inbox(N, c + g.x) ? at(c, p + g.x, p) : U;
+    }
+  }
+}
+
+template <int CH, bool LEFT>
+__device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const X64Pt &x, int m, int oct,
+                                      double2 *sp) {
+  const int N = P.N;
+  const Geom g = geom(CH, N, m);
+  const int D = g.D, D16 = d16(D), nk = (CH == CH_DPH ? 2 : 1) * (D16 / KS);
+  const int line0 = oct * PAN_LINES, nl = min(PAN_LINES, (LEFT ? D : N) - line0);
+  if (nl <= 0) return;
+  const int tid = threadIdx.x;
+  const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
+  __shared__ unsigned smax[PAN_LINES];
+  double2 *sw = sp + (CH == CH_DPH ? 2 : 1) * D16 * PAN_PITCH;
+  if (tid < PAN_LINES) smax[tid] = 0u;
+  if (LEFT) {
+    const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
+    const double2 *L = CH == CH_PP ? P.Lpp + (size_t)m * N : P.Lph + (size_t)(CH == CH_DPH ? 2 * N - 2 - m : m) * N;
+    for (int k = tid; k < D; k += PAN_T) sw[k] = cscale(L[g.p_lo + k], sc);
+  }
+  __syncthreads();
+  // the right pp operand is contiguous along its lines, the others along k or
+  // along neither
+  constexpr bool LINE_FAST = CH == CH_PP && !LEFT;
+  const int line = LINE_FAST ? tid & 7 : tid >> 4, k0 = LINE_FAST ? tid >> 3 : tid & 15;
+  unsigned um = 0u;
+  for (int kb = k0; kb < D16; kb += 64) {
+    double2 v[4], v2[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u] = v2[u] = make_double2(0.0, 0.0);
+      const int k = kb + 16 * u;
+      if (k < D && line < nl)
+        gather<CH, LEFT>(P, V, g, line0 + line, k, LEFT ? sw[k] : make_double2(0.0, 0.0), v[u], v2[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = kb + 16 * u;
+      if (k < D16) {
+        sp[k * PAN_PITCH + line] = v[u];
+        um = max(um, mag(v[u]));
+        if (CH == CH_DPH) {
+          sp[(D16 + k) * PAN_PITCH + line] = v2[u];
+          um = max(um, mag(v2[u]));
+        }
+      }
+    }
+  }
+  atomicMax(&smax[line], um);
+  __syncthreads();
+  const uint4 pr = x.prod[(size_t)CH * (2 * N - 1) + m];
+  const int tile = line0 / LINES, l0 = line0 & (LINES - 1);
+  const int ln = tid & 7;
+  const unsigned mx = smax[ln];
+  int e = line_exp(mx);
+  if (tid < nl) {
+    if (LEFT)
+      x.eL[(size_t)(pr.z + tile) * LINES + l0 + tid] = e;
+    else
+      x.eR[((size_t)(CH * (2 * N - 1) + m) * ((N + LINES - 1) / LINES) + tile) * LINES + l0 + tid] = e;
+    if ((mx >> 20) == 0x7ffu || e > E_LIM || e < -E_LIM) atomicOr(x.bad, 1);
+  }
+  e = max(-E_LIM, min(E_LIM, e));  // (a marked point's values are not used)
+  ulonglong2 *dst = (LEFT ? x.L + (size_t)(pr.x + tile * nk) * BLK : x.R + (size_t)(pr.y + tile * nk) * BLK) + l0 + ln;
+  if (ln < nl)
+    for (int k = tid >> 3; k < nk * KS; k += PAN_T / 8) {
+      const double2 v = sp[k * PAN_PITCH + ln];
+      dst[(size_t)k * LINES] = make_ulonglong2(to_fixed(v.x, e), to_fixed(v.y, e));
+    }
+}
+
+// grid: (line octets of the left, then of the right operand; transfers;
+// point x channel)
+__global__ void __launch_bounds__(PAN_T) k_x64_panels(const PointDesc *__restrict__ pts,
+                                                      const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
+                                                      int p0, int chmask) {
+  extern __shared__ double2 sp[];
+  const int pi = p0 + blockIdx.z / 3, ch = blockIdx.z % 3;
+  const RhsIO &o = io[pi];
+  const X64Pt &x = xp[pi];
+  if (!o.active || !x.prod || !(chmask >> ch & 1)) return;
+  const PointDesc &P = pts[pi];
+  const int m = blockIdx.y, half = gridDim.x / 2;
+  if (m >= 2 * P.N - 1) return;
+  const int b = blockIdx.x;
+  if (b < half) {
+    if (ch == CH_PP)
+      panel<CH_PP, true>(P, o, x, m, b, sp);
+    else if (ch == CH_DPH)
+      panel<CH_DPH, true>(P, o, x, m, b, sp);
+    else
+      panel<CH_XPH, true>(P, o, x, m, b, sp);
+  } else {
+    if (ch == CH_PP)
+      panel<CH_PP, false>(P, o, x, m, b - half, sp);
+    else if (ch == CH_DPH)
+      panel<CH_DPH, false>(P, o, x, m, b - half, sp);
+    else
+      panel<CH_XPH, false>(P, o, x, m, b - half, sp);
+  }
+}
+
+// ------------------------------------------------------------ products ----
+// A tile is 64 complex rows x 64 complex columns of one product.  Real form of
+// the complex product on the left operand: accumulator rows 0-63 hold Re,
+// rows 64-127 Im of the product, from A = [Re a; Im a] against Re b and
+// A = [-Im a; Re a] against Im b, so three planes of the left digits are kept.
+// Accumulator g (digit weight 256^-g) takes the 64 columns from 64 g on, and
+// the B digits of one k-step lie one after the other, so that one instruction
+// multiplies digit i of A with several consecutive digits of B: N up to 224.
+// Roles: warps 0-7 epilogue, 8 MMA issue, 9 loader (bulk copies, two blocks per
+// k-step), 10-17 transform (fixed-point values -> FP16 digit tiles).
+// Bound by the tensor cores (28 products of K' = 32 per k-step; the operand
+// reads of those products from shared memory come close behind).
+constexpr int EPI_W = 8, MMA_W = 8, LOAD_W = 9, XF_W0 = 10, N_XF = 8;
+constexpr int THREADS = 32 * (XF_W0 + N_XF);
+constexpr int NRAW = 2, NOP = 2;
+constexpr int RAW_STAGE = 2 * BLK_BYTES;
+// Operand tiles, K-major without swizzle: core matrices of 8 lines x 16 bytes.
+// A: [digit][k half][plane -Im, Re, Im][8 line groups][8 lines][16 B]
+// B: [plane Re, Im][k half][digit][8 line groups][8 lines][16 B]
+constexpr int PLANE = 1024;
+constexpr int A_KC = 3 * PLANE, A_DIG = 2 * A_KC, A_BYTES = SL * A_DIG;
+constexpr int B_KC = SL * PLANE, B_PL = 2 * B_KC, B_BYTES = 2 * B_PL;
+constexpr int OP_STAGE = A_BYTES + B_BYTES;
+constexpr int EPI_COLS = 8;
+constexpr int EPI_BUF = 32 * EPI_COLS * 16;  // one warp pair's 32 rows x 8 columns
+constexpr int SMEM = 1024 + NOP * OP_STAGE + NRAW * RAW_STAGE + 4 * EPI_BUF + 256;
+static_assert(SMEM <= 232448, "shared memory budget");
+
+struct Work {
+  int point;
+  short m, ch, rt, ct;
+};
+
+// Shared-memory matrix descriptor, K-major, no swizzle: lbo between the two
+// 16-byte columns of K, sbo between groups of eight lines.
+__device__ __forceinline__ uint64_t desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | (uint64_t)(lbo >> 4) << 16 | (uint64_t)(sbo >> 4) << 32 | 1ull << 46;
+}
+// D f32, A and B f16, K-major, M = 128, N = n.
+__host__ __device__ constexpr uint32_t idesc(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
+// Whether a predicate holds in both warps of an epilogue pair.
+__device__ __forceinline__ bool pair_all(bool v, int pair) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %1, 0;\n bar.red.and.pred q, %2, 64, p;\n selp.b32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)v), "r"(1 + pair)
+      : "memory");
+  return r != 0;
+}
+
+struct Tile {
+  int N, D, nk, r0, c0;
+  Geom g;
+  const ulonglong2 *L, *R;
+  const int *eL, *eR;
+};
+__device__ __forceinline__ bool tile_of(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
+                                        const X64Pt *__restrict__ xp, const Work &w, Tile &t) {
+  if (!io[w.point].active) return false;
+  const PointDesc &P = pts[w.point];
+  const X64Pt &x = xp[w.point];
+  t.N = P.N;
+  t.g = geom(w.ch, P.N, w.m);
+  t.D = t.g.D;
+  t.nk = (w.ch == CH_DPH ? 2 : 1) * (d16(t.D) / KS);
+  t.r0 = w.rt * LINES;
+  t.c0 = w.ct * LINES;
+  const int pi = w.ch * (2 * P.N - 1) + w.m, nct = (P.N + LINES - 1) / LINES;
+  const uint4 pr = x.prod[pi];
+  t.L = x.L + (size_t)(pr.x + w.rt * t.nk) * BLK;
+  t.R = x.R + (size_t)(pr.y + w.ct * t.nk) * BLK;
+  t.eL = x.eL + (size_t)(pr.z + w.rt) * LINES;
+  t.eR = x.eR + ((size_t)pi * nct + w.ct) * LINES;
+  return true;
+}
+
+// Digits `sel` of two values as a pair of FP16.  hi: the byte lies in the high
+// word, whose top byte is the FP16 exponent byte already.
+__device__ __forceinline__ uint32_t sub2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+constexpr uint32_t C1152 = 0x64806480u;  // (1152, 1152): 1024 + 128
+template <int I>
+__device__ __forceinline__ uint32_t biased(uint2 a, uint2 b) {
+  if constexpr (I < 3) {
+    constexpr uint32_t y = 2 - I;  // byte of the high word
+    return __byte_perm(a.y, b.y, y | 3u << 4 | (4 + y) << 8 | 7u << 12);
+  } else {
+    constexpr uint32_t y = 6 - I;  // byte of the low word
+    return (__byte_perm(a.x, b.x, y | y << 4 | (4 + y) << 8 | (4 + y) << 12) & 0x00ff00ffu) | 0x64006400u;
+  }
+}
+// Digit I of the eight values of one line: Re, Im and (left operand) -Im.
+template <int I, bool LEFT>
+__device__ __forceinline__ void store_digit(uint8_t *dst, const uint4 (&v)[8]) {
+  uint4 re, im, ni;
+  uint32_t *r = &re.x, *i = &im.x, *n = &ni.x;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint4 a = v[2 * q], b = v[2 * q + 1];
+    const uint32_t br = biased<I>(make_uint2(a.x, a.y), make_uint2(b.x, b.y));
+    const uint32_t bi = biased<I>(make_uint2(a.z, a.w), make_uint2(b.z, b.w));
+    r[q] = sub2(br, C1152);
+    i[q] = sub2(bi, C1152);
+    if (LEFT) n[q] = sub2(C1152, bi);
+  }
+  if (LEFT) {
+    uint8_t *p = dst + I * A_DIG;
+    *reinterpret_cast<uint4 *>(p) = ni;
+    *reinterpret_cast<uint4 *>(p + PLANE) = re;
+    *reinterpret_cast<uint4 *>(p + 2 * PLANE) = im;
+  } else {
+    uint8_t *p = dst + I * PLANE;
+    *reinterpret_cast<uint4 *>(p) = re;
+    *reinterpret_cast<uint4 *>(p + B_PL) = im;
+  }
+}
+template <bool LEFT>
+__device__ __forceinline__ void store_digits(uint8_t *dst, const uint4 (&v)[8]) {
+  store_digit<0, LEFT>(dst, v);
+  store_digit<1, LEFT>(dst, v);
+  store_digit<2, LEFT>(dst, v);
+  store_digit<3, LEFT>(dst, v);
+  store_digit<4, LEFT>(dst, v);
+  store_digit<5, LEFT>(dst, v);
+  store_digit<6, LEFT>(dst, v);
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+// s 2^e as FP64, rounded once, on the integer pipe (e within +-900: normal).
+__device__ __forceinline__ double scaled(long long s, int e) {
+  const unsigned long long sg = (unsigned long long)s & 0x8000000000000000ull;
+  unsigned long long a = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
+  if (a == 0ull) return 0.0;
+  const int lz = __clzll((long long)a);
+  a <<= lz;
+  // 53 leading bits, the implicit one included (it carries into the exponent)
+  const unsigned long long mant = (a >> 11) + ((a >> 10) & 1ull);
+  return __longlong_as_double((long long)(((unsigned long long)(1023 + 63 - lz + e - 1) << 52) + mant | sg));
+}
+
+// Row pointer of local row rr in the channel's own layout (pp: natural, dph: X,
+// xph: W).
+__device__ __forceinline__ double2 *out_row(int ch, double2 *kN, const X64Pt &x, const Tile &t, int rr) {
+  const int N = t.N, a = t.g.row_lo + rr;
+  if (ch == CH_PP) return kN + ((size_t)a * N + (t.g.x - a)) * N;
+  if (ch == CH_DPH) return x.PX + ((size_t)a * N + (a + t.g.x)) * N;
+  return x.PW + ((size_t)(a + t.g.x) * N + a) * N;
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
+    k_x64_products(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
+                   const Work *__restrict__ work, const int *__restrict__ cta_start, unsigned *__restrict__ err) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  uint8_t *ops = smem, *raws = ops + NOP * OP_STAGE, *epi = raws + NRAW * RAW_STAGE;
+  uint64_t *raw_full = reinterpret_cast<uint64_t *>(epi + 4 * EPI_BUF), *raw_empty = raw_full + NRAW;
+  uint64_t *op_full = raw_empty + NRAW, *op_empty = op_full + NOP, *tfull = op_empty + NOP, *tempty = tfull + 1;
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tempty + 1);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int j = 0; j < NRAW; ++j) {
+      mbar_init(&raw_full[j], 1);
+      mbar_init(&raw_empty[j], N_XF);
+    }
+    for (int s = 0; s < NOP; ++s) {
+      mbar_init(&op_full[s], N_XF);
+      mbar_init(&op_empty[s], 1);
+    }
+    mbar_init(tfull, 1);
+    mbar_init(tempty, EPI_W);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == MMA_W) tmem_alloc(tmem_slot, 512);
+  tc_before();
+  __syncthreads();
+  tc_after();
+  const uint32_t tmem = *tmem_slot;
+  const int w0 = cta_start[blockIdx.x], w1 = cta_start[blockIdx.x + 1];
+
+  if (warp == LOAD_W) {
+    uint32_t it = 0;
+    bool ok = true;
+    for (int wi = w0; wi < w1 && ok; ++wi) {
+      Tile t;
+      if (!tile_of(pts, io, xp, work[wi], t)) continue;
+      for (int kb = 0; kb < t.nk; ++kb, ++it) {
+        const int j = it % NRAW;
+        if (!(ok = wwait(&raw_empty[j], ((it / NRAW) & 1u) ^ 1u, err, abort_flag))) break;
+        if (lane == 0) {
+          arrive_expect_tx(&raw_full[j], RAW_STAGE);
+          bulk_copy(raws + j * RAW_STAGE, t.L + (size_t)kb * BLK, BLK_BYTES, &raw_full[j]);
+          bulk_copy(raws + j * RAW_STAGE + BLK_BYTES, t.R + (size_t)kb * BLK, BLK_BYTES, &raw_full[j]);
+        }
+        __syncwarp();
+      }
+    }
+    // copies still in flight must land before the CTA leaves
+    for (uint32_t k = it > (uint32_t)NRAW ? it - NRAW : 0u; k < it; ++k)
+      wwait(&raw_full[k % NRAW], (k / NRAW) & 1u, err, abort_flag);
+  } else if (warp >= XF_W0) {
+    // warps 0-3 of the role: left lines, 4-7: right lines; one line and eight
+    // of the 16 k per thread
+    const int xt = tid - 32 * XF_W0, side = xt >> 7, oct = (xt >> 6) & 1, line = xt & 63;
+    const uint32_t src = side * BLK_BYTES + (oct * 8 * LINES + line) * 16;
+    const uint32_t at = (side ? A_BYTES + oct * B_KC : oct * A_KC) + line * 16;
+    uint32_t it = 0;
+    bool ok = true;
+    for (int wi = w0; wi < w1 && ok; ++wi) {
+      Tile t;
+      if (!tile_of(pts, io, xp, work[wi], t)) continue;
+      for (int kb = 0; kb < t.nk; ++kb, ++it) {
+        const int j = it % NRAW, s = it % NOP;
+        if (!(ok = wwait(&raw_full[j], (it / NRAW) & 1u, err, abort_flag))) break;
+        const uint8_t *raw = raws + j * RAW_STAGE + src;
+        uint4 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = *reinterpret_cast<const uint4 *>(raw + q * LINES * 16);
+        // the loader's next copy into this stage is an async-proxy write: order
+        // the reads above before it
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&raw_empty[j]);
+        if (!(ok = wwait(&op_empty[s], ((it / NOP) & 1u) ^ 1u, err, abort_flag))) break;
+        uint8_t *dst = ops + s * OP_STAGE + at;
+        if (side == 0)
+          store_digits<true>(dst, v);
+        else
+          store_digits<false>(dst, v);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&op_full[s]);
+      }
+    }
+  } else if (warp == MMA_W) {
+    uint32_t it = 0, use = 0;
+    bool ok = true;
+    for (int wi = w0; wi < w1 && ok; ++wi) {
+      Tile t;
+      if (!tile_of(pts, io, xp, work[wi], t)) continue;
+      if (!(ok = wwait(tempty, (use & 1u) ^ 1u, err, abort_flag))) break;
+      ++use;
+      tc_after();
+      for (int kb = 0; kb < t.nk; ++kb, ++it) {
+        const int s = it % NOP;
+        if (!(ok = wwait(&op_full[s], (it / NOP) & 1u, err, abort_flag))) break;
+        tc_after();
+        if (lane == 0) {
+          const uint32_t a0 = smem_u32(ops + s * OP_STAGE), b0 = a0 + A_BYTES;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            // q = 0: [Re; Im] (planes 1, 2) x Re b; q = 1: [-Im; Re] (planes 0, 1) x Im b
+            const uint32_t aq = a0 + (q == 0 ? PLANE : 0), bq = b0 + q * B_PL;
+#pragma unroll
+            for (int i = 0; i < SL; ++i) {
+              const int cols = LINES * (SL - i), n1 = cols > 256 ? cols / 2 : cols;
+              const uint64_t da = desc(aq + i * A_DIG, A_KC, 128);
+              const uint32_t d = tmem + LINES * i;
+              mma_f16(d, da, desc(bq, B_KC, 128), idesc(n1), (kb | q | i) ? 1u : 0u);
+              if (cols > 256)  // the second half of the columns: n1 / 8 line groups further on
+                mma_f16(d + n1, da, desc(bq + n1 / 8 * 128, B_KC, 128), idesc(n1), (kb | q | i) ? 1u : 0u);
+            }
+          }
+          mma_commit(&op_empty[s]);
+        }
+        __syncwarp();
+      }
+      if (!ok) break;
+      if (lane == 0) mma_commit(tfull);
+      __syncwarp();
+    }
+  } else {
+    // warps w and w ^ 2 (w & 4 the same) hold Re and Im of the same 32 rows and
+    // take 32 of the 64 columns, eight at a time, through a common staging buffer
+    const int quarter = warp & 3, comp = quarter >> 1, pair = (quarter & 1) | (warp >> 2) << 1;
+    uint8_t *buf = epi + pair * EPI_BUF;
+    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
+    uint32_t use = 0;
+    bool ok = true;
+    for (int wi = w0; wi < w1 && ok; ++wi) {
+      Tile t;
+      const Work w = work[wi];
+      if (!tile_of(pts, io, xp, w, t)) continue;
+      // both warps of a pair leave together when a wait gave up
+      if (!(ok = pair_all(wwait(tfull, use & 1u, err, abort_flag), pair))) break;
+      ++use;
+      tc_after();
+      double2 *kN = static_cast<double2 *>(io[w.point].dgam);
+      const X64Pt &x = xp[w.point];
+      const int rl = 32 * (quarter & 1);  // first row of this warp's half
+      const int el = t.r0 + rl + lane < t.D ? t.eL[rl + lane] : 0;
+      for (int ci = 0; ci < 4; ++ci) {
+        const int cb = 32 * (warp >> 2) + ci * EPI_COLS;
+        float v[SL][EPI_COLS];
+#pragma unroll
+        for (int g = 0; g < SL; ++g) tmem_ld8(tl + g * LINES + cb, v[g]);
+        tmem_wait_ld();
+        if (ci == 3) {
+          tc_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty);
+        }
+#pragma unroll
+        for (int c = 0; c < EPI_COLS; ++c) {
+          const long long hi = (long long)__float2int_rn(v[2][c]) + (long long)__float2int_rn(v[1][c]) * 256 +
+                               (long long)__float2int_rn(v[0][c]) * 65536;
+          const long long lo = (long long)__float2int_rn(v[6][c]) + (long long)__float2int_rn(v[5][c]) * 256 +
+                               (long long)__float2int_rn(v[4][c]) * 65536 +
+                               (long long)__float2int_rn(v[3][c]) * 16777216;
+          const int er = t.c0 + cb + c < t.N ? t.eR[cb + c] : 0;
+          // sum of the integers X_L X_R in units of 2^57
+          const double r = scaled((hi << 23) + ((lo + 256) >> 9), el + er + 57 - 2 * FIX);
+          *reinterpret_cast<double *>(buf + lane * (EPI_COLS * 16) + ((c ^ (lane & 7)) << 4) + comp * 8) = r;
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
+        // each warp of the pair stores 16 of the 32 rows, 128 bytes a row
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = comp * 16 + (lane >> 3) + 4 * i, c = lane & 7;
+          const double2 z = *reinterpret_cast<const double2 *>(buf + row * (EPI_COLS * 16) + ((c ^ (row & 7)) << 4));
+          const int rr = t.r0 + rl + row, cc = t.c0 + cb + c;
+          if (rr < t.D && cc < t.N) out_row(w.ch, kN, x, t, rr)[cc] = z;
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
+      }
+    }
+  }
+  tc_before();
+  __syncthreads();
+  tc_after();
+  if (warp == MMA_W) tmem_dealloc(tmem, 512);
+}
+
+// ------------------------------------------------------------- combine ----
+// dGamma = (pp + direct) + crossed, the enabled channels, into the natural
+// layout (the pp products are there already).  A thread takes four consecutive
+// i1 of one (i2, i3): 64 contiguous bytes of a W row; a warp covers 4 i2 (64
+// bytes of each X row) x 8 i3 (128 bytes of each natural row).
+__global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict__ pts,
+                                                     const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
+                                                     int p0, int nz, int chmask) {
+  const int pi = p0 + blockIdx.z / nz;
+  const RhsIO &o = io[pi];
+  const X64Pt &x = xp[pi];
+  if (!o.active || !x.prod) return;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z % nz == 0 && threadIdx.x == 0) *x.bad = 0;
+  const int N = pts[pi].N, t = threadIdx.x;
+  const int i1 = 4 * (blockIdx.z % nz), i2 = 8 * blockIdx.y + 4 * (t >> 7) + ((t >> 3) & 3),
+            i3 = 32 * blockIdx.x + 8 * ((t >> 5) & 3) + (t & 7);
+  if (i1 >= N || i2 >= N || i3 >= N) return;
+  double2 *out = static_cast<double2 *>(o.dgam);
+  const double2 z = make_double2(0.0, 0.0);
+  double2 a[4], b[4], c[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const bool in = i1 + j < N;
+    a[j] = in && (chmask & 1) ? out[((size_t)(i1 + j) * N + i2) * N + i3] : z;
+    b[j] = in && (chmask & 2) ? x.PX[((size_t)(i1 + j) * N + i3) * N + i2] : z;
+    c[j] = in && (chmask & 4) ? x.PW[((size_t)i2 * N + i3) * N + i1 + j] : z;
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (i1 + j < N) out[((size_t)(i1 + j) * N + i2) * N + i3] = cadd(cadd(a[j], b[j]), c[j]);
+}
+}  // namespace x64
+
+// ---------------------------------------------------------------- plan ----
+struct X64Plan {
+  struct Sched {
+    x64::Work *d_work = nullptr;
+    int *d_start = nullptr;
+    int grid = 0;
+  };
+  struct Group {
+    int p0, p1, maxN;
+    Sched all;
+  };
+  std::vector<X64Pt> h;
+  std::vector<int> N;          // per point, 0: not on this path
+  std::vector<Sched> one;      // per point
+  std::vector<Group> groups;   // points whose operands share the workspace, one group after another
+  X64Pt *d_x = nullptr;
+  int *d_bad = nullptr;
+  char *ws = nullptr;
+  std::vector<void *> tables;
+  unsigned *d_err = nullptr;
+};
+
+namespace {
+// Operands of one group of points at most (a single point may need more: 2.9 GB
+// at N = 256): a large batch reuses the workspace group by group, so that the
+// path never takes more than a small part of the device's memory.
+constexpr size_t X64_WS_CAP = (size_t)4 << 30;
+constexpr int X64_GROUP = 512;  // points per group: grid.z stays below 65536
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+bool upload_sched(X64Plan::Sched &out, std::vector<std::pair<int, x64::Work>> &tiles, int sms) {
+  std::stable_sort(tiles.begin(), tiles.end(), [](auto &a, auto &b) { return a.first > b.first; });
+  out.grid = std::min((int)tiles.size(), sms);
+  if (!out.grid) return true;
+  // longest tile first, each to the CTA with the least work so far
+  std::vector<std::vector<x64::Work>> per(out.grid);
+  std::priority_queue<std::pair<long, int>, std::vector<std::pair<long, int>>, std::greater<std::pair<long, int>>> q;
+  for (int c = 0; c < out.grid; ++c) q.push({0, c});
+  for (auto &t : tiles) {
+    auto [load, c] = q.top();
+    q.pop();
+    per[c].push_back(t.second);
+    q.push({load + t.first, c});
+  }
+  std::vector<x64::Work> flat;
+  std::vector<int> start(1, 0);
+  for (auto &v : per) {
+    flat.insert(flat.end(), v.begin(), v.end());
+    start.push_back((int)flat.size());
+  }
+  return cudaMalloc(&out.d_work, sizeof(x64::Work) * flat.size()) == cudaSuccess &&
+         cudaMalloc(&out.d_start, sizeof(int) * start.size()) == cudaSuccess &&
+         cudaMemcpy(out.d_work, flat.data(), sizeof(x64::Work) * flat.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+         cudaMemcpy(out.d_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+}
+}  // namespace
+
+int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, unsigned *d_err) {
+  *out = nullptr;
+  const int n = (int)pts.size();
+  bool any = false;
+  for (const PointDesc &P : pts) any = any || P.N >= X64_MIN_N;
+  if (!any || !(chmask & 7)) return 0;
+  int dev = 0, sms = 0, maj = 0, min_ = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&maj, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&min_, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess)
+    return -3;
+  if (maj != 10 || min_ != 3) return 0;
+  X64Plan *p = new X64Plan();
+  p->d_err = d_err;
+  p->h.assign(n, X64Pt{});
+  p->N.assign(n, 0);
+  p->one.resize(n);
+  // per point: product table, tiles, and the sizes of its operands
+  struct Size {
+    size_t blkL = 0, blkR = 0, tileL = 0, tileR = 0, n3 = 0;
+  };
+  std::vector<Size> size(n);
+  std::vector<std::vector<uint4>> tab(n);
+  std::vector<std::vector<std::pair<int, x64::Work>>> tiles(n);
+  for (int i = 0; i < n; ++i) {
+    const int N = pts[i].N;
+    if (N < X64_MIN_N) continue;
+    p->N[i] = N;
+    Size &s = size[i];
+    s.n3 = (size_t)N * N * N;
+    tab[i].resize(3 * (2 * N - 1));
+    const int nct = (N + x64::LINES - 1) / x64::LINES;
+    s.tileR = (size_t)3 * (2 * N - 1) * nct;
+    for (int ch = 0; ch < 3; ++ch) {
+      if (!(chmask >> ch & 1)) continue;
+      for (int m = 0; m < 2 * N - 1; ++m) {
+        const Geom g = geom(ch, N, m);
+        const int nk = (ch == CH_DPH ? 2 : 1) * (x64::d16(g.D) / x64::KS);
+        const int nrt = (g.D + x64::LINES - 1) / x64::LINES;
+        tab[i][ch * (2 * N - 1) + m] = make_uint4((unsigned)s.blkL, (unsigned)s.blkR, (unsigned)s.tileL, 0u);
+        s.blkL += (size_t)nrt * nk;
+        s.blkR += (size_t)nct * nk;
+        s.tileL += nrt;
+        // the drain of a tile's accumulators costs about two k-steps
+        for (int rt = 0; rt < nrt; ++rt)
+          for (int ct = 0; ct < nct; ++ct)
+            tiles[i].push_back({nk + 2, x64::Work{i, (short)m, (short)ch, (short)rt, (short)ct}});
+      }
+    }
+  }
+  auto bytes = [&](const Size &s) {
+    return align256(s.blkL * x64::BLK_BYTES) + align256(s.blkR * x64::BLK_BYTES) + align256(s.tileL * x64::LINES * 4) +
+           align256(s.tileR * x64::LINES * 4) + 2 * align256(s.n3 * sizeof(double2));
+  };
+  // consecutive points share the workspace up to its cap
+  size_t ws = 0;
+  std::vector<size_t> base(n, 0);
+  for (int i = 0; i < n;) {
+    size_t sum = 0;
+    int j = i, maxN = 0;
+    for (; j < n && j < i + X64_GROUP && (j == i || sum + bytes(size[j]) <= X64_WS_CAP); ++j) {
+      base[j] = sum;
+      sum += bytes(size[j]);
+      maxN = std::max(maxN, p->N[j]);
+    }
+    if (maxN) p->groups.push_back({i, j, maxN, {}});
+    ws = std::max(ws, sum);
+    i = j;
+  }
+  if (cudaMalloc(&p->ws, ws) != cudaSuccess) {
+    cudaGetLastError();
+    x64_destroy(p);
+    return 0;
+  }
+  bool ok = cudaMalloc(&p->d_x, sizeof(X64Pt) * n) == cudaSuccess &&
+            cudaMalloc(&p->d_bad, sizeof(int) * n) == cudaSuccess &&
+            cudaMemset(p->d_bad, 0, sizeof(int) * n) == cudaSuccess &&
+            cudaFuncSetAttribute(x64::k_x64_products, cudaFuncAttributeMaxDynamicSharedMemorySize, x64::SMEM) ==
+                cudaSuccess &&
+            cudaFuncSetAttribute(x64::k_x64_panels, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)x64::panel_smem(FRG_MAX_N)) == cudaSuccess;
+  for (int i = 0; i < n && ok; ++i) {
+    if (!p->N[i]) continue;
+    X64Pt &x = p->h[i];
+    const Size &s = size[i];
+    char *b = p->ws + base[i];
+    x.L = reinterpret_cast<ulonglong2 *>(b);
+    b += align256(s.blkL * x64::BLK_BYTES);
+    x.R = reinterpret_cast<ulonglong2 *>(b);
+    b += align256(s.blkR * x64::BLK_BYTES);
+    x.eL = reinterpret_cast<int *>(b);
+    b += align256(s.tileL * x64::LINES * 4);
+    x.eR = reinterpret_cast<int *>(b);
+    b += align256(s.tileR * x64::LINES * 4);
+    x.PX = reinterpret_cast<double2 *>(b);
+    b += align256(s.n3 * sizeof(double2));
+    x.PW = reinterpret_cast<double2 *>(b);
+    x.bad = p->d_bad + i;
+    void *t = nullptr;
+    ok = cudaMalloc(&t, sizeof(uint4) * tab[i].size()) == cudaSuccess;
+    if (!ok) break;
+    p->tables.push_back(t);
+    x.prod = static_cast<const uint4 *>(t);
+    ok = cudaMemcpy(t, tab[i].data(), sizeof(uint4) * tab[i].size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+         upload_sched(p->one[i], tiles[i], sms);
+  }
+  for (X64Plan::Group &g : p->groups) {
+    if (!ok) break;
+    std::vector<std::pair<int, x64::Work>> all;
+    for (int i = g.p0; i < g.p1; ++i) all.insert(all.end(), tiles[i].begin(), tiles[i].end());
+    ok = upload_sched(g.all, all, sms);
+  }
+  if (!ok) {
+    x64_destroy(p);
+    return -3;
+  }
+  *out = p;
+  return 0;
+}
+
+void x64_set_work(X64Plan *p, int point, int ch, const WorkItem *d_work, int n) {
+  p->h[point].work[ch] = d_work;
+  p->h[point].nwork[ch] = n;
+}
+
+int x64_upload(X64Plan *p) {
+  return cudaMemcpy(p->d_x, p->h.data(), sizeof(X64Pt) * p->h.size(), cudaMemcpyHostToDevice) == cudaSuccess ? 0 : -3;
+}
+
+void x64_destroy(X64Plan *p) {
+  if (!p) return;
+  auto drop = [](X64Plan::Sched &s) {
+    cudaFree(s.d_work);
+    cudaFree(s.d_start);
+  };
+  for (auto &s : p->one) drop(s);
+  for (auto &g : p->groups) drop(g.all);
+  for (void *t : p->tables) cudaFree(t);
+  cudaFree(p->d_x);
+  cudaFree(p->d_bad);
+  cudaFree(p->ws);
+  delete p;
+}
+
+bool x64_has(const X64Plan *p, int point) { return p && p->N[point] > 0; }
+
+int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st) {
+  for (size_t gi = 0; gi < p->groups.size(); ++gi) {
+    X64Plan::Group &g = p->groups[gi];
+    int p0 = g.p0, p1 = g.p1, maxN = g.maxN;
+    const X64Plan::Sched *s = &g.all;
+    if (point >= 0) {
+      if (point < g.p0 || point >= g.p1) continue;
+      p0 = point;
+      p1 = point + 1;
+      maxN = p->N[point];
+      s = &p->one[point];
+    }
+    const int oct = (maxN + x64::PAN_LINES - 1) / x64::PAN_LINES, np = p1 - p0;
+    x64::k_x64_panels<<<dim3(2 * oct, 2 * maxN - 1, 3 * np), x64::PAN_T, x64::panel_smem(maxN), st>>>(d_pts, d_io, p->d_x,
+                                                                                                  p0, chmask);
+    x64::k_x64_products<<<s->grid, x64::THREADS, x64::SMEM, st>>>(d_pts, d_io, p->d_x, s->d_work, s->d_start, p->d_err);
+    FRG_COUNT(2);
+    if (launch_x64_fallback(d_pts, d_io, p->d_x, p0, p1, chmask, st) != 0) return -3;
+    const int nz = (maxN + 3) / 4;
+    x64::k_x64_combine<<<dim3((maxN + 31) / 32, (maxN + 7) / 8, nz * np), 256, 0, st>>>(d_pts, d_io, p->d_x, p0, nz,
+                                                                                      chmask);
+    FRG_COUNT(1);
+  }
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
+}  // namespace frg
