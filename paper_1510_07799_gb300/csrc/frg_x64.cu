@@ -29,7 +29,7 @@
 // channels into the natural layout.  Lines that cannot be converted (non-finite
 // values, exponents beyond 2^+-400) mark their point, whose products the
 // CUDA-core kernel then forms instead (k_x64_fallback in frg_fp64.cu).
-// Measured, one rhs (all channels): N = 128 6086 -> 452 us, N = 64 674 -> 89 us
+// Measured, one rhs (all channels): N = 128 6086 -> 330 us, N = 64 674 -> 78 us
 // (CUDA cores -> slices).
 #include <cuda_runtime.h>
 
@@ -59,19 +59,23 @@ constexpr int E_LIM = 400;                  // line exponents the path accepts
 
 // -------------------------------------------------------------- panels ----
 // One block: eight lines of one operand of one product over its whole
-// contraction range.  The lines are gathered (and weighted: the factor
-// +-T Lambda goes into the bubble weights) into shared memory, their largest
-// magnitudes give the exponents, and the values leave as fixed-point blocks in
-// 128-byte segments.  Bound by the FP64 multiplications of the weights and by
-// the gathers (16-byte elements, one 32-byte sector each wherever the line and
-// the contraction index both stride through the vertex).
-constexpr int PAN_T = 128, PAN_LINES = 8, PAN_PITCH = PAN_LINES + 1;
+// contraction range.  Eight lanes take the eight lines at one k, so that the
+// blocks are written in 128-byte segments; a thread gathers (and weights: the
+// factor +-T Lambda goes into the bubble weights) all its k of one line into
+// registers, the block finds each line's largest magnitude, and the values leave
+// in fixed point.  Bound by the FP64 multiplications of the weights and by the
+// gathers (16-byte elements, one 32-byte sector each wherever the line and the
+// contraction index both stride through the vertex): 114 us at N = 128 for 302 MB
+// written and 15 M entries gathered, the FP64 pipe half busy; 159 us with the
+// lines staged in shared memory between the gather and the conversion.
+constexpr int PAN_LINES = 8;
+constexpr int PAN_U = 4;  // k per thread and range
 // Elements along the contraction axis: one or two (direct channel) ranges of D
 // padded to whole blocks.
 __host__ __device__ inline int d16(int D) { return (D + KS - 1) / KS * KS; }
-static size_t panel_smem(int maxN) {
-  return (size_t)(2 * d16(maxN) * PAN_PITCH + d16(maxN)) * sizeof(double2);
-}
+// Threads of a block: eight per k, and at most PAN_U k each.
+static int panel_threads(int maxN) { return std::max(64, (d16(maxN) + 15) / 16 * 32); }
+static_assert(2 * PAN_U == PAN_LINES, "a block of twice as many threads as k takes PAN_U of them per thread");
 
 __device__ __forceinline__ unsigned mag(double2 v) {
   const unsigned a = (unsigned)__double2hiint(v.x) & 0x7fffffffu, b = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
@@ -83,52 +87,47 @@ __device__ __forceinline__ int line_exp(unsigned m) {
   const int E = (int)(m >> 20);
   return (E ? E : 1) - 1022 + ((m & 0xfffffu) >= 0xfc000u ? 1 : 0);
 }
-// rint(x 2^(FIX - e)) + BIAS (ties away from zero), for |x| < 0.993 2^e.
+// rint(x 2^(FIX - e)) + BIAS (ties away from zero), for |x| < 0.993 2^e, e >= -E_LIM.
 __device__ __forceinline__ unsigned long long to_fixed(double x, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int E = (int)(b >> 52) & 0x7ff;
-  unsigned long long m = (b & 0xfffffffffffffull) | (E ? 1ull << 52 : 0ull);
-  const int sh = (E ? E : 1) - 1075 + FIX - e;
-  if (sh >= 0) {
-    m <<= sh & 3;  // at most 2
-  } else {
-    const int r = min(-sh, 63);
-    m = (m + (1ull << (r - 1))) >> r;
-  }
-  return ((long long)b < 0 ? 0ull - m : m) + BIAS;
+  const int h = __double2hiint(x);
+  const int E = (h >> 20) & 0x7ff;
+  // the 53-bit significand, three bits up (zero and denormals: the implicit bit
+  // set here is shifted out with the rest), then right to one bit below the
+  // fixed point
+  const unsigned long long m = (unsigned long long)((unsigned)h & 0xfffffu | 0x100000u) << 32 | (unsigned)__double2loint(x);
+  const unsigned long long r = (((m << 3) >> min(e + 1022 - E, 63)) + 1ull) >> 1;
+  const unsigned long long s = (unsigned long long)(long long)(h >> 31);  // all ones for x < 0
+  return (r ^ s) + (BIAS - s);
 }
 
+// The vertex entries of one element: the pp and crossed operands and the direct
+// channel's A and C (left) or B and D (right).
 template <int CH, bool LEFT>
 __device__ __forceinline__ void gather(const PointDesc &P, const double2 *__restrict__ V, const Geom &g, int line,
-                                       int k, double2 w, double2 &v, double2 &v2) {
-  const int N = P.N;
-  auto at = [&](int i1, int i2, int i3) { return V[((size_t)i1 * N + i2) * N + i3]; };
+                                       int k, double2 &v, double2 &v2) {
+  const int N = P.N, p = g.p_lo + k;
+  auto at = [&](int i1, int i2, int i3) { return V[(i1 * N + i2) * N + i3]; };
   if (LEFT) {
     // every index is in the box for valid rows and k
-    const int p = g.p_lo + k;
+    const int r = g.row_lo + line;
     if (CH == CH_PP) {
-      const int a = g.row_lo + line;
-      v = cmul(at(a, g.x - a, p), w);
+      v = at(r, g.x - r, p);
     } else if (CH == CH_DPH) {
-      const int k1 = g.row_lo + line, t = g.x;
-      const double2 A = at(k1, p, k1 + t), C = at(k1, p, p - t);
-      v = cmul(make_double2(2.0 * A.x - C.x, 2.0 * A.y - C.y), w);
-      v2 = cmul(make_double2(-A.x, -A.y), w);
+      v = at(r, p, r + g.x);
+      v2 = at(r, p, p - g.x);
     } else {
-      const int k3 = g.row_lo + line;
-      v = cmul(at(p, k3 + g.x, k3), w);
+      v = at(p, r + g.x, r);
     }
   } else {
-    const int p = g.p_lo + k, c = line;
+    const int c = line;
     const double2 U = make_double2(P.U, 0.0);
     if (CH == CH_PP) {
       v = inbox(N, g.x - c) ? at(p, g.x - p, c) : U;
     } else if (CH == CH_DPH) {
-      const int t = g.x;
       // the fourth index of B and the third of D are both c - t
-      const bool in = inbox(N, c - t);
-      v = in ? at(p - t, c, p) : U;
-      v2 = in ? at(p - t, c, c - t) : U;
+      const bool in = inbox(N, c - g.x);
+      v = in ? at(p - g.x, c, p) : U;
+      v2 = in ? at(p - g.x, c, c - g.x) : U;
     } else {
       v = inbox(N, c + g.x) ? at(c, p + g.x, p) : U;
     }
@@ -137,79 +136,80 @@ __device__ __forceinline__ void gather(const PointDesc &P, const double2 *__rest
 
 template <int CH, bool LEFT>
 __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const X64Pt &x, int m, int oct,
-                                      double2 *sp) {
+                                      double2 *sw, unsigned *smax) {
   const int N = P.N;
   const Geom g = geom(CH, N, m);
   const int D = g.D, D16 = d16(D), nk = (CH == CH_DPH ? 2 : 1) * (D16 / KS);
   const int line0 = oct * PAN_LINES, nl = min(PAN_LINES, (LEFT ? D : N) - line0);
   if (nl <= 0) return;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, line = tid & 7, kstep = blockDim.x >> 3;
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
-  __shared__ unsigned smax[PAN_LINES];
-  double2 *sw = sp + (CH == CH_DPH ? 2 : 1) * D16 * PAN_PITCH;
   if (tid < PAN_LINES) smax[tid] = 0u;
   if (LEFT) {
     const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
     const double2 *L = CH == CH_PP ? P.Lpp + (size_t)m * N : P.Lph + (size_t)(CH == CH_DPH ? 2 * N - 2 - m : m) * N;
-    for (int k = tid; k < D; k += PAN_T) sw[k] = cscale(L[g.p_lo + k], sc);
+    for (int k = tid; k < D; k += blockDim.x) sw[k] = cscale(L[g.p_lo + k], sc);
   }
+  double2 v[PAN_U], v2[PAN_U];
+#pragma unroll
+  for (int u = 0; u < PAN_U; ++u) {
+    const int k = (tid >> 3) + u * kstep;
+    v[u] = v2[u] = make_double2(0.0, 0.0);
+    if (k < D && line < nl) gather<CH, LEFT>(P, V, g, line0 + line, k, v[u], v2[u]);
+  }
+  const uint4 pr = x.prod[(size_t)CH * (2 * N - 1) + m];
   __syncthreads();
-  // the right pp operand is contiguous along its lines, the others along k or
-  // along neither
-  constexpr bool LINE_FAST = CH == CH_PP && !LEFT;
-  const int line = LINE_FAST ? tid & 7 : tid >> 4, k0 = LINE_FAST ? tid >> 3 : tid & 15;
   unsigned um = 0u;
-  for (int kb = k0; kb < D16; kb += 64) {
-    double2 v[4], v2[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      v[u] = v2[u] = make_double2(0.0, 0.0);
-      const int k = kb + 16 * u;
-      if (k < D && line < nl)
-        gather<CH, LEFT>(P, V, g, line0 + line, k, LEFT ? sw[k] : make_double2(0.0, 0.0), v[u], v2[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int k = kb + 16 * u;
-      if (k < D16) {
-        sp[k * PAN_PITCH + line] = v[u];
-        um = max(um, mag(v[u]));
-        if (CH == CH_DPH) {
-          sp[(D16 + k) * PAN_PITCH + line] = v2[u];
-          um = max(um, mag(v2[u]));
-        }
+  for (int u = 0; u < PAN_U; ++u) {
+    const int k = (tid >> 3) + u * kstep;
+    if (LEFT && k < D) {
+      const double2 w = sw[k];
+      if (CH == CH_DPH) {
+        const double2 A = v[u], C = v2[u];
+        v[u] = cmul(make_double2(2.0 * A.x - C.x, 2.0 * A.y - C.y), w);
+        v2[u] = cmul(make_double2(-A.x, -A.y), w);
+      } else {
+        v[u] = cmul(v[u], w);
       }
     }
+    um = max(um, mag(v[u]));
+    if (CH == CH_DPH) um = max(um, mag(v2[u]));
   }
-  atomicMax(&smax[line], um);
+  um = max(um, __shfl_xor_sync(0xffffffffu, um, 8));
+  um = max(um, __shfl_xor_sync(0xffffffffu, um, 16));
+  if ((tid & 31) < PAN_LINES) atomicMax(&smax[line], um);
   __syncthreads();
-  const uint4 pr = x.prod[(size_t)CH * (2 * N - 1) + m];
-  const int tile = line0 / LINES, l0 = line0 & (LINES - 1);
-  const int ln = tid & 7;
-  const unsigned mx = smax[ln];
+  const int tile = line0 / LINES, l0 = (line0 & (LINES - 1)) + line;
+  const unsigned mx = smax[line];
   int e = line_exp(mx);
   if (tid < nl) {
     if (LEFT)
-      x.eL[(size_t)(pr.z + tile) * LINES + l0 + tid] = e;
+      x.eL[(size_t)(pr.z + tile) * LINES + l0] = e;
     else
-      x.eR[((size_t)(CH * (2 * N - 1) + m) * ((N + LINES - 1) / LINES) + tile) * LINES + l0 + tid] = e;
+      x.eR[((size_t)(CH * (2 * N - 1) + m) * ((N + LINES - 1) / LINES) + tile) * LINES + l0] = e;
     if ((mx >> 20) == 0x7ffu || e > E_LIM || e < -E_LIM) atomicOr(x.bad, 1);
   }
   e = max(-E_LIM, min(E_LIM, e));  // (a marked point's values are not used)
-  ulonglong2 *dst = (LEFT ? x.L + (size_t)(pr.x + tile * nk) * BLK : x.R + (size_t)(pr.y + tile * nk) * BLK) + l0 + ln;
-  if (ln < nl)
-    for (int k = tid >> 3; k < nk * KS; k += PAN_T / 8) {
-      const double2 v = sp[k * PAN_PITCH + ln];
-      dst[(size_t)k * LINES] = make_ulonglong2(to_fixed(v.x, e), to_fixed(v.y, e));
-    }
+  ulonglong2 *dst = (LEFT ? x.L + (size_t)(pr.x + tile * nk) * BLK : x.R + (size_t)(pr.y + tile * nk) * BLK) + l0;
+  if (line >= nl) return;
+#pragma unroll
+  for (int u = 0; u < PAN_U; ++u) {
+    const int k = (tid >> 3) + u * kstep;
+    if (k >= D16) break;
+    dst[(size_t)k * LINES] = make_ulonglong2(to_fixed(v[u].x, e), to_fixed(v[u].y, e));
+    if (CH == CH_DPH)
+      dst[(size_t)(D16 + k) * LINES] = make_ulonglong2(to_fixed(v2[u].x, e), to_fixed(v2[u].y, e));
+  }
 }
 
 // grid: (line octets of the left, then of the right operand; transfers;
 // point x channel)
-__global__ void __launch_bounds__(PAN_T) k_x64_panels(const PointDesc *__restrict__ pts,
+__global__ void __launch_bounds__(2 * FRG_MAX_N, 2) k_x64_panels(const PointDesc *__restrict__ pts,
                                                       const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
                                                       int p0, int chmask) {
-  extern __shared__ double2 sp[];
+  __shared__ double2 sw[FRG_MAX_N];
+  __shared__ unsigned smax[PAN_LINES];
   const int pi = p0 + blockIdx.z / 3, ch = blockIdx.z % 3;
   const RhsIO &o = io[pi];
   const X64Pt &x = xp[pi];
@@ -220,18 +220,18 @@ __global__ void __launch_bounds__(PAN_T) k_x64_panels(const PointDesc *__restric
   const int b = blockIdx.x;
   if (b < half) {
     if (ch == CH_PP)
-      panel<CH_PP, true>(P, o, x, m, b, sp);
+      panel<CH_PP, true>(P, o, x, m, b, sw, smax);
     else if (ch == CH_DPH)
-      panel<CH_DPH, true>(P, o, x, m, b, sp);
+      panel<CH_DPH, true>(P, o, x, m, b, sw, smax);
     else
-      panel<CH_XPH, true>(P, o, x, m, b, sp);
+      panel<CH_XPH, true>(P, o, x, m, b, sw, smax);
   } else {
     if (ch == CH_PP)
-      panel<CH_PP, false>(P, o, x, m, b - half, sp);
+      panel<CH_PP, false>(P, o, x, m, b - half, sw, smax);
     else if (ch == CH_DPH)
-      panel<CH_DPH, false>(P, o, x, m, b - half, sp);
+      panel<CH_DPH, false>(P, o, x, m, b - half, sw, smax);
     else
-      panel<CH_XPH, false>(P, o, x, m, b - half, sp);
+      panel<CH_XPH, false>(P, o, x, m, b - half, sw, smax);
   }
 }
 
@@ -243,11 +243,15 @@ __global__ void __launch_bounds__(PAN_T) k_x64_panels(const PointDesc *__restric
 // Accumulator g (digit weight 256^-g) takes the 64 columns from 64 g on, and
 // the B digits of one k-step lie one after the other, so that one instruction
 // multiplies digit i of A with several consecutive digits of B: N up to 224.
-// Roles: warps 0-7 epilogue, 8 MMA issue, 9 loader (bulk copies, two blocks per
-// k-step), 10-17 transform (fixed-point values -> FP16 digit tiles).
-// Bound by the tensor cores (28 products of K' = 32 per k-step; the operand
-// reads of those products from shared memory come close behind).
-constexpr int EPI_W = 8, MMA_W = 8, LOAD_W = 9, XF_W0 = 10, N_XF = 8;
+// Roles: warps 0-15 epilogue, 16 MMA issue, 17 loader (bulk copies, two blocks
+// per k-step), 18-25 transform (fixed-point values -> FP16 digit tiles).
+// Bound by the tensor cores (28 products of K' = 32 per k-step) for the k-steps
+// and by the drain of the accumulators between tiles: N = 128 172 us, of which
+// the tensor pipe is busy 58 %; without the drain 131 us.  The drain first joins
+// every entry in registers and frees TMEM (16 warps, 16 columns each), then
+// rounds and stores beside the next tile's products: 172 against 246 us with
+// eight warps that round as they read.
+constexpr int EPI_W = 16, MMA_W = 16, LOAD_W = 17, XF_W0 = 18, N_XF = 8;
 constexpr int THREADS = 32 * (XF_W0 + N_XF);
 constexpr int NRAW = 2, NOP = 2;
 constexpr int RAW_STAGE = 2 * BLK_BYTES;
@@ -258,9 +262,10 @@ constexpr int PLANE = 1024;
 constexpr int A_KC = 3 * PLANE, A_DIG = 2 * A_KC, A_BYTES = SL * A_DIG;
 constexpr int B_KC = SL * PLANE, B_PL = 2 * B_KC, B_BYTES = 2 * B_PL;
 constexpr int OP_STAGE = A_BYTES + B_BYTES;
-constexpr int EPI_COLS = 8;
-constexpr int EPI_BUF = 32 * EPI_COLS * 16;  // one warp pair's 32 rows x 8 columns
-constexpr int SMEM = 1024 + NOP * OP_STAGE + NRAW * RAW_STAGE + 4 * EPI_BUF + 256;
+constexpr int EPI_CPW = 64 / (EPI_W / 4);    // columns per epilogue warp
+constexpr int EPI_COLS = 4;
+constexpr int EPI_BUF = 32 * EPI_COLS * 16;  // one warp pair's 32 rows x 4 columns
+constexpr int SMEM = 1024 + NOP * OP_STAGE + NRAW * RAW_STAGE + EPI_W / 2 * EPI_BUF + 256;
 static_assert(SMEM <= 232448, "shared memory budget");
 
 struct Work {
@@ -375,24 +380,40 @@ __device__ __forceinline__ void store_digits(uint8_t *dst, const uint4 (&v)[8]) 
   store_digit<6, LEFT>(dst, v);
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, float &a, float &b) {
+  uint32_t r0, r1;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(taddr));
+  a = __uint_as_float(r0);
+  b = __uint_as_float(r1);
+}
+// The seven accumulators of one entry as one integer: the sum of the X_L X_R in
+// units of 2^57.  (The two last join in FP32 first, which loses less than
+// 2^-4 of the result's unit.)
+__device__ __forceinline__ long long join(const float (&d)[SL]) {
+  const long long hi = (long long)__float2int_rn(d[0]) * 65536 +
+                       ((long long)__float2int_rn(d[1]) * 256 + __float2int_rn(d[2]));
+  const long long lo = (long long)__float2int_rn(d[3]) * 32768 +
+                       ((long long)__float2int_rn(d[4]) * 128 + __float2int_rn(fmaf(d[6], 1.f / 512.f, 0.5f * d[5])));
+  return (hi << 23) + lo;
 }
 // s 2^e as FP64, rounded once, on the integer pipe (e within +-900: normal).
 __device__ __forceinline__ double scaled(long long s, int e) {
-  const unsigned long long sg = (unsigned long long)s & 0x8000000000000000ull;
-  unsigned long long a = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
-  if (a == 0ull) return 0.0;
-  const int lz = __clzll((long long)a);
-  a <<= lz;
+  const unsigned sg = (unsigned)(s >> 32) & 0x80000000u;
+  const unsigned long long a = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
+  unsigned h = (unsigned)(a >> 32), l = (unsigned)a;
+  if (h == 0u) {  // a cancelled sum: bring its bits up, or an exact zero
+    if (l == 0u) return 0.0;
+    h = l;
+    l = 0u;
+    e -= 32;
+  }
+  const int lz = __clz((int)h);
+  h = __funnelshift_l(l, h, lz);
+  l <<= lz;
   // 53 leading bits, the implicit one included (it carries into the exponent)
-  const unsigned long long mant = (a >> 11) + ((a >> 10) & 1ull);
-  return __longlong_as_double((long long)(((unsigned long long)(1023 + 63 - lz + e - 1) << 52) + mant | sg));
+  const unsigned long long mant = ((unsigned long long)(h >> 11) << 32 | __funnelshift_r(l, h, 11)) + (l >> 10 & 1u);
+  return __hiloint2double((int)(((unsigned)(1023 + 63 - 1 + e - lz) << 20) + (unsigned)(mant >> 32) | sg),
+                          (int)(unsigned)mant);
 }
 
 // Row pointer of local row rr in the channel's own layout (pp: natural, dph: X,
@@ -410,7 +431,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint8_t *ops = smem, *raws = ops + NOP * OP_STAGE, *epi = raws + NRAW * RAW_STAGE;
-  uint64_t *raw_full = reinterpret_cast<uint64_t *>(epi + 4 * EPI_BUF), *raw_empty = raw_full + NRAW;
+  uint64_t *raw_full = reinterpret_cast<uint64_t *>(epi + EPI_W / 2 * EPI_BUF), *raw_empty = raw_full + NRAW;
   uint64_t *op_full = raw_empty + NRAW, *op_empty = op_full + NOP, *tfull = op_empty + NOP, *tempty = tfull + 1;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tempty + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
@@ -528,55 +549,65 @@ __global__ void __launch_bounds__(THREADS, 1)
       __syncwarp();
     }
   } else {
-    // warps w and w ^ 2 (w & 4 the same) hold Re and Im of the same 32 rows and
-    // take 32 of the 64 columns, eight at a time, through a common staging buffer
+    // warp w reads TMEM lanes 32 (w % 4) on (Re of the rows 0-31 and 32-63, then
+    // their Im) and the columns 16 (w / 4) on.  First the accumulators of all its
+    // entries are joined in registers, so that the next tile's products can
+    // start; then the entries are rounded and stored, four columns at a time,
+    // through a buffer that warps w and w ^ 2 (Re and Im of the same rows) share.
     const int quarter = warp & 3, comp = quarter >> 1, pair = (quarter & 1) | (warp >> 2) << 1;
+    const int cb = EPI_CPW * (warp >> 2);
     uint8_t *buf = epi + pair * EPI_BUF;
-    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16) + cb;
+    const int rl = 32 * (quarter & 1);  // first row of this warp's half
     uint32_t use = 0;
     bool ok = true;
     for (int wi = w0; wi < w1 && ok; ++wi) {
       Tile t;
       const Work w = work[wi];
       if (!tile_of(pts, io, xp, w, t)) continue;
+      double2 *kN = static_cast<double2 *>(io[w.point].dgam);
+      const X64Pt &x = xp[w.point];
+      const int el = (t.r0 + rl + lane < t.D ? t.eL[rl + lane] : 0) + 57 - 2 * FIX;
+      const int er = lane < EPI_CPW && t.c0 + cb + lane < t.N ? t.eR[cb + lane] : 0;
       // both warps of a pair leave together when a wait gave up
       if (!(ok = pair_all(wwait(tfull, use & 1u, err, abort_flag), pair))) break;
       ++use;
       tc_after();
-      double2 *kN = static_cast<double2 *>(io[w.point].dgam);
-      const X64Pt &x = xp[w.point];
-      const int rl = 32 * (quarter & 1);  // first row of this warp's half
-      const int el = t.r0 + rl + lane < t.D ? t.eL[rl + lane] : 0;
-      for (int ci = 0; ci < 4; ++ci) {
-        const int cb = 32 * (warp >> 2) + ci * EPI_COLS;
-        float v[SL][EPI_COLS];
+      long long s[EPI_CPW];
+      // two columns at a time, the next two on their way meanwhile
+      float a[2][SL], b[2][SL];
 #pragma unroll
-        for (int g = 0; g < SL; ++g) tmem_ld8(tl + g * LINES + cb, v[g]);
+      for (int g = 0; g < SL; ++g) tmem_ld2(tl + g * LINES, a[0][g], b[0][g]);
+#pragma unroll
+      for (int c = 0; c < EPI_CPW; c += 2) {
+        const int f = (c >> 1) & 1;
         tmem_wait_ld();
-        if (ci == 3) {
-          tc_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty);
-        }
+        if (c + 2 < EPI_CPW) {
 #pragma unroll
-        for (int c = 0; c < EPI_COLS; ++c) {
-          const long long hi = (long long)__float2int_rn(v[2][c]) + (long long)__float2int_rn(v[1][c]) * 256 +
-                               (long long)__float2int_rn(v[0][c]) * 65536;
-          const long long lo = (long long)__float2int_rn(v[6][c]) + (long long)__float2int_rn(v[5][c]) * 256 +
-                               (long long)__float2int_rn(v[4][c]) * 65536 +
-                               (long long)__float2int_rn(v[3][c]) * 16777216;
-          const int er = t.c0 + cb + c < t.N ? t.eR[cb + c] : 0;
-          // sum of the integers X_L X_R in units of 2^57
-          const double r = scaled((hi << 23) + ((lo + 256) >> 9), el + er + 57 - 2 * FIX);
-          *reinterpret_cast<double *>(buf + lane * (EPI_COLS * 16) + ((c ^ (lane & 7)) << 4) + comp * 8) = r;
+          for (int g = 0; g < SL; ++g) tmem_ld2(tl + g * LINES + c + 2, a[f ^ 1][g], b[f ^ 1][g]);
         }
+        s[c] = join(a[f]);
+        s[c + 1] = join(b[f]);
+      }
+      tc_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty);
+      const bool live = t.c0 + cb < t.N;  // (uniform over the pair)
+#pragma unroll
+      for (int c0 = 0; c0 < EPI_CPW; c0 += EPI_COLS) {
+        if (!live) break;
+#pragma unroll
+        for (int c = 0; c < EPI_COLS; ++c)
+          *reinterpret_cast<double *>(buf + lane * (EPI_COLS * 16) + ((c ^ ((lane >> 1) & 3)) << 4) + comp * 8) =
+              scaled(s[c0 + c], el + __shfl_sync(0xffffffffu, er, c0 + c));
         asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
-        // each warp of the pair stores 16 of the 32 rows, 128 bytes a row
+        // each warp of the pair stores 16 of the 32 rows, 64 bytes a row
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int row = comp * 16 + (lane >> 3) + 4 * i, c = lane & 7;
-          const double2 z = *reinterpret_cast<const double2 *>(buf + row * (EPI_COLS * 16) + ((c ^ (row & 7)) << 4));
-          const int rr = t.r0 + rl + row, cc = t.c0 + cb + c;
+        for (int i = 0; i < 2; ++i) {
+          const int row = comp * 16 + (lane >> 2) + 8 * i, c = lane & 3;
+          const double2 z =
+              *reinterpret_cast<const double2 *>(buf + row * (EPI_COLS * 16) + ((c ^ ((row >> 1) & 3)) << 4));
+          const int rr = t.r0 + rl + row, cc = t.c0 + cb + c0 + c;
           if (rr < t.D && cc < t.N) out_row(w.ch, kN, x, t, rr)[cc] = z;
         }
         asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
@@ -758,9 +789,7 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
             cudaMalloc(&p->d_bad, sizeof(int) * n) == cudaSuccess &&
             cudaMemset(p->d_bad, 0, sizeof(int) * n) == cudaSuccess &&
             cudaFuncSetAttribute(x64::k_x64_products, cudaFuncAttributeMaxDynamicSharedMemorySize, x64::SMEM) ==
-                cudaSuccess &&
-            cudaFuncSetAttribute(x64::k_x64_panels, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)x64::panel_smem(FRG_MAX_N)) == cudaSuccess;
+                cudaSuccess;
   for (int i = 0; i < n && ok; ++i) {
     if (!p->N[i]) continue;
     X64Pt &x = p->h[i];
@@ -839,8 +868,8 @@ int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, in
       s = &p->one[point];
     }
     const int oct = (maxN + x64::PAN_LINES - 1) / x64::PAN_LINES, np = p1 - p0;
-    x64::k_x64_panels<<<dim3(2 * oct, 2 * maxN - 1, 3 * np), x64::PAN_T, x64::panel_smem(maxN), st>>>(d_pts, d_io, p->d_x,
-                                                                                                  p0, chmask);
+    x64::k_x64_panels<<<dim3(2 * oct, 2 * maxN - 1, 3 * np), x64::panel_threads(maxN), 0, st>>>(d_pts, d_io, p->d_x, p0,
+                                                                                             chmask);
     x64::k_x64_products<<<s->grid, x64::THREADS, x64::SMEM, st>>>(d_pts, d_io, p->d_x, s->d_work, s->d_start, p->d_err);
     FRG_COUNT(2);
     if (launch_x64_fallback(d_pts, d_io, p->d_x, p0, p1, chmask, st) != 0) return -3;
