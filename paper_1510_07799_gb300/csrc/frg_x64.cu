@@ -13,15 +13,19 @@
 //  * X is cut into seven digits of base 256 in [-128, 127] (one 64-bit add of
 //    128 in every byte, done when X is stored, makes its bytes the digits + 128),
 //    each an exact FP16 value.
-//  * Digit products i + j = g <= 6 (i, j counted from the leading digit) of all
-//    k go to accumulator g: 28 products.  Each is an integer of at most 2^14, and
+//  * Digit products i + j = g <= 7 (i, j counted from the leading digit) of all
+//    k go to accumulator g: 34 products.  Each is an integer of at most 2^14, and
 //    an FP32 accumulator adds integers exactly up to 2^24.  The products left
-//    out (i + j >= 7) are below 2^-56 of the lines' bounds per term.
-//  * The epilogue adds the seven accumulators as 64-bit integers and rounds the
-//    sum once to FP64, on the integer pipe.
+//    out (i + j >= 8) are below 2^-62 of the lines' bounds per term.  (Without
+//    those of i + j = 7, a fifth of the work, what is left out adds up to the
+//    rounding of a few FP64 additions where the bubble weights are sharply
+//    peaked: error 8.2e-16 against 7.4e-16 of the CUDA cores at N = 48 and
+//    Lambda = 0.02.)
+//  * The epilogue adds the accumulators as 64-bit integers and rounds the sum
+//    once to FP64, on the integer pipe.
 // So the sum over k itself is exact to 2^-53 of the lines' bounds, where a chain
-// of K fused multiply-adds rounds K times: measured error against 64-bit exact
-// sums below that of the CUDA-core path (tests/test_gpu_x64.py).
+// of K fused multiply-adds rounds K times: the error against extended precision
+// is below that of the CUDA cores (tests/test_gpu_x64.py).
 //
 // Three launches per rhs: k_x64_panels gathers, weights and converts the
 // operands into blocks of 16 k x 64 lines; k_x64_products multiplies them
@@ -47,6 +51,7 @@ namespace x64 {
 using namespace tc;
 
 constexpr int SL = 7;                       // digits per value
+constexpr int NACC = 8;                     // accumulators: digit products i + j = 0 .. 7
 constexpr int LINES = 64;                   // lines of an operand block (rows or columns of a tile)
 constexpr int KS = 16;                      // complex k per block
 constexpr int BLK = LINES * KS;             // elements (re, im) of a block: 16 KB
@@ -60,9 +65,8 @@ constexpr int E_LIM = 400;                  // line exponents the path accepts
 // -------------------------------------------------------------- panels ----
 // One block: eight lines of one operand of one product over its whole
 // contraction range.  Eight lanes take the eight lines at one k, so that the
-// blocks are written in 128-byte segments; a thread gathers (and weights: the
-// factor +-T Lambda goes into the bubble weights) all its k of one line into
-// registers, the block finds each line's largest magnitude, and the values leave
+// blocks are written in 128-byte segments; a thread gathers (and weights) all
+// its k of one line into registers, the block finds each line's largest magnitude, and the values leave
 // in fixed point.  Bound by the FP64 multiplications of the weights and by the
 // gathers (16-byte elements, one 32-byte sector each wherever the line and the
 // contraction index both stride through the vertex): 114 us at N = 128 for 302 MB
@@ -146,9 +150,8 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
   if (tid < PAN_LINES) smax[tid] = 0u;
   if (LEFT) {
-    const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
     const double2 *L = CH == CH_PP ? P.Lpp + (size_t)m * N : P.Lph + (size_t)(CH == CH_DPH ? 2 * N - 2 - m : m) * N;
-    for (int k = tid; k < D; k += blockDim.x) sw[k] = cscale(L[g.p_lo + k], sc);
+    for (int k = tid; k < D; k += blockDim.x) sw[k] = L[g.p_lo + k];
   }
   double2 v[PAN_U], v2[PAN_U];
 #pragma unroll
@@ -240,12 +243,13 @@ __global__ void __launch_bounds__(2 * FRG_MAX_N, 2) k_x64_panels(const PointDesc
 // the complex product on the left operand: accumulator rows 0-63 hold Re,
 // rows 64-127 Im of the product, from A = [Re a; Im a] against Re b and
 // A = [-Im a; Re a] against Im b, so three planes of the left digits are kept.
-// Accumulator g (digit weight 256^-g) takes the 64 columns from 64 g on, and
-// the B digits of one k-step lie one after the other, so that one instruction
-// multiplies digit i of A with several consecutive digits of B: N up to 224.
+// Accumulator g (digit weight 256^-g) takes the 64 columns from 64 g on (eight
+// fill TMEM), and the B digits of one k-step lie one after the other, so that
+// one instruction multiplies digit i of A with several consecutive digits of B:
+// N up to 256.
 // Roles: warps 0-15 epilogue, 16 MMA issue, 17 loader (bulk copies, two blocks
 // per k-step), 18-25 transform (fixed-point values -> FP16 digit tiles).
-// Bound by the tensor cores (28 products of K' = 32 per k-step) for the k-steps
+// Bound by the tensor cores (34 products of K' = 32 per k-step) for the k-steps
 // and by the drain of the accumulators between tiles: N = 128 172 us, of which
 // the tensor pipe is busy 58 %; without the drain 131 us.  The drain first joins
 // every entry in registers and frees TMEM (16 warps, 16 columns each), then
@@ -386,14 +390,14 @@ __device__ __forceinline__ void tmem_ld2(uint32_t taddr, float &a, float &b) {
   a = __uint_as_float(r0);
   b = __uint_as_float(r1);
 }
-// The seven accumulators of one entry as one integer: the sum of the X_L X_R in
-// units of 2^57.  (The two last join in FP32 first, which loses less than
-// 2^-4 of the result's unit.)
-__device__ __forceinline__ long long join(const float (&d)[SL]) {
+// The accumulators of one entry as one integer: the sum of the X_L X_R in units
+// of 2^57.  (The three last join in FP32 first, which loses less than 2^-3 of
+// the result's unit.)
+__device__ __forceinline__ long long join(const float (&d)[NACC]) {
   const long long hi = (long long)__float2int_rn(d[0]) * 65536 +
                        ((long long)__float2int_rn(d[1]) * 256 + __float2int_rn(d[2]));
   const long long lo = (long long)__float2int_rn(d[3]) * 32768 +
-                       ((long long)__float2int_rn(d[4]) * 128 + __float2int_rn(fmaf(d[6], 1.f / 512.f, 0.5f * d[5])));
+                       ((long long)__float2int_rn(d[4]) * 128 + __float2int_rn(fmaf(fmaf(d[7], 1.f / 256.f, d[6]), 1.f / 512.f, 0.5f * d[5])));
   return (hi << 23) + lo;
 }
 // s 2^e as FP64, rounded once, on the integer pipe (e within +-900: normal).
@@ -532,12 +536,22 @@ __global__ void __launch_bounds__(THREADS, 1)
             const uint32_t aq = a0 + (q == 0 ? PLANE : 0), bq = b0 + q * B_PL;
 #pragma unroll
             for (int i = 0; i < SL; ++i) {
-              const int cols = LINES * (SL - i), n1 = cols > 256 ? cols / 2 : cols;
+              const int digits = SL < NACC - i ? SL : NACC - i, cols = LINES * digits;
+              const int n1 = cols > 256 ? cols / 2 : cols;
               const uint64_t da = desc(aq + i * A_DIG, A_KC, 128);
               const uint32_t d = tmem + LINES * i;
-              mma_f16(d, da, desc(bq, B_KC, 128), idesc(n1), (kb | q | i) ? 1u : 0u);
-              if (cols > 256)  // the second half of the columns: n1 / 8 line groups further on
-                mma_f16(d + n1, da, desc(bq + n1 / 8 * 128, B_KC, 128), idesc(n1), (kb | q | i) ? 1u : 0u);
+              // the first k-step starts accumulators 0-6 with digit 0 of A, and
+              // accumulator 7 with the last 64 columns of digit 1
+              const uint32_t acc = (kb | q | i) ? 1u : 0u;
+              if (i == 1) {
+                mma_f16(d, da, desc(bq, B_KC, 128), idesc(192), 1u);
+                mma_f16(d + 192, da, desc(bq + 192 / 8 * 128, B_KC, 128), idesc(192), 1u);
+                mma_f16(d + 384, da, desc(bq + 384 / 8 * 128, B_KC, 128), idesc(64), (kb | q) ? 1u : 0u);
+              } else {
+                mma_f16(d, da, desc(bq, B_KC, 128), idesc(n1), acc);
+                if (cols > 256)  // the second half of the columns: n1 / 8 line groups further on
+                  mma_f16(d + n1, da, desc(bq + n1 / 8 * 128, B_KC, 128), idesc(n1), acc);
+              }
             }
           }
           mma_commit(&op_empty[s]);
@@ -574,20 +588,14 @@ __global__ void __launch_bounds__(THREADS, 1)
       ++use;
       tc_after();
       long long s[EPI_CPW];
-      // two columns at a time, the next two on their way meanwhile
-      float a[2][SL], b[2][SL];
-#pragma unroll
-      for (int g = 0; g < SL; ++g) tmem_ld2(tl + g * LINES, a[0][g], b[0][g]);
 #pragma unroll
       for (int c = 0; c < EPI_CPW; c += 2) {
-        const int f = (c >> 1) & 1;
-        tmem_wait_ld();
-        if (c + 2 < EPI_CPW) {
+        float a[NACC], b[NACC];
 #pragma unroll
-          for (int g = 0; g < SL; ++g) tmem_ld2(tl + g * LINES + c + 2, a[f ^ 1][g], b[f ^ 1][g]);
-        }
-        s[c] = join(a[f]);
-        s[c + 1] = join(b[f]);
+        for (int g = 0; g < NACC; ++g) tmem_ld2(tl + g * LINES + c, a[g], b[g]);
+        tmem_wait_ld();
+        s[c] = join(a);
+        s[c + 1] = join(b);
       }
       tc_before();
       __syncwarp();
@@ -621,8 +629,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // ------------------------------------------------------------- combine ----
-// dGamma = (pp + direct) + crossed, the enabled channels, into the natural
-// layout (the pp products are there already).  A thread takes four consecutive
+// dGamma = T Lambda ((direct - pp) - crossed), the enabled channels, into the
+// natural layout (the pp products are there already).  A thread takes four consecutive
 // i1 of one (i2, i3): 64 contiguous bytes of a W row; a warp covers 4 i2 (64
 // bytes of each X row) x 8 i3 (128 bytes of each natural row).
 __global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict__ pts,
@@ -638,6 +646,7 @@ __global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict
             i3 = 32 * blockIdx.x + 8 * ((t >> 5) & 3) + (t & 7);
   if (i1 >= N || i2 >= N || i3 >= N) return;
   double2 *out = static_cast<double2 *>(o.dgam);
+  const double sc = pts[pi].T * (*o.lam);
   const double2 z = make_double2(0.0, 0.0);
   double2 a[4], b[4], c[4];
 #pragma unroll
@@ -649,7 +658,9 @@ __global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict
   }
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    if (i1 + j < N) out[((size_t)(i1 + j) * N + i2) * N + i3] = cadd(cadd(a[j], b[j]), c[j]);
+    if (i1 + j < N)
+      out[((size_t)(i1 + j) * N + i2) * N + i3] =
+          make_double2(sc * ((b[j].x - a[j].x) - c[j].x), sc * ((b[j].y - a[j].y) - c[j].y));
 }
 }  // namespace x64
 

@@ -101,8 +101,9 @@ def extended_rhs(p, Lam, V, sig, idx):
 
 
 @pytest.mark.parametrize("N", [24, 48, 64])
+@pytest.mark.parametrize("Lam", [0.02, 0.2])
 @pytest.mark.parametrize("spread", [0.0, 3.0])
-def test_error_is_no_larger_than_the_cuda_cores(N, spread):
+def test_error_is_no_larger_than_the_cuda_cores(N, Lam, spread):
     """Root-mean-square error against extended precision, also for vertices
     whose entries spread over decades.  The sliced sum rounds once, the chain
     of fused multiply-adds at every term; both carry the rounding of the bubble
@@ -113,11 +114,11 @@ def test_error_is_no_larger_than_the_cuda_cores(N, spread):
         V = V * 10.0 ** np.random.default_rng(N).uniform(-spread, 0.0, V.shape)
     sig = inputs.random_sigma(N, seed=6)
     idx = np.random.default_rng(7).integers(0, N, (1500, 3))
-    ref = extended_rhs(p, 0.2, V, sig, idx)
+    ref = extended_rhs(p, Lam, V, sig, idx)
     at = (idx[:, 0], idx[:, 1], idx[:, 2])
     with frg.Context([p]) as ctx:
-        sliced = ctx_rhs(ctx, 0.2, V, sig)[0][at]
-    core = core_rhs(p, 0.2, V, sig)[0][at]
+        sliced = ctx_rhs(ctx, Lam, V, sig)[0][at]
+    core = core_rhs(p, Lam, V, sig)[0][at]
     rms = [float(np.sqrt(np.mean(np.abs(x - ref) ** 2) / np.mean(np.abs(ref) ** 2))) for x in (sliced, core)]
     assert rms[0] <= 1.25 * rms[1] and rms[0] < 2e-15, rms
 
