@@ -62,7 +62,7 @@ extern "C" {
  * error of one rhs below 1e-6 for FRG_3XTF32 and 5e-5 for FRG_BF16X3 on the
  * test inputs; whole flows within 1e-6 of the FP64 oracle).
  */
-#define FRG_FP64 0    /* FP64 throughout; grids of 24 frequencies on form the channel products from exact tcgen05 slices */
+#define FRG_FP64 0    /* FP64 throughout; grids of 28 frequencies on form the channel products from exact tcgen05 slices */
 #define FRG_3XTF32 1  /* split-TF32 (hi*hi + hi*lo + lo*hi) on tcgen05, FP32 accumulate */
 #define FRG_BF16X3 2  /* three BF16 slices, six products, on tcgen05, FP32 accumulate */
 
@@ -382,22 +382,16 @@ int frg_autotune(frg_ctx *ctx, frg_tune *out);
  * reading d_gamma (N^3 complex128) and d_sigma (N complex128, may be NULL) and
  * writing d_dgamma and d_dsigma, all device pointers on the current device,
  * asynchronously on cuda_stream (a cudaStream_t, NULL for the legacy stream).
- * It calls no cudaMalloc, cudaFree or other allocating routine: its whole
- * workspace is one file-scope device array of about 290 KB that every GPU
- * which loads this library holds until the process exits.
- *  - Limit: N_f <= FRG_NOALLOC_MAX_N (even, >= 2); larger sizes, T <= 0,
- *    Delta <= 0, Lambda <= 0, non-finite parameters, NULL output pointers, or
- *    a channel_mask with FRG_TAILS, FRG_REVERSAL, FRG_NO_REVERSAL or
- *    FRG_CROSSING (anything above FRG_CH_ALL) return FRG_EINVAL without
- *    touching the device.
- *  - The first call on a device looks up the array's device address
- *    (cudaGetSymbolAddress) and caches it with the device's current context;
- *    the first call after that context changed (cudaDeviceReset, or another
- *    context made current) looks it up again.  Make such a first call before
- *    any stream capture on that device.
- *  - Every call on a device shares the array and leaves its contents behind;
- *    each call rewrites everything it reads.  Calls that overlap on the GPU
- *    (for example on two streams) race on the array: serialise them.
+ * It calls no cudaMalloc, cudaFree or other allocating routine and keeps no
+ * device memory: one launch, whose parameters travel by value and whose
+ * workspace is the shared memory of its blocks.
+ *  - Limit: N_f <= FRG_NOALLOC_MAX_N (even, >= 2; the shared memory of a block);
+ *    larger sizes, T <= 0, Delta <= 0, Lambda <= 0, non-finite parameters, NULL
+ *    output pointers, or a channel_mask with FRG_TAILS, FRG_REVERSAL,
+ *    FRG_NO_REVERSAL or FRG_CROSSING (anything above FRG_CH_ALL) return
+ *    FRG_EINVAL without touching the device.
+ *  - Calls share nothing, so they may overlap (on several streams or threads)
+ *    as long as their outputs do not.
  * Returns FRG_OK, FRG_EINVAL or FRG_ECUDA (launch failure).
  */
 #define FRG_NOALLOC_MAX_N 64

@@ -16,6 +16,7 @@
 #include "frg_layout.cuh"
 #include "frg_lblock.cuh"
 #include "frg_misc.cuh"
+#include "frg_small.cuh"
 #include "frg_tc.cuh"
 #include "frg_x64.cuh"
 
@@ -185,6 +186,11 @@ void build_work(int ch, int pi, int N, std::vector<std::pair<int, WorkItem>> &ou
 
 }  // namespace
 
+// Whether an FP64 point's rhs is one launch of frg_small.cu.
+static bool small_point(const frg_ctx *ctx, int i) {
+  return !ctx->split && (ctx->mask & 7) && ctx->hpts[i].N < X64_MIN_N;
+}
+
 // ------------------------------------------------------------ rhs pipeline ----
 // ev (optional, 6 events): start, after the bubble weights and the self-energy
 // (one fused kernel), after the operand regather, after the channel products,
@@ -209,8 +215,15 @@ static int run_rhs(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cudaEvent
       CK(cudaEventRecord(ctx->ev_tails, ctx->sstream), "tails");
     }
   } else {
-    LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->split, ctx->mask, st),
-       "bubble weights and self-energy");
+    // FP64 points below X64_MIN_N take their whole rhs from one launch
+    const int p0 = point < 0 ? 0 : point, p1 = point < 0 ? ctx->n : point + 1;
+    bool small = false, large = false;
+    for (int i = p0; i < p1; ++i) (small_point(ctx, i) ? small : large) = true;
+    if (large)
+      LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->split, ctx->mask, st),
+         "bubble weights and self-energy");
+    if (small)
+      LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, st), "small rhs");
     if (tails) LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st), "tail sums");
   }
   if (ev) CK(cudaEventRecord(ev[1], st), "event");
@@ -229,8 +242,8 @@ static int run_rhs(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cudaEvent
     }
     if (ev) CK(cudaEventRecord(ev[2], st), "event");
     if (chmask) {
-      // the whole context's CUDA-core lists leave out the sliced points
-      if (point < 0 || !x64_has(ctx->x64, point))
+      // the whole context's CUDA-core lists leave out the small and the sliced points
+      if (point < 0 || (!x64_has(ctx->x64, point) && !small_point(ctx, point)))
         LK(launch_contract_fp64(ctx->d_pts, d_io, w, nw, chmask, st), "fp64 contraction");
       if (point < 0 ? ctx->x64 != nullptr : x64_has(ctx->x64, point))
         LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st), "sliced fp64 contraction");
@@ -668,7 +681,7 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
         build_work(ch, i, ctx->params[i].N_f, one);
         std::stable_sort(one.begin(), one.end(), [](auto &a, auto &b) { return a.first > b.first; });
         for (auto &x : one) per.push_back(x.second);
-        if (!x64_has(ctx->x64, i)) all.insert(all.end(), one.begin(), one.end());
+        if (!x64_has(ctx->x64, i) && !small_point(ctx, i)) all.insert(all.end(), one.begin(), one.end());
         ctx->work_off[ch].push_back((int)per.size());
       }
       std::stable_sort(all.begin(), all.end(), [](auto &a, auto &b) { return a.first > b.first; });

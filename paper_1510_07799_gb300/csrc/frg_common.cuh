@@ -329,7 +329,6 @@ struct StageArgs {
 // ------------------------------------------------- host-side launchers ----
 namespace frg {
 struct Workspace;
-int launch_bubble(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split, cudaStream_t st);
 int launch_contract_fp64(const PointDesc *d_pts, const RhsIO *d_io, const WorkItem *const d_work[3],
                          const int nwork[3], int mask, cudaStream_t st);
 // Propagators (16 frequencies per block), then both bubble-weight tables and
@@ -349,6 +348,4 @@ int launch_tail_sums(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
                      int parts = TAIL_WINDOW | TAIL_FINISH);
 // ... and their addition to the vertex derivative (after the contraction).
 int launch_add_tails(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, cudaStream_t st);
-// Self-energy rhs from FP64 input alone (after launch_bubble).
-int launch_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int mask, cudaStream_t st);
 }  // namespace frg

@@ -35,130 +35,6 @@ __global__ void k_bubble_gs(const PointDesc *__restrict__ pts, const RhsIO *__re
   P.S[i] = s;
 }
 
-// Lpp[s][p] = Lb(p, s-p), Lph[Q+N-1][p] = Lb(p, p+Q); grid (2N-1, 2, points).
-// Split paths also get the FP32 tables and the per-row maximum of |Re|, |Im|.
-__global__ void k_bubble_tables(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io) {
-  const int pi = blockIdx.z;
-  if (!io[pi].active) return;
-  const PointDesc &P = pts[pi];
-  const int N = P.N;
-  const int row = blockIdx.x;
-  if (row >= 2 * N - 1) return;
-  const int which = blockIdx.y;
-  float m = 0.f;
-  for (int p = threadIdx.x; p < N; p += blockDim.x) {
-    int q = which == 0 ? row - p : p + (row - (N - 1));
-    double2 v = make_double2(0.0, 0.0);
-    if (inbox(N, q)) {
-      double2 gp = P.G[p], sp = P.S[p], gq = P.G[q], sq = P.S[q];
-      v = cadd(cmul(sp, gq), cmul(gp, sq));
-    }
-    (which == 0 ? P.Lpp : P.Lph)[(size_t)row * N + p] = v;
-    if (P.Lpp32) {
-      const float2 f = make_float2((float)v.x, (float)v.y);
-      (which == 0 ? P.Lpp32 : P.Lph32)[(size_t)row * N + p] = f;
-      m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
-    }
-  }
-  if (P.kord) {
-    // order of the row's 16-wide k-chunks (starting at the first valid p) by
-    // increasing max |Lb|: the tensor-core accumulator loses up to an ulp of
-    // its running sum per addition, so small terms go first
-    __shared__ float am[FRG_MAX_N];
-    __shared__ float cmax[16];
-    const int Q = which == 0 ? 0 : row - (N - 1);
-    const int p_lo = which == 0 ? (row - (N - 1) > 0 ? row - (N - 1) : 0) : (Q < 0 ? -Q : 0);
-    const int D = which == 0 ? N - (row >= N - 1 ? row - (N - 1) : (N - 1) - row) : N - (Q >= 0 ? Q : -Q);
-    const int nch = (D + 15) / 16;
-    for (int p = threadIdx.x; p < N; p += blockDim.x) {
-      const float2 f = (which == 0 ? P.Lpp32 : P.Lph32)[(size_t)row * N + p];
-      am[p] = fmaxf(fabsf(f.x), fabsf(f.y));
-    }
-    __syncthreads();
-    if (threadIdx.x < nch) {
-      float mx = 0.f;
-      for (int j = 0; j < 16; ++j) {
-        const int p = p_lo + 16 * threadIdx.x + j;
-        if (p < p_lo + D) mx = fmaxf(mx, am[p]);
-      }
-      cmax[threadIdx.x] = mx;
-    }
-    __syncthreads();
-    if (threadIdx.x < 16) {
-      unsigned char *ord = P.kord + ((size_t)which * (2 * N - 1) + row) * 16;
-      if (threadIdx.x < nch) {
-        // rank of chunk c: chunks smaller than it, ties by index
-        const int c = threadIdx.x;
-        int rank = 0;
-        for (int j = 0; j < nch; ++j)
-          if (cmax[j] < cmax[c] || (cmax[j] == cmax[c] && j < c)) ++rank;
-        ord[rank] = (unsigned char)c;
-      }
-    }
-  }
-  if (P.Lmax) {
-    __shared__ float wm[32];
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float r = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = fmaxf(r, wm[w]);
-      P.Lmax[which * (2 * N - 1) + row] = r;
-    }
-  }
-}
-
-int launch_bubble(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split,
-                  cudaStream_t st) {
-  (void)split;
-  k_bubble_gs<<<dim3((maxN + GS_PER_BLOCK - 1) / GS_PER_BLOCK, n_points), GS_PER_BLOCK, 0, st>>>(d_pts, d_io);
-  FRG_COUNT(1);
-  dim3 g(2 * maxN - 1, 2, n_points);
-  k_bubble_tables<<<g, 128, 0, st>>>(d_pts, d_io);
-  FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
-}
-
-// ------------------------------------------------------------ self-energy ----
-// dSigma(w)/dl = L T sum_p S(p) [2 V(w,p,w) - V(w,p,p)]; one warp per w, FP64
-// input (the allocation-free entry point; the context paths use the fused
-// k_bubble_sigma).
-__global__ void k_sigma(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, int enabled) {
-  const int pi = blockIdx.y;
-  const RhsIO &o = io[pi];
-  if (!o.active) return;
-  const PointDesc &P = pts[pi];
-  const int N = P.N;
-  const int w = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (w >= N) return;
-  double2 acc = make_double2(0.0, 0.0);
-  if (enabled) {
-    for (int p = lane; p < N; p += 32) {
-      double2 a = vload<false>(o.gam, N, P.U, w, p, w);
-      double2 b = vload<false>(o.gam, N, P.U, w, p, p);
-      double2 t = make_double2(2.0 * a.x - b.x, 2.0 * a.y - b.y);
-      cfma(acc, P.S[p], t);
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-    }
-  }
-  if (lane == 0) {
-    const double f = (*o.lam) * P.T;
-    o.dsig[w] = make_double2(acc.x * f, acc.y * f);
-  }
-}
-
-int launch_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int mask, cudaStream_t st) {
-  dim3 g((maxN + 3) / 4, n_points);
-  k_sigma<<<g, 128, 0, st>>>(d_pts, d_io, (mask & 8) != 0);
-  FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
-}
-
 // ------------------------------------ bubble weights + self-energy, fused ----
 // Everything that needs only the propagators, in one launch after k_bubble_gs
 // (which forms G and S once per frequency: FP64 divisions are slow on this

@@ -1,0 +1,201 @@
+// frg_small.cu -- the whole FP64 right-hand side of a small grid in one launch.
+//
+// On a grid of some 16 frequencies every step of the rhs is latency: propagators,
+// bubble tables, three channel products and the self-energy were seven
+// dependent launches, and the products ran 32 x 32 tiles of which most was
+// padding, on 31 of the 152 SMs (the FP64 units do two multiply-adds per cycle
+// and SM, so a padded tile of 16 k takes 16 us).  Here a block takes the entries
+// of one k1 and R neighbouring k3, all k2.  It forms the propagators and the
+// bubble-weighted operands that its entries share in shared memory,
+//   W1[k2][p] = V(k1,k2,p) Lb(p,s-p)                         (pp)
+//   Wa[k3][p] = (2 V(k1,p,k3) - V(k1,p,p-t)) Lb(p,p-t), Wb[k3][p] = -V(k1,p,k3) Lb(p,p-t)   (direct)
+//   W3[Q][p]  = V(k1,p+Q,p) Lb(p,p+Q)                        (crossed)
+// and sums the four products of every entry over the valid p only: no padding,
+// no table in memory, one store per entry.  The last blocks form the
+// self-energy rhs.  Bound by the FP64 units: 16 multiply-adds per entry and p
+// plus the shared weights (R keeps their share below a third).
+// Measured (whole call of the allocation-free entry point): N = 16 100 -> 14 us.
+#include <cuda_runtime.h>
+
+#include "frg.h"
+#include "frg_common.cuh"
+#include "frg_small.cuh"
+
+namespace frg {
+namespace small {
+
+constexpr int T = 256;
+
+// k3 per block, and lanes that share an entry's p: enough blocks for the SMs on
+// the smallest grids, little repeated weight work on the larger ones.
+__host__ __device__ inline int rows(int N) { return N <= 24 ? 2 : N <= 40 ? 4 : 8; }
+__host__ __device__ inline int lanes(int N) {
+  int l = 8;
+  while (l > 1 && N * rows(N) * l > T) l >>= 1;
+  return l;
+}
+__host__ __device__ inline int pitch(int N) { return N + 1; }
+__host__ __device__ inline int blocks(int N) {
+  return N * ((N + rows(N) - 1) / rows(N)) + (N + T / 32 - 1) / (T / 32);
+}
+// G, S, W1, Wa, Wb, W3
+__host__ __device__ inline size_t smem(int N) {
+  const int R = rows(N);
+  return (size_t)(2 * N + (N + 2 * R + N + R - 1) * pitch(N)) * sizeof(double2);
+}
+
+__device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int b, double2 *sm) {
+  const int N = P.N, R = rows(N), PL = lanes(N), W = pitch(N), tid = threadIdx.x;
+  const int nb = (N + R - 1) / R;
+  if (b >= blocks(N)) return;
+  const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
+  double2 *G = sm, *S = G + N, *W1 = S + N, *Wa = W1 + N * W, *Wb = Wa + R * W, *W3 = Wb + R * W;
+  for (int i = tid; i < N; i += T) {
+    double2 g, s;
+    propagator_at(P, i, lam, o.sig ? o.sig[i] : make_double2(0.0, 0.0), g, s);
+    G[i] = g;
+    S[i] = s;
+  }
+  __syncthreads();
+  const double sc = P.T * lam;
+  if (b >= N * nb) {
+    // self-energy: one warp per frequency
+    const int w = (b - N * nb) * (T / 32) + (tid >> 5), lane = tid & 31;
+    if (w >= N) return;
+    double2 acc = make_double2(0.0, 0.0);
+    if (mask & FRG_CH_SIGMA)
+      for (int p = lane; p < N; p += 32) {
+        const double2 a = V[(w * N + p) * N + w], c = V[(w * N + p) * N + p];
+        cfma(acc, S[p], make_double2(2.0 * a.x - c.x, 2.0 * a.y - c.y));
+      }
+    for (int off = 16; off > 0; off >>= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+    }
+    if (lane == 0) o.dsig[w] = cscale(acc, sc);
+    return;
+  }
+  const int k1 = b / nb, c0 = (b % nb) * R;
+  const double2 U = make_double2(P.U, 0.0);
+  auto bub = [&](int p, int q) { return cadd(cmul(S[p], G[q]), cmul(G[p], S[q])); };
+  if (mask & FRG_CH_PP)
+    for (int e = tid; e < N * N; e += T) {
+      const int k2 = e / N, p = e - k2 * N, q = k1 + k2 - p;
+      if (inbox(N, q)) W1[k2 * W + p] = cmul(V[(k1 * N + k2) * N + p], bub(p, q));
+    }
+  if (mask & FRG_CH_DPH)
+    for (int e = tid; e < R * N; e += T) {
+      const int r = e / N, p = e - r * N, k3 = c0 + r, q = p - (k3 - k1);
+      if (k3 < N && inbox(N, q)) {
+        const double2 L = bub(p, q), A = V[(k1 * N + p) * N + k3], C = V[(k1 * N + p) * N + q];
+        Wa[r * W + p] = cmul(make_double2(2.0 * A.x - C.x, 2.0 * A.y - C.y), L);
+        Wb[r * W + p] = cmul(make_double2(-A.x, -A.y), L);
+      }
+    }
+  const int Q0 = -(c0 + R - 1);
+  if (mask & FRG_CH_XPH)
+    for (int e = tid; e < (N + R - 1) * N; e += T) {
+      const int d = e / N, p = e - d * N, Q = Q0 + d, q = p + Q;
+      if (inbox(N, q))
+        W3[d * W + p] = cmul(inbox(N, k1 + Q) ? V[(k1 * N + q) * N + p] : U, bub(p, q));
+    }
+  __syncthreads();
+  const int l = tid & (PL - 1), ne = N * R, step = T / PL;
+  double2 *out = static_cast<double2 *>(o.dgam);
+  for (int eb = 0; eb < ne; eb += step) {  // (the same trips in every thread: the fold below is warp-wide)
+    const int e = eb + tid / PL, k2 = e / R, r = e - k2 * R, k3 = c0 + r;
+    const bool on = e < ne && k3 < N;
+    const int s = k1 + k2, t = k3 - k1, Q = k2 - k3, k4 = s - k3;
+    const bool in4 = inbox(N, k4);
+    double2 pp = make_double2(0.0, 0.0), dd = pp, xx = pp;
+    if (on && (mask & FRG_CH_PP)) {
+      const double2 *w = W1 + k2 * W;
+      const int hi = min(N - 1, s);
+#pragma unroll 4
+      for (int p = max(0, s - (N - 1)) + l; p <= hi; p += PL)
+        cfma(pp, w[p], in4 ? V[(p * N + s - p) * N + k3] : U);
+    }
+    if (on && (mask & FRG_CH_DPH)) {
+      const double2 *wa = Wa + r * W, *wb = Wb + r * W;
+      const int hi = min(N - 1, N - 1 + t);
+#pragma unroll 2
+      for (int p = max(0, t) + l; p <= hi; p += PL) {
+        const int row = ((p - t) * N + k2) * N;
+        cfma(dd, wa[p], in4 ? V[row + p] : U);
+        cfma(dd, wb[p], in4 ? V[row + k4] : U);
+      }
+    }
+    if (on && (mask & FRG_CH_XPH)) {
+      const double2 *w = W3 + (Q - Q0) * W;
+      const int hi = min(N - 1, N - 1 - Q);
+#pragma unroll 4
+      for (int p = max(0, -Q) + l; p <= hi; p += PL) cfma(xx, w[p], V[(p * N + k2) * N + k3]);
+      // a non-finite sum again with the weight on the other factor, as the tiled
+      // products have it (which of infinity and NaN an infinite entry gives
+      // depends on that)
+      if (!isfinite(xx.x) || !isfinite(xx.y)) {
+        xx = make_double2(0.0, 0.0);
+        for (int p = max(0, -Q) + l; p <= hi; p += PL)
+          cfma(xx, cmul(V[(p * N + k2) * N + k3], bub(p, p + Q)), in4 ? V[(k1 * N + p + Q) * N + p] : U);
+      }
+    }
+    double2 v = cadd(cadd(cscale(pp, -sc), cscale(dd, sc)), cscale(xx, -sc));
+    for (int off = PL >> 1; off > 0; off >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
+    }
+    if (on && l == 0) out[(k1 * N + k2) * N + k3] = v;
+  }
+}
+
+__global__ void __launch_bounds__(T) k_rhs_small(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
+                                                 int n_below, int mask) {
+  extern __shared__ double2 sm[];
+  const PointDesc &P = pts[blockIdx.y];
+  const RhsIO &o = io[blockIdx.y];
+  if (!o.active || P.N >= n_below) return;
+  rhs(P, o, *o.lam, mask, blockIdx.x, sm);
+}
+
+__global__ void __launch_bounds__(T) k_rhs_small_value(const __grid_constant__ PointDesc P,
+                                                       const __grid_constant__ RhsIO o, double lam, int mask) {
+  extern __shared__ double2 sm[];
+  rhs(P, o, lam, mask, blockIdx.x, sm);
+}
+
+// (a host-side setting of the current device's context: set on every call, as
+// the context may have changed)
+template <typename K>
+bool room(K kernel, size_t bytes) {
+  return bytes <= 48 * 1024 ||
+         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
+}  // namespace small
+
+int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int n_below, int mask,
+                     cudaStream_t st) {
+  const int N = maxN < n_below ? maxN : n_below - 1;
+  // the shared weights and the block count both grow with N within a row count,
+  // and the row count's steps keep the larger N ahead; sizes between them are
+  // covered by the maxima over the range
+  size_t bytes = 0;
+  int blocks = 0;
+  for (int n = 2; n <= N; n += 2) {
+    bytes = small::smem(n) > bytes ? small::smem(n) : bytes;
+    blocks = small::blocks(n) > blocks ? small::blocks(n) : blocks;
+  }
+  if (!small::room(small::k_rhs_small, bytes)) return -3;
+  small::k_rhs_small<<<dim3(blocks, n_points), small::T, bytes, st>>>(d_pts, d_io, n_below, mask);
+  FRG_COUNT(1);
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
+int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int mask, cudaStream_t st) {
+  const size_t bytes = small::smem(P.N);
+  if (!small::room(small::k_rhs_small_value, bytes)) return -3;
+  small::k_rhs_small_value<<<small::blocks(P.N), small::T, bytes, st>>>(P, o, lam, mask);
+  FRG_COUNT(1);
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
+}  // namespace frg

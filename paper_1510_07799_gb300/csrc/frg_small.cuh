@@ -1,0 +1,12 @@
+// frg_small.cuh -- FP64 right-hand sides of small grids in one launch.
+#pragma once
+#include "frg_common.cuh"
+
+namespace frg {
+constexpr int SMALL_MAX_N = 64;  // limited by the block's shared memory
+// Vertex and self-energy rhs of every active point with N < n_below (<= 65).
+int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int n_below, int mask,
+                     cudaStream_t st);
+// The same for one point (N <= SMALL_MAX_N) given by value: no device memory.
+int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int mask, cudaStream_t st);
+}  // namespace frg

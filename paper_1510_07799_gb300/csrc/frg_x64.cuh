@@ -6,10 +6,10 @@
 
 namespace frg {
 
-// Smallest grid whose FP64 channel products take the sliced tensor-core path:
-// four dependent launches of a few microseconds each against the CUDA cores'
-// N^4 work.
-constexpr int X64_MIN_N = 24;
+// Smallest grid whose FP64 channel products take the sliced tensor-core path; the
+// ones below take the one-launch rhs (frg_small.cu).  Measured per rhs: N = 24 44
+// (sliced) against 29 us, N = 28 47 us either way, N = 32 48 against 57 us.
+constexpr int X64_MIN_N = 28;
 
 // Device-side operands of one point (frg_x64.cu).
 struct X64Pt {

@@ -1,4 +1,4 @@
-"""FP64 channel products by exact slices on the tensor cores (grids with N_f >= 24)
+"""FP64 channel products by exact slices on the tensor cores (grids with N_f >= 28)
 against the oracle and against extended-precision sums, at the edges of their
 tiles (64 rows and columns, 16 k), for values that cannot be sliced, and for
 contexts whose operands do not fit one workspace."""
@@ -40,7 +40,7 @@ def core_rhs(p, Lam, V, sig):
 
 
 @pytest.mark.parametrize("mask", [0xF, 0x1, 0x2, 0x4, 0x6])
-@pytest.mark.parametrize("N", [24, 30, 32, 48, 62, 66, 82, 96])
+@pytest.mark.parametrize("N", [28, 30, 32, 48, 62, 66, 82, 96])
 def test_rhs_matches_oracle_at_tile_edges(N, mask):
     p = params(N)
     V = inputs.random_vertex(N, p.U, seed=N + mask, crossing=False)
@@ -100,7 +100,7 @@ def extended_rhs(p, Lam, V, sig, idx):
     return np.array(out)
 
 
-@pytest.mark.parametrize("N", [24, 48, 64])
+@pytest.mark.parametrize("N", [28, 48, 64])
 @pytest.mark.parametrize("Lam", [0.02, 0.2])
 @pytest.mark.parametrize("spread", [0.0, 3.0])
 def test_error_is_no_larger_than_the_cuda_cores(N, Lam, spread):
