@@ -397,9 +397,7 @@ static int run_split_stage(frg_ctx *ctx, int s, bool err, bool fused, bool defer
                             chmask | (tails ? FRG_TAILS : 0), st, stage_grid(ctx), ctx->n, ctx->lb_want),
        "scatter-add and stage sum");
   else
-    LK(launch_stage(ctx->d_pts, ctx->d_ctl, seg(ctx), ctx->nseg, s, 1, io, st, stage_grid(ctx), ctx->n,
-                    ctx->lb_want),
-       "stage sum");
+    LK(launch_stage(ctx->d_pts, ctx->d_ctl, s, st, stage_grid(ctx), ctx->n, ctx->lb_want), "stage sum");
   CK(cudaEventRecord(ctx->ev_stage, st), "stage");
   CK(cudaStreamWaitEvent(ss, ctx->ev_stage, 0), "stage");
   // with the channel products and no tails, the contraction's epilogue warps
@@ -455,11 +453,11 @@ static int issue_step(frg_ctx *ctx) {
       // stage sums 2..6 that read them
       if ((rc = run_split_stage(ctx, s, s == 6, s >= 2, s <= 5))) return rc;
     } else {
-      LK(launch_stage(ctx->d_pts, ctx->d_ctl, seg(ctx), ctx->nseg, s, 0, ctx->d_io_stage, st), "stage sum");
+      LK(launch_stage_fp64(ctx->d_pts, ctx->d_ctl, s, ctx->d_io_stage, st, ctx->n, ctx->maxN), "stage sum");
       if ((rc = run_rhs(ctx, ctx->d_io_stage, -1))) return rc;
     }
   }
-  if (!ctx->split) LK(launch_error(ctx->d_pts, ctx->d_ctl, seg(ctx), ctx->nseg, 0, st), "error norm");
+  if (!ctx->split) LK(launch_error(ctx->d_pts, ctx->d_ctl, st, ctx->n, ctx->maxN), "error norm");
   LK(launch_controller(ctx->d_pts, ctx->d_ctl, ctx->n, st), "controller");
   return FRG_OK;
 }
@@ -1027,9 +1025,7 @@ int frg_autotune(frg_ctx *ctx, frg_tune *out) {
     if (!fs.ok) return fail(ctx, FRG_ECUDA, "flow stream ordering");
     cudaStream_t st = ctx->stream;
     // stage input of the current state of every point
-    LK(launch_stage(ctx->d_pts, ctx->d_ctl, seg(ctx), ctx->nseg, 0, 1, ctx->d_io_stage, st, stage_grid(ctx), ctx->n,
-                    ctx->lb_want),
-       "stage 0");
+    LK(launch_stage(ctx->d_pts, ctx->d_ctl, 0, st, stage_grid(ctx), ctx->n, ctx->lb_want), "stage 0");
     LK(launch_sigma_stage(ctx->d_pts, ctx->d_ctl, ctx->d_io_stage, 0, ctx->n, st, ctx->mask), "self-energy stage 0");
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0), "events");

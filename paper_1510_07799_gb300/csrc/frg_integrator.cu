@@ -10,6 +10,8 @@
 // real and imaginary parts of vertex and self-energy; accept iff err <= 1;
 // new step = h * clamp(0.9 err^{-1/5}, 0.2, 5) (rejection: lower clamp only);
 // the last step is clipped to end exactly at ln Lambda_f.
+#include <math_constants.h>
+
 #include "frg_common.cuh"
 #include "frg_integrator.cuh"
 #include "frg_split.cuh"
@@ -159,29 +161,40 @@ __global__ void k_finish_k1(Ctl *__restrict__ ctl, const RhsIO *__restrict__ io,
 }
 
 // Step begin: step-attempt budget, clipping of the last step, stage scales.
+// Eight lanes per point, one exponential each (3.6 us, against 7.2 us for
+// one thread's seven in turn).
 __global__ void k_prepare(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl, int n) {
-  const int pi = blockIdx.x * blockDim.x + threadIdx.x;
+  const int pi = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, s = threadIdx.x & 7;
   if (pi >= n) return;
   Ctl &c = ctl[pi];
-  if (c.done) return;
   const PointDesc &P = pts[pi];
-  if (c.steps >= P.max_steps) {
-    c.status = -5;
-    c.done = 1;
+  const unsigned grp = 0xffu << (threadIdx.x & 24);  // the point's lanes
+  const bool done = c.done, out = c.steps >= P.max_steps;
+  const double t = c.t, l_end = P.l_end;
+  double h = c.h;
+  // l decreases towards l_end (direction -1)
+  const bool last = -(t + h - l_end) >= 0.0;
+  if (last) h = l_end - t;
+  __syncwarp(grp);  // every lane has read the state
+  if (done) return;
+  if (out) {
+    if (s == 0) {
+      c.status = -5;
+      c.done = 1;
+    }
     return;
   }
-  c.steps++;
-  c.last = 0;
-  // l decreases towards l_end (direction -1)
-  if (-(c.t + c.h - P.l_end) >= 0.0) {
-    c.h = P.l_end - c.t;
-    c.last = 1;
+  if (s < 7) {
+    c.lam_stage[s] = exp(t + dC[s] * h);
+  } else {
+    c.steps++;
+    c.last = last;
+    c.h = h;
+    c.errbits = 0ull;
+    c.nonfinite = 0;
+    c.ymax_acc = 0ull;
+    c.smax_acc = 0ull;
   }
-  for (int s = 0; s < 7; ++s) c.lam_stage[s] = exp(c.t + dC[s] * c.h);
-  c.errbits = 0ull;
-  c.nonfinite = 0;
-  c.ymax_acc = 0ull;
-  c.smax_acc = 0ull;
 }
 
 // Block-wide max of a non-negative float, folded into *dst (float bits).
@@ -200,42 +213,61 @@ __device__ __forceinline__ void block_max_to(float v, unsigned *dst) {
 
 // ---------------------------------------------------------- stage sums ----
 // Y_s = y + h sum_{j<s} a_sj k_j, FP64 path.  Stage 6 (the seventh) is the
-// fifth-order candidate, kept as ynew.  (The split paths use k_stage_split.)
-__global__ void __launch_bounds__(256) k_stage(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl,
-                                               SegTable seg, int s, RhsIO *__restrict__ io) {
-  const int b = blockIdx.x;
-  const int pi = seg.point[b];
+// fifth-order candidate, kept as ynew; it also leaves the partial error sum
+// sum_{j != 7} E_j k_j in the place of k2, which nothing reads any more (its
+// fifth-order and error weights are zero).  (The split paths use k_stage_split.)
+// One element per thread, all of its loads in flight together: bound by the
+// FP64 units (2 (s + 1) multiply-adds per element, 22 for the seventh stage).
+// Measured at N = 64: 6-11 us per stage and 16 us for the seventh, against 13-25
+// us with eight elements per thread in turn on 129 blocks; N = 16 5 against
+// 12-25 us.
+constexpr int ST_T = 256;
+template <int S>
+__global__ void __launch_bounds__(ST_T) k_stage(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl,
+                                                RhsIO *__restrict__ io) {
+  const int pi = blockIdx.y;
+  const PointDesc &P = pts[pi];
   // the first block of the point also writes the stage's rhs IO record
-  if (io && seg.base[b] == 0 && threadIdx.x == 0) write_stage_io(pts[pi], ctl[pi], io + pi, s, 0);
+  if (blockIdx.x == 0 && threadIdx.x == 0) write_stage_io(P, ctl[pi], io + pi, S, 0);
   const Ctl &c = ctl[pi];
   if (c.done) return;
-  const PointDesc &P = pts[pi];
   const int n3 = P.n3, n = n3 + P.N;
-  const int base = seg.base[b];
+  const int i = blockIdx.x * ST_T + threadIdx.x;
+  if (i >= n) return;
   const double h = c.h;
-  const double2 *y = P.ybuf[c.yslot];
-  double2 *ynew = P.ybuf[c.yslot ^ 1];
-  double a[6];
+  const int ys = c.yslot;
+  double2 k[S];
 #pragma unroll
-  for (int j = 0; j < 6; ++j) a[j] = dA[s][j];
-  for (int e = threadIdx.x; e < SEG_ELEMS; e += blockDim.x) {
-    const int i = base + e;
-    if (i >= n) break;
-    double2 acc = make_double2(0.0, 0.0);
+  for (int j = 0; j < S; ++j) {
+    if (S == 6 && j == 1) continue;  // the fifth-order weight of k2 is zero: no read
+    const int kj = c.kslot[j];
+    k[j] = i < n3 ? static_cast<const double2 *>(P.kG[kj])[i] : P.kS[kj][i - n3];
+  }
+  const double2 yi = P.ybuf[ys][i];
+  double2 acc = make_double2(0.0, 0.0);
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      if (j < s) {
-        const double2 k = i < n3 ? static_cast<const double2 *>(P.kG[c.kslot[j]])[i] : P.kS[c.kslot[j]][i - n3];
-        acc.x += a[j] * k.x;
-        acc.y += a[j] * k.y;
-      }
+  for (int j = 0; j < S; ++j) {
+    if (S == 6 && j == 1) continue;
+    acc.x += dA[S][j] * k[j].x;
+    acc.y += dA[S][j] * k[j].y;
+  }
+  const double2 Y = make_double2(yi.x + h * acc.x, yi.y + h * acc.y);
+  if (S < 6) {
+    P.Y64[i] = Y;
+  } else {
+    P.ybuf[ys ^ 1][i] = Y;
+    double2 e = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+      if (j == 1) continue;
+      e.x += dE[j] * k[j].x;
+      e.y += dE[j] * k[j].y;
     }
-    const double2 yi = y[i];
-    const double2 Y = make_double2(yi.x + h * acc.x, yi.y + h * acc.y);
-    if (s < 6)
-      P.Y64[i] = Y;
+    const int k2 = c.kslot[1];
+    if (i < n3)
+      static_cast<double2 *>(P.kG[k2])[i] = e;
     else
-      ynew[i] = Y;
+      P.kS[k2][i - n3] = e;
   }
 }
 
@@ -468,59 +500,67 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long *addr, doub
 }
 
 // Error norm of the FP64 path (the split paths complete theirs in the scatter-add
-// of the seventh rhs, k_combine in frg_layout.cu).
-__global__ void __launch_bounds__(256) k_error(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl,
-                                               SegTable seg) {
-  const int b = blockIdx.x;
-  const int pi = seg.point[b];
+// of the seventh rhs, k_combine in frg_layout.cu): e = h (e' + E_7 k7) with the
+// partial sum e' of the seventh stage.  The FP64 division of the scaled error is
+// what costs on this part, and only the largest ratio matters: a ratio in FP32
+// finds the entries within 2^-16 of the block's largest, and those alone are
+// divided in FP64 (the maximum is the same, bit for bit).  Measured at N = 64:
+// 15 us, against 36 us for summing all stages and dividing every entry.
+__device__ __forceinline__ double maxabs(double a, double b) {
+  const long long x = __double_as_longlong(a) & 0x7fffffffffffffffll, y = __double_as_longlong(b) & 0x7fffffffffffffffll;
+  return __longlong_as_double(x > y ? x : y);
+}
+constexpr int ERR_T = 512;
+__global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl) {
+  const int pi = blockIdx.y;
   Ctl &c = ctl[pi];
   if (c.done) return;
   const PointDesc &P = pts[pi];
   const int n3 = P.n3, n = n3 + P.N;
-  const int base = seg.base[b];
-  const double h = c.h, rtol = P.rtol, atol = P.atol;
-  const double2 *y = P.ybuf[c.yslot];
-  const double2 *yn = P.ybuf[c.yslot ^ 1];
-  double emax = 0.0;
+  if (blockIdx.x * ERR_T >= n) return;
+  const int i = blockIdx.x * ERR_T + threadIdx.x;
+  __shared__ unsigned wmax[ERR_T / 32];
+  __shared__ unsigned long long emax;
+  if (threadIdx.x == 0) emax = 0ull;
+  const double h = c.h;
+  double2 acc = make_double2(0.0, 0.0), yi = acc, yni = acc;
   int bad = 0;
-  for (int e = threadIdx.x; e < SEG_ELEMS; e += blockDim.x) {
-    const int i = base + e;
-    if (i >= n) break;
-    double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-    for (int j = 0; j < 7; ++j) {
-      const double2 k = i < n3 ? static_cast<const double2 *>(P.kG[c.kslot[j]])[i] : P.kS[c.kslot[j]][i - n3];
-      acc.x += dE[j] * k.x;
-      acc.y += dE[j] * k.y;
-    }
-    const double2 yi = y[i], yni = yn[i];
-    const double rx = fabs(h * acc.x) / (atol + rtol * fmax(fabs(yi.x), fabs(yni.x)));
-    const double ry = fabs(h * acc.y) / (atol + rtol * fmax(fabs(yi.y), fabs(yni.y)));
-    if (!isfinite(rx) || !isfinite(ry) || !isfinite(yni.x) || !isfinite(yni.y)) bad = 1;
-    else emax = fmax(emax, fmax(rx, ry));
+  float rx = 0.f, ry = 0.f;
+  const bool on = i < n;
+  if (on) {
+    const int k2 = c.kslot[1], k7 = c.kslot[6];
+    acc = i < n3 ? static_cast<const double2 *>(P.kG[k2])[i] : P.kS[k2][i - n3];
+    const double2 k = i < n3 ? static_cast<const double2 *>(P.kG[k7])[i] : P.kS[k7][i - n3];
+    yi = P.ybuf[c.yslot][i];
+    yni = P.ybuf[c.yslot ^ 1][i];
+    acc.x += dE[6] * k.x;
+    acc.y += dE[6] * k.y;
+    bad = !isfinite(yni.x) || !isfinite(yni.y);
+    const float hf = fabsf(d2f(h)), at = d2f(P.atol), rt = d2f(P.rtol);
+    const float fx = fabsf(d2f(acc.x)), fy = fabsf(d2f(acc.y));
+    rx = hf * fx / (at + rt * d2f(maxabs(yi.x, yni.x)));
+    ry = hf * fy / (at + rt * d2f(maxabs(yi.y, yni.y)));
+    // a sum that FP32 flushes to zero has no FP32 ratio
+    if ((fx == 0.f && acc.x != 0.0) || (fy == 0.f && acc.y != 0.0)) rx = CUDART_INF_F;
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, off));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, off);
-  }
-  __shared__ double wmax[8];
-  __shared__ int wbad[8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    wmax[wid] = emax;
-    wbad[wid] = bad;
-  }
+  // (bits of non-negative floats order as integers, a NaN above infinity)
+  const unsigned bx = __float_as_uint(rx) & 0x7fffffffu, by = __float_as_uint(ry) & 0x7fffffffu;
+  unsigned m = __reduce_max_sync(0xffffffffu, max(bx, by));
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = 0.0;
-    int bb = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      m = fmax(m, wmax[w]);
-      bb |= wbad[w];
-    }
-    atomic_max_nonneg(&c.errbits, m);
-    if (bb) atomicOr(&c.nonfinite, 1);
+  m = 0u;
+  for (int w = 0; w < ERR_T / 32; ++w) m = max(m, wmax[w]);
+  // 2^-16 below the maximum (a NaN or an infinity in FP32, or ratios near its
+  // smallest: every entry)
+  const unsigned cut = m >= 0x7f800000u || m < 0x01000000u ? 0u : m - 0x80u;
+  if (on && max(bx, by) >= cut) {
+    const double ex = fabs(h * acc.x) / (P.atol + P.rtol * maxabs(yi.x, yni.x));
+    const double ey = fabs(h * acc.y) / (P.atol + P.rtol * maxabs(yi.y, yni.y));
+    if (!isfinite(ex) || !isfinite(ey)) bad = 1;
+    else atomicMax(&emax, (unsigned long long)__double_as_longlong(fmax(ex, ey)));
   }
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&c.nonfinite, 1);
+  if (threadIdx.x == 0 && emax) atomicMax(&c.errbits, emax);
 }
 
 // ----------------------------------------------------------- controller ----
@@ -592,7 +632,7 @@ int launch_finish_k1(Ctl *d_ctl, const RhsIO *d_io, int n, cudaStream_t st) {
 }
 
 int launch_prepare(const PointDesc *d_pts, Ctl *d_ctl, int n, cudaStream_t st) {
-  k_prepare<<<(n + 127) / 128, 128, 0, st>>>(d_pts, d_ctl, n);
+  k_prepare<<<(8 * n + 127) / 128, 128, 0, st>>>(d_pts, d_ctl, n);
   FRG_COUNT(1);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -617,26 +657,37 @@ int stage_split_init() {
   return ok ? 0 : -3;
 }
 
-int launch_stage(const PointDesc *d_pts, Ctl *d_ctl, SegTable seg, int nblk, int s, int split, RhsIO *d_io,
-                 cudaStream_t st, int lb_grid, int n_points, int want) {
-  if (split) {
-    const dim3 g(lb_grid, n_points);
-    const int cv = step_carveout(n_points);
-    const Ctl *c = d_ctl;
-    cudaError_t e;
-    switch (s) {
-      case 0: e = launch_with_carveout(k_stage_split<0>, g, stage_threads<0>(), LB_SMEM, st, cv, d_pts, c, want); break;
-      case 1: e = launch_with_carveout(k_stage_split<1>, g, stage_threads<1>(), LB_SMEM, st, cv, d_pts, c, want); break;
-      case 2: e = launch_with_carveout(k_stage_split<2>, g, stage_threads<2>(), LB_SMEM, st, cv, d_pts, c, want); break;
-      case 3: e = launch_with_carveout(k_stage_split<3>, g, stage_threads<3>(), LB_SMEM, st, cv, d_pts, c, want); break;
-      case 4: e = launch_with_carveout(k_stage_split<4>, g, stage_threads<4>(), LB_SMEM, st, cv, d_pts, c, want); break;
-      case 5: e = launch_with_carveout(k_stage_split<5>, g, stage_threads<5>(), LB_SMEM, st, cv, d_pts, c, want); break;
-      default: e = launch_with_carveout(k_stage_split<6>, g, stage_threads<6>(), LB_SMEM, st, cv, d_pts, c, want); break;
-    }
-    if (e != cudaSuccess) return -3;
-  } else {
-    k_stage<<<nblk, 256, 0, st>>>(d_pts, d_ctl, seg, s, d_io);
+int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cudaStream_t st, int n_points,
+                      int maxN) {
+  const dim3 g((maxN * maxN * maxN + maxN + ST_T - 1) / ST_T, n_points);
+  switch (s) {
+    case 1: k_stage<1><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
+    case 2: k_stage<2><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
+    case 3: k_stage<3><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
+    case 4: k_stage<4><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
+    case 5: k_stage<5><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
+    case 6: k_stage<6><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
+    default: return -1;
   }
+  FRG_COUNT(1);
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
+int launch_stage(const PointDesc *d_pts, Ctl *d_ctl, int s, cudaStream_t st, int lb_grid, int n_points, int want) {
+  const dim3 g(lb_grid, n_points);
+  const int cv = step_carveout(n_points);
+  const Ctl *c = d_ctl;
+  cudaError_t e;
+  switch (s) {
+    case 0: e = launch_with_carveout(k_stage_split<0>, g, stage_threads<0>(), LB_SMEM, st, cv, d_pts, c, want); break;
+    case 1: e = launch_with_carveout(k_stage_split<1>, g, stage_threads<1>(), LB_SMEM, st, cv, d_pts, c, want); break;
+    case 2: e = launch_with_carveout(k_stage_split<2>, g, stage_threads<2>(), LB_SMEM, st, cv, d_pts, c, want); break;
+    case 3: e = launch_with_carveout(k_stage_split<3>, g, stage_threads<3>(), LB_SMEM, st, cv, d_pts, c, want); break;
+    case 4: e = launch_with_carveout(k_stage_split<4>, g, stage_threads<4>(), LB_SMEM, st, cv, d_pts, c, want); break;
+    case 5: e = launch_with_carveout(k_stage_split<5>, g, stage_threads<5>(), LB_SMEM, st, cv, d_pts, c, want); break;
+    default: e = launch_with_carveout(k_stage_split<6>, g, stage_threads<6>(), LB_SMEM, st, cv, d_pts, c, want); break;
+  }
+  if (e != cudaSuccess) return -3;
   FRG_COUNT(1);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -684,9 +735,8 @@ int launch_sigma_stage(const PointDesc *d_pts, Ctl *d_ctl, RhsIO *d_io, int s, i
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int launch_error(const PointDesc *d_pts, Ctl *d_ctl, SegTable seg, int nblk, int split, cudaStream_t st) {
-  (void)split;  // the split paths' error norm is part of their scatter-add (frg_layout.cu)
-  k_error<<<nblk, 256, 0, st>>>(d_pts, d_ctl, seg);
+int launch_error(const PointDesc *d_pts, Ctl *d_ctl, cudaStream_t st, int n_points, int maxN) {
+  k_error<<<dim3((maxN * maxN * maxN + maxN + ERR_T - 1) / ERR_T, n_points), ERR_T, 0, st>>>(d_pts, d_ctl);
   FRG_COUNT(1);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }

@@ -28,14 +28,15 @@ int launch_set_stage_io(const PointDesc *d_pts, Ctl *d_ctl, RhsIO *d_io, int sta
                         cudaStream_t st);
 int launch_finish_k1(Ctl *d_ctl, const RhsIO *d_io, int n, cudaStream_t st);
 int launch_prepare(const PointDesc *d_pts, Ctl *d_ctl, int n, cudaStream_t st);
-// Stage sum s of every point.  FP64 path: nblk segments of the table seg; with
-// d_io non-null the first block of each point also writes the stage's rhs IO
-// record (as launch_set_stage_io).  Split paths: the vertex part only, on a
-// grid of lb_grid x n_points layout blocks (frg_lblock.cuh; lb_grid = the
-// largest point's vertex blocks), also writing the W / X / Z copies in `want`;
+// FP64 path: stage sum s (1..6) of every point; the first block of each point
+// also writes the stage's rhs IO record (as launch_set_stage_io), and the seventh
+// stage leaves the partial error sum in the place of k2.
+int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cudaStream_t st, int n_points, int maxN);
+// Split paths: stage sum s of every point, the vertex part only, on a grid of
+// lb_grid x n_points layout blocks (frg_lblock.cuh; lb_grid = the largest
+// point's vertex blocks), also writing the W / X / Z copies in `want`;
 // launch_sigma_stage does the self-energy part and the IO record.
-int launch_stage(const PointDesc *d_pts, Ctl *d_ctl, SegTable seg, int nblk, int s, int split, RhsIO *d_io,
-                 cudaStream_t st, int lb_grid = 0, int n_points = 0, int want = 0);
+int launch_stage(const PointDesc *d_pts, Ctl *d_ctl, int s, cudaStream_t st, int lb_grid, int n_points, int want);
 // Split flows: the scatter-add of the rhs of stage s - 1 (channel bits and
 // FRG_TAILS of mask) fused with the vertex part of stage sum s (s = 2..6; rev:
 // the reversal reduction's canonical half and mirrored reads; vmax: keep the
@@ -49,7 +50,8 @@ int launch_sigma_stage(const PointDesc *d_pts, Ctl *d_ctl, RhsIO *d_io, int s, i
                        int mask);
 // Dynamic shared-memory limits of the split stage kernels (once per set-up).
 int stage_split_init();
-int launch_error(const PointDesc *d_pts, Ctl *d_ctl, SegTable seg, int nblk, int split, cudaStream_t st);
+// FP64 path's error norm of the step (after the seventh rhs).
+int launch_error(const PointDesc *d_pts, Ctl *d_ctl, cudaStream_t st, int n_points, int maxN);
 int launch_controller(const PointDesc *d_pts, Ctl *d_ctl, int n, cudaStream_t st);
 
 }  // namespace frg
