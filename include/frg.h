@@ -310,12 +310,14 @@ int frg_set_state(frg_ctx *ctx, int point, const void *d_gamma, const void *d_si
 int frg_stats(frg_ctx *ctx, frg_flow_stats *stats);
 
 /*
- * Diagnostics.  frg_rhs_timed evaluates exactly like frg_rhs and records CUDA
- * events on the context stream around its phases; ms[0..4] (host) receive the
- * durations of the bubble-weight (with the self-energy, which the same kernel
- * computes), operand-regather, channel-contraction and combine (scatter-add)
- * phases, and ms[4] the addition of the frequency-box tails (FRG_TAILS; 0
- * without them); 0 for a phase the path does not have.  Synchronises.
+ * Diagnostics.  frg_rhs_timed evaluates exactly like frg_rhs, its kernels in turn
+ * on the context stream, and records CUDA events around its phases; ms[0..4]
+ * (host) receive the durations of the bubble-weight, operand-regather,
+ * channel-contraction and combine (scatter-add) phases, and ms[4] the addition
+ * of the frequency-box tails on the FP64 path; 0 for a phase the path does not
+ * have.  The self-energy rhs is part of the contraction on the split paths (of
+ * the regather phase with FRG_TAILS), and of the first phase on the FP64 path.
+ * Synchronises.
  * frg_kernel_launches returns the number of kernels this library has launched
  * in the process so far.
  */

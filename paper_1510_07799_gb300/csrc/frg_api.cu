@@ -66,11 +66,7 @@ struct frg_ctx {
   // host-buffer entry point staging (per point, lazily)
   std::vector<double2 *> user_in, user_out;
   TcPlan *tc = nullptr;  // split-precision contraction plan
-  struct UserScratch {
-    double2 *s64 = nullptr;
-    float2 *kout = nullptr;
-  };
-  std::vector<UserScratch> user_split;
+  std::vector<float2 *> user_kout;  // stand-alone split evaluations: pp output, per point, lazily
   bool need_k1 = true;
   // flow driver: one DP5 step attempt of every point is captured once as a
   // CUDA graph and replayed on an internal stream, ordered after and before
@@ -192,43 +188,30 @@ static bool small_point(const frg_ctx *ctx, int i) {
 }
 
 // ------------------------------------------------------------ rhs pipeline ----
-// ev (optional, 6 events): start, after the bubble weights and the self-energy
-// (one fused kernel), after the operand regather, after the channel products,
-// after the combine; the last event follows the combine directly.
-static int run_rhs(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cudaEvent_t *ev = nullptr) {
+// FP64 path.  ev (optional, 6 events): start, after the bubble weights and the
+// self-energy (one fused kernel; the whole rhs of the small points), twice
+// after the channel products (no regather), and after the tails.
+static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cudaEvent_t *ev = nullptr,
+                        bool sig_in_place = false) {
   cudaStream_t st = ctx->stream;
   if (ev) CK(cudaEventRecord(ev[0], st), "event");
-  // untimed split evaluations overlap the bubble weights with the relayout
-  const bool fork = !ev && ctx->split && ctx->sstream;
   const bool tails = (ctx->mask & FRG_TAILS) != 0;
-  if (fork) {
-    CK(cudaEventRecord(ctx->ev_fork, st), "fork");
-    CK(cudaStreamWaitEvent(ctx->sstream, ctx->ev_fork, 0), "fork");
-    LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->split, ctx->mask, ctx->sstream),
-       "bubble weights and self-energy");
-    CK(cudaEventRecord(ctx->ev_join, ctx->sstream), "join");
-    // the tail constants are needed only after the contraction: they run on
-    // the side stream while the main stream regathers and contracts (the
-    // self-energy's is added to the self-energy rhs, which has run)
-    if (tails) {
-      LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ctx->sstream), "tail sums");
-      CK(cudaEventRecord(ctx->ev_tails, ctx->sstream), "tails");
-    }
-  } else {
-    // FP64 points below X64_MIN_N take their whole rhs from one launch
-    const int p0 = point < 0 ? 0 : point, p1 = point < 0 ? ctx->n : point + 1;
-    bool small = false, large = false;
-    for (int i = p0; i < p1; ++i) (small_point(ctx, i) ? small : large) = true;
-    if (large)
-      LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->split, ctx->mask, st),
-         "bubble weights and self-energy");
-    if (small)
-      LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, st), "small rhs");
-    if (tails) LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st), "tail sums");
-  }
-  if (ev) CK(cudaEventRecord(ev[1], st), "event");
   const int chmask = ctx->mask & 7;
-  if (!ctx->split) {
+  // points below X64_MIN_N take their whole rhs from one launch
+  const int p0 = point < 0 ? 0 : point, p1 = point < 0 ? ctx->n : point + 1;
+  bool small = false, large = false;
+  for (int i = p0; i < p1; ++i) (small_point(ctx, i) ? small : large) = true;
+  if (large)
+    LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 0, ctx->mask, st), "bubble weights and self-energy");
+  if (small)
+    LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, sig_in_place, st),
+       "small rhs");
+  if (tails) LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st), "tail sums");
+  if (ev) CK(cudaEventRecord(ev[1], st), "event");
+  if (ev) CK(cudaEventRecord(ev[2], st), "event");
+  if (!chmask) {
+    LK(launch_zero_vertex(ctx->d_pts, d_io, ctx->n, ctx->maxN, st), "zero vertex");
+  } else {
     const WorkItem *w[3];
     int nw[3];
     for (int ch = 0; ch < 3; ++ch) {
@@ -240,38 +223,83 @@ static int run_rhs(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cudaEvent
         nw[ch] = ctx->work_off[ch][point + 1] - ctx->work_off[ch][point];
       }
     }
-    if (ev) CK(cudaEventRecord(ev[2], st), "event");
-    if (chmask) {
-      // the whole context's CUDA-core lists leave out the small and the sliced points
-      if (point < 0 || (!x64_has(ctx->x64, point) && !small_point(ctx, point)))
-        LK(launch_contract_fp64(ctx->d_pts, d_io, w, nw, chmask, st), "fp64 contraction");
-      if (point < 0 ? ctx->x64 != nullptr : x64_has(ctx->x64, point))
-        LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st), "sliced fp64 contraction");
-    } else {
-      LK(launch_zero_vertex(ctx->d_pts, d_io, ctx->n, ctx->maxN, st), "zero vertex");
-    }
-    if (ev) CK(cudaEventRecord(ev[3], st), "event");
-  } else {
-    if (chmask) {
-      // the reversal reduction's transfers: flows while it is on, every call
-      // when the caller asserts the symmetry
-      const bool half = d_io == ctx->d_io_stage ? ctx->rev_on : ctx->rev_mode == 2;
-      // flow evaluations: the split stage kernels have written the layouts
-      LK(tc_run(ctx->tc, ctx->d_pts, d_io, point, chmask, st, ev ? ev[2] : nullptr, ev ? ev[3] : nullptr, ctx->n,
-                ctx->maxN, fork ? ctx->ev_join : nullptr, tails, (fork && tails) ? ctx->ev_tails : nullptr,
-                d_io == ctx->d_io_stage, half, false, ctx->cross),
-         "split contraction");
-    } else {
-      if (ev) CK(cudaEventRecord(ev[2], st), "event");
-      if (fork) CK(cudaStreamWaitEvent(st, ctx->ev_join, 0), "join");
-      LK(launch_zero_vertex(ctx->d_pts, d_io, ctx->n, ctx->maxN, st), "zero vertex");
-      if (ev) CK(cudaEventRecord(ev[3], st), "event");
-    }
+    // the whole context's CUDA-core lists leave out the small and the sliced points
+    if (point < 0 || (!x64_has(ctx->x64, point) && !small_point(ctx, point)))
+      LK(launch_contract_fp64(ctx->d_pts, d_io, w, nw, chmask, st), "fp64 contraction");
+    if (point < 0 ? ctx->x64 != nullptr : x64_has(ctx->x64, point))
+      LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st), "sliced fp64 contraction");
   }
-  // the split contraction's combine adds the tails itself
-  if (tails && !(ctx->split && chmask)) {
-    if (fork) CK(cudaStreamWaitEvent(st, ctx->ev_tails, 0), "tails");
-    LK(launch_add_tails(ctx->d_pts, d_io, ctx->n, ctx->maxN, st), "tails");
+  if (ev) CK(cudaEventRecord(ev[3], st), "event");
+  if (ev) CK(cudaEventRecord(ev[4], st), "event");
+  if (tails) LK(launch_add_tails(ctx->d_pts, d_io, ctx->n, ctx->maxN, st), "tails");
+  if (ev) CK(cudaEventRecord(ev[5], st), "event");
+  return FRG_OK;
+}
+
+// Split paths.  gam (a stand-alone evaluation of one point): the FP64 vertex,
+// regathered here into the operand copies; null: a flow's stage input, whose
+// copies the stage kernels have written.  Side stream: the propagators and the
+// bubble weights (they need the self-energy input alone) beside the regather,
+// then the tail constants.  The contraction's epilogue warps form the self-energy
+// rhs, except with the tails or without channel products: a kernel on the side
+// stream after the regather, then the tails' last kernel, which adds the
+// self-energy's constant to it.  ev (optional, 6 events; everything in turn on
+// the main stream): start, after the bubble weights, after the regather (and
+// such a self-energy kernel), after the channel products (with the self-energy
+// rhs otherwise), after the combine, and the same again.
+static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, const double2 *gam,
+                         cudaEvent_t *ev = nullptr) {
+  cudaStream_t st = ctx->stream, ss = ev ? st : ctx->sstream;
+  const bool fork = !ev, tails = (ctx->mask & FRG_TAILS) != 0;
+  const int chmask = ctx->mask & 7;
+  // the reversal reduction's transfers: flows while it is on, every call when
+  // the caller asserts the symmetry
+  const bool half = gam ? ctx->rev_mode == 2 : ctx->rev_on;
+  if (ev) CK(cudaEventRecord(ev[0], st), "event");
+  if (fork) {
+    CK(cudaEventRecord(ctx->ev_fork, st), "fork");
+    CK(cudaStreamWaitEvent(ss, ctx->ev_fork, 0), "fork");
+  }
+  LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES), "bubble weights");
+  if (fork) CK(cudaEventRecord(ctx->ev_join, ss), "join");
+  if (tails)
+    LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ss, TAIL_WINDOW), "tail sums");
+  if (ev) CK(cudaEventRecord(ev[1], st), "event");
+  if (gam)
+    LK(launch_relayout(ctx->d_pts + point, gam, ctx->hpts[point].N, ctx->lb_want, ctx->precision == FRG_BF16X3, st),
+       "regather");
+  const bool sig_in_tc = chmask && !tails;
+  if (!sig_in_tc) {
+    if (fork) {
+      CK(cudaEventRecord(ctx->ev_stage, st), "regather");
+      CK(cudaStreamWaitEvent(ss, ctx->ev_stage, 0), "regather");
+    }
+    LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_SIGMA), "self-energy rhs");
+    if (tails)
+      LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ss, TAIL_FINISH), "tail constants");
+    if (fork) CK(cudaEventRecord(ctx->ev_sig, ss), "self-energy");
+  }
+  if (ev) CK(cudaEventRecord(ev[2], st), "event");
+  if (chmask) {
+    TcRun r;
+    r.ev_contract = ev ? ev[3] : nullptr;
+    r.wait_before = fork ? ctx->ev_join : nullptr;
+    r.wait_combine = fork && !sig_in_tc ? ctx->ev_sig : nullptr;
+    r.tails = tails;
+    r.half = half;
+    r.canon = half && !gam;
+    r.out64 = gam != nullptr;
+    r.cross = ctx->cross;
+    r.sigma = sig_in_tc ? 1 | ((ctx->mask & 8) ? 2 : 0) : 0;
+    LK(tc_run(ctx->tc, ctx->d_pts, d_io, point, chmask, st, ctx->n, ctx->maxN, r), "split contraction");
+  } else {
+    // no vertex channel: the scatter-add writes the zero (or tail-only) vertex
+    // derivative
+    if (ev) CK(cudaEventRecord(ev[3], st), "event");
+    if (fork) CK(cudaStreamWaitEvent(st, ctx->ev_sig, 0), "self-energy");
+    const int cmask = (tails ? FRG_TAILS : 0) | (half ? FRG_REVERSAL : 0);
+    LK(launch_combine(ctx->d_pts, d_io, ctx->n, ctx->maxN, cmask, st, false, half && !gam, gam != nullptr),
+       "scatter-add");
   }
   if (ev) CK(cudaEventRecord(ev[4], st), "event");
   if (ev) CK(cudaEventRecord(ev[5], st), "event");
@@ -415,10 +443,16 @@ static int run_split_stage(frg_ctx *ctx, int s, bool err, bool fused, bool defer
   }
   CK(cudaEventRecord(ctx->ev_sig, ss), "self-energy");
   if (chmask) {
-    LK(tc_run(ctx->tc, ctx->d_pts, io, -1, chmask, st, nullptr, nullptr, ctx->n, ctx->maxN, ctx->ev_join, tails,
-              ctx->ev_sig, true, ctx->rev_on, err, ctx->cross, !deferred,
-              sig_in_tc ? 1 | ((ctx->mask & 8) ? 2 : 0) : 0),
-       "split contraction");
+    TcRun r;
+    r.wait_before = ctx->ev_join;
+    r.wait_combine = ctx->ev_sig;
+    r.tails = tails;
+    r.half = r.canon = ctx->rev_on;
+    r.err = err;
+    r.cross = ctx->cross;
+    r.combine = !deferred;
+    r.sigma = sig_in_tc ? 1 | ((ctx->mask & 8) ? 2 : 0) : 0;
+    LK(tc_run(ctx->tc, ctx->d_pts, io, -1, chmask, st, ctx->n, ctx->maxN, r), "split contraction");
   } else if (!deferred) {
     // no vertex channel: the scatter-add writes the zero (or tail-only)
     // vertex derivative and, for k7, completes the error estimate
@@ -436,7 +470,7 @@ static int issue_k1(frg_ctx *ctx) {
     if ((rc = run_split_stage(ctx, 0, false, false, false))) return rc;
   } else {
     LK(launch_set_stage_io(ctx->d_pts, ctx->d_ctl, ctx->d_io_stage, 0, ctx->split, ctx->n, st), "stage io");
-    if ((rc = run_rhs(ctx, ctx->d_io_stage, -1))) return rc;
+    if ((rc = run_rhs_fp64(ctx, ctx->d_io_stage, -1))) return rc;
   }
   LK(launch_finish_k1(ctx->d_ctl, ctx->d_io_stage, ctx->n, st), "finish k1");
   return FRG_OK;
@@ -454,7 +488,7 @@ static int issue_step(frg_ctx *ctx) {
       if ((rc = run_split_stage(ctx, s, s == 6, s >= 2, s <= 5))) return rc;
     } else {
       LK(launch_stage_fp64(ctx->d_pts, ctx->d_ctl, s, ctx->d_io_stage, st, ctx->n, ctx->maxN), "stage sum");
-      if ((rc = run_rhs(ctx, ctx->d_io_stage, -1))) return rc;
+      if ((rc = run_rhs_fp64(ctx, ctx->d_io_stage, -1))) return rc;
     }
   }
   if (!ctx->split) LK(launch_error(ctx->d_pts, ctx->d_ctl, st, ctx->n, ctx->maxN), "error norm");
@@ -737,7 +771,7 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
   }
   ctx->user_in.assign(n_points, nullptr);
   ctx->user_out.assign(n_points, nullptr);
-  ctx->user_split.assign(n_points, frg_ctx::UserScratch());
+  ctx->user_kout.assign(n_points, nullptr);
   if (launch_init(ctx->d_pts, ctx->d_ctl, seg(ctx), ctx->nseg, n_points, ctx->stream) != 0) return bail(FRG_ECUDA);
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return bail(FRG_ECUDA);
   *out = ctx;
@@ -798,6 +832,9 @@ const char *frg_last_error(const frg_ctx *ctx) {
   return ctx->err.c_str();
 }
 
+// Whether the self-energy output overlaps the input (a derivative taken in place).
+static bool sigma_overlap(const RhsIO &o, int N) { return o.sig && o.sig < o.dsig + N && o.dsig < o.sig + N; }
+
 static int rhs_impl(frg_ctx *ctx, int point, double Lambda, const void *d_gamma, const void *d_sigma,
                     void *d_dgamma, void *d_dsigma, cudaEvent_t *ev) {
   if (!ctx) return FRG_EINVAL;
@@ -805,48 +842,28 @@ static int rhs_impl(frg_ctx *ctx, int point, double Lambda, const void *d_gamma,
   if (!(Lambda > 0.0) || !std::isfinite(Lambda)) return fail(ctx, FRG_EINVAL, "Lambda must be > 0");
   if (!d_gamma || !d_dgamma || !d_dsigma) return fail(ctx, FRG_EINVAL, "null buffer");
   DevGuard g(ctx->dev);
-  RhsIO o;
+  const PointDesc &P = ctx->hpts[point];
+  RhsIO o = {};
   o.gam = d_gamma;
   o.sig = static_cast<const double2 *>(d_sigma);
   o.dgam = d_dgamma;
   o.dsig = static_cast<double2 *>(d_dsigma);
-  o.lam = nullptr;
   o.active = 1;
-  o.out_f32 = 0;
-  o.canon = 0;
-  o.ctl = nullptr;
-  o.par = 0;
   if (!ctx->split) {
     LK(launch_set_user_io(ctx->d_io_user, ctx->d_ctl, ctx->n, point, o, Lambda, ctx->stream), "user io");
-    return run_rhs(ctx, ctx->d_io_user, point, ev);
+    return run_rhs_fp64(ctx, ctx->d_io_user, point, ev, sigma_overlap(o, P.N));
   }
-  // split path: convert the input to float pairs, evaluate into float2, widen.
-  // Scratch of its own so that a stand-alone call leaves the flow state intact.
-  const PointDesc &P = ctx->hpts[point];
-  // the stage input buffers (FP32 vertex and its layouts) are scratch between
-  // stages, and the contraction's tensor maps point at them
-  frg_ctx::UserScratch &u = ctx->user_split[point];
-  if (!u.kout) {
-    if (!(u.s64 = dalloc<double2>(ctx, P.N)) || !(u.kout = dalloc<float2>(ctx, P.n3)))
-      return fail(ctx, FRG_ENOMEM, "stand-alone rhs scratch");
-  }
-  LK(launch_split_input(P.Y32, u.s64, static_cast<const double2 *>(d_gamma), o.sig, P.n3, P.N, (float)P.U, P.vmax,
-                        ctx->stream),
-     "split input");
-  RhsIO s = o;
-  s.gam = P.Y32;
-  s.sig = u.s64;
-  s.dgam = u.kout;
-  s.out_f32 = 1;
-  LK(launch_set_user_io(ctx->d_io_user, ctx->d_ctl, ctx->n, point, s, Lambda, ctx->stream), "user io");
-  int rc = run_rhs(ctx, ctx->d_io_user, point, ev);
-  if (rc) return rc;
-  // the relayout above rewrote every entry of the point's layouts: the flow's
-  // next step attempt writes every entry again (not only the half the
-  // reversal reduction reads)
-  CK(cudaMemsetAsync(&ctx->d_ctl[point].lay_both, 1, sizeof(int), ctx->stream), "layout flag");
-  LK(launch_widen(static_cast<double2 *>(d_dgamma), u.kout, P.n3, ctx->stream), "widen output");
-  return FRG_OK;
+  // split path: the vertex goes into the FP32 operand copies (scratch between
+  // the stages of a flow; the contraction's tensor maps point at them), the
+  // channels' pp part into a buffer of its own, and the sum out in FP64
+  float2 *&kout = ctx->user_kout[point];
+  if (!kout && !(kout = dalloc<float2>(ctx, P.n3))) return fail(ctx, FRG_ENOMEM, "stand-alone rhs scratch");
+  o.gam = P.Y32;
+  o.dgam = kout;
+  o.out64 = static_cast<double2 *>(d_dgamma);
+  o.out_f32 = 1;
+  LK(launch_set_user_io(ctx->d_io_user, ctx->d_ctl, ctx->n, point, o, Lambda, ctx->stream, true), "user io");
+  return run_rhs_split(ctx, ctx->d_io_user, point, static_cast<const double2 *>(d_gamma), ev);
 }
 
 int frg_rhs(frg_ctx *ctx, int point, double Lambda, const void *d_gamma, const void *d_sigma, void *d_dgamma,
@@ -1053,7 +1070,7 @@ int frg_autotune(frg_ctx *ctx, frg_tune *out) {
         float ms = 1e30f;
         for (int r = 0; r < 4 && rc == FRG_OK; ++r) {
           if (cudaEventRecord(e0, st) != cudaSuccess) rc = FRG_ECUDA;
-          if (rc == FRG_OK) rc = run_rhs(ctx, ctx->d_io_stage, -1);
+          if (rc == FRG_OK) rc = run_rhs_split(ctx, ctx->d_io_stage, -1, nullptr);
           if (rc == FRG_OK && cudaEventRecord(e1, st) != cudaSuccess) rc = FRG_ECUDA;
           if (rc == FRG_OK && cudaEventSynchronize(e1) != cudaSuccess) rc = FRG_ECUDA;
           float x = 0.f;

@@ -112,7 +112,8 @@ __host__ __device__ constexpr int comb_threads() { return (REV && !ERR) ? LB_THR
 // One layout block of the scatter-add (an active point's): TPB threads,
 // the block in sm (LB x LAP float2); VMAX: reset the vertex bound of the stage
 // input (BF16 slicing) for the next stage.
-template <bool REV, bool ERR, int TPB, bool VMAX>
+// OUT64: the result widened to FP64 into RhsIO.out64 (stand-alone evaluations).
+template <bool REV, bool ERR, int TPB, bool VMAX, bool OUT64 = false>
 __device__ __forceinline__ void combine_block(const PointDesc &P, const RhsIO &o, int mask, const ErrWeights &ew,
                                               float2 *__restrict__ sm) {
   const int N = P.N, M = N - 1, nrow = 2 * N - 1;
@@ -243,7 +244,13 @@ __device__ __forceinline__ void combine_block(const PointDesc &P, const RhsIO &o
       }
       v = make_float4(v.x + (ta.x + tb0.x), v.y + (ta.y + tb0.y), v.z + (ta.x + tb1.x), v.w + (ta.y + tb1.y));
     }
-    K4[((ga * N + gb) * N + gc) >> 1] = make_float4(v.x + vk.x, v.y + vk.y, v.z + vk.z, v.w + vk.w);
+    const int i = (ga * N + gb) * N + gc;
+    if (OUT64) {
+      o.out64[i] = make_double2((double)(v.x + vk.x), (double)(v.y + vk.y));
+      o.out64[i + 1] = make_double2((double)(v.z + vk.z), (double)(v.w + vk.w));
+    } else {
+      K4[i >> 1] = make_float4(v.x + vk.x, v.y + vk.y, v.z + vk.z, v.w + vk.w);
+    }
   }
   if constexpr (!ERR) return;
   if (!o.ctl) return;

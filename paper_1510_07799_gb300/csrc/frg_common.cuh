@@ -105,6 +105,9 @@ struct RhsIO {
   const double *lam;   // scale (device)
   int active;          // 0: skip this point
   int out_f32;         // vertex output as float2
+  // stand-alone evaluations of the split paths: the vertex output in FP64 (dgam
+  // then holds the pp products of the contraction only); null otherwise
+  double2 *out64;
   int canon;           // 1: only the entries i < n3/2 of the vertex output are wanted (dgam holds n3/2)
   // split paths, the seventh rhs of a step (k7): the scatter-add that forms it
   // also completes the embedded error estimate of the step (ctl: the point's

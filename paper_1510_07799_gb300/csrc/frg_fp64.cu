@@ -272,10 +272,9 @@ __global__ void k_tail_finish(const PointDesc *__restrict__ pts, const RhsIO *__
   }
 }
 
-// dGamma(k1,k2,k3) += tail_pp[k1 + k2] + tail_xph[k2 - k3] (FP32 or FP64
-// output, the constants rounded to the output's precision; k_tail_finish has
-// added the self-energy's).  A block takes TAIL_ROWS rows (k1, k2); thread k3
-// walks them.
+// dGamma(k1,k2,k3) += tail_pp[k1 + k2] + tail_xph[k2 - k3], FP64 path
+// (k_tail_finish has added the self-energy's; the split paths' scatter-add adds
+// theirs).  A block takes TAIL_ROWS rows (k1, k2); thread k3 walks them.
 constexpr int TAIL_ROWS = 16;
 __global__ void __launch_bounds__(FRG_MAX_N) k_add_tails(const PointDesc *__restrict__ pts,
                                                          const RhsIO *__restrict__ io) {
@@ -288,43 +287,22 @@ __global__ void __launch_bounds__(FRG_MAX_N) k_add_tails(const PointDesc *__rest
   const int r0 = blockIdx.x * TAIL_ROWS;
   if (r0 >= N * N) return;
   __shared__ double2 tab[2 * (2 * FRG_MAX_N - 1)];
-  __shared__ float2 tabf[2 * (2 * FRG_MAX_N - 1)];
-  for (int j = threadIdx.x; j < 2 * nrow; j += blockDim.x) {
-    tab[j] = P.tail[o.par * tail_set(N) + j];
-    tabf[j] = make_float2((float)tab[j].x, (float)tab[j].y);
-  }
+  for (int j = threadIdx.x; j < 2 * nrow; j += blockDim.x) tab[j] = P.tail[o.par * tail_set(N) + j];
   __syncthreads();
   const int i3 = threadIdx.x;
-  // half storage: the rows (i1, i2) with i1 < N/2 only
-  const int nrows = o.canon ? N * N / 2 : N * N;
-  if (i3 >= N || r0 >= nrows) return;
-  const int nr = min(TAIL_ROWS, nrows - r0);
+  if (i3 >= N) return;
+  const int nr = min(TAIL_ROWS, N * N - r0);
   // all loads of the thread first, then the updates (one round trip)
-  if (o.out_f32) {
-    float2 *d = static_cast<float2 *>(o.dgam) + (size_t)r0 * N + i3;
-    float2 v[TAIL_ROWS];
+  double2 *d = static_cast<double2 *>(o.dgam) + (size_t)r0 * N + i3;
+  double2 v[TAIL_ROWS];
 #pragma unroll
-    for (int k = 0; k < TAIL_ROWS; ++k)
-      if (k < nr) v[k] = d[(size_t)k * N];
+  for (int k = 0; k < TAIL_ROWS; ++k)
+    if (k < nr) v[k] = d[(size_t)k * N];
 #pragma unroll
-    for (int k = 0; k < TAIL_ROWS; ++k) {
-      if (k >= nr) break;
-      const int r = r0 + k, i1 = r / N, i2 = r - i1 * N;
-      const float2 ta = tabf[i1 + i2], tb = tabf[nrow + i2 - i3 + N - 1];
-      d[(size_t)k * N] = make_float2(v[k].x + (ta.x + tb.x), v[k].y + (ta.y + tb.y));
-    }
-  } else {
-    double2 *d = static_cast<double2 *>(o.dgam) + (size_t)r0 * N + i3;
-    double2 v[TAIL_ROWS];
-#pragma unroll
-    for (int k = 0; k < TAIL_ROWS; ++k)
-      if (k < nr) v[k] = d[(size_t)k * N];
-#pragma unroll
-    for (int k = 0; k < TAIL_ROWS; ++k) {
-      if (k >= nr) break;
-      const int r = r0 + k, i1 = r / N, i2 = r - i1 * N;
-      d[(size_t)k * N] = cadd(v[k], cadd(tab[i1 + i2], tab[nrow + i2 - i3 + N - 1]));
-    }
+  for (int k = 0; k < TAIL_ROWS; ++k) {
+    if (k >= nr) break;
+    const int r = r0 + k, i1 = r / N, i2 = r - i1 * N;
+    d[(size_t)k * N] = cadd(v[k], cadd(tab[i1 + i2], tab[nrow + i2 - i3 + N - 1]));
   }
 }
 

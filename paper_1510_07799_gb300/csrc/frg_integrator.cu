@@ -136,6 +136,7 @@ __device__ __forceinline__ void write_stage_io(const PointDesc &P, Ctl &c, RhsIO
   o.dgam = P.kG[c.kslot[stage]];
   o.dsig = P.kS[c.kslot[stage]];
   o.out_f32 = split;
+  o.out64 = nullptr;
   o.canon = split ? P.rev_half : 0;
   // the scatter-add of k7 completes the split paths' error estimate
   o.ctl = (split && stage == 6) ? &c : nullptr;

@@ -12,11 +12,10 @@
 // (in Z both direct-channel operands C and D have i2 - i3 = t: C's rows are
 // k1, D's rows p - t, both contiguous along i2), and each channel's output
 // tile is a run of rows in one layout as well (pp: N, dph: X, xph: W).
-// k_relayout writes the W, X and Z copies of the stage input from layout
-// blocks of 8 x 8 x 128 entries (frg_lblock.cuh; the split stage kernels write
-// the same copies themselves in a flow); k_combine adds the three channel
-// outputs into the natural layout through 16^3 tiles in shared memory, every
-// global access a 128-byte row.
+// k_relayout writes the natural, W, X and Z copies of a stand-alone evaluation's
+// FP64 vertex through layout blocks (frg_lblock.cuh; the split stage kernels
+// write the same copies themselves in a flow); k_combine adds the three channel
+// outputs into the natural layout through the same blocks.
 #include "frg.h"
 #include "frg_common.cuh"
 #include "frg_layout.cuh"
@@ -28,37 +27,58 @@
 namespace frg {
 
 
-// W, X and Z copies of each active point's FP32 stage input (io.gam), one
-// layout block (frg_lblock.cuh) per CTA: whole natural rows in (16-byte
-// loads, all issued before the first shared-memory store), 64-byte row
-// segments of each layout out.
-__global__ void __launch_bounds__(LB_THREADS, LB_MINBLOCKS) k_relayout(const PointDesc *__restrict__ pts,
-                                                         const RhsIO *__restrict__ io, int want) {
+// A stand-alone evaluation's vertex (FP64, natural layout) as the FP32 operand
+// copies of the contraction: the natural copy (bare U wherever the fourth
+// frequency leaves the box) and the W, X and Z copies in `want`, one layout block
+// (frg_lblock.cuh) per CTA: whole natural rows in (16-byte loads, all issued
+// before the first store), 64-byte row segments of each layout out.  VMAX
+// (BF16x3): fold the largest |Re|, |Im| into P.vmax[0].  One pass over the input
+// instead of two with an FP32 copy between them: N = 128 20 us against 28 + 13.
+template <bool VMAX>
+__global__ void __launch_bounds__(LB_THREADS, 5)
+    k_relayout(const PointDesc *__restrict__ pt, const double2 *__restrict__ G, int want) {
   extern __shared__ float4 lsm4[];
   float2 *sm = reinterpret_cast<float2 *>(lsm4);
-  const int pi = blockIdx.y;
-  const RhsIO &o = io[pi];
-  if (!o.active) return;
-  const PointDesc &P = pts[pi];
+  const PointDesc &P = *pt;
   const int N = P.N;
   const LBlock k = lblock(N, N, blockIdx.x);
   if (!k.ok) return;
-  const float4 *__restrict__ Y = static_cast<const float4 *>(o.gam);
+  const float2 U = make_float2((float)P.U, 0.f);
   // rows (a, b) of n3 elements from g3: pairs of complex values (N is even)
   constexpr int PAIRS = LB * LB * (LC / 2), PER = PAIRS / LB_THREADS;
-  float4 v[PER];
+  double2 v[PER][2];
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int e = threadIdx.x + u * LB_THREADS;
     const int c2 = e % (LC / 2), r = e / (LC / 2), b = r % LB, a = r / LB;
-    if (a < k.n1 && b < k.n2 && 2 * c2 < k.n3)
-      v[u] = Y[(((size_t)(k.g1 + a) * N + (k.g2 + b)) * N + k.g3) / 2 + c2];
+    if (a < k.n1 && b < k.n2 && 2 * c2 < k.n3) {
+      const double2 *g = G + ((k.g1 + a) * N + (k.g2 + b)) * N + k.g3 + 2 * c2;
+      v[u][0] = g[0];
+      v[u][1] = g[1];
+    }
   }
+  float vm = 0.f;
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int e = threadIdx.x + u * LB_THREADS;
     const int c2 = e % (LC / 2), r = e / (LC / 2), b = r % LB, a = r / LB;
-    if (a < k.n1 && b < k.n2 && 2 * c2 < k.n3) *reinterpret_cast<float4 *>(sm + lsidx(a, b, 2 * c2)) = v[u];
+    if (a < k.n1 && b < k.n2 && 2 * c2 < k.n3) {
+      const int i1 = k.g1 + a, i2 = k.g2 + b, i3 = k.g3 + 2 * c2, i4 = i1 + i2 - i3;
+      float2 x = round_c64(v[u][0]), y = round_c64(v[u][1]);
+      if (VMAX) vm = fmaxf(vm, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y))));
+      if (!inbox(N, i4)) x = U;
+      if (!inbox(N, i4 - 1)) y = U;
+      const float4 f = make_float4(x.x, x.y, y.x, y.y);
+      *reinterpret_cast<float4 *>(P.Y32 + ((i1 * N + i2) * N + i3)) = f;
+      *reinterpret_cast<float4 *>(sm + lsidx(a, b, 2 * c2)) = f;
+    }
+  }
+  if (VMAX) {
+    vm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(vm)));
+    if ((threadIdx.x & 31) == 0) {
+      if (!(vm <= 3.0e38f)) vm = 3.0e38f;
+      atomicMax(P.vmax, __float_as_uint(vm));
+    }
   }
   __syncthreads();
   lblock_write<false>(P, sm, k, want);
@@ -83,25 +103,29 @@ __global__ void k_fill_z(const PointDesc *__restrict__ pts) {
   }
 }
 
-template <bool REV, bool ERR>
+template <bool REV, bool ERR, bool OUT64>
 __global__ void __launch_bounds__(comb_threads<REV, ERR>(), ERR ? 4 : REV ? LB_MINBLOCKS_WIDE : LB_MINBLOCKS)
     k_combine(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, int mask, ErrWeights ew) {
   __shared__ __align__(16) float2 sm[LB * LAP];
   const RhsIO &o = io[blockIdx.y];
   if (!o.active) return;
-  combine_block<REV, ERR, comb_threads<REV, ERR>(), true>(pts[blockIdx.y], o, mask, ew, sm);
+  combine_block<REV, ERR, comb_threads<REV, ERR>(), true, OUT64>(pts[blockIdx.y], o, mask, ew, sm);
 }
 
 int layout_init() {
-  return cudaFuncSetAttribute(k_relayout, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LB_SMEM) == cudaSuccess
+  return cudaFuncSetAttribute(k_relayout<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LB_SMEM) ==
+                     cudaSuccess &&
+                 cudaFuncSetAttribute(k_relayout<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LB_SMEM) ==
+                     cudaSuccess
              ? 0
              : -3;
 }
 
-int launch_relayout(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int want_w, int want_x,
-                    int want_z, cudaStream_t st) {
-  const int want = (want_w ? LAY_W : 0) | (want_x ? LAY_X : 0) | (want_z ? LAY_Z : 0);
-  k_relayout<<<dim3(lblocks(maxN, maxN), n_points), LB_THREADS, LB_SMEM, st>>>(d_pts, d_io, want);
+int launch_relayout(const PointDesc *d_pt, const double2 *gam, int N, int want, bool vmax, cudaStream_t st) {
+  if (vmax)
+    k_relayout<true><<<lblocks(N, N), LB_THREADS, LB_SMEM, st>>>(d_pt, gam, want);
+  else
+    k_relayout<false><<<lblocks(N, N), LB_THREADS, LB_SMEM, st>>>(d_pt, gam, want);
   FRG_COUNT(1);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -113,21 +137,27 @@ int launch_fill_z(const PointDesc *d_pts, int n_points, cudaStream_t st) {
 }
 
 int launch_combine(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int mask, cudaStream_t st,
-                   bool err, bool canon_half) {
+                   bool err, bool canon_half, bool out64) {
   const dim3 g(lblocks(maxN, canon_half ? maxN / 2 : maxN), n_points);
   const ErrWeights ew = host_error_weights();
   const bool rev = (mask & FRG_REVERSAL) != 0;
   const int cv = step_carveout(n_points);
   cudaError_t e;
   if (rev && err)
-    e = launch_with_carveout(k_combine<true, true>, g, comb_threads<true, true>(), 0, st, cv, d_pts, d_io, mask, ew);
+    e = launch_with_carveout(k_combine<true, true, false>, g, comb_threads<true, true>(), 0, st, cv, d_pts, d_io, mask, ew);
+  else if (rev && out64)
+    e = launch_with_carveout(k_combine<true, false, true>, g, comb_threads<true, false>(), 0, st, cv, d_pts, d_io,
+                             mask, ew);
   else if (rev)
-    e = launch_with_carveout(k_combine<true, false>, g, comb_threads<true, false>(), 0, st, cv, d_pts, d_io, mask, ew);
+    e = launch_with_carveout(k_combine<true, false, false>, g, comb_threads<true, false>(), 0, st, cv, d_pts, d_io, mask, ew);
   else if (err)
-    e = launch_with_carveout(k_combine<false, true>, g, comb_threads<false, true>(), 0, st, cv, d_pts, d_io, mask, ew);
+    e = launch_with_carveout(k_combine<false, true, false>, g, comb_threads<false, true>(), 0, st, cv, d_pts, d_io, mask, ew);
+  else if (out64)
+    e = launch_with_carveout(k_combine<false, false, true>, g, comb_threads<false, false>(), 0, st, cv, d_pts, d_io,
+                             mask, ew);
   else
-    e = launch_with_carveout(k_combine<false, false>, g, comb_threads<false, false>(), 0, st, cv, d_pts, d_io, mask,
-                             ew);
+    e = launch_with_carveout(k_combine<false, false, false>, g, comb_threads<false, false>(), 0, st, cv, d_pts, d_io,
+                             mask, ew);
   FRG_COUNT(1);
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -3;
 }

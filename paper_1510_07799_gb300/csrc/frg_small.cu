@@ -14,7 +14,8 @@
 // no table in memory, one store per entry.  The last blocks form the
 // self-energy rhs.  Bound by the FP64 units: 16 multiply-adds per entry and p
 // plus the shared weights (R keeps their share below a third).
-// Measured (whole call of the allocation-free entry point): N = 16 100 -> 14 us.
+// Measured (whole call of the allocation-free entry point): N = 16 100 -> 14 us, N =
+// 32 183 -> 51, N = 48 353 -> 187, N = 64 572 -> 503 us.
 #include <cuda_runtime.h>
 
 #include "frg.h"
@@ -27,7 +28,9 @@ namespace small {
 constexpr int T = 256;
 
 // k3 per block, and lanes that share an entry's p: enough blocks for the SMs on
-// the smallest grids, little repeated weight work on the larger ones.
+// the smallest grids, little repeated weight work on the larger ones.  (Splitting
+// p further, so that the warps fill the SM's four partitions evenly, gains
+// nothing: N = 40 138 us with four lanes against 127 us with one.)
 __host__ __device__ inline int rows(int N) { return N <= 24 ? 2 : N <= 40 ? 4 : 8; }
 __host__ __device__ inline int lanes(int N) {
   int l = 8;
@@ -38,18 +41,23 @@ __host__ __device__ inline int pitch(int N) { return N + 1; }
 __host__ __device__ inline int blocks(int N) {
   return N * ((N + rows(N) - 1) / rows(N)) + (N + T / 32 - 1) / (T / 32);
 }
-// G, S, W1, Wa, Wb, W3
+// G, S, B, W1, Wa, Wb, W3
 __host__ __device__ inline size_t smem(int N) {
   const int R = rows(N);
-  return (size_t)(2 * N + (N + 2 * R + N + R - 1) * pitch(N)) * sizeof(double2);
+  return (size_t)(2 * N + (N + N + 2 * R + N + R - 1) * pitch(N)) * sizeof(double2);
 }
 
-__device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int b, double2 *sm) {
+// Which part of the rhs a launch covers: everything, or (in-place self-energy) the
+// vertex blocks and then the self-energy by one block.
+enum Part { ALL, VERTEX, SIGMA };
+
+__device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int part, int b,
+                                    double2 *sm) {
   const int N = P.N, R = rows(N), PL = lanes(N), W = pitch(N), tid = threadIdx.x;
   const int nb = (N + R - 1) / R;
-  if (b >= blocks(N)) return;
+  if (b >= (part == VERTEX ? N * nb : part == SIGMA ? 1 : blocks(N))) return;
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
-  double2 *G = sm, *S = G + N, *W1 = S + N, *Wa = W1 + N * W, *Wb = Wa + R * W, *W3 = Wb + R * W;
+  double2 *G = sm, *S = G + N, *B = S + N, *W1 = B + N * W, *Wa = W1 + N * W, *Wb = Wa + R * W, *W3 = Wb + R * W;
   for (int i = tid; i < N; i += T) {
     double2 g, s;
     propagator_at(P, i, lam, o.sig ? o.sig[i] : make_double2(0.0, 0.0), g, s);
@@ -58,26 +66,34 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
   }
   __syncthreads();
   const double sc = P.T * lam;
-  if (b >= N * nb) {
+  if (part == SIGMA || b >= N * nb) {
     // self-energy: one warp per frequency
-    const int w = (b - N * nb) * (T / 32) + (tid >> 5), lane = tid & 31;
-    if (w >= N) return;
-    double2 acc = make_double2(0.0, 0.0);
-    if (mask & FRG_CH_SIGMA)
-      for (int p = lane; p < N; p += 32) {
-        const double2 a = V[(w * N + p) * N + w], c = V[(w * N + p) * N + p];
-        cfma(acc, S[p], make_double2(2.0 * a.x - c.x, 2.0 * a.y - c.y));
+    const int lane = tid & 31;
+    int w = (part == SIGMA ? 0 : b - N * nb) * (T / 32) + (tid >> 5);
+    for (; w < N; w += part == SIGMA ? T / 32 : N) {
+      double2 acc = make_double2(0.0, 0.0);
+      if (mask & FRG_CH_SIGMA)
+        for (int p = lane; p < N; p += 32) {
+          const double2 a = V[(w * N + p) * N + w], c = V[(w * N + p) * N + p];
+          cfma(acc, S[p], make_double2(2.0 * a.x - c.x, 2.0 * a.y - c.y));
+        }
+      for (int off = 16; off > 0; off >>= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
       }
-    for (int off = 16; off > 0; off >>= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+      if (lane == 0) o.dsig[w] = cscale(acc, sc);
     }
-    if (lane == 0) o.dsig[w] = cscale(acc, sc);
     return;
   }
   const int k1 = b / nb, c0 = (b % nb) * R;
   const double2 U = make_double2(P.U, 0.0);
-  auto bub = [&](int p, int q) { return cadd(cmul(S[p], G[q]), cmul(G[p], S[q])); };
+  // every weight below is a bubble Lb(p, q) = Lb(q, p) of two box frequencies
+  for (int e = tid; e < N * N; e += T) {
+    const int p = e / N, q = e - p * N;
+    if (p <= q) B[p * W + q] = B[q * W + p] = cadd(cmul(S[p], G[q]), cmul(G[p], S[q]));
+  }
+  __syncthreads();
+  auto bub = [&](int p, int q) { return B[p * W + q]; };
   if (mask & FRG_CH_PP)
     for (int e = tid; e < N * N; e += T) {
       const int k2 = e / N, p = e - k2 * N, q = k1 + k2 - p;
@@ -149,18 +165,19 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
 }
 
 __global__ void __launch_bounds__(T) k_rhs_small(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                                                 int n_below, int mask) {
+                                                 int n_below, int mask, int part) {
   extern __shared__ double2 sm[];
   const PointDesc &P = pts[blockIdx.y];
   const RhsIO &o = io[blockIdx.y];
   if (!o.active || P.N >= n_below) return;
-  rhs(P, o, *o.lam, mask, blockIdx.x, sm);
+  rhs(P, o, *o.lam, mask, part, blockIdx.x, sm);
 }
 
 __global__ void __launch_bounds__(T) k_rhs_small_value(const __grid_constant__ PointDesc P,
-                                                       const __grid_constant__ RhsIO o, double lam, int mask) {
+                                                       const __grid_constant__ RhsIO o, double lam, int mask,
+                                                       int part) {
   extern __shared__ double2 sm[];
-  rhs(P, o, lam, mask, blockIdx.x, sm);
+  rhs(P, o, lam, mask, part, blockIdx.x, sm);
 }
 
 // (a host-side setting of the current device's context: set on every call, as
@@ -173,11 +190,10 @@ bool room(K kernel, size_t bytes) {
 }  // namespace small
 
 int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int n_below, int mask,
-                     cudaStream_t st) {
+                     bool sig_in_place, cudaStream_t st) {
+  // shared memory and blocks for every size below the bound (both drop where the
+  // rows per block step up)
   const int N = maxN < n_below ? maxN : n_below - 1;
-  // the shared weights and the block count both grow with N within a row count,
-  // and the row count's steps keep the larger N ahead; sizes between them are
-  // covered by the maxima over the range
   size_t bytes = 0;
   int blocks = 0;
   for (int n = 2; n <= N; n += 2) {
@@ -185,16 +201,27 @@ int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
     blocks = small::blocks(n) > blocks ? small::blocks(n) : blocks;
   }
   if (!small::room(small::k_rhs_small, bytes)) return -3;
-  small::k_rhs_small<<<dim3(blocks, n_points), small::T, bytes, st>>>(d_pts, d_io, n_below, mask);
+  const int first = sig_in_place ? small::VERTEX : small::ALL;
+  small::k_rhs_small<<<dim3(blocks, n_points), small::T, bytes, st>>>(d_pts, d_io, n_below, mask, first);
   FRG_COUNT(1);
+  if (sig_in_place) {
+    small::k_rhs_small<<<dim3(1, n_points), small::T, bytes, st>>>(d_pts, d_io, n_below, mask, small::SIGMA);
+    FRG_COUNT(1);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int mask, cudaStream_t st) {
+int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int mask, bool sig_in_place,
+                           cudaStream_t st) {
   const size_t bytes = small::smem(P.N);
   if (!small::room(small::k_rhs_small_value, bytes)) return -3;
-  small::k_rhs_small_value<<<small::blocks(P.N), small::T, bytes, st>>>(P, o, lam, mask);
+  const int first = sig_in_place ? small::VERTEX : small::ALL;
+  small::k_rhs_small_value<<<small::blocks(P.N), small::T, bytes, st>>>(P, o, lam, mask, first);
   FRG_COUNT(1);
+  if (sig_in_place) {
+    small::k_rhs_small_value<<<1, small::T, bytes, st>>>(P, o, lam, mask, small::SIGMA);
+    FRG_COUNT(1);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 

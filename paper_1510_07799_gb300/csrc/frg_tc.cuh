@@ -31,24 +31,24 @@ void tc_plan_destroy(TcPlan *plan);
 int tc_wait_selftest(unsigned *d_err, double limit_ms, cudaStream_t st);
 // Evaluate the enabled vertex channels of every active point (point = -1) or of
 // one point, writing the float2 vertex output of each active RhsIO.
-// Relayout of the stage input (skipped with layouts_ready: the split stage
-// kernels of a flow write the W, X and Z copies themselves), the channel
-// products (with half: the reversal reduction's schedule, transfers m <= N - 1,
-// the combine taking the others from the mirrored entries), and the combine
-// into the natural layout (with err also the step's error estimate: the
-// seventh rhs of a flow step; with half and cross the crossing-reduced
-// tiles; without combine the caller runs the scatter-add itself, e.g. fused
-// with the next stage sum).  ev_gather / ev_contract
-// (optional) are recorded after the relayout and after the products; the
-// products wait for wait_before (optional: the bubble weights computed on
-// another stream), the combine for wait_combine (optional: the tail constants
-// and the self-energy rhs computed on another stream).  sigma (flows of all
-// points, point = -1): the contraction also forms the self-energy rhs of every
-// active point (bit 0: on; bit 1: the self-energy channel is enabled, else
-// the rhs is zero).
+// The channel products over the layouts of the stage input (with half: the
+// reversal reduction's schedule, transfers m <= N - 1, the combine taking the
+// others from the mirrored entries), and the combine into the natural layout
+// (canon: the canonical half only, a flow under the reversal reduction; out64:
+// in FP64 to io.out64; with err also the step's error estimate: the seventh rhs
+// of a flow step; with half and cross the crossing-reduced tiles; without
+// combine the caller runs the scatter-add itself, e.g. fused with the next stage
+// sum).  ev_contract (optional) is recorded after the products; the products
+// wait for wait_before (optional: the bubble weights computed on another
+// stream), the combine for wait_combine (optional: the tail constants and the
+// self-energy rhs computed on another stream).  sigma: the contraction also
+// forms the self-energy rhs of the active points it covers (bit 0: on; bit 1:
+// the self-energy channel is enabled, else the rhs is zero).
+struct TcRun {
+  cudaEvent_t ev_contract = nullptr, wait_before = nullptr, wait_combine = nullptr;
+  bool tails = false, half = false, canon = false, out64 = false, err = false, cross = false, combine = true;
+  int sigma = 0;
+};
 int tc_run(TcPlan *plan, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st,
-           cudaEvent_t ev_gather, cudaEvent_t ev_contract, int n_points, int maxN,
-           cudaEvent_t wait_before = nullptr, int tails = 0, cudaEvent_t wait_combine = nullptr,
-           bool layouts_ready = false, bool half = false, bool err = false, bool cross = false,
-           bool combine = true, int sigma = 0);
+           int n_points, int maxN, const TcRun &r);
 }  // namespace frg

@@ -248,9 +248,9 @@ class Context:
                                  _ptr(dsigma)))
 
     def rhs_timed(self, point, Lambda, gamma, sigma, dgamma, dsigma):
-        """Like rhs(); returns the phase durations in ms (bubble weights with the
-        self-energy, operand regather, channel contractions, combine, and 0)
-        measured with CUDA events on the context stream."""
+        """Like rhs(); returns the phase durations in ms (bubble weights, operand
+        regather, channel contractions, combine, tails) measured with CUDA events
+        on the context stream (frg_rhs_timed says where the self-energy counts)."""
         N = self.N(point)
         _check_dev(gamma, (N, N, N), "gamma")
         _check_dev(dgamma, (N, N, N), "dgamma")

@@ -51,3 +51,20 @@ def test_batch_of_small_and_sliced_points():
             one.advance(2)
             g1, s1, _, _ = one.get_state(0)
         assert torch.equal(g, g1) and torch.equal(s, s1)
+
+
+@pytest.mark.parametrize("N", [16, 64])
+def test_self_energy_rhs_in_place(N):
+    """The self-energy output may be the input's own buffer."""
+    p = frg.Params(U=1.3, T=0.64 / N, eps_d=-0.4, N_f=N)
+    V = torch.from_numpy(inputs.random_vertex(N, p.U, seed=N)).cuda()
+    sig = torch.from_numpy(inputs.random_sigma(N, seed=N)).cuda()
+    calls = [lambda *a: frg.rhs_noalloc(p, 0.25, *a)]
+    with frg.Context([p]) as ctx, frg.Context([p], precision="3xtf32") as split:
+        calls += [lambda *a: ctx.rhs(0, 0.25, *a), lambda *a: split.rhs(0, 0.25, *a)]
+        for call in calls:
+            dg, ds, dg2, buf = torch.empty_like(V), torch.empty_like(sig), torch.empty_like(V), sig.clone()
+            call(V, sig, dg, ds)
+            call(V, buf, dg2, buf)
+            torch.cuda.synchronize()
+            assert torch.equal(dg, dg2) and torch.equal(ds, buf)
