@@ -68,10 +68,6 @@ struct Tr<FRG_BF16X3> {
   static constexpr int SLICES = 3, ROWB = 64, SWZ_MODE = 4, ATOM = 512;
 };
 
-struct TcWork {
-  int point, m, rt, ct, cx;
-};
-
 // ---------------------------------------------------------------- PTX ----
 // Shared-memory matrix descriptor (K-major, swizzled): start address, stride
 // between 8-row atoms (SBO), version bits 46-48 = 0b001, swizzle mode.
@@ -232,37 +228,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
-template <int CH>
-__device__ __forceinline__ bool tile_info(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                                          const TcWork &w, const int *__restrict__ nt_of, TileInfo &ti) {
-  ti.point = w.point;
-  const PointDesc &P = pts[w.point];
-  ti.N = P.N;
-  ti.NTb = nt_of[w.point];
-  ti.g = geom(CH, P.N, w.m);
-  ti.D16 = (ti.g.D + KSTEP - 1) / KSTEP * KSTEP;
-  ti.nk = (CH == CH_DPH ? 2 : 1) * ti.D16 / KSTEP;
-  ti.r0 = w.rt * MROWS;
-  if (w.cx) {
-    const CrossTile x = cross_tile(CH, P.N, ti.NTb, w.m, w.rt);
-    ti.c0 = x.c0;
-    ti.NT = x.nt;
-    ti.own_lo = x.own_lo;
-    ti.own_hi = x.own_hi;
-    ti.m_lo = x.m_lo;
-    ti.m_hi = x.m_hi;
-    ti.m_row = x.m_row;
-  } else {
-    ti.NT = ti.NTb;
-    ti.c0 = w.ct * ti.NT;
-    ti.own_lo = 0;
-    ti.own_hi = P.N;
-    ti.m_lo = ti.m_hi = 0;
-    ti.m_row = -1;
-  }
-  return io[w.point].active != 0;
-}
-
 // ===================================================================
 // The persistent contraction over the tiles of all channels and points.
 //
@@ -374,12 +339,7 @@ __device__ __forceinline__ Step step_of(const TileInfo &ti, int kb) {
 
 // k-step processed i-th in a tile: chunks in increasing max |Lb| (table
 // written by the bubble kernel, one 16-byte row per transfer, read once per
-// tile), both halves of the direct channel interleaved.
-template <int CH>
-__device__ __forceinline__ uint4 korder_row(const PointDesc &P, int N, int m) {
-  const int row = CH == CH_PP ? m : (2 * N - 1) + (CH == CH_XPH ? m : 2 * N - 2 - m);
-  return *reinterpret_cast<const uint4 *>(P.kord + (size_t)row * 16);
-}
+// tile through StWork.kord), both halves of the direct channel interleaved.
 __device__ __forceinline__ int kord_byte(const uint4 &o, int i) {
   const uint32_t w = (i & 8) ? ((i & 4) ? o.w : o.z) : ((i & 4) ? o.y : o.x);
   return (int)((w >> (8 * (i & 3))) & 0xFFu);
@@ -391,12 +351,18 @@ __device__ __forceinline__ int kstep_at(const uint4 &ord, const TileInfo &ti, in
 }
 
 // One tile of the channel product: channel, point, transfer index, row tile,
-// column tile.  The work list holds every tile of every enabled channel; the
-// host assigns the tiles to the persistent CTAs (longest first, each to the
-// least loaded CTA) and stores them CTA by CTA.
-struct StWork {
+// column tile, and what a role needs to start on it without a chain of dependent
+// loads (each a cache miss of some 700 cycles: the grid, the box width and the
+// transfer's row of the k-chunk order and of the bubble-weight maxima).  The
+// work list holds every tile of every enabled channel; the host assigns the
+// tiles to the persistent CTAs (longest first, each to the least loaded CTA) and
+// stores them CTA by CTA.
+struct __align__(16) StWork {
   int point;
-  short m, ch, rt, ct, cx, pad_;  // cx: a crossing-reduced tile (cross_tile)
+  short m, ch, rt, ct, cx;  // cx: a crossing-reduced tile (cross_tile)
+  short N, NTb, pad_;       // NTb: column width of the raw right-operand box (the point's column-tile width)
+  const unsigned char *kord;
+  const float *lmax;
 };
 
 // Shared pipeline state of one CTA.
@@ -413,43 +379,86 @@ struct Pipe {
 // X: the kernel instance that runs crossing-reduced schedules (the other one
 // ignores the tile mark, so its tiles keep the plain geometry at no cost).
 template <int CH>
-__device__ __forceinline__ bool st_tile_info(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                                             const StWork &w, const int *__restrict__ nt_of, TileInfo &ti,
-                                             bool X) {
-  return tile_info<CH>(pts, io, TcWork{w.point, w.m, w.rt, w.ct, X ? (int)w.cx : 0}, nt_of, ti);
+__device__ __forceinline__ void tile_info(const StWork &w, TileInfo &ti, bool X) {
+  ti.point = w.point;
+  ti.N = w.N;
+  ti.NTb = w.NTb;
+  ti.g = geom(CH, w.N, w.m);
+  ti.D16 = (ti.g.D + KSTEP - 1) / KSTEP * KSTEP;
+  ti.nk = (CH == CH_DPH ? 2 : 1) * ti.D16 / KSTEP;
+  ti.r0 = w.rt * MROWS;
+  if (X && w.cx) {
+    const CrossTile x = cross_tile(CH, w.N, ti.NTb, w.m, w.rt);
+    ti.c0 = x.c0;
+    ti.NT = x.nt;
+    ti.own_lo = x.own_lo;
+    ti.own_hi = x.own_hi;
+    ti.m_lo = x.m_lo;
+    ti.m_hi = x.m_hi;
+    ti.m_row = x.m_row;
+  } else {
+    ti.NT = ti.NTb;
+    ti.c0 = w.ct * ti.NT;
+    ti.own_lo = 0;
+    ti.own_hi = w.N;
+    ti.m_lo = ti.m_hi = 0;
+    ti.m_row = -1;
+  }
+}
+
+// Brings what the roles read first on the CTA's next tiles into the L1 cache, one
+// tile ahead (the loader's idle lanes: plain loads whose values nothing waits
+// for).
+__device__ __forceinline__ void touch(const void *p) {
+  uint32_t v;
+  asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(v) : "l"(p));
+}
+__device__ __forceinline__ void look_ahead(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
+                                           const StWork *__restrict__ work, int wi, int w1, int lane) {
+  if (wi + 1 < w1) {
+    const StWork n = work[wi + 1];
+    if (lane == 1) touch(n.kord);
+    if (lane == 2) touch(n.lmax);
+    if (lane == 3) touch(&io[n.point].active);
+    if (lane == 4) touch(&io[n.point].lam);
+    if (lane == 5) touch(&pts[n.point].T);
+    if (lane == 6) touch(&pts[n.point].PX);
+  }
+  if (wi + 2 < w1 && (lane == 7 || lane == 8)) touch(reinterpret_cast<const char *>(work + wi + 2) + (lane - 7) * 32);
 }
 
 // Loader (one warp, lane 0 issues): the raw rows of every k-step of a tile by
 // tensor-map TMA, NRAW k-steps ahead.  Returns false when a wait gave up.
 template <int CH>
-__device__ __forceinline__ bool load_tile(const Pipe &S, const PointDesc *__restrict__ pts,
-                                          const RhsIO *__restrict__ io, const StWork &w,
-                                          const int *__restrict__ nt_of, const CUtensorMap *__restrict__ maps,
-                                          uint32_t &it, int lane, bool X) {
+__device__ __forceinline__ bool load_tile(const Pipe &S, const RhsIO *__restrict__ io, const StWork &w,
+                                          const CUtensorMap *__restrict__ maps, uint32_t &it, int lane, bool X) {
+  if (!io[w.point].active) return true;
   TileInfo ti;
-  if (!st_tile_info<CH>(pts, io, w, nt_of, ti, X)) return true;
-  const uint4 ord = korder_row<CH>(pts[ti.point], ti.N, w.m);
+  tile_info<CH>(w, ti, X);
+  const uint4 ord = *reinterpret_cast<const uint4 *>(w.kord);
   const CUtensorMap *mp = maps + (size_t)ti.point * M_COUNT;
   for (int ki = 0; ki < ti.nk; ++ki, ++it) {
     const int j = it % NRAW;
-    if (!wwait(&S.raw_empty[j], ((it / NRAW) & 1u) ^ 1u, S.err, S.abort_flag)) return false;
+    // everything about the k-step before the wait: from the hand-back of a raw
+    // stage to its next rows is the pipeline's longest chain
     const Step q = step_of<CH>(ti, kstep_at<CH>(ord, ti, ki));
     const bool two = CH == CH_DPH && !q.half;
     uint8_t *raw = S.raws + j * RAW_STAGE;
     const uint32_t bytes = (uint32_t)(RAW_A * (two ? 2 : 1) + KS * ti.NTb * 8 + RA * 8);
+    uint64_t *bar = &S.raw_full[j];
+    const int xa = 2 * q.a0, xb = 2 * ti.c0, x = ti.g.x, kr = q.kl;
+    if (!wwait(&S.raw_empty[j], ((it / NRAW) & 1u) ^ 1u, S.err, S.abort_flag)) return false;
     if (lane == 0) {
-      uint64_t *bar = &S.raw_full[j];
       arrive_expect_tx(bar, bytes);
-      const int xa = 2 * q.a0, xb = 2 * ti.c0, x = ti.g.x;
       if (CH == CH_PP) {
+        tma3(raw + 2 * RAW_A, mp + M_PB, xb, ti.g.p_lo + kr, x, bar);
         tma3(raw, mp + M_PA, xa, ti.g.row_lo + ti.r0, x, bar);
-        tma3(raw + 2 * RAW_A, mp + M_PB, xb, ti.g.p_lo + q.kl, x, bar);
         tma2(raw + 2 * RAW_A + RAW_B, mp + M_LPP, xa, x, bar);
       } else if (CH == CH_XPH) {
         const bool d2 = x >= 0;
         const int z = x >= 0 ? x : -x;
+        tma3(raw + 2 * RAW_A, mp + (d2 ? M_W2B : M_W1B), xb, kr, z, bar);
         tma3(raw, mp + (d2 ? M_W2A : M_W1A), xa, ti.r0, z, bar);
-        tma3(raw + 2 * RAW_A, mp + (d2 ? M_W2B : M_W1B), xb, q.kl, z, bar);
         tma2(raw + 2 * RAW_A + RAW_B, mp + M_LPH, xa, x + ti.N - 1, bar);
       } else {
         const bool d1 = x >= 0;
@@ -457,12 +466,12 @@ __device__ __forceinline__ bool load_tile(const Pipe &S, const PointDesc *__rest
         // A (k1, p, k1+t) from X; C (k1, p, p-t) = Z[k1][t+N-1][p]; B (p-t, k2, p)
         // from X; D (p-t, k2, k2-t) = Z[p-t][t+N-1][k2], rows p - t = row_lo + kl + j
         const int zd = x + ti.N - 1;
+        if (q.half)
+          tma3(raw + 2 * RAW_A, mp + M_ZB, xb, ti.g.row_lo + kr, zd, bar);
+        else
+          tma3(raw + 2 * RAW_A, mp + (d1 ? M_X1B : M_X2B), xb, kr, z, bar);
         tma3(raw, mp + (d1 ? M_X1A : M_X2A), xa, ti.r0, z, bar);
         if (two) tma3(raw + RAW_A, mp + M_ZA, xa, ti.g.row_lo + ti.r0, zd, bar);
-        if (q.half)
-          tma3(raw + 2 * RAW_A, mp + M_ZB, xb, ti.g.row_lo + q.kl, zd, bar);
-        else
-          tma3(raw + 2 * RAW_A, mp + (d1 ? M_X1B : M_X2B), xb, q.kl, z, bar);
         tma2(raw + 2 * RAW_A + RAW_B, mp + M_LPH, xa, -x + ti.N - 1, bar);
       }
     }
@@ -656,19 +665,19 @@ __device__ __forceinline__ void xf_right(XfV<PREC> &o, const float2 *rB, const X
 // parts, for the left one.
 template <int CH, int PREC>
 __device__ __forceinline__ bool xf_tile(const Pipe &S, const PointDesc *__restrict__ pts,
-                                        const RhsIO *__restrict__ io, const StWork &w,
-                                        const int *__restrict__ nt_of, uint32_t &it, int xt, int lane, bool X) {
+                                        const RhsIO *__restrict__ io, const StWork &w, uint32_t &it, int xt,
+                                        int lane, bool X) {
   using L = OpL<PREC>;
+  if (!io[w.point].active) return true;
   TileInfo ti;
-  if (!st_tile_info<CH>(pts, io, w, nt_of, ti, X)) return true;
-  const PointDesc &P = pts[ti.point];
-  const uint4 ord = korder_row<CH>(P, ti.N, w.m);
+  tile_info<CH>(w, ti, X);
+  const uint4 ord = *reinterpret_cast<const uint4 *>(w.kord);
   typename XfV<PREC>::Scale scA{}, scB{};
   if constexpr (PREC == FRG_BF16X3) {
+    const PointDesc &P = pts[ti.point];
     const float vb = fmaxf(__uint_as_float(P.vmax[io[ti.point].par]), fabsf((float)P.U));
-    const int row = CH == CH_PP ? w.m : (2 * ti.N - 1) + (CH == CH_XPH ? w.m : 2 * ti.N - 2 - w.m);
     scB = slice_grid(bound_exp(vb));
-    scA = slice_grid(bound_exp(P.Lmax[row] * vb * (CH == CH_DPH ? 6.f : 2.f)));
+    scA = slice_grid(bound_exp(*w.lmax * vb * (CH == CH_DPH ? 6.f : 2.f)));
   }
   // warps 0-7: left item xt and right item xt; warps 8-11: right items xt and xt + 128
   const bool lr = xt < 256;
@@ -676,9 +685,9 @@ __device__ __forceinline__ bool xf_tile(const Pipe &S, const PointDesc *__restri
   const XfAt a1 = xf_right_at<PREC>(lr ? xt : xt + 128, ti.NT, ti.NTb);
   for (int ki = 0; ki < ti.nk; ++ki, ++it) {
     const int j = it % NRAW, s = it % NOP;
-    if (!wwait(&S.raw_full[j], (it / NRAW) & 1u, S.err, S.abort_flag)) return false;
     const Step q = step_of<CH>(ti, kstep_at<CH>(ord, ti, ki));
     const int off = q.p0 - q.a0;
+    if (!wwait(&S.raw_full[j], (it / NRAW) & 1u, S.err, S.abort_flag)) return false;
     const uint8_t *raw = S.raws + j * RAW_STAGE;
     const float2 *rA = reinterpret_cast<const float2 *>(raw);
     const float2 *rC = reinterpret_cast<const float2 *>(raw + RAW_A);
@@ -744,12 +753,12 @@ __device__ __forceinline__ TSlot tslot_next(TBuf &t, int NT) {
 // slices are integers times a power of two below 2^8), the five products of
 // order up to 4 beyond it into the second.
 template <int CH, int PREC>
-__device__ __forceinline__ bool mma_tile(const Pipe &S, const PointDesc *__restrict__ pts,
-                                         const RhsIO *__restrict__ io, const StWork &w,
-                                         const int *__restrict__ nt_of, uint32_t &it, TBuf &tb, int lane, bool X) {
+__device__ __forceinline__ bool mma_tile(const Pipe &S, const RhsIO *__restrict__ io, const StWork &w, uint32_t &it,
+                                         TBuf &tb, int lane, bool X) {
   using L = OpL<PREC>;
+  if (!io[w.point].active) return true;
   TileInfo ti;
-  if (!st_tile_info<CH>(pts, io, w, nt_of, ti, X)) return true;
+  tile_info<CH>(w, ti, X);
   const TSlot ts = tslot_next(tb, ti.NT);
   uint32_t &e = ts.b ? tb.e1 : tb.e0;
   if (!wwait(&S.tempty[ts.b], (e & 1u) ^ 1u, S.err, S.abort_flag)) return false;
@@ -828,10 +837,11 @@ __device__ __forceinline__ void st_pair(float2 *row, int x, float2 a, float2 b, 
 }
 template <int CH>
 __device__ __forceinline__ bool epi_tile(const Pipe &S, const PointDesc *__restrict__ pts,
-                                         const RhsIO *__restrict__ io, const StWork &w,
-                                         const int *__restrict__ nt_of, TBuf &tb, int warp, int lane, bool X) {
+                                         const RhsIO *__restrict__ io, const StWork &w, TBuf &tb, int warp, int lane,
+                                         bool X) {
+  if (!io[w.point].active) return true;
   TileInfo ti;
-  if (!st_tile_info<CH>(pts, io, w, nt_of, ti, X)) return true;
+  tile_info<CH>(w, ti, X);
   const TSlot ts = tslot_next(tb, ti.NT);
   uint32_t &f = ts.b ? tb.f1 : tb.f0;
   if (!wwait(&S.tfull[ts.b], f & 1u, S.err, S.abort_flag)) return false;
@@ -964,7 +974,7 @@ __device__ __forceinline__ void sigma_rhs(const PointDesc *__restrict__ pts, con
 template <int PREC, bool X>
 __device__ __forceinline__ void contract(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
                                          const StWork *__restrict__ work, const int *__restrict__ cta_start,
-                                         const int *__restrict__ nt_of, unsigned *__restrict__ err,
+                                         unsigned *__restrict__ err,
                                          const CUtensorMap *__restrict__ maps, int half, int sig_p0, int sig_p1, int sig_on) {
   extern __shared__ uint8_t smem_raw[];
   // offset the shared array itself (keeps the shared state space for ld/st.shared)
@@ -1018,7 +1028,8 @@ __device__ __forceinline__ void contract(const PointDesc *__restrict__ pts, cons
     uint32_t it = 0;
     for (int wi = w0; wi < w1; ++wi) {
       const StWork w = work[wi];
-      if (!FRG_BY_CH(load_tile, S, pts, io, w, nt_of, maps, it, lane, X)) break;
+      look_ahead(pts, io, work, wi, w1, lane);
+      if (!FRG_BY_CH(load_tile, S, io, w, maps, it, lane, X)) break;
     }
     // copies still in flight must land before the CTA leaves
     for (uint32_t k = it > (uint32_t)NRAW ? it - NRAW : 0u; k < it; ++k)
@@ -1028,21 +1039,21 @@ __device__ __forceinline__ void contract(const PointDesc *__restrict__ pts, cons
     uint32_t it = 0;
     for (int wi = w0; wi < w1; ++wi) {
       const StWork w = work[wi];
-      if (!FRG_BY_CH_P(xf_tile, S, pts, io, w, nt_of, it, xt, lane, X)) break;
+      if (!FRG_BY_CH_P(xf_tile, S, pts, io, w, it, xt, lane, X)) break;
     }
   } else if (warp == MMA_W) {
     uint32_t it = 0;
     TBuf tb;
     for (int wi = w0; wi < w1; ++wi) {
       const StWork w = work[wi];
-      if (!FRG_BY_CH_P(mma_tile, S, pts, io, w, nt_of, it, tb, lane, X)) break;
+      if (!FRG_BY_CH_P(mma_tile, S, io, w, it, tb, lane, X)) break;
     }
   } else {
     if (sig_p1 > sig_p0) sigma_rhs(pts, io, sig_p0, sig_p1, sig_on != 0, warp, lane, S.epi_stg);
     TBuf tb;
     for (int wi = w0; wi < w1; ++wi) {
       const StWork w = work[wi];
-      if (!FRG_BY_CH(epi_tile, S, pts, io, w, nt_of, tb, warp, lane, X)) break;
+      if (!FRG_BY_CH(epi_tile, S, pts, io, w, tb, warp, lane, X)) break;
     }
   }
 #undef FRG_BY_CH
@@ -1055,31 +1066,28 @@ __device__ __forceinline__ void contract(const PointDesc *__restrict__ pts, cons
 
 __global__ void __launch_bounds__(THREADS, 1)
     k_contract_tf32(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, const StWork *__restrict__ work,
-                    const int *__restrict__ cta_start, const int *__restrict__ nt_of, unsigned *__restrict__ err,
+                    const int *__restrict__ cta_start, unsigned *__restrict__ err,
                     const CUtensorMap *__restrict__ maps, int half, int sig_p0, int sig_p1, int sig_on) {
-  contract<FRG_3XTF32, false>(pts, io, work, cta_start, nt_of, err, maps, half, sig_p0, sig_p1, sig_on);
+  contract<FRG_3XTF32, false>(pts, io, work, cta_start, err, maps, half, sig_p0, sig_p1, sig_on);
 }
 __global__ void __launch_bounds__(THREADS, 1)
     k_contract_bf16x3(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                      const StWork *__restrict__ work, const int *__restrict__ cta_start,
-                      const int *__restrict__ nt_of, unsigned *__restrict__ err, const CUtensorMap *__restrict__ maps,
+                      const StWork *__restrict__ work, const int *__restrict__ cta_start, unsigned *__restrict__ err, const CUtensorMap *__restrict__ maps,
                       int half, int sig_p0, int sig_p1, int sig_on) {
-  contract<FRG_BF16X3, false>(pts, io, work, cta_start, nt_of, err, maps, half, sig_p0, sig_p1, sig_on);
+  contract<FRG_BF16X3, false>(pts, io, work, cta_start, err, maps, half, sig_p0, sig_p1, sig_on);
 }
 // The same for crossing-reduced schedules (cross_tile).
 __global__ void __launch_bounds__(THREADS, 1)
     k_contract_tf32_x(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                      const StWork *__restrict__ work, const int *__restrict__ cta_start,
-                      const int *__restrict__ nt_of, unsigned *__restrict__ err, const CUtensorMap *__restrict__ maps,
+                      const StWork *__restrict__ work, const int *__restrict__ cta_start, unsigned *__restrict__ err, const CUtensorMap *__restrict__ maps,
                       int half, int sig_p0, int sig_p1, int sig_on) {
-  contract<FRG_3XTF32, true>(pts, io, work, cta_start, nt_of, err, maps, half, sig_p0, sig_p1, sig_on);
+  contract<FRG_3XTF32, true>(pts, io, work, cta_start, err, maps, half, sig_p0, sig_p1, sig_on);
 }
 __global__ void __launch_bounds__(THREADS, 1)
     k_contract_bf16x3_x(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                        const StWork *__restrict__ work, const int *__restrict__ cta_start,
-                        const int *__restrict__ nt_of, unsigned *__restrict__ err,
+                        const StWork *__restrict__ work, const int *__restrict__ cta_start, unsigned *__restrict__ err,
                         const CUtensorMap *__restrict__ maps, int half, int sig_p0, int sig_p1, int sig_on) {
-  contract<FRG_BF16X3, true>(pts, io, work, cta_start, nt_of, err, maps, half, sig_p0, sig_p1, sig_on);
+  contract<FRG_BF16X3, true>(pts, io, work, cta_start, err, maps, half, sig_p0, sig_p1, sig_on);
 }
 }  // namespace st
 
@@ -1113,7 +1121,6 @@ struct TcPlan {
   int precision = FRG_3XTF32;
   int sms = 0;
   int n = 0;
-  int *d_nt = nullptr;
   unsigned *d_err = nullptr;  // owned by the context
   // one launch for all enabled channels; schedule [0] covers every point,
   // [1 + i] point i alone; sched: every transfer, sched_half: the reversal
@@ -1149,6 +1156,8 @@ static bool build_sched(TcPlan *p, const std::vector<PointDesc> &pts, const std:
         const Geom g = geom(ch, N, m);
         const int nk = (ch == CH_DPH ? 2 : 1) * ((g.D + tc::KSTEP - 1) / tc::KSTEP);
         const bool cx = half && cross && nt[i] >= N && g.D > tc::MROWS;
+        // the transfer's row of the bubble-weight tables: pp m, crossed Q = m, direct -t
+        const int row = ch == CH_PP ? m : (2 * N - 1) + (ch == CH_XPH ? m : 2 * N - 2 - m);
         for (int rt = 0; rt * tc::MROWS < g.D; ++rt)
           for (int ct = 0; ct * nt[i] < N; ++ct) {
             int w = 256;
@@ -1158,7 +1167,8 @@ static bool build_sched(TcPlan *p, const std::vector<PointDesc> &pts, const std:
               w = 128 + 128 * x.nt / nt[i];
             }
             tiles.push_back({(nk + EPI_COST) * w,
-                             tc::st::StWork{i, (short)m, (short)ch, (short)rt, (short)ct, (short)(cx ? 1 : 0), 0}});
+                             tc::st::StWork{i, (short)m, (short)ch, (short)rt, (short)ct, (short)(cx ? 1 : 0), (short)N,
+                                           (short)nt[i], 0, pts[i].kord + (size_t)row * 16, pts[i].Lmax + row}});
           }
       }
     }
@@ -1292,8 +1302,7 @@ int tc_plan_create(TcPlan **out, const std::vector<PointDesc> &pts, const std::v
   p->tune = tune;
   std::vector<int> nt(p->n);
   for (int i = 0; i < p->n; ++i) nt[i] = std::min(tune.nt_cap, (pts[i].N + 15) / 16 * 16);
-  bool ok = cudaMalloc(&p->d_nt, sizeof(int) * p->n) == cudaSuccess &&
-            cudaMemcpy(p->d_nt, nt.data(), sizeof(int) * p->n, cudaMemcpyHostToDevice) == cudaSuccess;
+  bool ok = true;
   p->mask = (params.empty() ? FRG_CH_ALL : params[0].channel_mask) & 7;
   for (int h = 0; h < 3 && ok; ++h) {
     if (!(schedules & (h == 0 ? TC_FULL : h == 1 ? TC_HALF : TC_CROSS))) continue;
@@ -1334,7 +1343,6 @@ int tc_plan_create(TcPlan **out, const std::vector<PointDesc> &pts, const std::v
 void tc_plan_destroy(TcPlan *p) {
   if (!p) return;
   cudaFree(p->d_maps);
-  cudaFree(p->d_nt);
   for (auto *v : {&p->sched, &p->sched_half, &p->sched_cross})
     for (auto &sc : *v) {
       cudaFree(sc.d_work);
@@ -1370,7 +1378,7 @@ int tc_run(TcPlan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int 
                                            : (x ? tc::st::k_contract_bf16x3_x : tc::st::k_contract_bf16x3);
     const int smem = p->precision == FRG_3XTF32 ? tc::st::OpL<FRG_3XTF32>::SMEM : tc::st::OpL<FRG_BF16X3>::SMEM;
     const int s0 = point < 0 ? 0 : point, s1 = r.sigma ? (point < 0 ? n_points : point + 1) : s0;
-    kern<<<sc.grid, tc::st::THREADS, smem, st>>>(d_pts, d_io, sc.d_work, sc.d_start, p->d_nt, p->d_err, p->d_maps,
+    kern<<<sc.grid, tc::st::THREADS, smem, st>>>(d_pts, d_io, sc.d_work, sc.d_start, p->d_err, p->d_maps,
                                                  r.half ? 1 : 0, s0, s1, (r.sigma & 2) ? 1 : 0);
     FRG_COUNT(1);
     if (cudaGetLastError() != cudaSuccess) return -3;
