@@ -406,10 +406,10 @@ struct F64Smem {
   double2 Rs[F64_TK][F64_TN + 1];
 };
 
-// One tile of one channel: store(geometry, local row, column, sc x sum) for
-// every entry.
+// One tile of one channel: store(geometry, local row, column, value) for every
+// entry.
 template <int CH, typename Store>
-__device__ __forceinline__ void f64_tile(const PointDesc &P, const RhsIO &o, const WorkItem &w, double sc, F64Smem &sm,
+__device__ __forceinline__ void f64_tile(const PointDesc &P, const RhsIO &o, const WorkItem &w, F64Smem &sm,
                                          Store store) {
   auto &Ls = sm.Ls;
   auto &Rs = sm.Rs;
@@ -451,6 +451,7 @@ __device__ __forceinline__ void f64_tile(const PointDesc &P, const RhsIO &o, con
     }
     __syncthreads();
   }
+  const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -470,8 +471,7 @@ __global__ void __launch_bounds__(F64_THREADS)
   if (!o.active) return;
   const PointDesc &P = pts[w.point];
   double2 *out = static_cast<double2 *>(o.dgam);
-  const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
-  f64_tile<CH>(P, o, w, sc, sm, [&](const Geom &g, int r, int c, double2 v) {
+  f64_tile<CH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) {
     const size_t at = out_index<CH>(P.N, g, r, c);
     out[at] = ACCUM ? cadd(out[at], v) : v;
   });
@@ -495,11 +495,11 @@ __global__ void __launch_bounds__(F64_THREADS)
       for (int i = blockIdx.x; i < x.nwork[ch]; i += gridDim.x) {
         const WorkItem w = x.work[ch][i];
         if (ch == CH_PP)
-          f64_tile<CH_PP>(P, o, w, 1.0, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_PP>(P.N, g, r, c)] = v; });
+          f64_tile<CH_PP>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_PP>(P.N, g, r, c)] = v; });
         else if (ch == CH_DPH)
-          f64_tile<CH_DPH>(P, o, w, 1.0, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_DPH>(P.N, g, r, c)] = v; });
+          f64_tile<CH_DPH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_DPH>(P.N, g, r, c)] = v; });
         else
-          f64_tile<CH_XPH>(P, o, w, 1.0, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_XPH>(P.N, g, r, c)] = v; });
+          f64_tile<CH_XPH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_XPH>(P.N, g, r, c)] = v; });
       }
     }
   }

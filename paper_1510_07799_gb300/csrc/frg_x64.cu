@@ -65,8 +65,9 @@ constexpr int E_LIM = 400;                  // line exponents the path accepts
 // -------------------------------------------------------------- panels ----
 // One block: eight lines of one operand of one product over its whole
 // contraction range.  Eight lanes take the eight lines at one k, so that the
-// blocks are written in 128-byte segments; a thread gathers (and weights) all
-// its k of one line into registers, the block finds each line's largest magnitude, and the values leave
+// blocks are written in 128-byte segments; a thread gathers (and weights: the
+// factor +-T Lambda goes into the bubble weights) all its k of one line into
+// registers, the block finds each line's largest magnitude, and the values leave
 // in fixed point.  Bound by the FP64 multiplications of the weights and by the
 // gathers (16-byte elements, one 32-byte sector each wherever the line and the
 // contraction index both stride through the vertex): 114 us at N = 128 for 302 MB
@@ -150,8 +151,9 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
   if (tid < PAN_LINES) smax[tid] = 0u;
   if (LEFT) {
+    const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
     const double2 *L = CH == CH_PP ? P.Lpp + (size_t)m * N : P.Lph + (size_t)(CH == CH_DPH ? 2 * N - 2 - m : m) * N;
-    for (int k = tid; k < D; k += blockDim.x) sw[k] = L[g.p_lo + k];
+    for (int k = tid; k < D; k += blockDim.x) sw[k] = cscale(L[g.p_lo + k], sc);
   }
   double2 v[PAN_U], v2[PAN_U];
 #pragma unroll
@@ -190,7 +192,7 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
     if (LEFT)
       x.eL[(size_t)(pr.z + tile) * LINES + l0] = e;
     else
-      x.eR[((size_t)(CH * (2 * N - 1) + m) * ((N + LINES - 1) / LINES) + tile) * LINES + l0] = e;
+      x.eR[(size_t)(pr.w + tile) * LINES + l0] = e;
     if ((mx >> 20) == 0x7ffu || e > E_LIM || e < -E_LIM) atomicOr(x.bad, 1);
   }
   e = max(-E_LIM, min(E_LIM, e));  // (a marked point's values are not used)
@@ -272,9 +274,13 @@ constexpr int EPI_BUF = 32 * EPI_COLS * 16;  // one warp pair's 32 rows x 4 colu
 constexpr int SMEM = 1024 + NOP * OP_STAGE + NRAW * RAW_STAGE + EPI_W / 2 * EPI_BUF + 256;
 static_assert(SMEM <= 232448, "shared memory budget");
 
-struct Work {
+// One tile, with what every role needs to start on it without a chain of
+// dependent loads: its k-steps, where its operand blocks and line exponents start.
+struct __align__(16) Work {
   int point;
   short m, ch, rt, ct;
+  int nk;
+  unsigned bl, br, el, er;  // first left and right block, left and right tile of exponents
 };
 
 // Shared-memory matrix descriptor, K-major, no swizzle: lbo between the two
@@ -304,30 +310,24 @@ __device__ __forceinline__ bool pair_all(bool v, int pair) {
   return r != 0;
 }
 
-struct Tile {
-  int N, D, nk, r0, c0;
-  Geom g;
-  const ulonglong2 *L, *R;
-  const int *eL, *eR;
-};
-__device__ __forceinline__ bool tile_of(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                                        const X64Pt *__restrict__ xp, const Work &w, Tile &t) {
-  if (!io[w.point].active) return false;
-  const PointDesc &P = pts[w.point];
-  const X64Pt &x = xp[w.point];
-  t.N = P.N;
-  t.g = geom(w.ch, P.N, w.m);
-  t.D = t.g.D;
-  t.nk = (w.ch == CH_DPH ? 2 : 1) * (d16(t.D) / KS);
-  t.r0 = w.rt * LINES;
-  t.c0 = w.ct * LINES;
-  const int pi = w.ch * (2 * P.N - 1) + w.m, nct = (P.N + LINES - 1) / LINES;
-  const uint4 pr = x.prod[pi];
-  t.L = x.L + (size_t)(pr.x + w.rt * t.nk) * BLK;
-  t.R = x.R + (size_t)(pr.y + w.ct * t.nk) * BLK;
-  t.eL = x.eL + (size_t)(pr.z + w.rt) * LINES;
-  t.eR = x.eR + ((size_t)pi * nct + w.ct) * LINES;
-  return true;
+// What the roles read first on the CTA's next tiles, brought into the L1 cache one
+// tile ahead by the loader's idle lanes (plain loads whose values nothing waits
+// for).
+__device__ __forceinline__ void touch(const void *p) {
+  uint32_t v;
+  asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(v) : "l"(p));
+}
+__device__ __forceinline__ void look_ahead(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
+                                           const X64Pt *__restrict__ xp, const Work *__restrict__ work, int wi, int w1,
+                                           int lane) {
+  if (wi + 1 < w1) {
+    const Work n = work[wi + 1];
+    if (lane == 1) touch(&io[n.point].active);
+    if (lane == 2) touch(&pts[n.point].N);
+    if (lane == 3) touch(&xp[n.point].L);
+    if (lane == 4) touch(&xp[n.point].PX);
+  }
+  if (wi + 2 < w1 && lane == 5) touch(work + wi + 2);
 }
 
 // Digits `sel` of two values as a pair of FP16.  hi: the byte lies in the high
@@ -384,20 +384,25 @@ __device__ __forceinline__ void store_digits(uint8_t *dst, const uint4 (&v)[8]) 
   store_digit<6, LEFT>(dst, v);
 }
 
-__device__ __forceinline__ void tmem_ld2(uint32_t taddr, float &a, float &b) {
-  uint32_t r0, r1;
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(taddr));
-  a = __uint_as_float(r0);
-  b = __uint_as_float(r1);
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
 }
 // The accumulators of one entry as one integer: the sum of the X_L X_R in units
 // of 2^57.  (The three last join in FP32 first, which loses less than 2^-3 of
 // the result's unit.)
-__device__ __forceinline__ long long join(const float (&d)[NACC]) {
-  const long long hi = (long long)__float2int_rn(d[0]) * 65536 +
-                       ((long long)__float2int_rn(d[1]) * 256 + __float2int_rn(d[2]));
-  const long long lo = (long long)__float2int_rn(d[3]) * 32768 +
-                       ((long long)__float2int_rn(d[4]) * 128 + __float2int_rn(fmaf(fmaf(d[7], 1.f / 256.f, d[6]), 1.f / 512.f, 0.5f * d[5])));
+template <int W>
+__device__ __forceinline__ long long join(const float (&d)[NACC][W], int c) {
+  const long long hi = (long long)__float2int_rn(d[0][c]) * 65536 +
+                       ((long long)__float2int_rn(d[1][c]) * 256 + __float2int_rn(d[2][c]));
+  const long long lo =
+      (long long)__float2int_rn(d[3][c]) * 32768 +
+      ((long long)__float2int_rn(d[4][c]) * 128 +
+       __float2int_rn(fmaf(fmaf(d[7][c], 1.f / 256.f, d[6][c]), 1.f / 512.f, 0.5f * d[5][c])));
   return (hi << 23) + lo;
 }
 // s 2^e as FP64, rounded once, on the integer pipe (e within +-900: normal).
@@ -422,11 +427,11 @@ __device__ __forceinline__ double scaled(long long s, int e) {
 
 // Row pointer of local row rr in the channel's own layout (pp: natural, dph: X,
 // xph: W).
-__device__ __forceinline__ double2 *out_row(int ch, double2 *kN, const X64Pt &x, const Tile &t, int rr) {
-  const int N = t.N, a = t.g.row_lo + rr;
-  if (ch == CH_PP) return kN + ((size_t)a * N + (t.g.x - a)) * N;
-  if (ch == CH_DPH) return x.PX + ((size_t)a * N + (a + t.g.x)) * N;
-  return x.PW + ((size_t)(a + t.g.x) * N + a) * N;
+__device__ __forceinline__ double2 *out_row(int ch, double2 *kN, const X64Pt &x, int N, const Geom &g, int rr) {
+  const int a = g.row_lo + rr;
+  if (ch == CH_PP) return kN + ((size_t)a * N + (g.x - a)) * N;
+  if (ch == CH_DPH) return x.PX + ((size_t)a * N + (a + g.x)) * N;
+  return x.PW + ((size_t)(a + g.x) * N + a) * N;
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
@@ -465,15 +470,17 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t it = 0;
     bool ok = true;
     for (int wi = w0; wi < w1 && ok; ++wi) {
-      Tile t;
-      if (!tile_of(pts, io, xp, work[wi], t)) continue;
-      for (int kb = 0; kb < t.nk; ++kb, ++it) {
+      const Work w = work[wi];
+      look_ahead(pts, io, xp, work, wi, w1, lane);
+      if (!io[w.point].active) continue;
+      const ulonglong2 *L = xp[w.point].L + (size_t)w.bl * BLK, *R = xp[w.point].R + (size_t)w.br * BLK;
+      for (int kb = 0; kb < w.nk; ++kb, ++it) {
         const int j = it % NRAW;
         if (!(ok = wwait(&raw_empty[j], ((it / NRAW) & 1u) ^ 1u, err, abort_flag))) break;
         if (lane == 0) {
           arrive_expect_tx(&raw_full[j], RAW_STAGE);
-          bulk_copy(raws + j * RAW_STAGE, t.L + (size_t)kb * BLK, BLK_BYTES, &raw_full[j]);
-          bulk_copy(raws + j * RAW_STAGE + BLK_BYTES, t.R + (size_t)kb * BLK, BLK_BYTES, &raw_full[j]);
+          bulk_copy(raws + j * RAW_STAGE, L + (size_t)kb * BLK, BLK_BYTES, &raw_full[j]);
+          bulk_copy(raws + j * RAW_STAGE + BLK_BYTES, R + (size_t)kb * BLK, BLK_BYTES, &raw_full[j]);
         }
         __syncwarp();
       }
@@ -490,9 +497,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t it = 0;
     bool ok = true;
     for (int wi = w0; wi < w1 && ok; ++wi) {
-      Tile t;
-      if (!tile_of(pts, io, xp, work[wi], t)) continue;
-      for (int kb = 0; kb < t.nk; ++kb, ++it) {
+      const Work w = work[wi];
+      if (!io[w.point].active) continue;
+      for (int kb = 0; kb < w.nk; ++kb, ++it) {
         const int j = it % NRAW, s = it % NOP;
         if (!(ok = wwait(&raw_full[j], (it / NRAW) & 1u, err, abort_flag))) break;
         const uint8_t *raw = raws + j * RAW_STAGE + src;
@@ -519,12 +526,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t it = 0, use = 0;
     bool ok = true;
     for (int wi = w0; wi < w1 && ok; ++wi) {
-      Tile t;
-      if (!tile_of(pts, io, xp, work[wi], t)) continue;
+      const Work w = work[wi];
+      if (!io[w.point].active) continue;
       if (!(ok = wwait(tempty, (use & 1u) ^ 1u, err, abort_flag))) break;
       ++use;
       tc_after();
-      for (int kb = 0; kb < t.nk; ++kb, ++it) {
+      for (int kb = 0; kb < w.nk; ++kb, ++it) {
         const int s = it % NOP;
         if (!(ok = wwait(&op_full[s], (it / NOP) & 1u, err, abort_flag))) break;
         tc_after();
@@ -576,38 +583,38 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t use = 0;
     bool ok = true;
     for (int wi = w0; wi < w1 && ok; ++wi) {
-      Tile t;
       const Work w = work[wi];
-      if (!tile_of(pts, io, xp, w, t)) continue;
+      if (!io[w.point].active) continue;
+      const int N = pts[w.point].N, r0 = w.rt * LINES + rl, c0 = w.ct * LINES + cb;
+      const Geom g = geom(w.ch, N, w.m);
       double2 *kN = static_cast<double2 *>(io[w.point].dgam);
       const X64Pt &x = xp[w.point];
-      const int el = (t.r0 + rl + lane < t.D ? t.eL[rl + lane] : 0) + 57 - 2 * FIX;
-      const int er = lane < EPI_CPW && t.c0 + cb + lane < t.N ? t.eR[cb + lane] : 0;
+      const int el = (r0 + lane < g.D ? x.eL[(size_t)w.el * LINES + rl + lane] : 0) + 57 - 2 * FIX;
+      const int er = lane < EPI_CPW && c0 + lane < N ? x.eR[(size_t)w.er * LINES + cb + lane] : 0;
       // both warps of a pair leave together when a wait gave up
       if (!(ok = pair_all(wwait(tfull, use & 1u, err, abort_flag), pair))) break;
       ++use;
       tc_after();
       long long s[EPI_CPW];
 #pragma unroll
-      for (int c = 0; c < EPI_CPW; c += 2) {
-        float a[NACC], b[NACC];
+      for (int c = 0; c < EPI_CPW; c += 4) {
+        float a[NACC][4];
 #pragma unroll
-        for (int g = 0; g < NACC; ++g) tmem_ld2(tl + g * LINES + c, a[g], b[g]);
+        for (int q = 0; q < NACC; ++q) tmem_ld4(tl + q * LINES + c, a[q]);
         tmem_wait_ld();
-        s[c] = join(a);
-        s[c + 1] = join(b);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[c + i] = join(a, i);
       }
       tc_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty);
-      const bool live = t.c0 + cb < t.N;  // (uniform over the pair)
 #pragma unroll
-      for (int c0 = 0; c0 < EPI_CPW; c0 += EPI_COLS) {
-        if (!live) break;
+      for (int cc = 0; cc < EPI_CPW; cc += EPI_COLS) {
+        if (c0 + cc >= N) break;  // (uniform over the pair)
 #pragma unroll
         for (int c = 0; c < EPI_COLS; ++c)
           *reinterpret_cast<double *>(buf + lane * (EPI_COLS * 16) + ((c ^ ((lane >> 1) & 3)) << 4) + comp * 8) =
-              scaled(s[c0 + c], el + __shfl_sync(0xffffffffu, er, c0 + c));
+              scaled(s[cc + c], el + __shfl_sync(0xffffffffu, er, cc + c));
         asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
         // each warp of the pair stores 16 of the 32 rows, 64 bytes a row
 #pragma unroll
@@ -615,8 +622,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           const int row = comp * 16 + (lane >> 2) + 8 * i, c = lane & 3;
           const double2 z =
               *reinterpret_cast<const double2 *>(buf + row * (EPI_COLS * 16) + ((c ^ ((row >> 1) & 3)) << 4));
-          const int rr = t.r0 + rl + row, cc = t.c0 + cb + c0 + c;
-          if (rr < t.D && cc < t.N) out_row(w.ch, kN, x, t, rr)[cc] = z;
+          const int col = c0 + cc + c;
+          if (r0 + row < g.D && col < N) out_row(w.ch, kN, x, N, g, r0 + row)[col] = z;
         }
         asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
       }
@@ -629,8 +636,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // ------------------------------------------------------------- combine ----
-// dGamma = T Lambda ((direct - pp) - crossed), the enabled channels, into the
-// natural layout (the pp products are there already).  A thread takes four consecutive
+// dGamma = (pp + direct) + crossed, the enabled channels, into the natural
+// layout (the pp products are there already).  A thread takes four consecutive
 // i1 of one (i2, i3): 64 contiguous bytes of a W row; a warp covers 4 i2 (64
 // bytes of each X row) x 8 i3 (128 bytes of each natural row).
 __global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict__ pts,
@@ -646,7 +653,6 @@ __global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict
             i3 = 32 * blockIdx.x + 8 * ((t >> 5) & 3) + (t & 7);
   if (i1 >= N || i2 >= N || i3 >= N) return;
   double2 *out = static_cast<double2 *>(o.dgam);
-  const double sc = pts[pi].T * (*o.lam);
   const double2 z = make_double2(0.0, 0.0);
   double2 a[4], b[4], c[4];
 #pragma unroll
@@ -658,9 +664,7 @@ __global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict
   }
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    if (i1 + j < N)
-      out[((size_t)(i1 + j) * N + i2) * N + i3] =
-          make_double2(sc * ((b[j].x - a[j].x) - c[j].x), sc * ((b[j].y - a[j].y) - c[j].y));
+    if (i1 + j < N) out[((size_t)(i1 + j) * N + i2) * N + i3] = cadd(cadd(a[j], b[j]), c[j]);
 }
 }  // namespace x64
 
@@ -754,21 +758,23 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
     s.n3 = (size_t)N * N * N;
     tab[i].resize(3 * (2 * N - 1));
     const int nct = (N + x64::LINES - 1) / x64::LINES;
-    s.tileR = (size_t)3 * (2 * N - 1) * nct;
     for (int ch = 0; ch < 3; ++ch) {
       if (!(chmask >> ch & 1)) continue;
       for (int m = 0; m < 2 * N - 1; ++m) {
         const Geom g = geom(ch, N, m);
         const int nk = (ch == CH_DPH ? 2 : 1) * (x64::d16(g.D) / x64::KS);
         const int nrt = (g.D + x64::LINES - 1) / x64::LINES;
-        tab[i][ch * (2 * N - 1) + m] = make_uint4((unsigned)s.blkL, (unsigned)s.blkR, (unsigned)s.tileL, 0u);
+        const uint4 t = make_uint4((unsigned)s.blkL, (unsigned)s.blkR, (unsigned)s.tileL, (unsigned)s.tileR);
+        tab[i][ch * (2 * N - 1) + m] = t;
         s.blkL += (size_t)nrt * nk;
         s.blkR += (size_t)nct * nk;
         s.tileL += nrt;
+        s.tileR += nct;
         // the drain of a tile's accumulators costs about two k-steps
         for (int rt = 0; rt < nrt; ++rt)
           for (int ct = 0; ct < nct; ++ct)
-            tiles[i].push_back({nk + 2, x64::Work{i, (short)m, (short)ch, (short)rt, (short)ct}});
+            tiles[i].push_back({nk + 2, x64::Work{i, (short)m, (short)ch, (short)rt, (short)ct, nk, t.x + rt * nk,
+                                                  t.y + ct * nk, t.z + rt, t.w + ct}});
       }
     }
   }

@@ -13,7 +13,8 @@ constexpr int X64_MIN_N = 28;
 
 // Device-side operands of one point (frg_x64.cu).
 struct X64Pt {
-  const uint4 *prod;   // per ch * (2N - 1) + m: first left and right operand block, first left tile; null: not on this path
+  const uint4 *prod;   // per ch * (2N - 1) + m: first left and right operand block, first left and right tile of
+                       // exponents; null: not on this path
   ulonglong2 *L, *R;   // fixed-point operand blocks (re, im), 16 k x 64 lines each
   int *eL, *eR;        // line exponents, 64 per tile
   double2 *PX, *PW;    // direct (layout X) and crossed (layout W) channel outputs
