@@ -39,7 +39,8 @@ struct frg_ctx {
   unsigned *h_err = nullptr;   // pinned mirror
   RhsIO *d_io_stage = nullptr; // flow evaluations
   RhsIO *d_io_user = nullptr;  // stand-alone evaluations
-  // contraction work lists: [ch] all points cost-sorted; per-point slices
+  // CUDA-core contraction work lists (FP64 points that are neither small nor
+  // sliced): [ch] all points cost-sorted; per-point slices
   WorkItem *d_work_all[3] = {nullptr, nullptr, nullptr};
   int nwork_all[3] = {0, 0, 0};
   WorkItem *d_work_pt[3] = {nullptr, nullptr, nullptr};
@@ -710,10 +711,10 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
       ctx->work_off[ch].push_back(0);
       for (int i = 0; i < n_points; ++i) {
         one.clear();
-        build_work(ch, i, ctx->params[i].N_f, one);
+        if (!x64_has(ctx->x64, i) && !small_point(ctx, i)) build_work(ch, i, ctx->params[i].N_f, one);
         std::stable_sort(one.begin(), one.end(), [](auto &a, auto &b) { return a.first > b.first; });
         for (auto &x : one) per.push_back(x.second);
-        if (!x64_has(ctx->x64, i) && !small_point(ctx, i)) all.insert(all.end(), one.begin(), one.end());
+        all.insert(all.end(), one.begin(), one.end());
         ctx->work_off[ch].push_back((int)per.size());
       }
       std::stable_sort(all.begin(), all.end(), [](auto &a, auto &b) { return a.first > b.first; });
@@ -725,12 +726,7 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
         return bail(FRG_ENOMEM);
       cudaMemcpy(ctx->d_work_all[ch], allw.data(), sizeof(WorkItem) * allw.size(), cudaMemcpyHostToDevice);
       cudaMemcpy(ctx->d_work_pt[ch], per.data(), sizeof(WorkItem) * per.size(), cudaMemcpyHostToDevice);
-      for (int i = 0; i < n_points; ++i)
-        if (x64_has(ctx->x64, i))
-          x64_set_work(ctx->x64, i, ch, ctx->d_work_pt[ch] + ctx->work_off[ch][i],
-                       ctx->work_off[ch][i + 1] - ctx->work_off[ch][i]);
     }
-    if (ctx->x64 && x64_upload(ctx->x64) != 0) return bail(FRG_ECUDA);
   } else {
     int rc = tc_plan_create(&ctx->tc, ctx->hpts, ctx->params, ctx->precision, ctx->d_pts, ctx->d_err, why,
                             TcTune(), tc_schedules(ctx));

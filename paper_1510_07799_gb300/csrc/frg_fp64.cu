@@ -12,8 +12,8 @@
 
 #include "frg.h"
 #include "frg_common.cuh"
+#include "frg_f64elem.cuh"
 #include "frg_split.cuh"
-#include "frg_x64.cuh"
 
 namespace frg {
 
@@ -336,47 +336,6 @@ int launch_add_tails(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
 // ------------------------------------------------- FP64 contraction ----
 constexpr int F64_TK = 16, F64_THREADS = 256;  // tile rows / columns: F64_TM, F64_TN (frg_common.cuh)
 
-// Left[r][k] (r local row, k in [0,K)) of channel CH for transfer geometry g.
-template <int CH>
-__device__ __forceinline__ double2 left_elem(const PointDesc &P, const void *gam, const Geom &g, int r, int k) {
-  const int N = P.N;
-  if (CH == CH_PP) {
-    const int a = g.row_lo + r, p = g.p_lo + k, s = g.x;
-    return cmul(vload<false>(gam, N, P.U, a, s - a, p), P.Lpp[(size_t)s * N + p]);
-  } else if (CH == CH_DPH) {
-    const int t = g.x, k1 = g.row_lo + r;
-    const int half = k >= g.D;
-    const int p = g.p_lo + (half ? k - g.D : k);
-    const double2 L = P.Lph[(size_t)(-t + N - 1) * N + p];
-    const double2 A = vload<false>(gam, N, P.U, k1, p, k1 + t);
-    if (!half) {
-      const double2 C = vload<false>(gam, N, P.U, k1, p, p - t);
-      return cmul(make_double2(2.0 * A.x - C.x, 2.0 * A.y - C.y), L);
-    }
-    return cmul(make_double2(-A.x, -A.y), L);
-  } else {
-    const int Q = g.x, k3 = g.row_lo + r, p = g.p_lo + k;
-    return cmul(vload<false>(gam, N, P.U, p, k3 + Q, k3), P.Lph[(size_t)(Q + N - 1) * N + p]);
-  }
-}
-
-template <int CH>
-__device__ __forceinline__ double2 right_elem(const PointDesc &P, const void *gam, const Geom &g, int k, int c) {
-  const int N = P.N;
-  if (CH == CH_PP) {
-    const int p = g.p_lo + k, s = g.x;
-    return vload<false>(gam, N, P.U, p, s - p, c);
-  } else if (CH == CH_DPH) {
-    const int t = g.x;
-    const int half = k >= g.D;
-    const int p = g.p_lo + (half ? k - g.D : k);
-    return half ? vload<false>(gam, N, P.U, p - t, c, c - t) : vload<false>(gam, N, P.U, p - t, c, p);
-  } else {
-    const int Q = g.x, p = g.p_lo + k;
-    return vload<false>(gam, N, P.U, c, p + Q, p);
-  }
-}
-
 // Output element (local row r, column c) -> flat vertex index.
 template <int CH>
 __device__ __forceinline__ size_t out_index(int N, const Geom &g, int r, int c) {
@@ -390,15 +349,6 @@ __device__ __forceinline__ size_t out_index(int N, const Geom &g, int r, int c) 
     const int k3 = g.row_lo + r;
     return ((size_t)c * N + (k3 + g.x)) * N + k3;
   }
-}
-
-// Output element in the channel's own layout (dph: X, xph: W).
-template <int CH>
-__device__ __forceinline__ size_t own_index(int N, const Geom &g, int r, int c) {
-  const int a = g.row_lo + r;
-  if (CH == CH_PP) return out_index<CH>(N, g, r, c);
-  if (CH == CH_DPH) return ((size_t)a * N + (a + g.x)) * N + c;
-  return ((size_t)(a + g.x) * N + a) * N + c;
 }
 
 struct F64Smem {
@@ -475,41 +425,6 @@ __global__ void __launch_bounds__(F64_THREADS)
     const size_t at = out_index<CH>(P.N, g, r, c);
     out[at] = ACCUM ? cadd(out[at], v) : v;
   });
-}
-
-// The same tiles for the points whose operands the sliced tensor-core products
-// could not take (X64Pt.bad), into the buffers those products write; returns at
-// once for the others.
-__global__ void __launch_bounds__(F64_THREADS)
-    k_x64_fallback(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
-                   int p0, int p1, int chmask) {
-  __shared__ F64Smem sm;
-  for (int pi = p0; pi < p1; ++pi) {
-    const X64Pt &x = xp[pi];
-    const RhsIO &o = io[pi];
-    if (!x.prod || !o.active || *x.bad == 0) continue;
-    const PointDesc &P = pts[pi];
-    for (int ch = 0; ch < 3; ++ch) {
-      if (!(chmask >> ch & 1)) continue;
-      double2 *out = ch == CH_PP ? static_cast<double2 *>(o.dgam) : ch == CH_DPH ? x.PX : x.PW;
-      for (int i = blockIdx.x; i < x.nwork[ch]; i += gridDim.x) {
-        const WorkItem w = x.work[ch][i];
-        if (ch == CH_PP)
-          f64_tile<CH_PP>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_PP>(P.N, g, r, c)] = v; });
-        else if (ch == CH_DPH)
-          f64_tile<CH_DPH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_DPH>(P.N, g, r, c)] = v; });
-        else
-          f64_tile<CH_XPH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) { out[own_index<CH_XPH>(P.N, g, r, c)] = v; });
-      }
-    }
-  }
-}
-
-int launch_x64_fallback(const PointDesc *d_pts, const RhsIO *d_io, const X64Pt *d_x, int p0, int p1, int chmask,
-                        cudaStream_t st) {
-  k_x64_fallback<<<304, F64_THREADS, 0, st>>>(d_pts, d_io, d_x, p0, p1, chmask);
-  FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 // pp stores, dph and xph accumulate: the three channels run in this order so

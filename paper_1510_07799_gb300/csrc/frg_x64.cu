@@ -31,9 +31,9 @@
 // operands into blocks of 16 k x 64 lines; k_x64_products multiplies them
 // (persistent CTAs over a longest-first tile schedule); k_x64_combine sums the
 // channels into the natural layout.  Lines that cannot be converted (non-finite
-// values, exponents beyond 2^+-400) mark their point, whose products the
-// CUDA-core kernel then forms instead (k_x64_fallback in frg_fp64.cu).
-// Measured, one rhs (all channels): N = 128 6086 -> 330 us, N = 64 674 -> 78 us
+// values, exponents beyond 2^+-400) mark their point, whose entries k_x64_combine
+// then sums in FP64 instead.
+// Measured, one rhs (all channels): N = 128 6086 -> 330 us, N = 64 674 -> 73 us
 // (CUDA cores -> slices).
 #include <cuda_runtime.h>
 
@@ -43,6 +43,7 @@
 
 #include "frg.h"
 #include "frg_common.cuh"
+#include "frg_f64elem.cuh"
 #include "frg_ptx.cuh"
 #include "frg_x64.cuh"
 
@@ -70,17 +71,22 @@ constexpr int E_LIM = 400;                  // line exponents the path accepts
 // registers, the block finds each line's largest magnitude, and the values leave
 // in fixed point.  Bound by the FP64 multiplications of the weights and by the
 // gathers (16-byte elements, one 32-byte sector each wherever the line and the
-// contraction index both stride through the vertex): 114 us at N = 128 for 302 MB
-// written and 15 M entries gathered, the FP64 pipe half busy; 159 us with the
-// lines staged in shared memory between the gather and the conversion.
+// contraction index both stride through the vertex): 99 us at N = 128 for 302 MB
+// written and 15 M entries gathered; 159 us with the lines staged in shared memory
+// between the gather and the conversion.  (The two operands as launches of their
+// own, the right one beside the bubble weights: 130 us, the left one alone takes
+// as long as both at N = 64.)
 constexpr int PAN_LINES = 8;
-constexpr int PAN_U = 4;  // k per thread and range
+// k per thread and range: eight on the larger grids (more gathers in flight: N =
+// 128 99 against 111 us), four on the smaller ones (more warps: N = 64 18.0
+// against 19.3 us).
+static int panel_u(int maxN) { return maxN > 80 ? 8 : 4; }
 // Elements along the contraction axis: one or two (direct channel) ranges of D
 // padded to whole blocks.
 __host__ __device__ inline int d16(int D) { return (D + KS - 1) / KS * KS; }
-// Threads of a block: eight per k, and at most PAN_U k each.
-static int panel_threads(int maxN) { return std::max(64, (d16(maxN) + 15) / 16 * 32); }
-static_assert(2 * PAN_U == PAN_LINES, "a block of twice as many threads as k takes PAN_U of them per thread");
+// Threads of a block: eight per k, and at most U k each (8 / U threads per k of the
+// padded range, in whole warps).
+static int panel_threads(int maxN) { return std::max(64, (d16(maxN) * (PAN_LINES / panel_u(maxN)) + 31) / 32 * 32); }
 
 __device__ __forceinline__ unsigned mag(double2 v) {
   const unsigned a = (unsigned)__double2hiint(v.x) & 0x7fffffffu, b = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
@@ -139,7 +145,7 @@ __device__ __forceinline__ void gather(const PointDesc &P, const double2 *__rest
   }
 }
 
-template <int CH, bool LEFT>
+template <int CH, bool LEFT, int U>
 __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const X64Pt &x, int m, int oct,
                                       double2 *sw, unsigned *smax) {
   const int N = P.N;
@@ -155,9 +161,9 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
     const double2 *L = CH == CH_PP ? P.Lpp + (size_t)m * N : P.Lph + (size_t)(CH == CH_DPH ? 2 * N - 2 - m : m) * N;
     for (int k = tid; k < D; k += blockDim.x) sw[k] = cscale(L[g.p_lo + k], sc);
   }
-  double2 v[PAN_U], v2[PAN_U];
+  double2 v[U], v2[U];
 #pragma unroll
-  for (int u = 0; u < PAN_U; ++u) {
+  for (int u = 0; u < U; ++u) {
     const int k = (tid >> 3) + u * kstep;
     v[u] = v2[u] = make_double2(0.0, 0.0);
     if (k < D && line < nl) gather<CH, LEFT>(P, V, g, line0 + line, k, v[u], v2[u]);
@@ -166,13 +172,13 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
   __syncthreads();
   unsigned um = 0u;
 #pragma unroll
-  for (int u = 0; u < PAN_U; ++u) {
+  for (int u = 0; u < U; ++u) {
     const int k = (tid >> 3) + u * kstep;
     if (LEFT && k < D) {
       const double2 w = sw[k];
       if (CH == CH_DPH) {
         const double2 A = v[u], C = v2[u];
-        v[u] = cmul(make_double2(2.0 * A.x - C.x, 2.0 * A.y - C.y), w);
+        v[u] = cmul(make_double2(fma(2.0, A.x, -C.x), fma(2.0, A.y, -C.y)), w);
         v2[u] = cmul(make_double2(-A.x, -A.y), w);
       } else {
         v[u] = cmul(v[u], w);
@@ -199,7 +205,7 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
   ulonglong2 *dst = (LEFT ? x.L + (size_t)(pr.x + tile * nk) * BLK : x.R + (size_t)(pr.y + tile * nk) * BLK) + l0;
   if (line >= nl) return;
 #pragma unroll
-  for (int u = 0; u < PAN_U; ++u) {
+  for (int u = 0; u < U; ++u) {
     const int k = (tid >> 3) + u * kstep;
     if (k >= D16) break;
     dst[(size_t)k * LINES] = make_ulonglong2(to_fixed(v[u].x, e), to_fixed(v[u].y, e));
@@ -210,9 +216,10 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
 
 // grid: (line octets of the left, then of the right operand; transfers;
 // point x channel)
-__global__ void __launch_bounds__(2 * FRG_MAX_N, 2) k_x64_panels(const PointDesc *__restrict__ pts,
-                                                      const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
-                                                      int p0, int chmask) {
+template <int U>
+__global__ void __launch_bounds__(FRG_MAX_N *PAN_LINES / U, U == 8 ? 3 : 2)
+    k_x64_panels(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp, int p0,
+                 int chmask) {
   __shared__ double2 sw[FRG_MAX_N];
   __shared__ unsigned smax[PAN_LINES];
   const int pi = p0 + blockIdx.z / 3, ch = blockIdx.z % 3;
@@ -225,18 +232,18 @@ __global__ void __launch_bounds__(2 * FRG_MAX_N, 2) k_x64_panels(const PointDesc
   const int b = blockIdx.x;
   if (b < half) {
     if (ch == CH_PP)
-      panel<CH_PP, true>(P, o, x, m, b, sw, smax);
+      panel<CH_PP, true, U>(P, o, x, m, b, sw, smax);
     else if (ch == CH_DPH)
-      panel<CH_DPH, true>(P, o, x, m, b, sw, smax);
+      panel<CH_DPH, true, U>(P, o, x, m, b, sw, smax);
     else
-      panel<CH_XPH, true>(P, o, x, m, b, sw, smax);
+      panel<CH_XPH, true, U>(P, o, x, m, b, sw, smax);
   } else {
     if (ch == CH_PP)
-      panel<CH_PP, false>(P, o, x, m, b - half, sw, smax);
+      panel<CH_PP, false, U>(P, o, x, m, b - half, sw, smax);
     else if (ch == CH_DPH)
-      panel<CH_DPH, false>(P, o, x, m, b - half, sw, smax);
+      panel<CH_DPH, false, U>(P, o, x, m, b - half, sw, smax);
     else
-      panel<CH_XPH, false>(P, o, x, m, b - half, sw, smax);
+      panel<CH_XPH, false, U>(P, o, x, m, b - half, sw, smax);
   }
 }
 
@@ -640,28 +647,59 @@ __global__ void __launch_bounds__(THREADS, 1)
 // layout (the pp products are there already).  A thread takes four consecutive
 // i1 of one (i2, i3): 64 contiguous bytes of a W row; a warp covers 4 i2 (64
 // bytes of each X row) x 8 i3 (128 bytes of each natural row).
-__global__ void __launch_bounds__(256) k_x64_combine(const PointDesc *__restrict__ pts,
+// The entries of a marked point are summed here, term by term as the tiles of the
+// CUDA-core products do (k_contract_fp64).
+template <int CH>
+__device__ double2 entry_sum(const PointDesc &P, const void *gam, int m, int row, int col) {
+  const Geom g = geom(CH, P.N, m);
+  double2 acc = make_double2(0.0, 0.0);
+  for (int k = 0; k < g.K; ++k)
+    cfma(acc, left_elem<CH>(P, gam, g, row - g.row_lo, k), right_elem<CH>(P, gam, g, k, col));
+  return acc;
+}
+__device__ __noinline__ void marked_entry(const PointDesc &P, const RhsIO &o, int i1, int i2, int i3, int chmask) {
+  const int N = P.N;
+  const double sc = P.T * (*o.lam);
+  double2 v = make_double2(0.0, 0.0);
+  if (chmask & 1) v = cscale(entry_sum<CH_PP>(P, o.gam, i1 + i2, i1, i3), -sc);
+  if (chmask & 2) v = cadd(v, cscale(entry_sum<CH_DPH>(P, o.gam, i3 - i1 + N - 1, i1, i2), sc));
+  if (chmask & 4) v = cadd(v, cscale(entry_sum<CH_XPH>(P, o.gam, i2 - i3 + N - 1, i3, i1), -sc));
+  static_cast<double2 *>(o.dgam)[((size_t)i1 * N + i2) * N + i3] = v;
+}
+__global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restrict__ pts,
                                                      const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
                                                      int p0, int nz, int chmask) {
   const int pi = p0 + blockIdx.z / nz;
   const RhsIO &o = io[pi];
   const X64Pt &x = xp[pi];
   if (!o.active || !x.prod) return;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z % nz == 0 && threadIdx.x == 0) *x.bad = 0;
-  const int N = pts[pi].N, t = threadIdx.x;
-  const int i1 = 4 * (blockIdx.z % nz), i2 = 8 * blockIdx.y + 4 * (t >> 7) + ((t >> 3) & 3),
-            i3 = 32 * blockIdx.x + 8 * ((t >> 5) & 3) + (t & 7);
-  if (i1 >= N || i2 >= N || i3 >= N) return;
+  const PointDesc &P = pts[pi];
+  const int N = P.N, t = threadIdx.x;
+  const int i1 = 4 * (blockIdx.z % nz), b2 = 8 * blockIdx.y, b3 = 32 * blockIdx.x;
+  if (i1 >= N || b2 >= N || b3 >= N) return;
+  const int i2 = b2 + 4 * (t >> 7) + ((t >> 3) & 3), i3 = b3 + 8 * ((t >> 5) & 3) + (t & 7);
+  const int bad = x.bad[0];
   double2 *out = static_cast<double2 *>(o.dgam);
   const double2 z = make_double2(0.0, 0.0);
+  const bool on = i2 < N && i3 < N;
   double2 a[4], b[4], c[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const bool in = i1 + j < N;
+    const bool in = on && i1 + j < N;
     a[j] = in && (chmask & 1) ? out[((size_t)(i1 + j) * N + i2) * N + i3] : z;
     b[j] = in && (chmask & 2) ? x.PX[((size_t)(i1 + j) * N + i3) * N + i2] : z;
     c[j] = in && (chmask & 4) ? x.PW[((size_t)i2 * N + i3) * N + i1 + j] : z;
   }
+  if (bad) {
+    if (on)
+      for (int j = 0; j < 4 && i1 + j < N; ++j) marked_entry(P, o, i1 + j, i2, i3, chmask);
+    // the point's last block (every block has read the mark) clears it
+    __syncthreads();
+    const int blocks = ((N + 3) / 4) * ((N + 7) / 8) * ((N + 31) / 32);
+    if (t == 0 && atomicAdd(&x.bad[1], 1) == blocks - 1) x.bad[0] = x.bad[1] = 0;
+    return;
+  }
+  if (!on) return;
 #pragma unroll
   for (int j = 0; j < 4; ++j)
     if (i1 + j < N) out[((size_t)(i1 + j) * N + i2) * N + i3] = cadd(cadd(a[j], b[j]), c[j]);
@@ -803,8 +841,8 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
     return 0;
   }
   bool ok = cudaMalloc(&p->d_x, sizeof(X64Pt) * n) == cudaSuccess &&
-            cudaMalloc(&p->d_bad, sizeof(int) * n) == cudaSuccess &&
-            cudaMemset(p->d_bad, 0, sizeof(int) * n) == cudaSuccess &&
+            cudaMalloc(&p->d_bad, sizeof(int) * 2 * n) == cudaSuccess &&
+            cudaMemset(p->d_bad, 0, sizeof(int) * 2 * n) == cudaSuccess &&
             cudaFuncSetAttribute(x64::k_x64_products, cudaFuncAttributeMaxDynamicSharedMemorySize, x64::SMEM) ==
                 cudaSuccess;
   for (int i = 0; i < n && ok; ++i) {
@@ -823,7 +861,7 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
     x.PX = reinterpret_cast<double2 *>(b);
     b += align256(s.n3 * sizeof(double2));
     x.PW = reinterpret_cast<double2 *>(b);
-    x.bad = p->d_bad + i;
+    x.bad = p->d_bad + 2 * i;
     void *t = nullptr;
     ok = cudaMalloc(&t, sizeof(uint4) * tab[i].size()) == cudaSuccess;
     if (!ok) break;
@@ -838,21 +876,13 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
     for (int i = g.p0; i < g.p1; ++i) all.insert(all.end(), tiles[i].begin(), tiles[i].end());
     ok = upload_sched(g.all, all, sms);
   }
+  ok = ok && cudaMemcpy(p->d_x, p->h.data(), sizeof(X64Pt) * n, cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) {
     x64_destroy(p);
     return -3;
   }
   *out = p;
   return 0;
-}
-
-void x64_set_work(X64Plan *p, int point, int ch, const WorkItem *d_work, int n) {
-  p->h[point].work[ch] = d_work;
-  p->h[point].nwork[ch] = n;
-}
-
-int x64_upload(X64Plan *p) {
-  return cudaMemcpy(p->d_x, p->h.data(), sizeof(X64Pt) * p->h.size(), cudaMemcpyHostToDevice) == cudaSuccess ? 0 : -3;
 }
 
 void x64_destroy(X64Plan *p) {
@@ -885,15 +915,16 @@ int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, in
       s = &p->one[point];
     }
     const int oct = (maxN + x64::PAN_LINES - 1) / x64::PAN_LINES, np = p1 - p0;
-    x64::k_x64_panels<<<dim3(2 * oct, 2 * maxN - 1, 3 * np), x64::panel_threads(maxN), 0, st>>>(d_pts, d_io, p->d_x, p0,
-                                                                                             chmask);
+    const dim3 pg(2 * oct, 2 * maxN - 1, 3 * np);
+    if (x64::panel_u(maxN) == 8)
+      x64::k_x64_panels<8><<<pg, x64::panel_threads(maxN), 0, st>>>(d_pts, d_io, p->d_x, p0, chmask);
+    else
+      x64::k_x64_panels<4><<<pg, x64::panel_threads(maxN), 0, st>>>(d_pts, d_io, p->d_x, p0, chmask);
     x64::k_x64_products<<<s->grid, x64::THREADS, x64::SMEM, st>>>(d_pts, d_io, p->d_x, s->d_work, s->d_start, p->d_err);
-    FRG_COUNT(2);
-    if (launch_x64_fallback(d_pts, d_io, p->d_x, p0, p1, chmask, st) != 0) return -3;
     const int nz = (maxN + 3) / 4;
     x64::k_x64_combine<<<dim3((maxN + 31) / 32, (maxN + 7) / 8, nz * np), 256, 0, st>>>(d_pts, d_io, p->d_x, p0, nz,
                                                                                       chmask);
-    FRG_COUNT(1);
+    FRG_COUNT(3);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }

@@ -18,25 +18,16 @@ struct X64Pt {
   ulonglong2 *L, *R;   // fixed-point operand blocks (re, im), 16 k x 64 lines each
   int *eL, *eR;        // line exponents, 64 per tile
   double2 *PX, *PW;    // direct (layout X) and crossed (layout W) channel outputs
-  int *bad;            // set when a line cannot be sliced (non-finite or extreme values)
-  const WorkItem *work[3];  // CUDA-core tiles of the three channels, for such a point
-  int nwork[3];
+  int *bad;            // [0] set when a line cannot be sliced (non-finite or extreme values); [1] blocks that have seen it
 };
 
 struct X64Plan;
 // Plan for the points with N >= X64_MIN_N.  *out stays null when there is none
 // or the device has no room for the operands (the caller then keeps those
-// points on the CUDA-core path).  work / nwork: per point the CUDA-core tiles.
-// Returns 0, or -3 when a CUDA call failed.
+// points on the CUDA-core path).  Returns 0, or -3 when a CUDA call failed.
 int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, unsigned *d_err);
-void x64_set_work(X64Plan *p, int point, int ch, const WorkItem *d_work, int n);
-int x64_upload(X64Plan *p);
 void x64_destroy(X64Plan *p);
 bool x64_has(const X64Plan *p, int point);
 // Channel products of every point of the plan (point < 0) or of one point.
 int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st);
-// CUDA-core products of the points whose operands could not be sliced
-// (frg_fp64.cu); a single small launch when there is none.
-int launch_x64_fallback(const PointDesc *d_pts, const RhsIO *d_io, const X64Pt *d_x, int p0, int p1, int chmask,
-                        cudaStream_t st);
 }  // namespace frg
