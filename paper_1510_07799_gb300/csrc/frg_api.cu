@@ -240,8 +240,8 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
 // Split paths.  gam (a stand-alone evaluation of one point): the FP64 vertex,
 // regathered here into the operand copies; null: a flow's stage input, whose
 // copies the stage kernels have written.  Side stream: the propagators and the
-// bubble weights (they need the self-energy input alone) beside the regather,
-// then the tail constants.  The contraction's epilogue warps form the self-energy
+// bubble weights (they need the self-energy input alone) beside the regather; the
+// window sums of the tails on a third one.  The contraction's epilogue warps form the self-energy
 // rhs, except with the tails or without channel products: a kernel on the side
 // stream after the regather, then the tails' last kernel, which adds the
 // self-energy's constant to it.  ev (optional, 6 events; everything in turn on
@@ -249,8 +249,8 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
 // such a self-energy kernel), after the channel products (with the self-energy
 // rhs otherwise), after the combine, and the same again.
 static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, const double2 *gam,
-                         cudaEvent_t *ev = nullptr) {
-  cudaStream_t st = ctx->stream, ss = ev ? st : ctx->sstream;
+                         cudaEvent_t *ev = nullptr, bool sig_in_place = false) {
+  cudaStream_t st = ctx->stream, ss = ev ? st : ctx->sstream, ts = ev ? st : ctx->tstream;
   const bool fork = !ev, tails = (ctx->mask & FRG_TAILS) != 0;
   const int chmask = ctx->mask & 7;
   // the reversal reduction's transfers: flows while it is on, every call when
@@ -260,11 +260,12 @@ static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, con
   if (fork) {
     CK(cudaEventRecord(ctx->ev_fork, st), "fork");
     CK(cudaStreamWaitEvent(ss, ctx->ev_fork, 0), "fork");
+    if (tails) CK(cudaStreamWaitEvent(ts, ctx->ev_fork, 0), "fork");
   }
   LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES), "bubble weights");
   if (fork) CK(cudaEventRecord(ctx->ev_join, ss), "join");
   if (tails)
-    LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ss, TAIL_WINDOW), "tail sums");
+    LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ts, TAIL_WINDOW), "tail sums");
   if (ev) CK(cudaEventRecord(ev[1], st), "event");
   if (gam)
     LK(launch_relayout(ctx->d_pts + point, gam, ctx->hpts[point].N, ctx->lb_want, ctx->precision == FRG_BF16X3, st),
@@ -274,10 +275,15 @@ static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, con
     if (fork) {
       CK(cudaEventRecord(ctx->ev_stage, st), "regather");
       CK(cudaStreamWaitEvent(ss, ctx->ev_stage, 0), "regather");
+      if (tails) CK(cudaEventRecord(ctx->ev_tails, ts), "tails");
+      // (the window propagators read the self-energy input that this rhs overwrites)
+      if (tails && sig_in_place) CK(cudaStreamWaitEvent(ss, ctx->ev_tails, 0), "tails");
     }
     LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_SIGMA), "self-energy rhs");
-    if (tails)
+    if (tails) {
+      if (fork) CK(cudaStreamWaitEvent(ss, ctx->ev_tails, 0), "tails");
       LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ss, TAIL_FINISH), "tail constants");
+    }
     if (fork) CK(cudaEventRecord(ctx->ev_sig, ss), "self-energy");
   }
   if (ev) CK(cudaEventRecord(ev[2], st), "event");
@@ -859,7 +865,7 @@ static int rhs_impl(frg_ctx *ctx, int point, double Lambda, const void *d_gamma,
   o.out64 = static_cast<double2 *>(d_dgamma);
   o.out_f32 = 1;
   LK(launch_set_user_io(ctx->d_io_user, ctx->d_ctl, ctx->n, point, o, Lambda, ctx->stream, true), "user io");
-  return run_rhs_split(ctx, ctx->d_io_user, point, static_cast<const double2 *>(d_gamma), ev);
+  return run_rhs_split(ctx, ctx->d_io_user, point, static_cast<const double2 *>(d_gamma), ev, sigma_overlap(o, P.N));
 }
 
 int frg_rhs(frg_ctx *ctx, int point, double Lambda, const void *d_gamma, const void *d_sigma, void *d_dgamma,
@@ -1124,7 +1130,7 @@ int frg_get_state(frg_ctx *ctx, int point, void *d_gamma, void *d_sigma, double 
   const Ctl &c = ctx->h_ctl[point];
   const PointDesc &P = ctx->hpts[point];
   const double2 *y = P.ybuf[c.yslot];
-  if (ctx->split && ctx->rev_on) LK(launch_mirror_state(ctx->d_pts, ctx->n, ctx->stream), "copy state");
+  if (ctx->split && ctx->rev_on) LK(launch_mirror_state(ctx->d_pts + point, 1, ctx->stream), "copy state");
   if (d_gamma) CK(cudaMemcpyAsync(d_gamma, y, (size_t)P.n3 * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream), "copy state");
   if (d_sigma) CK(cudaMemcpyAsync(d_sigma, y + P.n3, (size_t)P.N * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream), "copy state");
   if (Lambda) *Lambda = std::exp(c.t);
@@ -1141,9 +1147,6 @@ int frg_set_state(frg_ctx *ctx, int point, const void *d_gamma, const void *d_si
   if (h > 0.0) return fail(ctx, FRG_EINVAL, "h must be <= 0");
   DevGuard g(ctx->dev);
   const PointDesc &P = ctx->hpts[point];
-  // the other points' states whole before the flows may switch to every
-  // transfer (their stage kernels then read whole states)
-  if (ctx->split && ctx->rev_on) LK(launch_mirror_state(ctx->d_pts, ctx->n, ctx->stream), "set state");
   CK(cudaMemcpyAsync(P.ybuf[0], d_gamma, (size_t)P.n3 * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream), "set state");
   if (d_sigma)
     CK(cudaMemcpyAsync(P.ybuf[0] + P.n3, d_sigma, (size_t)P.N * sizeof(double2), cudaMemcpyDeviceToDevice, ctx->stream), "set state");
@@ -1161,6 +1164,13 @@ int frg_set_state(frg_ctx *ctx, int point, const void *d_gamma, const void *d_si
   CK(cudaStreamSynchronize(ctx->stream), "set state");
   if (ctx->rev_mode == 1) {
     ctx->sym[point] = *ctx->h_asym == 0;
+    // the other points' states whole before the flows switch to every transfer
+    // (their stage kernels then read whole states)
+    if (ctx->rev_on && !ctx->sym[point]) {
+      if (point > 0) LK(launch_mirror_state(ctx->d_pts, point, ctx->stream), "set state");
+      if (point + 1 < ctx->n)
+        LK(launch_mirror_state(ctx->d_pts + point + 1, ctx->n - point - 1, ctx->stream), "set state");
+    }
     int rc = update_reversal(ctx);
     if (rc) return rc;
     CK(cudaStreamSynchronize(ctx->stream), "set state");
@@ -1180,7 +1190,7 @@ int frg_observables(frg_ctx *ctx, int point, frg_obs *out) {
   std::vector<double2> sig(N);
   double2 ueff;
   const double2 *y = P.ybuf[c.yslot];
-  if (ctx->split && ctx->rev_on) LK(launch_mirror_state(ctx->d_pts, ctx->n, ctx->stream), "observables");
+  if (ctx->split && ctx->rev_on) LK(launch_mirror_state(ctx->d_pts + point, 1, ctx->stream), "observables");
   CK(cudaMemcpyAsync(sig.data(), y + P.n3, N * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream), "observables");
   CK(cudaMemcpyAsync(&ueff, y + ((size_t)hN * N + hN) * N + hN, sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream),
      "observables");

@@ -66,7 +66,7 @@ __global__ void k_check_reversal(const double2 *__restrict__ y, int N, int *asym
 // candidate state's vertex for the canonical half only; the readers of a
 // whole state (frg_get_state, frg_observables, a switch to full flows) first
 // fill in the other half as conjugates: y[n3 - 1 - i] = conj(y[i]), i < n3/2,
-// in both state slots of every point whose flow keeps the canonical half.
+// in both state slots of every point of pts whose flow keeps the canonical half.
 __global__ void k_mirror_state(const PointDesc *__restrict__ pts) {
   const PointDesc &P = pts[blockIdx.y];
   if (!P.rev_half) return;

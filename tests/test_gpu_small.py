@@ -60,8 +60,9 @@ def test_self_energy_rhs_in_place(N):
     V = torch.from_numpy(inputs.random_vertex(N, p.U, seed=N)).cuda()
     sig = torch.from_numpy(inputs.random_sigma(N, seed=N)).cuda()
     calls = [lambda *a: frg.rhs_noalloc(p, 0.25, *a)]
-    with frg.Context([p]) as ctx, frg.Context([p], precision="3xtf32") as split:
-        calls += [lambda *a: ctx.rhs(0, 0.25, *a), lambda *a: split.rhs(0, 0.25, *a)]
+    with frg.Context([p]) as ctx, frg.Context([p], precision="3xtf32") as split, \
+            frg.Context([p], precision="bf16x3", channel_mask=frg.CH_ALL | frg.TAILS) as tails:
+        calls += [lambda *a, c=c: c.rhs(0, 0.25, *a) for c in (ctx, split, tails)]
         for call in calls:
             dg, ds, dg2, buf = torch.empty_like(V), torch.empty_like(sig), torch.empty_like(V), sig.clone()
             call(V, sig, dg, ds)
