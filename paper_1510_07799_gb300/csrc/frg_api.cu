@@ -680,6 +680,10 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
         !(P.Lpp = dalloc<double2>(ctx, (size_t)(2 * N - 1) * N)) ||
         !(P.Lph = dalloc<double2>(ctx, (size_t)(2 * N - 1) * N)))
       return bail(FRG_ENOMEM);
+    if (!ctx->split && N >= X64_MIN_N &&
+        (!(P.LppS = dalloc<double2>(ctx, (size_t)(2 * N - 1) * N)) ||
+         !(P.LphS = dalloc<double2>(ctx, (size_t)(2 * N - 1) * N))))
+      return bail(FRG_ENOMEM);
   }
   if (!(ctx->d_pts = dalloc<PointDesc>(ctx, n_points)) || !(ctx->d_ctl = dalloc<Ctl>(ctx, n_points)) ||
       !(ctx->d_io_stage = dalloc<RhsIO>(ctx, n_points)) || !(ctx->d_io_user = dalloc<RhsIO>(ctx, n_points)))

@@ -42,6 +42,7 @@ struct PointDesc {
   double2 *G, *S;    // propagators on the box (N)
   double2 *Lpp;      // Lpp[s*N + p] = Lb(p, s-p) (0 outside the box), s in [0, 2N-1)
   double2 *Lph;      // Lph[(Q+N-1)*N + p] = Lb(p, p+Q) (0 outside the box)
+  double2 *LppS, *LphS;  // FP64 sliced products: the two tables times T Lambda (null otherwise)
   float2 *Lpp32, *Lph32;  // FP32 copies of the two tables (split paths)
   float *Lmax;       // split paths: max over p of |Re|,|Im| of each table row: [pp rows | ph rows]
   float2 *yhi[2], *ylo[2];  // split paths: vertex part of ybuf[] as float pairs (hi + lo)

@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(128)
     double2 v = make_double2(0.0, 0.0);
     if (inbox(N, q)) v = cadd(cmul(Sp[p], Gp[q]), cmul(Gp[p], Sp[q]));
     (which == 0 ? P.Lpp : P.Lph)[(size_t)row * N + p] = v;
+    if (!SPLIT && P.LppS) (which == 0 ? P.LppS : P.LphS)[(size_t)row * N + p] = cscale(v, P.T * L);
     if (P.Lpp32) {
       const float2 f = make_float2((float)v.x, (float)v.y);
       (which == 0 ? P.Lpp32 : P.Lph32)[(size_t)row * N + p] = f;

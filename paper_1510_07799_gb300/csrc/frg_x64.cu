@@ -66,9 +66,8 @@ constexpr int E_LIM = 400;                  // line exponents the path accepts
 // -------------------------------------------------------------- panels ----
 // One block: eight lines of one operand of one product over its whole
 // contraction range.  Eight lanes take the eight lines at one k, so that the
-// blocks are written in 128-byte segments; a thread gathers (and weights: the
-// factor +-T Lambda goes into the bubble weights) all its k of one line into
-// registers, the block finds each line's largest magnitude, and the values leave
+// blocks are written in 128-byte segments; a thread gathers (and weights, with the
+// table that carries T Lambda) all its k of one line into registers, the block finds each line's largest magnitude, and the values leave
 // in fixed point.  Bound by the FP64 multiplications of the weights and by the
 // gathers (16-byte elements, one 32-byte sector each wherever the line and the
 // contraction index both stride through the vertex): 99 us at N = 128 for 302 MB
@@ -157,9 +156,8 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
   if (tid < PAN_LINES) smax[tid] = 0u;
   if (LEFT) {
-    const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
-    const double2 *L = CH == CH_PP ? P.Lpp + (size_t)m * N : P.Lph + (size_t)(CH == CH_DPH ? 2 * N - 2 - m : m) * N;
-    for (int k = tid; k < D; k += blockDim.x) sw[k] = cscale(L[g.p_lo + k], sc);
+    const double2 *L = CH == CH_PP ? P.LppS + (size_t)m * N : P.LphS + (size_t)(CH == CH_DPH ? 2 * N - 2 - m : m) * N;
+    for (int k = tid; k < D; k += blockDim.x) sw[k] = L[g.p_lo + k];
   }
   double2 v[U], v2[U];
 #pragma unroll
@@ -181,7 +179,7 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
         v[u] = cmul(make_double2(fma(2.0, A.x, -C.x), fma(2.0, A.y, -C.y)), w);
         v2[u] = cmul(make_double2(-A.x, -A.y), w);
       } else {
-        v[u] = cmul(v[u], w);
+        v[u] = cmul(make_double2(-v[u].x, -v[u].y), w);
       }
     }
     um = max(um, mag(v[u]));
@@ -222,13 +220,16 @@ __global__ void __launch_bounds__(FRG_MAX_N *PAN_LINES / U, U == 8 ? 3 : 2)
                  int chmask) {
   __shared__ double2 sw[FRG_MAX_N];
   __shared__ unsigned smax[PAN_LINES];
-  const int pi = p0 + blockIdx.z / 3, ch = blockIdx.z % 3;
+  // the direct channel's blocks first, and each channel's largest transfers (m =
+  // N - 1 and outwards) first: the light blocks fill in at the end
+  const int pi = p0 + blockIdx.z / 3, z = blockIdx.z % 3, ch = z == 0 ? CH_DPH : z == 1 ? CH_PP : CH_XPH;
   const RhsIO &o = io[pi];
   const X64Pt &x = xp[pi];
   if (!o.active || !x.prod || !(chmask >> ch & 1)) return;
   const PointDesc &P = pts[pi];
-  const int m = blockIdx.y, half = gridDim.x / 2;
-  if (m >= 2 * P.N - 1) return;
+  const int half = gridDim.x / 2, y = blockIdx.y;
+  if (y >= 2 * P.N - 1) return;
+  const int m = P.N - 1 + (y & 1 ? (y + 1) / 2 : -(y / 2));
   const int b = blockIdx.x;
   if (b < half) {
     if (ch == CH_PP)
