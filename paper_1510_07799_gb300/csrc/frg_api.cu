@@ -58,6 +58,7 @@ struct frg_ctx {
   // use it now; sym: per point, whether its state is symmetric
   int rev_mode = 0;
   bool rev_on = false;
+  bool capturing = false;  // the step graph is being recorded
   // crossing reduction of the products (FRG_CROSSING, split paths): used
   // wherever the reversal reduction's schedule is
   bool cross = false;
@@ -198,14 +199,21 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
   if (ev) CK(cudaEventRecord(ev[0], st), "event");
   const bool tails = (ctx->mask & FRG_TAILS) != 0;
   const int chmask = ctx->mask & 7;
+  // under a caller's capture the launches keep ordinary edges
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (!ctx->capturing) CK(cudaStreamIsCapturing(st, &cap), "capture status");
+  const bool chain = cap == cudaStreamCaptureStatusNone;
   // points below X64_MIN_N take their whole rhs from one launch
   const int p0 = point < 0 ? 0 : point, p1 = point < 0 ? ctx->n : point + 1;
   bool small = false, large = false;
   for (int i = p0; i < p1; ++i) (small_point(ctx, i) ? small : large) = true;
   if (large)
-    LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 0, ctx->mask, st), "bubble weights and self-energy");
+    LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 0, ctx->mask, st,
+                           BUBBLE_TABLES | BUBBLE_SIGMA, chain),
+       "bubble weights and self-energy");
   if (small)
-    LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, sig_in_place, st),
+    LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, sig_in_place, st,
+                        chain),
        "small rhs");
   if (tails) LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st), "tail sums");
   if (ev) CK(cudaEventRecord(ev[1], st), "event");
@@ -228,7 +236,7 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
     if (point < 0 || (!x64_has(ctx->x64, point) && !small_point(ctx, point)))
       LK(launch_contract_fp64(ctx->d_pts, d_io, w, nw, chmask, st), "fp64 contraction");
     if (point < 0 ? ctx->x64 != nullptr : x64_has(ctx->x64, point))
-      LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st), "sliced fp64 contraction");
+      LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st, chain), "sliced fp64 contraction");
   }
   if (ev) CK(cudaEventRecord(ev[3], st), "event");
   if (ev) CK(cudaEventRecord(ev[4], st), "event");
@@ -525,8 +533,10 @@ struct FlowStream {
 static int build_step_graph(frg_ctx *ctx) {
   cudaGraph_t gr = nullptr;
   const long l0 = g_kernel_launches;
+  ctx->capturing = true;
   CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal), "begin step capture");
   const int rc = issue_step(ctx);
+  ctx->capturing = false;
   const cudaError_t e = cudaStreamEndCapture(ctx->stream, &gr);
   ctx->step_launches = g_kernel_launches - l0;
   g_kernel_launches = l0;  // counted when the graph runs

@@ -232,23 +232,55 @@ __device__ __forceinline__ void propagator_at(const PointDesc &P, int i, double 
   s = cscale(cmul(cmul(g, g), gi), -dthinv);
 }
 
-// Launch of a kernel with a shared-memory carveout preference for this launch
-// (carveout in percent of the unified L1/shared storage, or -1: the default).
+// Kernel launch with two options.
+// carveout: shared-memory carveout preference of this launch, in percent of the
+// unified L1/shared storage, or -1: the default.
+// chain: the kernel follows another one of this library on the same stream, and its
+// blocks may become resident while the predecessor's last ones still run, which takes
+// the launch itself off the serial chain of a rhs (five kernels of 5-30 us at N = 64:
+// 72.7 -> 59.8 us).  Such a kernel calls chain_wait() before it touches anything that
+// another kernel reads or writes: it returns once the predecessor has completed and
+// its writes are visible.  The trigger comes after the wait, so at most two neighbours
+// of a chain are on the GPU at a time (a kernel that holds TMEM never meets another
+// one of its chain), and successors come in only when every block of the predecessor
+// is resident, so no block of it waits for room.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_with_carveout(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                        cudaStream_t st, int carveout, Args... args) {
+inline cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             int carveout, bool chain, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute a[1];
-  a[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-  a[0].val.sharedMemCarveout = carveout < 0 ? 0u : (unsigned)carveout;
+  cudaLaunchAttribute a[2];
+  if (carveout >= 0) {
+    a[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    a[cfg.numAttrs++].val.sharedMemCarveout = (unsigned)carveout;
+  }
+  if (chain) {
+    a[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
   cfg.attrs = a;
-  cfg.numAttrs = carveout < 0 ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_with_carveout(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                        cudaStream_t st, int carveout, Args... args) {
+  return launch_ex(kernel, grid, block, smem, st, carveout, false, args...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                  bool chain, Args... args) {
+  return launch_ex(kernel, grid, block, smem, st, -1, chain, args...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+#endif
+
 // Vertex entry V(i1, i2, i3) of an input (FP64, or FP32 on the split paths)
 // under the box rule: the bare U wherever an index leaves the box.
 template <bool SPLIT>
@@ -342,7 +374,7 @@ int launch_contract_fp64(const PointDesc *d_pts, const RhsIO *d_io, const WorkIt
 // flow can compute the tables before the vertex stage input exists.
 constexpr int BUBBLE_TABLES = 1, BUBBLE_SIGMA = 2;
 int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split, int mask,
-                        cudaStream_t st, int parts = BUBBLE_TABLES | BUBBLE_SIGMA);
+                        cudaStream_t st, int parts = BUBBLE_TABLES | BUBBLE_SIGMA, bool chain = false);
 // Frequency-box tails: the window propagators and the sums over the window
 // (TAIL_WINDOW), then the constants, the self-energy's added to the
 // self-energy rhs (TAIL_FINISH: after launch_bubble_sigma's self-energy

@@ -23,6 +23,7 @@ namespace frg {
 // FP64 rate per SM is low).
 constexpr int GS_PER_BLOCK = 16;
 __global__ void k_bubble_gs(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io) {
+  chain_wait();
   const int pi = blockIdx.y;
   const RhsIO &o = io[pi];
   if (!o.active) return;
@@ -47,6 +48,7 @@ __global__ void k_bubble_gs(const PointDesc *__restrict__ pts, const RhsIO *__re
 template <bool SPLIT>
 __global__ void __launch_bounds__(128)
     k_bubble_sigma(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, int maxN, int sigma_on, int b0) {
+  chain_wait();
   const int pi = blockIdx.y;
   const RhsIO &o = io[pi];
   if (!o.active) return;
@@ -130,14 +132,15 @@ __global__ void __launch_bounds__(128)
 }
 
 int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split, int mask,
-                        cudaStream_t st, int parts) {
+                        cudaStream_t st, int parts, bool chain) {
   const int nrow_max = 2 * maxN - 1;
   // split flows run these beside the stage kernel
   const int cv = split ? side_carveout(n_points, mask) : -1;
   cudaError_t e = cudaSuccess;
   if (parts & BUBBLE_TABLES) {
-    e = launch_with_carveout(k_bubble_gs, dim3((maxN + GS_PER_BLOCK - 1) / GS_PER_BLOCK, n_points), GS_PER_BLOCK, 0,
-                             st, cv, d_pts, d_io);
+    const dim3 g((maxN + GS_PER_BLOCK - 1) / GS_PER_BLOCK, n_points);
+    e = split ? launch_with_carveout(k_bubble_gs, g, GS_PER_BLOCK, 0, st, cv, d_pts, d_io)
+              : launch_chained(k_bubble_gs, g, GS_PER_BLOCK, 0, st, chain, d_pts, d_io);
     FRG_COUNT(1);
   }
   // blocks [0, 2 nrow_max): table rows; [2 nrow_max, 2 nrow_max + maxN): self-energy entries
@@ -147,7 +150,7 @@ int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points,
     const dim3 g(b1 - b0, n_points);
     const int sig = (mask & 8) != 0;
     const cudaError_t e2 = split ? launch_with_carveout(k_bubble_sigma<true>, g, 128, 0, st, cv, d_pts, d_io, maxN, sig, b0)
-                                 : launch_with_carveout(k_bubble_sigma<false>, g, 128, 0, st, cv, d_pts, d_io, maxN, sig, b0);
+                                 : launch_chained(k_bubble_sigma<false>, g, 128, 0, st, chain, d_pts, d_io, maxN, sig, b0);
     if (e == cudaSuccess) e = e2;
     FRG_COUNT(1);
   }

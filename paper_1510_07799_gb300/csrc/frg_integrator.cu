@@ -165,6 +165,7 @@ __global__ void k_finish_k1(Ctl *__restrict__ ctl, const RhsIO *__restrict__ io,
 // Eight lanes per point, one exponential each (3.6 us, against 7.2 us for
 // one thread's seven in turn).
 __global__ void k_prepare(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl, int n) {
+  chain_wait();
   const int pi = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, s = threadIdx.x & 7;
   if (pi >= n) return;
   Ctl &c = ctl[pi];
@@ -226,6 +227,7 @@ constexpr int ST_T = 256;
 template <int S>
 __global__ void __launch_bounds__(ST_T) k_stage(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl,
                                                 RhsIO *__restrict__ io) {
+  chain_wait();
   const int pi = blockIdx.y;
   const PointDesc &P = pts[pi];
   // the first block of the point also writes the stage's rhs IO record
@@ -513,6 +515,7 @@ __device__ __forceinline__ double maxabs(double a, double b) {
 }
 constexpr int ERR_T = 512;
 __global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl) {
+  chain_wait();
   const int pi = blockIdx.y;
   Ctl &c = ctl[pi];
   if (c.done) return;
@@ -566,6 +569,7 @@ __global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ p
 
 // ----------------------------------------------------------- controller ----
 __global__ void k_controller(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl, int n) {
+  chain_wait();
   const int pi = blockIdx.x * blockDim.x + threadIdx.x;
   if (pi >= n) return;
   Ctl &c = ctl[pi];
@@ -661,17 +665,18 @@ int stage_split_init() {
 int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cudaStream_t st, int n_points,
                       int maxN) {
   const dim3 g((maxN * maxN * maxN + maxN + ST_T - 1) / ST_T, n_points);
+  cudaError_t e;
   switch (s) {
-    case 1: k_stage<1><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
-    case 2: k_stage<2><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
-    case 3: k_stage<3><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
-    case 4: k_stage<4><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
-    case 5: k_stage<5><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
-    case 6: k_stage<6><<<g, ST_T, 0, st>>>(d_pts, d_ctl, d_io); break;
+    case 1: e = launch_chained(k_stage<1>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
+    case 2: e = launch_chained(k_stage<2>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
+    case 3: e = launch_chained(k_stage<3>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
+    case 4: e = launch_chained(k_stage<4>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
+    case 5: e = launch_chained(k_stage<5>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
+    case 6: e = launch_chained(k_stage<6>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
     default: return -1;
   }
   FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  return e == cudaSuccess ? 0 : -3;
 }
 
 int launch_stage(const PointDesc *d_pts, Ctl *d_ctl, int s, cudaStream_t st, int lb_grid, int n_points, int want) {
@@ -737,15 +742,14 @@ int launch_sigma_stage(const PointDesc *d_pts, Ctl *d_ctl, RhsIO *d_io, int s, i
 }
 
 int launch_error(const PointDesc *d_pts, Ctl *d_ctl, cudaStream_t st, int n_points, int maxN) {
-  k_error<<<dim3((maxN * maxN * maxN + maxN + ERR_T - 1) / ERR_T, n_points), ERR_T, 0, st>>>(d_pts, d_ctl);
+  const dim3 g((maxN * maxN * maxN + maxN + ERR_T - 1) / ERR_T, n_points);
   FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  return launch_chained(k_error, g, ERR_T, 0, st, true, d_pts, d_ctl) == cudaSuccess ? 0 : -3;
 }
 
 int launch_controller(const PointDesc *d_pts, Ctl *d_ctl, int n, cudaStream_t st) {
-  k_controller<<<(n + 127) / 128, 128, 0, st>>>(d_pts, d_ctl, n);
   FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  return launch_chained(k_controller, (n + 127) / 128, 128, 0, st, true, d_pts, d_ctl, n) == cudaSuccess ? 0 : -3;
 }
 
 }  // namespace frg

@@ -167,6 +167,7 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
 __global__ void __launch_bounds__(T) k_rhs_small(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
                                                  int n_below, int mask, int part) {
   extern __shared__ double2 sm[];
+  chain_wait();
   const PointDesc &P = pts[blockIdx.y];
   const RhsIO &o = io[blockIdx.y];
   if (!o.active || P.N >= n_below) return;
@@ -190,7 +191,7 @@ bool room(K kernel, size_t bytes) {
 }  // namespace small
 
 int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int n_below, int mask,
-                     bool sig_in_place, cudaStream_t st) {
+                     bool sig_in_place, cudaStream_t st, bool chain) {
   // shared memory and blocks for every size below the bound (both drop where the
   // rows per block step up)
   const int N = maxN < n_below ? maxN : n_below - 1;
@@ -202,10 +203,14 @@ int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
   }
   if (!small::room(small::k_rhs_small, bytes)) return -3;
   const int first = sig_in_place ? small::VERTEX : small::ALL;
-  small::k_rhs_small<<<dim3(blocks, n_points), small::T, bytes, st>>>(d_pts, d_io, n_below, mask, first);
+  if (launch_chained(small::k_rhs_small, dim3(blocks, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
+                     first) != cudaSuccess)
+    return -3;
   FRG_COUNT(1);
   if (sig_in_place) {
-    small::k_rhs_small<<<dim3(1, n_points), small::T, bytes, st>>>(d_pts, d_io, n_below, mask, small::SIGMA);
+    if (launch_chained(small::k_rhs_small, dim3(1, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
+                       (int)small::SIGMA) != cudaSuccess)
+      return -3;
     FRG_COUNT(1);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;

@@ -28,6 +28,8 @@ struct X64Plan;
 int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, unsigned *d_err);
 void x64_destroy(X64Plan *p);
 bool x64_has(const X64Plan *p, int point);
-// Channel products of every point of the plan (point < 0) or of one point.
-int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st);
+// Channel products of every point of the plan (point < 0) or of one point; chain:
+// see launch_ex.
+int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st,
+            bool chain);
 }  // namespace frg
