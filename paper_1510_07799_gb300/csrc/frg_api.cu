@@ -190,6 +190,14 @@ static bool small_point(const frg_ctx *ctx, int i) {
 }
 
 // ------------------------------------------------------------ rhs pipeline ----
+// Whether a rhs chains its launches (launch_ex): always, except while a caller
+// records the stream, which keeps ordinary edges.
+static bool chain_launches(frg_ctx *ctx) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return ctx->capturing || (cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess &&
+                            cap == cudaStreamCaptureStatusNone);
+}
+
 // FP64 path.  ev (optional, 6 events): start, after the bubble weights and the
 // self-energy (one fused kernel; the whole rhs of the small points), twice
 // after the channel products (no regather), and after the tails.
@@ -199,10 +207,7 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
   if (ev) CK(cudaEventRecord(ev[0], st), "event");
   const bool tails = (ctx->mask & FRG_TAILS) != 0;
   const int chmask = ctx->mask & 7;
-  // under a caller's capture the launches keep ordinary edges
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (!ctx->capturing) CK(cudaStreamIsCapturing(st, &cap), "capture status");
-  const bool chain = cap == cudaStreamCaptureStatusNone;
+  const bool chain = chain_launches(ctx);
   // points below X64_MIN_N take their whole rhs from one launch
   const int p0 = point < 0 ? 0 : point, p1 = point < 0 ? ctx->n : point + 1;
   bool small = false, large = false;
@@ -261,6 +266,7 @@ static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, con
   cudaStream_t st = ctx->stream, ss = ev ? st : ctx->sstream, ts = ev ? st : ctx->tstream;
   const bool fork = !ev, tails = (ctx->mask & FRG_TAILS) != 0;
   const int chmask = ctx->mask & 7;
+  const bool chain = chain_launches(ctx);
   // the reversal reduction's transfers: flows while it is on, every call when
   // the caller asserts the symmetry
   const bool half = gam ? ctx->rev_mode == 2 : ctx->rev_on;
@@ -270,13 +276,14 @@ static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, con
     CK(cudaStreamWaitEvent(ss, ctx->ev_fork, 0), "fork");
     if (tails) CK(cudaStreamWaitEvent(ts, ctx->ev_fork, 0), "fork");
   }
-  LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES), "bubble weights");
+  LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES, chain), "bubble weights");
   if (fork) CK(cudaEventRecord(ctx->ev_join, ss), "join");
   if (tails)
     LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ts, TAIL_WINDOW), "tail sums");
   if (ev) CK(cudaEventRecord(ev[1], st), "event");
   if (gam)
-    LK(launch_relayout(ctx->d_pts + point, gam, ctx->hpts[point].N, ctx->lb_want, ctx->precision == FRG_BF16X3, st),
+    LK(launch_relayout(ctx->d_pts + point, gam, ctx->hpts[point].N, ctx->lb_want, ctx->precision == FRG_BF16X3, st,
+                       chain),
        "regather");
   const bool sig_in_tc = chmask && !tails;
   if (!sig_in_tc) {
@@ -304,6 +311,7 @@ static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, con
     r.half = half;
     r.canon = half && !gam;
     r.out64 = gam != nullptr;
+    r.chain = chain && !ev;
     r.cross = ctx->cross;
     r.sigma = sig_in_tc ? 1 | ((ctx->mask & 8) ? 2 : 0) : 0;
     LK(tc_run(ctx->tc, ctx->d_pts, d_io, point, chmask, st, ctx->n, ctx->maxN, r), "split contraction");
@@ -433,7 +441,7 @@ static int run_split_stage(frg_ctx *ctx, int s, bool err, bool fused, bool defer
     CK(cudaStreamWaitEvent(ts, ctx->ev_sst, 0), "self-energy stage");
     LK(launch_tail_sums(ctx->d_pts, io, ctx->n, ctx->maxN, ctx->mask, ts, TAIL_WINDOW), "tail sums");
   }
-  LK(launch_bubble_sigma(ctx->d_pts, io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES), "bubble weights");
+  LK(launch_bubble_sigma(ctx->d_pts, io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES, true), "bubble weights");
   CK(cudaEventRecord(ctx->ev_join, ss), "join");
   if (fused)
     LK(launch_combine_stage(ctx->d_pts, ctx->d_ctl, s, ctx->rev_on, ctx->precision == FRG_BF16X3,

@@ -139,8 +139,7 @@ int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points,
   cudaError_t e = cudaSuccess;
   if (parts & BUBBLE_TABLES) {
     const dim3 g((maxN + GS_PER_BLOCK - 1) / GS_PER_BLOCK, n_points);
-    e = split ? launch_with_carveout(k_bubble_gs, g, GS_PER_BLOCK, 0, st, cv, d_pts, d_io)
-              : launch_chained(k_bubble_gs, g, GS_PER_BLOCK, 0, st, chain, d_pts, d_io);
+    e = launch_ex(k_bubble_gs, g, GS_PER_BLOCK, 0, st, cv, chain, d_pts, d_io);
     FRG_COUNT(1);
   }
   // blocks [0, 2 nrow_max): table rows; [2 nrow_max, 2 nrow_max + maxN): self-energy entries
@@ -149,8 +148,8 @@ int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points,
   if (b1 > b0) {
     const dim3 g(b1 - b0, n_points);
     const int sig = (mask & 8) != 0;
-    const cudaError_t e2 = split ? launch_with_carveout(k_bubble_sigma<true>, g, 128, 0, st, cv, d_pts, d_io, maxN, sig, b0)
-                                 : launch_chained(k_bubble_sigma<false>, g, 128, 0, st, chain, d_pts, d_io, maxN, sig, b0);
+    const cudaError_t e2 = launch_ex(split ? k_bubble_sigma<true> : k_bubble_sigma<false>, g, 128, 0, st, cv, chain, d_pts,
+                                     d_io, maxN, sig, b0);
     if (e == cudaSuccess) e = e2;
     FRG_COUNT(1);
   }

@@ -468,6 +468,7 @@ constexpr int SIG_THREADS = 128;
 template <int S>
 __global__ void __launch_bounds__(SIG_THREADS) k_sigma_stage(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl,
                                                              RhsIO *__restrict__ io) {
+  chain_wait();
   const int pi = blockIdx.x;
   const PointDesc &P = pts[pi];
   if (threadIdx.x == 0) write_stage_io(P, ctl[pi], io + pi, S, 1);

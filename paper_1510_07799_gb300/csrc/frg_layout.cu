@@ -38,6 +38,7 @@ template <bool VMAX>
 __global__ void __launch_bounds__(LB_THREADS, 5)
     k_relayout(const PointDesc *__restrict__ pt, const double2 *__restrict__ G, int want) {
   extern __shared__ float4 lsm4[];
+  chain_wait();
   float2 *sm = reinterpret_cast<float2 *>(lsm4);
   const PointDesc &P = *pt;
   const int N = P.N;
@@ -107,6 +108,7 @@ template <bool REV, bool ERR, bool OUT64>
 __global__ void __launch_bounds__(comb_threads<REV, ERR>(), ERR ? 4 : REV ? LB_MINBLOCKS_WIDE : LB_MINBLOCKS)
     k_combine(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, int mask, ErrWeights ew) {
   __shared__ __align__(16) float2 sm[LB * LAP];
+  chain_wait();
   const RhsIO &o = io[blockIdx.y];
   if (!o.active) return;
   combine_block<REV, ERR, comb_threads<REV, ERR>(), true, OUT64>(pts[blockIdx.y], o, mask, ew, sm);
@@ -121,13 +123,13 @@ int layout_init() {
              : -3;
 }
 
-int launch_relayout(const PointDesc *d_pt, const double2 *gam, int N, int want, bool vmax, cudaStream_t st) {
-  if (vmax)
-    k_relayout<true><<<lblocks(N, N), LB_THREADS, LB_SMEM, st>>>(d_pt, gam, want);
-  else
-    k_relayout<false><<<lblocks(N, N), LB_THREADS, LB_SMEM, st>>>(d_pt, gam, want);
+int launch_relayout(const PointDesc *d_pt, const double2 *gam, int N, int want, bool vmax, cudaStream_t st,
+                    bool chain) {
   FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  return launch_chained(vmax ? k_relayout<true> : k_relayout<false>, lblocks(N, N), LB_THREADS, LB_SMEM, st, chain,
+                        d_pt, gam, want) == cudaSuccess
+             ? 0
+             : -3;
 }
 
 int launch_fill_z(const PointDesc *d_pts, int n_points, cudaStream_t st) {
@@ -137,7 +139,7 @@ int launch_fill_z(const PointDesc *d_pts, int n_points, cudaStream_t st) {
 }
 
 int launch_combine(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int mask, cudaStream_t st,
-                   bool err, bool canon_half, bool out64) {
+                   bool err, bool canon_half, bool out64, bool chain) {
   const dim3 g(lblocks(maxN, canon_half ? maxN / 2 : maxN), n_points);
   const ErrWeights ew = host_error_weights();
   const bool rev = (mask & FRG_REVERSAL) != 0;
@@ -146,15 +148,13 @@ int launch_combine(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int 
   if (rev && err)
     e = launch_with_carveout(k_combine<true, true, false>, g, comb_threads<true, true>(), 0, st, cv, d_pts, d_io, mask, ew);
   else if (rev && out64)
-    e = launch_with_carveout(k_combine<true, false, true>, g, comb_threads<true, false>(), 0, st, cv, d_pts, d_io,
-                             mask, ew);
+    e = launch_ex(k_combine<true, false, true>, g, comb_threads<true, false>(), 0, st, cv, chain, d_pts, d_io, mask, ew);
   else if (rev)
     e = launch_with_carveout(k_combine<true, false, false>, g, comb_threads<true, false>(), 0, st, cv, d_pts, d_io, mask, ew);
   else if (err)
     e = launch_with_carveout(k_combine<false, true, false>, g, comb_threads<false, true>(), 0, st, cv, d_pts, d_io, mask, ew);
   else if (out64)
-    e = launch_with_carveout(k_combine<false, false, true>, g, comb_threads<false, false>(), 0, st, cv, d_pts, d_io,
-                             mask, ew);
+    e = launch_ex(k_combine<false, false, true>, g, comb_threads<false, false>(), 0, st, cv, chain, d_pts, d_io, mask, ew);
   else
     e = launch_with_carveout(k_combine<false, false, false>, g, comb_threads<false, false>(), 0, st, cv, d_pts, d_io,
                              mask, ew);

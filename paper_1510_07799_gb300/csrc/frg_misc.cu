@@ -12,6 +12,7 @@ long g_kernel_launches = 0;
 // point's layouts, so the flow's next step attempt writes every entry again (not
 // only the half the reversal reduction reads).
 __global__ void k_set_user_io(RhsIO *io, Ctl *ctl, int n, int point, RhsIO o, double lam, int relaid) {
+  chain_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (i == point) {

@@ -1017,6 +1017,7 @@ __device__ __forceinline__ void contract(const PointDesc *__restrict__ pts, cons
   __syncthreads();
   tc_after();
   S.tmem = *tmem_slot;
+  chain_wait();
   const int w0 = cta_start[blockIdx.x], w1 = cta_start[blockIdx.x + 1];
 
 #define FRG_BY_CH(f, ...) \
@@ -1390,7 +1391,7 @@ int tc_run(TcPlan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int 
   // vertex bound that the BF16 slicing read
   if (r.wait_combine && cudaStreamWaitEvent(st, r.wait_combine, 0) != cudaSuccess) return -3;
   const int cmask = chmask | (r.tails ? FRG_TAILS : 0) | (r.half ? FRG_REVERSAL : 0);
-  if (launch_combine(d_pts, d_io, n_points, maxN, cmask, st, r.err, r.canon, r.out64) != 0) return -3;
+  if (launch_combine(d_pts, d_io, n_points, maxN, cmask, st, r.err, r.canon, r.out64, r.chain && !r.wait_combine) != 0) return -3;
   return 0;
 }
 

@@ -47,6 +47,7 @@ int tc_wait_selftest(unsigned *d_err, double limit_ms, cudaStream_t st);
 struct TcRun {
   cudaEvent_t ev_contract = nullptr, wait_before = nullptr, wait_combine = nullptr;
   bool tails = false, half = false, canon = false, out64 = false, err = false, cross = false, combine = true;
+  bool chain = false;  // the combine of a stand-alone evaluation follows the products at once (launch_ex)
   int sigma = 0;
 };
 int tc_run(TcPlan *plan, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st,
