@@ -46,8 +46,6 @@ struct frg_ctx {
   WorkItem *d_work_pt[3] = {nullptr, nullptr, nullptr};
   std::vector<int> work_off[3];  // per point offsets into d_work_pt
   X64Plan *x64 = nullptr;        // FP64 path: the points whose products run sliced on the tensor cores
-  int *d_seg_point = nullptr, *d_seg_base = nullptr;
-  int nseg = 0;
   // split stage kernels: layout blocks per point (the largest point's vertex
   // blocks plus one self-energy block) and the layouts its channels read
   int lb_grid = 0, lb_grid_half = 0, lb_want = 0;
@@ -374,8 +372,6 @@ static int flow_status(frg_ctx *ctx) {
   return FRG_OK;
 }
 
-static SegTable seg(frg_ctx *ctx) { return SegTable{ctx->d_seg_point, ctx->d_seg_base}; }
-
 // Contraction schedules the context needs: the reversal reduction's alone when
 // the caller asserts the symmetry, both when the flows switch automatically.
 static int tc_schedules(const frg_ctx *ctx) {
@@ -699,9 +695,9 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
         !(P.Lph = dalloc<double2>(ctx, (size_t)(2 * N - 1) * N)))
       return bail(FRG_ENOMEM);
     if (!ctx->split && N >= X64_MIN_N &&
-        (!(P.LppS = dalloc<double2>(ctx, (size_t)(2 * N - 1) * N)) ||
-         !(P.LphS = dalloc<double2>(ctx, (size_t)(2 * N - 1) * N))))
+        !(P.LppS = dalloc<double2>(ctx, 2 * (size_t)(2 * N - 1) * N)))
       return bail(FRG_ENOMEM);
+    if (P.LppS) P.LphS = P.LppS + (size_t)(2 * N - 1) * N;
   }
   if (!(ctx->d_pts = dalloc<PointDesc>(ctx, n_points)) || !(ctx->d_ctl = dalloc<Ctl>(ctx, n_points)) ||
       !(ctx->d_io_stage = dalloc<RhsIO>(ctx, n_points)) || !(ctx->d_io_user = dalloc<RhsIO>(ctx, n_points)))
@@ -749,6 +745,7 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
       std::vector<WorkItem> allw;
       for (auto &x : all) allw.push_back(x.second);
       ctx->nwork_all[ch] = (int)allw.size();
+      if (allw.empty()) continue;
       if (!(ctx->d_work_all[ch] = dalloc<WorkItem>(ctx, allw.size())) ||
           !(ctx->d_work_pt[ch] = dalloc<WorkItem>(ctx, per.size())))
         return bail(FRG_ENOMEM);
@@ -764,39 +761,10 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
     }
   }
 
-  // ---- segment table for the elementwise kernels
-  {
-    std::vector<int> sp, sb;
-    for (int i = 0; i < n_points; ++i) {
-      const PointDesc &P = ctx->hpts[i];
-      if (ctx->rev_mode == 2) {
-        // the vertex entries i < n3/2, then the self-energy
-        for (int b = 0; b < P.n3 / 2; b += SEG_ELEMS) {
-          sp.push_back(i);
-          sb.push_back(b);
-        }
-        for (int b = P.n3; b < P.n3 + P.N; b += SEG_ELEMS) {
-          sp.push_back(i);
-          sb.push_back(b);
-        }
-        continue;
-      }
-      const int nc = P.n3 + P.N;
-      for (int b = 0; b < nc; b += SEG_ELEMS) {
-        sp.push_back(i);
-        sb.push_back(b);
-      }
-    }
-    ctx->nseg = (int)sp.size();
-    if (!(ctx->d_seg_point = dalloc<int>(ctx, sp.size())) || !(ctx->d_seg_base = dalloc<int>(ctx, sb.size())))
-      return bail(FRG_ENOMEM);
-    cudaMemcpy(ctx->d_seg_point, sp.data(), sizeof(int) * sp.size(), cudaMemcpyHostToDevice);
-    cudaMemcpy(ctx->d_seg_base, sb.data(), sizeof(int) * sb.size(), cudaMemcpyHostToDevice);
-  }
   ctx->user_in.assign(n_points, nullptr);
   ctx->user_out.assign(n_points, nullptr);
   ctx->user_kout.assign(n_points, nullptr);
-  if (launch_init(ctx->d_pts, ctx->d_ctl, seg(ctx), ctx->nseg, n_points, ctx->stream) != 0) return bail(FRG_ECUDA);
+  if (launch_init(ctx->d_pts, ctx->d_ctl, ctx->maxN, n_points, ctx->stream) != 0) return bail(FRG_ECUDA);
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return bail(FRG_ECUDA);
   *out = ctx;
   return FRG_OK;

@@ -12,6 +12,8 @@
 // the last step is clipped to end exactly at ln Lambda_f.
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "frg_common.cuh"
 #include "frg_integrator.cuh"
 #include "frg_split.cuh"
@@ -88,18 +90,13 @@ __global__ void k_init_ctl(const PointDesc *__restrict__ pts, Ctl *__restrict__ 
   ctl[pi] = c;
 }
 
-__global__ void k_fill_bare(const PointDesc *__restrict__ pts, SegTable seg) {
-  const int b = blockIdx.x;
-  const int pi = seg.point[b];
-  const PointDesc &P = pts[pi];
-  const int n = P.n3 + P.N;
-  const int base = seg.base[b];
-  double2 *y = P.ybuf[0];
-  for (int e = threadIdx.x; e < SEG_ELEMS; e += blockDim.x) {
-    const int i = base + e;
-    if (i < n) y[i] = make_double2(i < P.n3 ? P.U : 0.0, 0.0);
-    // half-storage segments cover the entries i < n3/2: their mirrors too
-    if (P.rev_half && i < P.n3 / 2) y[P.n3 - 1 - i] = make_double2(P.U, 0.0);
+// The bare state of every point: grid (blocks, points).
+__global__ void k_fill_bare(const PointDesc *__restrict__ pts, int n_points) {
+  for (int pi = blockIdx.y; pi < n_points; pi += gridDim.y) {
+    const PointDesc &P = pts[pi];
+    double2 *y = P.ybuf[0];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n3 + P.N; i += gridDim.x * blockDim.x)
+      y[i] = make_double2(i < P.n3 ? P.U : 0.0, 0.0);
   }
 }
 
@@ -610,10 +607,11 @@ __global__ void k_controller(const PointDesc *__restrict__ pts, Ctl *__restrict_
 }
 
 // ------------------------------------------------------------ launchers ----
-int launch_init(const PointDesc *d_pts, Ctl *d_ctl, SegTable seg, int nblk, int n, cudaStream_t st) {
+int launch_init(const PointDesc *d_pts, Ctl *d_ctl, int maxN, int n, cudaStream_t st) {
   k_init_ctl<<<(n + 127) / 128, 128, 0, st>>>(d_pts, d_ctl, n);
   FRG_COUNT(1);
-  k_fill_bare<<<nblk, 256, 0, st>>>(d_pts, seg);
+  const int blocks = std::min(4096, (maxN * maxN * maxN + maxN + 255) / 256);
+  k_fill_bare<<<dim3(blocks, std::min(n, 65535)), 256, 0, st>>>(d_pts, n);
   FRG_COUNT(1);
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }

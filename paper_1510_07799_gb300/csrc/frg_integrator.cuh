@@ -4,14 +4,6 @@
 
 namespace frg {
 
-// Elementwise kernels over the (vertex | self-energy) state of every point:
-// block b handles elements [base[b], base[b] + SEG_ELEMS) of point point[b].
-constexpr int SEG_ELEMS = 2048;
-struct SegTable {
-  const int *point;
-  const int *base;
-};
-
 int upload_tableau();
 // Embedded error weights E_j = b_j - bstar_j of the Dormand-Prince pair (FP64)
 // and E_7 as a float pair, for the split paths' scatter-add of k7, which
@@ -22,7 +14,7 @@ struct ErrWeights {
 };
 ErrWeights host_error_weights();
 void host_tableau(double *c, double *a, double *bstar);
-int launch_init(const PointDesc *d_pts, Ctl *d_ctl, SegTable seg, int nblk, int n, cudaStream_t st);
+int launch_init(const PointDesc *d_pts, Ctl *d_ctl, int maxN, int n, cudaStream_t st);
 int launch_set_ctl(const PointDesc *d_pts, Ctl *d_ctl, int pi, double t, double h, cudaStream_t st);
 int launch_set_stage_io(const PointDesc *d_pts, Ctl *d_ctl, RhsIO *d_io, int stage, int split, int n,
                         cudaStream_t st);

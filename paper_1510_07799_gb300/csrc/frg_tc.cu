@@ -43,6 +43,7 @@
 #include "frg.h"
 #include "frg_layout.cuh"
 #include "frg_ptx.cuh"
+#include "frg_sched.cuh"
 #include "frg_tc.cuh"
 
 namespace frg {
@@ -1127,20 +1128,15 @@ struct TcPlan {
   // [1 + i] point i alone; sched: every transfer, sched_half: the reversal
   // reduction's transfers m <= N - 1, sched_cross: those with the crossing
   // reduction (each may be absent)
-  struct Sched {
-    tc::st::StWork *d_work = nullptr;
-    int *d_start = nullptr;
-    int grid = 0;
-  };
+  // (a context of one point has [0] alone)
+  using Sched = Schedule<tc::st::StWork>;
   std::vector<Sched> sched, sched_half, sched_cross;
   int mask = 7;
   TcTune tune;
 };
 
-// Longest-processing-time schedule of the tiles of points [first, last) over at
-// most `sms` persistent CTAs: tiles sorted by cost (k-steps plus an epilogue
-// allowance), each given to the CTA with the least work so far; stored CTA by
-// CTA with start offsets.
+// Schedule of the tiles of points [first, last); a tile's cost: its k-steps plus an
+// epilogue allowance.
 // cross (with half): the transfers with two row tiles of points whose one
 // column tile spans all N columns take the crossing-reduced tiles (cross_tile);
 // a tile's cost then scales with its width (the left operand's share and the
@@ -1174,30 +1170,7 @@ static bool build_sched(TcPlan *p, const std::vector<PointDesc> &pts, const std:
       }
     }
   }
-  std::stable_sort(tiles.begin(), tiles.end(), [](auto &a, auto &b) { return a.first > b.first; });
-  const int grid = std::min((int)tiles.size(), p->sms);
-  out.grid = grid;
-  if (!grid) return true;
-  std::vector<std::vector<tc::st::StWork>> per(grid);
-  std::vector<long> load(grid, 0);
-  for (auto &t : tiles) {
-    int best = 0;
-    for (int c = 1; c < grid; ++c)
-      if (load[c] < load[best]) best = c;
-    load[best] += t.first;
-    per[best].push_back(t.second);
-  }
-  std::vector<tc::st::StWork> flat;
-  std::vector<int> start(1, 0);
-  for (auto &v : per) {
-    flat.insert(flat.end(), v.begin(), v.end());
-    start.push_back((int)flat.size());
-  }
-  return cudaMalloc(&out.d_work, sizeof(tc::st::StWork) * flat.size()) == cudaSuccess &&
-         cudaMalloc(&out.d_start, sizeof(int) * start.size()) == cudaSuccess &&
-         cudaMemcpy(out.d_work, flat.data(), sizeof(tc::st::StWork) * flat.size(), cudaMemcpyHostToDevice) ==
-             cudaSuccess &&
-         cudaMemcpy(out.d_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+  return upload_schedule(out, tiles, p->sms);
 }
 
 // Tensor maps of the operand tiles (see MapId): box {2*RA floats, 64 rows} for
@@ -1308,9 +1281,9 @@ int tc_plan_create(TcPlan **out, const std::vector<PointDesc> &pts, const std::v
   for (int h = 0; h < 3 && ok; ++h) {
     if (!(schedules & (h == 0 ? TC_FULL : h == 1 ? TC_HALF : TC_CROSS))) continue;
     std::vector<TcPlan::Sched> &v = h == 0 ? p->sched : h == 1 ? p->sched_half : p->sched_cross;
-    v.resize(1 + p->n);
+    v.resize(p->n > 1 ? 1 + p->n : 1);
     ok = build_sched(p, pts, nt, 0, p->n, v[0], h != 0, h == 2);
-    for (int i = 0; i < p->n && ok; ++i) ok = build_sched(p, pts, nt, i, i + 1, v[1 + i], h != 0, h == 2);
+    for (int i = 0; i + 1 < (int)v.size() && ok; ++i) ok = build_sched(p, pts, nt, i, i + 1, v[1 + i], h != 0, h == 2);
   }
   if (ok) {
     std::string mw;
@@ -1345,10 +1318,7 @@ void tc_plan_destroy(TcPlan *p) {
   if (!p) return;
   cudaFree(p->d_maps);
   for (auto *v : {&p->sched, &p->sched_half, &p->sched_cross})
-    for (auto &sc : *v) {
-      cudaFree(sc.d_work);
-      cudaFree(sc.d_start);
-    }
+    for (auto &sc : *v) drop_schedule(sc);
   delete p;
 }
 
@@ -1372,14 +1342,14 @@ int tc_run(TcPlan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int 
   const bool x = r.half && r.cross;
   const std::vector<TcPlan::Sched> &scv = r.half ? (x ? p->sched_cross : p->sched_half) : p->sched;
   if ((chmask & 7) != p->mask || point >= p->n || scv.empty()) return -1;
-  const TcPlan::Sched &sc = scv[point < 0 ? 0 : 1 + point];
+  const TcPlan::Sched &sc = scv[point < 0 || p->n == 1 ? 0 : 1 + point];
   if (r.sigma && !sc.grid) return -1;
   if (sc.grid) {
     auto kern = p->precision == FRG_3XTF32 ? (x ? tc::st::k_contract_tf32_x : tc::st::k_contract_tf32)
                                            : (x ? tc::st::k_contract_bf16x3_x : tc::st::k_contract_bf16x3);
     const int smem = p->precision == FRG_3XTF32 ? tc::st::OpL<FRG_3XTF32>::SMEM : tc::st::OpL<FRG_BF16X3>::SMEM;
     const int s0 = point < 0 ? 0 : point, s1 = r.sigma ? (point < 0 ? n_points : point + 1) : s0;
-    kern<<<sc.grid, tc::st::THREADS, smem, st>>>(d_pts, d_io, sc.d_work, sc.d_start, p->d_err, p->d_maps,
+    kern<<<sc.grid, tc::st::THREADS, smem, st>>>(d_pts, d_io, sc.work, sc.start, p->d_err, p->d_maps,
                                                  r.half ? 1 : 0, s0, s1, (r.sigma & 2) ? 1 : 0);
     FRG_COUNT(1);
     if (cudaGetLastError() != cudaSuccess) return -3;

@@ -38,13 +38,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <queue>
 #include <vector>
 
 #include "frg.h"
 #include "frg_common.cuh"
 #include "frg_f64elem.cuh"
 #include "frg_ptx.cuh"
+#include "frg_sched.cuh"
 #include "frg_x64.cuh"
 
 namespace frg {
@@ -712,18 +712,14 @@ __global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restr
 
 // ---------------------------------------------------------------- plan ----
 struct X64Plan {
-  struct Sched {
-    x64::Work *d_work = nullptr;
-    int *d_start = nullptr;
-    int grid = 0;
-  };
+  using Sched = Schedule<x64::Work>;
   struct Group {
     int p0, p1, maxN;
     Sched all;
   };
   std::vector<X64Pt> h;
   std::vector<int> N;          // per point, 0: not on this path
-  std::vector<Sched> one;      // per point
+  std::vector<Sched> one;      // per point (a context of one point has its group's alone)
   std::vector<Group> groups;   // points whose operands share the workspace, one group after another
   X64Pt *d_x = nullptr;
   int *d_bad = nullptr;
@@ -739,32 +735,6 @@ namespace {
 constexpr size_t X64_WS_CAP = (size_t)4 << 30;
 constexpr int X64_GROUP = 512;  // points per group: grid.z stays below 65536
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-bool upload_sched(X64Plan::Sched &out, std::vector<std::pair<int, x64::Work>> &tiles, int sms) {
-  std::stable_sort(tiles.begin(), tiles.end(), [](auto &a, auto &b) { return a.first > b.first; });
-  out.grid = std::min((int)tiles.size(), sms);
-  if (!out.grid) return true;
-  // longest tile first, each to the CTA with the least work so far
-  std::vector<std::vector<x64::Work>> per(out.grid);
-  std::priority_queue<std::pair<long, int>, std::vector<std::pair<long, int>>, std::greater<std::pair<long, int>>> q;
-  for (int c = 0; c < out.grid; ++c) q.push({0, c});
-  for (auto &t : tiles) {
-    auto [load, c] = q.top();
-    q.pop();
-    per[c].push_back(t.second);
-    q.push({load + t.first, c});
-  }
-  std::vector<x64::Work> flat;
-  std::vector<int> start(1, 0);
-  for (auto &v : per) {
-    flat.insert(flat.end(), v.begin(), v.end());
-    start.push_back((int)flat.size());
-  }
-  return cudaMalloc(&out.d_work, sizeof(x64::Work) * flat.size()) == cudaSuccess &&
-         cudaMalloc(&out.d_start, sizeof(int) * start.size()) == cudaSuccess &&
-         cudaMemcpy(out.d_work, flat.data(), sizeof(x64::Work) * flat.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaMemcpy(out.d_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-}
 }  // namespace
 
 int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, unsigned *d_err) {
@@ -872,13 +842,13 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
     p->tables.push_back(t);
     x.prod = static_cast<const uint4 *>(t);
     ok = cudaMemcpy(t, tab[i].data(), sizeof(uint4) * tab[i].size(), cudaMemcpyHostToDevice) == cudaSuccess &&
-         upload_sched(p->one[i], tiles[i], sms);
+         (n == 1 || upload_schedule(p->one[i], tiles[i], sms));
   }
   for (X64Plan::Group &g : p->groups) {
     if (!ok) break;
     std::vector<std::pair<int, x64::Work>> all;
     for (int i = g.p0; i < g.p1; ++i) all.insert(all.end(), tiles[i].begin(), tiles[i].end());
-    ok = upload_sched(g.all, all, sms);
+    ok = upload_schedule(g.all, all, sms);
   }
   ok = ok && cudaMemcpy(p->d_x, p->h.data(), sizeof(X64Pt) * n, cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) {
@@ -891,12 +861,8 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
 
 void x64_destroy(X64Plan *p) {
   if (!p) return;
-  auto drop = [](X64Plan::Sched &s) {
-    cudaFree(s.d_work);
-    cudaFree(s.d_start);
-  };
-  for (auto &s : p->one) drop(s);
-  for (auto &g : p->groups) drop(g.all);
+  for (auto &s : p->one) drop_schedule(s);
+  for (auto &g : p->groups) drop_schedule(g.all);
   for (void *t : p->tables) cudaFree(t);
   cudaFree(p->d_x);
   cudaFree(p->d_bad);
@@ -917,7 +883,7 @@ int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, in
       p0 = point;
       p1 = point + 1;
       maxN = p->N[point];
-      s = &p->one[point];
+      if (p->N.size() > 1) s = &p->one[point];
     }
     const int oct = (maxN + x64::PAN_LINES - 1) / x64::PAN_LINES, np = p1 - p0;
     const dim3 pg(2 * oct, 2 * maxN - 1, 3 * np);
@@ -928,8 +894,8 @@ int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, in
     // and 37.8 against 35.8 ms per flow; nothing chained 327 and 65.0 us, 36.2 ms).
     if (launch_chained(x64::panel_u(maxN) == 8 ? x64::k_x64_panels<8> : x64::k_x64_panels<4>, pg,
                        x64::panel_threads(maxN), 0, st, chain, d_pts, d_io, p->d_x, p0, chmask) != cudaSuccess ||
-        launch_chained(x64::k_x64_products, s->grid, x64::THREADS, x64::SMEM, st, chain, d_pts, d_io, p->d_x, s->d_work,
-                       s->d_start, p->d_err) != cudaSuccess ||
+        launch_chained(x64::k_x64_products, s->grid, x64::THREADS, x64::SMEM, st, chain, d_pts, d_io, p->d_x, s->work,
+                       s->start, p->d_err) != cudaSuccess ||
         launch_chained(x64::k_x64_combine, dim3((maxN + 31) / 32, (maxN + 7) / 8, nz * np), 256, 0, st, false, d_pts,
                        d_io, p->d_x, p0, nz, chmask) != cudaSuccess)
       return -3;
