@@ -49,10 +49,10 @@ struct frg_ctx {
   // split stage kernels: layout blocks per point (the largest point's vertex
   // blocks plus one self-energy block) and the layouts its channels read
   int lb_grid = 0, lb_grid_half = 0, lb_want = 0;
-  // frequency-reversal reduction of the split paths: rev_mode 0 off (FP64,
-  // FRG_NO_REVERSAL), 1 automatic (flows use it while every point's state is
+  // frequency-reversal reduction: rev_mode 0 off (FRG_NO_REVERSAL, FP64 with the
+  // tails), 1 automatic (flows use it while every point's state is
   // reversal-symmetric, checked exactly by frg_set_state), 2 asserted by the
-  // caller (FRG_REVERSAL: every evaluation, half storage); rev_on: the flows
+  // caller (FRG_REVERSAL on the split paths: every evaluation, half storage); rev_on: the flows
   // use it now; sym: per point, whether its state is symmetric
   int rev_mode = 0;
   bool rev_on = false;
@@ -206,17 +206,18 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
   const bool tails = (ctx->mask & FRG_TAILS) != 0;
   const int chmask = ctx->mask & 7;
   const bool chain = chain_launches(ctx);
+  const bool half = point < 0 && ctx->rev_on;  // (flows alone)
   // points below X64_MIN_N take their whole rhs from one launch
   const int p0 = point < 0 ? 0 : point, p1 = point < 0 ? ctx->n : point + 1;
   bool small = false, large = false;
   for (int i = p0; i < p1; ++i) (small_point(ctx, i) ? small : large) = true;
   if (large)
     LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 0, ctx->mask, st,
-                           BUBBLE_TABLES | BUBBLE_SIGMA, chain),
+                           BUBBLE_TABLES | BUBBLE_SIGMA, chain, half),
        "bubble weights and self-energy");
   if (small)
     LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, sig_in_place, st,
-                        chain),
+                        chain, half),
        "small rhs");
   if (tails) LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st), "tail sums");
   if (ev) CK(cudaEventRecord(ev[1], st), "event");
@@ -239,7 +240,7 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
     if (point < 0 || (!x64_has(ctx->x64, point) && !small_point(ctx, point)))
       LK(launch_contract_fp64(ctx->d_pts, d_io, w, nw, chmask, st), "fp64 contraction");
     if (point < 0 ? ctx->x64 != nullptr : x64_has(ctx->x64, point))
-      LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st, chain), "sliced fp64 contraction");
+      LK(x64_run(ctx->x64, ctx->d_pts, d_io, point, chmask, st, chain, half), "sliced fp64 contraction");
   }
   if (ev) CK(cudaEventRecord(ev[3], st), "event");
   if (ev) CK(cudaEventRecord(ev[4], st), "event");
@@ -593,7 +594,10 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
   ctx->precision = ctx->params[0].precision;
   ctx->mask = ctx->params[0].channel_mask;
   ctx->split = ctx->precision != FRG_FP64;
-  ctx->rev_mode = !ctx->split ? 0 : (ctx->mask & FRG_REVERSAL) ? 2 : (ctx->mask & FRG_NO_REVERSAL) ? 0 : 1;
+  // (FP64: flows by the one-launch rhs and the sliced products; the tails' sums
+  // run in an order of their own for an entry and its mirror)
+  ctx->rev_mode = (ctx->mask & FRG_NO_REVERSAL) ? 0 : ctx->split ? ((ctx->mask & FRG_REVERSAL) ? 2 : 1)
+                                                : (ctx->mask & FRG_TAILS) || !(ctx->mask & 7) ? 0 : 1;
   ctx->rev_on = ctx->rev_mode != 0;
   ctx->cross = ctx->split && (ctx->mask & FRG_CROSSING) != 0;
   ctx->sym.assign(n_points, 1);
@@ -729,6 +733,8 @@ int frg_init(const frg_params *params, int n_points, void *cuda_stream, frg_ctx 
   // heavy-first so that long transfers start early and short ones fill in.
   if (!ctx->split) {
     if (x64_create(&ctx->x64, ctx->hpts, ctx->mask & 7, ctx->d_err) != 0) return bail(FRG_ECUDA);
+    for (int i = 0; i < n_points; ++i)
+      if (!x64_has(ctx->x64, i) && !small_point(ctx, i)) ctx->rev_mode = ctx->rev_on = 0;
     for (int ch = 0; ch < 3; ++ch) {
       std::vector<std::pair<int, WorkItem>> all, one;
       std::vector<WorkItem> per;
@@ -1156,7 +1162,7 @@ int frg_set_state(frg_ctx *ctx, int point, const void *d_gamma, const void *d_si
     ctx->sym[point] = *ctx->h_asym == 0;
     // the other points' states whole before the flows switch to every transfer
     // (their stage kernels then read whole states)
-    if (ctx->rev_on && !ctx->sym[point]) {
+    if (ctx->split && ctx->rev_on && !ctx->sym[point]) {
       if (point > 0) LK(launch_mirror_state(ctx->d_pts, point, ctx->stream), "set state");
       if (point + 1 < ctx->n)
         LK(launch_mirror_state(ctx->d_pts + point + 1, ctx->n - point - 1, ctx->stream), "set state");

@@ -371,10 +371,12 @@ int launch_contract_fp64(const PointDesc *d_pts, const RhsIO *d_io, const WorkIt
 // the self-energy rhs in one launch.  `parts` selects the propagators and the
 // tables (BUBBLE_TABLES: they need the self-energy input alone) and the
 // self-energy rhs (BUBBLE_SIGMA: it also reads the vertex input), so that a
-// flow can compute the tables before the vertex stage input exists.
+// flow can compute the tables before the vertex stage input exists.  half (FP64):
+// the self-energy rhs for the lower half of the frequencies, the others their
+// mirrors' conjugates (a reversal-symmetric input).
 constexpr int BUBBLE_TABLES = 1, BUBBLE_SIGMA = 2;
 int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split, int mask,
-                        cudaStream_t st, int parts = BUBBLE_TABLES | BUBBLE_SIGMA, bool chain = false);
+                        cudaStream_t st, int parts = BUBBLE_TABLES | BUBBLE_SIGMA, bool chain = false, bool half = false);
 // Frequency-box tails: the window propagators and the sums over the window
 // (TAIL_WINDOW), then the constants, the self-energy's added to the
 // self-energy rhs (TAIL_FINISH: after launch_bubble_sigma's self-energy

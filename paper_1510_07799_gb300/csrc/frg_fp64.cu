@@ -47,7 +47,7 @@ __global__ void k_bubble_gs(const PointDesc *__restrict__ pts, const RhsIO *__re
 // shared memory: a thread reads each value it needs about once.
 template <bool SPLIT>
 __global__ void __launch_bounds__(128)
-    k_bubble_sigma(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, int maxN, int sigma_on, int b0) {
+    k_bubble_sigma(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, int maxN, int sigma_on, int b0, int half) {
   chain_wait();
   const int pi = blockIdx.y;
   const RhsIO &o = io[pi];
@@ -60,13 +60,14 @@ __global__ void __launch_bounds__(128)
   const int which = table ? b / nrow_max : 0;
   const int row = table ? b % nrow_max : 0;
   const int w = table ? 0 : b - 2 * nrow_max;
-  if (table ? row >= 2 * N - 1 : w >= N) return;
+  if (table ? row >= 2 * N - 1 : w >= (half ? N / 2 : N)) return;
   const double2 *__restrict__ Gp = P.G;
   const double2 *__restrict__ Sp = P.S;
   const double L = *o.lam;
   if (!table) {
     __shared__ double2 part[4];
     sigma_entry<SPLIT>(P, o, w, threadIdx.x, sigma_on != 0, part, SyncBlock{});
+    if (half && threadIdx.x == 0) o.dsig[N - 1 - w] = make_double2(o.dsig[w].x, -o.dsig[w].y);
     return;
   }
   // Lpp[s][p] = Lb(p, s-p), Lph[Q+N-1][p] = Lb(p, p+Q); split paths also get
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(128)
 }
 
 int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split, int mask,
-                        cudaStream_t st, int parts, bool chain) {
+                        cudaStream_t st, int parts, bool chain, bool half) {
   const int nrow_max = 2 * maxN - 1;
   // split flows run these beside the stage kernel
   const int cv = split ? side_carveout(n_points, mask) : -1;
@@ -144,12 +145,12 @@ int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points,
   }
   // blocks [0, 2 nrow_max): table rows; [2 nrow_max, 2 nrow_max + maxN): self-energy entries
   const int b0 = (parts & BUBBLE_TABLES) ? 0 : 2 * nrow_max;
-  const int b1 = (parts & BUBBLE_SIGMA) ? 2 * nrow_max + maxN : 2 * nrow_max;
+  const int b1 = (parts & BUBBLE_SIGMA) ? 2 * nrow_max + (half ? maxN / 2 : maxN) : 2 * nrow_max;
   if (b1 > b0) {
     const dim3 g(b1 - b0, n_points);
     const int sig = (mask & 8) != 0;
     const cudaError_t e2 = launch_ex(split ? k_bubble_sigma<true> : k_bubble_sigma<false>, g, 128, 0, st, cv, chain, d_pts,
-                                     d_io, maxN, sig, b0);
+                                     d_io, maxN, sig, b0, half ? 1 : 0);
     if (e == cudaSuccess) e = e2;
     FRG_COUNT(1);
   }

@@ -38,8 +38,10 @@ __host__ __device__ inline int lanes(int N) {
   return l;
 }
 __host__ __device__ inline int pitch(int N) { return N + 1; }
-__host__ __device__ inline int blocks(int N) {
-  return N * ((N + rows(N) - 1) / rows(N)) + (N + T / 32 - 1) / (T / 32);
+// (half: a reversal-symmetric input, the rows k1 < N / 2 and their frequencies)
+__host__ __device__ inline int blocks(int N, bool half) {
+  const int n = half ? N / 2 : N;
+  return n * ((N + rows(N) - 1) / rows(N)) + (n + T / 32 - 1) / (T / 32);
 }
 // G, S, B, W1, Wa, Wb, W3
 __host__ __device__ inline size_t smem(int N) {
@@ -51,11 +53,11 @@ __host__ __device__ inline size_t smem(int N) {
 // vertex blocks and then the self-energy by one block.
 enum Part { ALL, VERTEX, SIGMA };
 
-__device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int part, int b,
-                                    double2 *sm) {
+__device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int part, bool half,
+                                    int b, double2 *sm) {
   const int N = P.N, R = rows(N), PL = lanes(N), W = pitch(N), tid = threadIdx.x;
-  const int nb = (N + R - 1) / R;
-  if (b >= (part == VERTEX ? N * nb : part == SIGMA ? 1 : blocks(N))) return;
+  const int nb = (N + R - 1) / R, nk = half ? N / 2 : N;
+  if (b >= (part == VERTEX ? nk * nb : part == SIGMA ? 1 : blocks(N, half))) return;
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
   double2 *G = sm, *S = G + N, *B = S + N, *W1 = B + N * W, *Wa = W1 + N * W, *Wb = Wa + R * W, *W3 = Wb + R * W;
   for (int i = tid; i < N; i += T) {
@@ -66,11 +68,11 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
   }
   __syncthreads();
   const double sc = P.T * lam;
-  if (part == SIGMA || b >= N * nb) {
+  if (part == SIGMA || b >= nk * nb) {
     // self-energy: one warp per frequency
     const int lane = tid & 31;
-    int w = (part == SIGMA ? 0 : b - N * nb) * (T / 32) + (tid >> 5);
-    for (; w < N; w += part == SIGMA ? T / 32 : N) {
+    int w = (part == SIGMA ? 0 : b - nk * nb) * (T / 32) + (tid >> 5);
+    for (; w < nk; w += part == SIGMA ? T / 32 : N) {
       double2 acc = make_double2(0.0, 0.0);
       if (mask & FRG_CH_SIGMA)
         for (int p = lane; p < N; p += 32) {
@@ -81,7 +83,11 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
         acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
       }
-      if (lane == 0) o.dsig[w] = cscale(acc, sc);
+      if (lane == 0) {
+        const double2 v = cscale(acc, sc);
+        o.dsig[w] = v;
+        if (half) o.dsig[N - 1 - w] = make_double2(v.x, -v.y);
+      }
     }
     return;
   }
@@ -160,25 +166,29 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
       v.x += __shfl_xor_sync(0xffffffffu, v.x, off);
       v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
     }
-    if (on && l == 0) out[(k1 * N + k2) * N + k3] = v;
+    if (on && l == 0) {
+      const int at = (k1 * N + k2) * N + k3;
+      out[at] = v;
+      if (half) out[N * N * N - 1 - at] = make_double2(v.x, -v.y);
+    }
   }
 }
 
 __global__ void __launch_bounds__(T) k_rhs_small(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                                                 int n_below, int mask, int part) {
+                                                 int n_below, int mask, int part, int half) {
   extern __shared__ double2 sm[];
   chain_wait();
   const PointDesc &P = pts[blockIdx.y];
   const RhsIO &o = io[blockIdx.y];
   if (!o.active || P.N >= n_below) return;
-  rhs(P, o, *o.lam, mask, part, blockIdx.x, sm);
+  rhs(P, o, *o.lam, mask, part, half != 0, blockIdx.x, sm);
 }
 
 __global__ void __launch_bounds__(T) k_rhs_small_value(const __grid_constant__ PointDesc P,
                                                        const __grid_constant__ RhsIO o, double lam, int mask,
                                                        int part) {
   extern __shared__ double2 sm[];
-  rhs(P, o, lam, mask, part, blockIdx.x, sm);
+  rhs(P, o, lam, mask, part, false, blockIdx.x, sm);
 }
 
 // (a host-side setting of the current device's context: set on every call, as
@@ -191,7 +201,7 @@ bool room(K kernel, size_t bytes) {
 }  // namespace small
 
 int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int n_below, int mask,
-                     bool sig_in_place, cudaStream_t st, bool chain) {
+                     bool sig_in_place, cudaStream_t st, bool chain, bool half) {
   // shared memory and blocks for every size below the bound (both drop where the
   // rows per block step up)
   const int N = maxN < n_below ? maxN : n_below - 1;
@@ -199,17 +209,17 @@ int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
   int blocks = 0;
   for (int n = 2; n <= N; n += 2) {
     bytes = small::smem(n) > bytes ? small::smem(n) : bytes;
-    blocks = small::blocks(n) > blocks ? small::blocks(n) : blocks;
+    blocks = small::blocks(n, half) > blocks ? small::blocks(n, half) : blocks;
   }
   if (!small::room(small::k_rhs_small, bytes)) return -3;
   const int first = sig_in_place ? small::VERTEX : small::ALL;
   if (launch_chained(small::k_rhs_small, dim3(blocks, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
-                     first) != cudaSuccess)
+                     first, half ? 1 : 0) != cudaSuccess)
     return -3;
   FRG_COUNT(1);
   if (sig_in_place) {
     if (launch_chained(small::k_rhs_small, dim3(1, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
-                       (int)small::SIGMA) != cudaSuccess)
+                       (int)small::SIGMA, half ? 1 : 0) != cudaSuccess)
       return -3;
     FRG_COUNT(1);
   }
@@ -221,7 +231,7 @@ int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int m
   const size_t bytes = small::smem(P.N);
   if (!small::room(small::k_rhs_small_value, bytes)) return -3;
   const int first = sig_in_place ? small::VERTEX : small::ALL;
-  small::k_rhs_small_value<<<small::blocks(P.N), small::T, bytes, st>>>(P, o, lam, mask, first);
+  small::k_rhs_small_value<<<small::blocks(P.N, false), small::T, bytes, st>>>(P, o, lam, mask, first);
   FRG_COUNT(1);
   if (sig_in_place) {
     small::k_rhs_small_value<<<1, small::T, bytes, st>>>(P, o, lam, mask, small::SIGMA);

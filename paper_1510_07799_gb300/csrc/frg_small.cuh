@@ -7,8 +7,10 @@ constexpr int SMALL_MAX_N = 64;  // limited by the block's shared memory
 // Vertex and self-energy rhs of every active point with N < n_below (<= 65).
 // sig_in_place: a self-energy output overlaps its input (the self-energy rhs then
 // takes a launch of one block per point, after every other block has read it).
+// chain: see launch_ex.  half: the inputs are reversal-symmetric, so the entries
+// with i1 < N / 2 give the others as conjugates.
 int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int n_below, int mask,
-                     bool sig_in_place, cudaStream_t st, bool chain);
+                     bool sig_in_place, cudaStream_t st, bool chain, bool half);
 // The same for one point (N <= SMALL_MAX_N) given by value: no device memory.
 int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int mask, bool sig_in_place,
                            cudaStream_t st);

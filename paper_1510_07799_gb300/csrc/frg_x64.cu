@@ -217,7 +217,7 @@ __device__ __forceinline__ void panel(const PointDesc &P, const RhsIO &o, const 
 template <int U>
 __global__ void __launch_bounds__(FRG_MAX_N *PAN_LINES / U, U == 8 ? 3 : 2)
     k_x64_panels(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp, int p0,
-                 int chmask) {
+                 int chmask, int rev) {
   __shared__ double2 sw[FRG_MAX_N];
   __shared__ unsigned smax[PAN_LINES];
   chain_wait();
@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(FRG_MAX_N *PAN_LINES / U, U == 8 ? 3 : 2)
   if (!o.active || !x.prod || !(chmask >> ch & 1)) return;
   const PointDesc &P = pts[pi];
   const int half = gridDim.x / 2, y = blockIdx.y;
-  if (y >= 2 * P.N - 1) return;
-  const int m = P.N - 1 + (y & 1 ? (y + 1) / 2 : -(y / 2));
+  if (y >= (rev ? P.N : 2 * P.N - 1)) return;
+  const int m = rev ? P.N - 1 - y : P.N - 1 + (y & 1 ? (y + 1) / 2 : -(y / 2));
   const int b = blockIdx.x;
   if (b < half) {
     if (ch == CH_PP)
@@ -660,15 +660,19 @@ __device__ double2 entry_sum(const PointDesc &P, const void *gam, int m, int row
     cfma(acc, left_elem<CH>(P, gam, g, row - g.row_lo, k), right_elem<CH>(P, gam, g, k, col));
   return acc;
 }
-__device__ __noinline__ void marked_entry(const PointDesc &P, const RhsIO &o, int i1, int i2, int i3, int chmask) {
+__device__ __noinline__ void marked_entry(const PointDesc &P, const RhsIO &o, int i1, int i2, int i3, int chmask,
+                                          bool rev) {
   const int N = P.N;
   const double sc = P.T * (*o.lam);
   double2 v = make_double2(0.0, 0.0);
   if (chmask & 1) v = cscale(entry_sum<CH_PP>(P, o.gam, i1 + i2, i1, i3), -sc);
   if (chmask & 2) v = cadd(v, cscale(entry_sum<CH_DPH>(P, o.gam, i3 - i1 + N - 1, i1, i2), sc));
   if (chmask & 4) v = cadd(v, cscale(entry_sum<CH_XPH>(P, o.gam, i2 - i3 + N - 1, i3, i1), -sc));
-  static_cast<double2 *>(o.dgam)[((size_t)i1 * N + i2) * N + i3] = v;
+  const size_t e = ((size_t)i1 * N + i2) * N + i3;
+  static_cast<double2 *>(o.dgam)[e] = v;
+  if (rev) static_cast<double2 *>(o.dgam)[(size_t)N * N * N - 1 - e] = make_double2(v.x, -v.y);
 }
+template <bool REV>
 __global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restrict__ pts,
                                                      const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
                                                      int p0, int nz, int chmask) {
@@ -678,9 +682,12 @@ __global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restr
   const X64Pt &x = xp[pi];
   if (!o.active || !x.prod) return;
   const PointDesc &P = pts[pi];
-  const int N = P.N, t = threadIdx.x;
+  // REV: the rows i1 < N / 2, each entry from its own transfer or, where that is
+  // above N - 1, as the conjugate of its mirror's, and its mirror as the conjugate
+  const int N = P.N, n1 = REV ? N / 2 : N, t = threadIdx.x;
+  const size_t end = (size_t)N * N * N - 1;
   const int i1 = 4 * (blockIdx.z % nz), b2 = 8 * blockIdx.y, b3 = 32 * blockIdx.x;
-  if (i1 >= N || b2 >= N || b3 >= N) return;
+  if (i1 >= n1 || b2 >= N || b3 >= N) return;
   const int i2 = b2 + 4 * (t >> 7) + ((t >> 3) & 3), i3 = b3 + 8 * ((t >> 5) & 3) + (t & 7);
   const int bad = x.bad[0];
   double2 *out = static_cast<double2 *>(o.dgam);
@@ -689,24 +696,35 @@ __global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restr
   double2 a[4], b[4], c[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const bool in = on && i1 + j < N;
-    a[j] = in && (chmask & 1) ? out[((size_t)(i1 + j) * N + i2) * N + i3] : z;
-    b[j] = in && (chmask & 2) ? x.PX[((size_t)(i1 + j) * N + i3) * N + i2] : z;
-    c[j] = in && (chmask & 4) ? x.PW[((size_t)i2 * N + i3) * N + i1 + j] : z;
+    const bool in = on && i1 + j < n1;
+    const size_t ea = ((size_t)(i1 + j) * N + i2) * N + i3, eb = ((size_t)(i1 + j) * N + i3) * N + i2,
+                 ec = ((size_t)i2 * N + i3) * N + i1 + j;
+    const bool ma = REV && i1 + j + i2 > N - 1, mb = REV && i3 > i1 + j, mc = REV && i2 > i3;
+    a[j] = in && (chmask & 1) ? out[ma ? end - ea : ea] : z;
+    b[j] = in && (chmask & 2) ? x.PX[mb ? end - eb : eb] : z;
+    c[j] = in && (chmask & 4) ? x.PW[mc ? end - ec : ec] : z;
+    if (ma) a[j].y = -a[j].y;
+    if (mb) b[j].y = -b[j].y;
+    if (mc) c[j].y = -c[j].y;
   }
   if (bad) {
     if (on)
-      for (int j = 0; j < 4 && i1 + j < N; ++j) marked_entry(P, o, i1 + j, i2, i3, chmask);
+      for (int j = 0; j < 4 && i1 + j < n1; ++j) marked_entry(P, o, i1 + j, i2, i3, chmask, REV);
     // the point's last block (every block has read the mark) clears it
     __syncthreads();
-    const int blocks = ((N + 3) / 4) * ((N + 7) / 8) * ((N + 31) / 32);
+    const int blocks = ((n1 + 3) / 4) * ((N + 7) / 8) * ((N + 31) / 32);
     if (t == 0 && atomicAdd(&x.bad[1], 1) == blocks - 1) x.bad[0] = x.bad[1] = 0;
     return;
   }
   if (!on) return;
 #pragma unroll
   for (int j = 0; j < 4; ++j)
-    if (i1 + j < N) out[((size_t)(i1 + j) * N + i2) * N + i3] = cadd(cadd(a[j], b[j]), c[j]);
+    if (i1 + j < n1) {
+      const size_t e = ((size_t)(i1 + j) * N + i2) * N + i3;
+      const double2 v = cadd(cadd(a[j], b[j]), c[j]);
+      out[e] = v;
+      if (REV) out[end - e] = make_double2(v.x, -v.y);
+    }
 }
 }  // namespace x64
 
@@ -715,7 +733,7 @@ struct X64Plan {
   using Sched = Schedule<x64::Work>;
   struct Group {
     int p0, p1, maxN;
-    Sched all;
+    Sched all, half;  // half: the transfers m < N
   };
   std::vector<X64Pt> h;
   std::vector<int> N;          // per point, 0: not on this path
@@ -848,7 +866,10 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
     if (!ok) break;
     std::vector<std::pair<int, x64::Work>> all;
     for (int i = g.p0; i < g.p1; ++i) all.insert(all.end(), tiles[i].begin(), tiles[i].end());
-    ok = upload_schedule(g.all, all, sms);
+    std::vector<std::pair<int, x64::Work>> low;
+    for (auto &t : all)
+      if (t.second.m < pts[t.second.point].N) low.push_back(t);
+    ok = upload_schedule(g.all, all, sms) && upload_schedule(g.half, low, sms);
   }
   ok = ok && cudaMemcpy(p->d_x, p->h.data(), sizeof(X64Pt) * n, cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) {
@@ -862,7 +883,10 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
 void x64_destroy(X64Plan *p) {
   if (!p) return;
   for (auto &s : p->one) drop_schedule(s);
-  for (auto &g : p->groups) drop_schedule(g.all);
+  for (auto &g : p->groups) {
+    drop_schedule(g.all);
+    drop_schedule(g.half);
+  }
   for (void *t : p->tables) cudaFree(t);
   cudaFree(p->d_x);
   cudaFree(p->d_bad);
@@ -873,11 +897,11 @@ void x64_destroy(X64Plan *p) {
 bool x64_has(const X64Plan *p, int point) { return p && p->N[point] > 0; }
 
 int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st,
-            bool chain) {
+            bool chain, bool half) {
   for (size_t gi = 0; gi < p->groups.size(); ++gi) {
     X64Plan::Group &g = p->groups[gi];
     int p0 = g.p0, p1 = g.p1, maxN = g.maxN;
-    const X64Plan::Sched *s = &g.all;
+    const X64Plan::Sched *s = half ? &g.half : &g.all;
     if (point >= 0) {
       if (point < g.p0 || point >= g.p1) continue;
       p0 = point;
@@ -886,18 +910,19 @@ int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, in
       if (p->N.size() > 1) s = &p->one[point];
     }
     const int oct = (maxN + x64::PAN_LINES - 1) / x64::PAN_LINES, np = p1 - p0;
-    const dim3 pg(2 * oct, 2 * maxN - 1, 3 * np);
-    const int nz = (maxN + 3) / 4;
+    const dim3 pg(2 * oct, half ? maxN : 2 * maxN - 1, 3 * np);
+    const int nz = ((half ? maxN / 2 : maxN) + 3) / 4, rev = half ? 1 : 0;
     // The combine is not chained: blocks that become resident beside the products' find
     // the SM's storage set up as shared memory and next to no L1, and so do the kernels
     // chained to them (N = 128 336 against 322 us per rhs, N = 64 62.0 against 59.8 us
     // and 37.8 against 35.8 ms per flow; nothing chained 327 and 65.0 us, 36.2 ms).
     if (launch_chained(x64::panel_u(maxN) == 8 ? x64::k_x64_panels<8> : x64::k_x64_panels<4>, pg,
-                       x64::panel_threads(maxN), 0, st, chain, d_pts, d_io, p->d_x, p0, chmask) != cudaSuccess ||
+                       x64::panel_threads(maxN), 0, st, chain, d_pts, d_io, p->d_x, p0, chmask, rev) != cudaSuccess ||
         launch_chained(x64::k_x64_products, s->grid, x64::THREADS, x64::SMEM, st, chain, d_pts, d_io, p->d_x, s->work,
                        s->start, p->d_err) != cudaSuccess ||
-        launch_chained(x64::k_x64_combine, dim3((maxN + 31) / 32, (maxN + 7) / 8, nz * np), 256, 0, st, false, d_pts,
-                       d_io, p->d_x, p0, nz, chmask) != cudaSuccess)
+        launch_chained(half ? x64::k_x64_combine<true> : x64::k_x64_combine<false>,
+                       dim3((maxN + 31) / 32, (maxN + 7) / 8, nz * np), 256, 0, st, false, d_pts, d_io, p->d_x, p0, nz,
+                       chmask) != cudaSuccess)
       return -3;
     FRG_COUNT(3);
   }

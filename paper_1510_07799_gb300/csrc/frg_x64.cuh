@@ -29,7 +29,9 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
 void x64_destroy(X64Plan *p);
 bool x64_has(const X64Plan *p, int point);
 // Channel products of every point of the plan (point < 0) or of one point; chain:
-// see launch_ex.
+// see launch_ex; half (every point): the inputs are reversal-symmetric, so the
+// transfers m < N give the others (V(N-1-i1, N-1-i2, N-1-i3) = conj V(i1, i2, i3)
+// takes transfer m of each channel to 2N - 2 - m).
 int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, int chmask, cudaStream_t st,
-            bool chain);
+            bool chain, bool half);
 }  // namespace frg
