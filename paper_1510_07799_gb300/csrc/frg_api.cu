@@ -507,11 +507,12 @@ static int issue_step(frg_ctx *ctx) {
       // stage sums 2..6 that read them
       if ((rc = run_split_stage(ctx, s, s == 6, s >= 2, s <= 5))) return rc;
     } else {
-      LK(launch_stage_fp64(ctx->d_pts, ctx->d_ctl, s, ctx->d_io_stage, st, ctx->n, ctx->maxN), "stage sum");
+      LK(launch_stage_fp64(ctx->d_pts, ctx->d_ctl, s, ctx->d_io_stage, st, ctx->n, ctx->maxN, ctx->rev_on),
+         "stage sum");
       if ((rc = run_rhs_fp64(ctx, ctx->d_io_stage, -1))) return rc;
     }
   }
-  if (!ctx->split) LK(launch_error(ctx->d_pts, ctx->d_ctl, st, ctx->n, ctx->maxN), "error norm");
+  if (!ctx->split) LK(launch_error(ctx->d_pts, ctx->d_ctl, st, ctx->n, ctx->maxN, ctx->rev_on), "error norm");
   LK(launch_controller(ctx->d_pts, ctx->d_ctl, ctx->n, st), "controller");
   return FRG_OK;
 }

@@ -219,11 +219,13 @@ __device__ __forceinline__ void block_max_to(float v, unsigned *dst) {
 // FP64 units (2 (s + 1) multiply-adds per element, 22 for the seventh stage).
 // Measured at N = 64: 6-11 us per stage and 16 us for the seventh, against 13-25
 // us with eight elements per thread in turn on 129 blocks; N = 16 5 against
-// 12-25 us.
+// 12-25 us.  half (a flow under the reversal reduction): the entries i < n3 / 2,
+// their mirrors n3 - 1 - i as conjugates (every operation here commutes with the
+// conjugation, so nothing changes but the work), and the self-energy.
 constexpr int ST_T = 256;
 template <int S>
 __global__ void __launch_bounds__(ST_T) k_stage(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl,
-                                                RhsIO *__restrict__ io) {
+                                                RhsIO *__restrict__ io, int half) {
   chain_wait();
   const int pi = blockIdx.y;
   const PointDesc &P = pts[pi];
@@ -231,19 +233,19 @@ __global__ void __launch_bounds__(ST_T) k_stage(const PointDesc *__restrict__ pt
   if (blockIdx.x == 0 && threadIdx.x == 0) write_stage_io(P, ctl[pi], io + pi, S, 0);
   const Ctl &c = ctl[pi];
   if (c.done) return;
-  const int n3 = P.n3, n = n3 + P.N;
+  const int n3 = P.n3, nv = half ? n3 / 2 : n3, n = nv + P.N;
   const int i = blockIdx.x * ST_T + threadIdx.x;
   if (i >= n) return;
   const double h = c.h;
-  const int ys = c.yslot;
+  const int ys = c.yslot, iy = i < nv ? i : n3 + (i - nv);  // (the self-energy follows the whole vertex)
   double2 k[S];
 #pragma unroll
   for (int j = 0; j < S; ++j) {
     if (S == 6 && j == 1) continue;  // the fifth-order weight of k2 is zero: no read
     const int kj = c.kslot[j];
-    k[j] = i < n3 ? static_cast<const double2 *>(P.kG[kj])[i] : P.kS[kj][i - n3];
+    k[j] = i < nv ? static_cast<const double2 *>(P.kG[kj])[i] : P.kS[kj][i - nv];
   }
-  const double2 yi = P.ybuf[ys][i];
+  const double2 yi = P.ybuf[ys][iy];
   double2 acc = make_double2(0.0, 0.0);
 #pragma unroll
   for (int j = 0; j < S; ++j) {
@@ -252,10 +254,10 @@ __global__ void __launch_bounds__(ST_T) k_stage(const PointDesc *__restrict__ pt
     acc.y += dA[S][j] * k[j].y;
   }
   const double2 Y = make_double2(yi.x + h * acc.x, yi.y + h * acc.y);
-  if (S < 6) {
-    P.Y64[i] = Y;
-  } else {
-    P.ybuf[ys ^ 1][i] = Y;
+  double2 *out = S < 6 ? P.Y64 : P.ybuf[ys ^ 1];
+  out[iy] = Y;
+  if (half && i < nv) out[n3 - 1 - i] = make_double2(Y.x, -Y.y);
+  if (S == 6) {
     double2 e = make_double2(0.0, 0.0);
 #pragma unroll
     for (int j = 0; j < S; ++j) {
@@ -264,10 +266,10 @@ __global__ void __launch_bounds__(ST_T) k_stage(const PointDesc *__restrict__ pt
       e.y += dE[j] * k[j].y;
     }
     const int k2 = c.kslot[1];
-    if (i < n3)
+    if (i < nv)
       static_cast<double2 *>(P.kG[k2])[i] = e;
     else
-      P.kS[k2][i - n3] = e;
+      P.kS[k2][i - nv] = e;
   }
 }
 
@@ -512,13 +514,13 @@ __device__ __forceinline__ double maxabs(double a, double b) {
   return __longlong_as_double(x > y ? x : y);
 }
 constexpr int ERR_T = 512;
-__global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl) {
+__global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl, int half) {
   chain_wait();
   const int pi = blockIdx.y;
   Ctl &c = ctl[pi];
   if (c.done) return;
   const PointDesc &P = pts[pi];
-  const int n3 = P.n3, n = n3 + P.N;
+  const int n3 = P.n3, nv = half ? n3 / 2 : n3, n = nv + P.N;
   if (blockIdx.x * ERR_T >= n) return;
   const int i = blockIdx.x * ERR_T + threadIdx.x;
   __shared__ unsigned wmax[ERR_T / 32];
@@ -531,10 +533,11 @@ __global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ p
   const bool on = i < n;
   if (on) {
     const int k2 = c.kslot[1], k7 = c.kslot[6];
-    acc = i < n3 ? static_cast<const double2 *>(P.kG[k2])[i] : P.kS[k2][i - n3];
-    const double2 k = i < n3 ? static_cast<const double2 *>(P.kG[k7])[i] : P.kS[k7][i - n3];
-    yi = P.ybuf[c.yslot][i];
-    yni = P.ybuf[c.yslot ^ 1][i];
+    const int iy = i < nv ? i : n3 + (i - nv);
+    acc = i < nv ? static_cast<const double2 *>(P.kG[k2])[i] : P.kS[k2][i - nv];
+    const double2 k = i < nv ? static_cast<const double2 *>(P.kG[k7])[i] : P.kS[k7][i - nv];
+    yi = P.ybuf[c.yslot][iy];
+    yni = P.ybuf[c.yslot ^ 1][iy];
     acc.x += dE[6] * k.x;
     acc.y += dE[6] * k.y;
     bad = !isfinite(yni.x) || !isfinite(yni.y);
@@ -662,16 +665,17 @@ int stage_split_init() {
 }
 
 int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cudaStream_t st, int n_points,
-                      int maxN) {
-  const dim3 g((maxN * maxN * maxN + maxN + ST_T - 1) / ST_T, n_points);
+                      int maxN, bool rev) {
+  const int n3 = maxN * maxN * maxN, half = rev ? 1 : 0;
+  const dim3 g(((rev ? n3 / 2 : n3) + maxN + ST_T - 1) / ST_T, n_points);
   cudaError_t e;
   switch (s) {
-    case 1: e = launch_chained(k_stage<1>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
-    case 2: e = launch_chained(k_stage<2>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
-    case 3: e = launch_chained(k_stage<3>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
-    case 4: e = launch_chained(k_stage<4>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
-    case 5: e = launch_chained(k_stage<5>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
-    case 6: e = launch_chained(k_stage<6>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io); break;
+    case 1: e = launch_chained(k_stage<1>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io, half); break;
+    case 2: e = launch_chained(k_stage<2>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io, half); break;
+    case 3: e = launch_chained(k_stage<3>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io, half); break;
+    case 4: e = launch_chained(k_stage<4>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io, half); break;
+    case 5: e = launch_chained(k_stage<5>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io, half); break;
+    case 6: e = launch_chained(k_stage<6>, g, ST_T, 0, st, true, d_pts, d_ctl, d_io, half); break;
     default: return -1;
   }
   FRG_COUNT(1);
@@ -740,10 +744,11 @@ int launch_sigma_stage(const PointDesc *d_pts, Ctl *d_ctl, RhsIO *d_io, int s, i
   return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int launch_error(const PointDesc *d_pts, Ctl *d_ctl, cudaStream_t st, int n_points, int maxN) {
-  const dim3 g((maxN * maxN * maxN + maxN + ERR_T - 1) / ERR_T, n_points);
+int launch_error(const PointDesc *d_pts, Ctl *d_ctl, cudaStream_t st, int n_points, int maxN, bool rev) {
+  const int n3 = maxN * maxN * maxN;
+  const dim3 g(((rev ? n3 / 2 : n3) + maxN + ERR_T - 1) / ERR_T, n_points);
   FRG_COUNT(1);
-  return launch_chained(k_error, g, ERR_T, 0, st, true, d_pts, d_ctl) == cudaSuccess ? 0 : -3;
+  return launch_chained(k_error, g, ERR_T, 0, st, true, d_pts, d_ctl, rev ? 1 : 0) == cudaSuccess ? 0 : -3;
 }
 
 int launch_controller(const PointDesc *d_pts, Ctl *d_ctl, int n, cudaStream_t st) {

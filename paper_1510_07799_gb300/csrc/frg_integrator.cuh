@@ -22,8 +22,10 @@ int launch_finish_k1(Ctl *d_ctl, const RhsIO *d_io, int n, cudaStream_t st);
 int launch_prepare(const PointDesc *d_pts, Ctl *d_ctl, int n, cudaStream_t st);
 // FP64 path: stage sum s (1..6) of every point; the first block of each point
 // also writes the stage's rhs IO record (as launch_set_stage_io), and the seventh
-// stage leaves the partial error sum in the place of k2.
-int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cudaStream_t st, int n_points, int maxN);
+// stage leaves the partial error sum in the place of k2.  rev (here and in
+// launch_error): the flow keeps the reversal reduction.
+int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cudaStream_t st, int n_points, int maxN,
+                      bool rev);
 // Split paths: stage sum s of every point, the vertex part only, on a grid of
 // lb_grid x n_points layout blocks (frg_lblock.cuh; lb_grid = the largest
 // point's vertex blocks), also writing the W / X / Z copies in `want`;
@@ -43,7 +45,7 @@ int launch_sigma_stage(const PointDesc *d_pts, Ctl *d_ctl, RhsIO *d_io, int s, i
 // Dynamic shared-memory limits of the split stage kernels (once per set-up).
 int stage_split_init();
 // FP64 path's error norm of the step (after the seventh rhs).
-int launch_error(const PointDesc *d_pts, Ctl *d_ctl, cudaStream_t st, int n_points, int maxN);
+int launch_error(const PointDesc *d_pts, Ctl *d_ctl, cudaStream_t st, int n_points, int maxN, bool rev);
 int launch_controller(const PointDesc *d_pts, Ctl *d_ctl, int n, cudaStream_t st);
 
 }  // namespace frg
