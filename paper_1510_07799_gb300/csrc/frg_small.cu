@@ -30,22 +30,26 @@ constexpr int T = 256;
 // k3 per block, and lanes that share an entry's p: enough blocks for the SMs on
 // the smallest grids, little repeated weight work on the larger ones.  (Splitting
 // p further, so that the warps fill the SM's four partitions evenly, gains
-// nothing: N = 40 138 us with four lanes against 127 us with one.)
-__host__ __device__ inline int rows(int N) { return N <= 24 ? 2 : N <= 40 ? 4 : 8; }
-__host__ __device__ inline int lanes(int N) {
-  int l = 8;
-  while (l > 1 && N * rows(N) * l > T) l >>= 1;
+// nothing: N = 40 138 us with four lanes against 127 us with one.)  Where one k3 per
+// block still fits the SMs in one go it halves a block's FP64 work: flow N = 16 7.05
+// -> 6.57 ms.  half: a reversal-symmetric input, the rows k1 < N / 2 and their
+// frequencies.
+__host__ __device__ inline int rows(int N, bool half) {
+  return (half ? N / 2 : N) * N <= 144 ? 1 : N <= 24 ? 2 : N <= 40 ? 4 : 8;
+}
+__host__ __device__ inline int lanes(int N, bool half) {
+  int l = 16;
+  while (l > 1 && N * rows(N, half) * l > T) l >>= 1;
   return l;
 }
 __host__ __device__ inline int pitch(int N) { return N + 1; }
-// (half: a reversal-symmetric input, the rows k1 < N / 2 and their frequencies)
 __host__ __device__ inline int blocks(int N, bool half) {
   const int n = half ? N / 2 : N;
-  return n * ((N + rows(N) - 1) / rows(N)) + (n + T / 32 - 1) / (T / 32);
+  return n * ((N + rows(N, half) - 1) / rows(N, half)) + (n + T / 32 - 1) / (T / 32);
 }
 // G, S, B, W1, Wa, Wb, W3
-__host__ __device__ inline size_t smem(int N) {
-  const int R = rows(N);
+__host__ __device__ inline size_t smem(int N, bool half) {
+  const int R = rows(N, half);
   return (size_t)(2 * N + (N + N + 2 * R + N + R - 1) * pitch(N)) * sizeof(double2);
 }
 
@@ -55,7 +59,7 @@ enum Part { ALL, VERTEX, SIGMA };
 
 __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int part, bool half,
                                     int b, double2 *sm) {
-  const int N = P.N, R = rows(N), PL = lanes(N), W = pitch(N), tid = threadIdx.x;
+  const int N = P.N, R = rows(N, half), PL = lanes(N, half), W = pitch(N), tid = threadIdx.x;
   const int nb = (N + R - 1) / R, nk = half ? N / 2 : N;
   if (b >= (part == VERTEX ? nk * nb : part == SIGMA ? 1 : blocks(N, half))) return;
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
@@ -208,7 +212,7 @@ int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
   size_t bytes = 0;
   int blocks = 0;
   for (int n = 2; n <= N; n += 2) {
-    bytes = small::smem(n) > bytes ? small::smem(n) : bytes;
+    bytes = small::smem(n, half) > bytes ? small::smem(n, half) : bytes;
     blocks = small::blocks(n, half) > blocks ? small::blocks(n, half) : blocks;
   }
   if (!small::room(small::k_rhs_small, bytes)) return -3;
@@ -228,7 +232,7 @@ int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
 
 int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int mask, bool sig_in_place,
                            cudaStream_t st) {
-  const size_t bytes = small::smem(P.N);
+  const size_t bytes = small::smem(P.N, false);
   if (!small::room(small::k_rhs_small_value, bytes)) return -3;
   const int first = sig_in_place ? small::VERTEX : small::ALL;
   small::k_rhs_small_value<<<small::blocks(P.N, false), small::T, bytes, st>>>(P, o, lam, mask, first);

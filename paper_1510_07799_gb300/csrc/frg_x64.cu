@@ -647,8 +647,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 // ------------------------------------------------------------- combine ----
 // dGamma = (pp + direct) + crossed, the enabled channels, into the natural
-// layout (the pp products are there already).  A thread takes four consecutive
-// i1 of one (i2, i3): 64 contiguous bytes of a W row; a warp covers 4 i2 (64
+// layout (the pp products are there already).  A thread takes IW consecutive
+// i1 of one (i2, i3): 32 contiguous bytes of a W row; a warp covers 4 i2 (64
 // bytes of each X row) x 8 i3 (128 bytes of each natural row).
 // The entries of a marked point are summed here, term by term as the tiles of the
 // CUDA-core products do (k_contract_fp64).
@@ -672,8 +672,12 @@ __device__ __noinline__ void marked_entry(const PointDesc &P, const RhsIO &o, in
   static_cast<double2 *>(o.dgam)[e] = v;
   if (rev) static_cast<double2 *>(o.dgam)[(size_t)N * N * N - 1 - e] = make_double2(v.x, -v.y);
 }
+// IW rows i1 per thread: two make a whole sector of the crossed output's layout, and
+// enough blocks (flow N = 64 25.9 ms, against 26.8 with four and 25.7 with one; N = 128
+// 320.8 us per rhs, against 322.5 and 324.4).
+constexpr int IW = 2;
 template <bool REV>
-__global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restrict__ pts,
+__global__ void __launch_bounds__(256, 6) k_x64_combine(const PointDesc *__restrict__ pts,
                                                      const RhsIO *__restrict__ io, const X64Pt *__restrict__ xp,
                                                      int p0, int nz, int chmask) {
   chain_wait();
@@ -686,16 +690,16 @@ __global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restr
   // above N - 1, as the conjugate of its mirror's, and its mirror as the conjugate
   const int N = P.N, n1 = REV ? N / 2 : N, t = threadIdx.x;
   const size_t end = (size_t)N * N * N - 1;
-  const int i1 = 4 * (blockIdx.z % nz), b2 = 8 * blockIdx.y, b3 = 32 * blockIdx.x;
+  const int i1 = IW * (blockIdx.z % nz), b2 = 8 * blockIdx.y, b3 = 32 * blockIdx.x;
   if (i1 >= n1 || b2 >= N || b3 >= N) return;
   const int i2 = b2 + 4 * (t >> 7) + ((t >> 3) & 3), i3 = b3 + 8 * ((t >> 5) & 3) + (t & 7);
   const int bad = x.bad[0];
   double2 *out = static_cast<double2 *>(o.dgam);
   const double2 z = make_double2(0.0, 0.0);
   const bool on = i2 < N && i3 < N;
-  double2 a[4], b[4], c[4];
+  double2 a[IW], b[IW], c[IW];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < IW; ++j) {
     const bool in = on && i1 + j < n1;
     const size_t ea = ((size_t)(i1 + j) * N + i2) * N + i3, eb = ((size_t)(i1 + j) * N + i3) * N + i2,
                  ec = ((size_t)i2 * N + i3) * N + i1 + j;
@@ -709,16 +713,16 @@ __global__ void __launch_bounds__(256, 4) k_x64_combine(const PointDesc *__restr
   }
   if (bad) {
     if (on)
-      for (int j = 0; j < 4 && i1 + j < n1; ++j) marked_entry(P, o, i1 + j, i2, i3, chmask, REV);
+      for (int j = 0; j < IW && i1 + j < n1; ++j) marked_entry(P, o, i1 + j, i2, i3, chmask, REV);
     // the point's last block (every block has read the mark) clears it
     __syncthreads();
-    const int blocks = ((n1 + 3) / 4) * ((N + 7) / 8) * ((N + 31) / 32);
+    const int blocks = ((n1 + IW - 1) / IW) * ((N + 7) / 8) * ((N + 31) / 32);
     if (t == 0 && atomicAdd(&x.bad[1], 1) == blocks - 1) x.bad[0] = x.bad[1] = 0;
     return;
   }
   if (!on) return;
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+  for (int j = 0; j < IW; ++j)
     if (i1 + j < n1) {
       const size_t e = ((size_t)(i1 + j) * N + i2) * N + i3;
       const double2 v = cadd(cadd(a[j], b[j]), c[j]);
@@ -911,7 +915,7 @@ int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, in
     }
     const int oct = (maxN + x64::PAN_LINES - 1) / x64::PAN_LINES, np = p1 - p0;
     const dim3 pg(2 * oct, half ? maxN : 2 * maxN - 1, 3 * np);
-    const int nz = ((half ? maxN / 2 : maxN) + 3) / 4, rev = half ? 1 : 0;
+    const int nz = ((half ? maxN / 2 : maxN) + x64::IW - 1) / x64::IW, rev = half ? 1 : 0;
     // The combine is not chained: blocks that become resident beside the products' find
     // the SM's storage set up as shared memory and next to no L1, and so do the kernels
     // chained to them (N = 128 336 against 322 us per rhs, N = 64 62.0 against 59.8 us
