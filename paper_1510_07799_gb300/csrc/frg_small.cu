@@ -27,15 +27,27 @@ namespace small {
 
 constexpr int T = 256;
 
-// k3 per block, and lanes that share an entry's p: enough blocks for the SMs on
-// the smallest grids, little repeated weight work on the larger ones.  (Splitting
-// p further, so that the warps fill the SM's four partitions evenly, gains
-// nothing: N = 40 138 us with four lanes against 127 us with one.)  Where one k3 per
-// block still fits the SMs in one go it halves a block's FP64 work: flow N = 16 7.05
-// -> 6.57 ms.  half: a reversal-symmetric input, the rows k1 < N / 2 and their
-// frequencies.
+// k3 per block, and lanes that share an entry's p.  A block's FP64 work is about
+// 1.2 + R units (the weights, and R entries per k2), and an SM takes its blocks' work
+// one after the other: the smallest R whose blocks still fit the 152 SMs in one go,
+// up to N = 36 (more than one block per SM costs N = 18 18.5 against 16.5 us, N = 36 92
+// against 77 us), and two or three goes of moderate R above (N = 40 127 us with R = 4,
+// 98 with 6, 125 with 14; N = 48 186 with 8, 162 with 16; N = 56 321 with 8, 390 with
+// 16).  half: a reversal-symmetric input, the rows k1 < N / 2 and their frequencies.
+// (Splitting p further, so that the warps fill the SM's four partitions evenly, gains
+// nothing.)
 __host__ __device__ inline int rows(int N, bool half) {
-  return (half ? N / 2 : N) * N <= 144 ? 1 : N <= 24 ? 2 : N <= 40 ? 4 : 8;
+  if (half) return N <= 16 ? 1 : N <= 24 ? 2 : 3;
+  return N <= 12   ? 1
+         : N <= 16 ? 2
+         : N <= 20 ? 3
+         : N <= 24 ? 4
+         : N <= 28 ? 6
+         : N <= 32 ? 8
+         : N <= 36 ? 9
+         : N <= 40 ? 6
+         : N <= 48 ? 16
+                   : 8;
 }
 __host__ __device__ inline int lanes(int N, bool half) {
   int l = 16;
@@ -57,11 +69,12 @@ __host__ __device__ inline size_t smem(int N, bool half) {
 // vertex blocks and then the self-energy by one block.
 enum Part { ALL, VERTEX, SIGMA };
 
-__device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int part, bool half,
+template <bool HALF>
+__device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double lam, int mask, int part,
                                     int b, double2 *sm) {
-  const int N = P.N, R = rows(N, half), PL = lanes(N, half), W = pitch(N), tid = threadIdx.x;
-  const int nb = (N + R - 1) / R, nk = half ? N / 2 : N;
-  if (b >= (part == VERTEX ? nk * nb : part == SIGMA ? 1 : blocks(N, half))) return;
+  const int N = P.N, R = rows(N, HALF), PL = lanes(N, HALF), W = pitch(N), tid = threadIdx.x;
+  const int nb = (N + R - 1) / R, nk = HALF ? N / 2 : N;
+  if (b >= (part == VERTEX ? nk * nb : part == SIGMA ? 1 : blocks(N, HALF))) return;
   const double2 *__restrict__ V = static_cast<const double2 *>(o.gam);
   double2 *G = sm, *S = G + N, *B = S + N, *W1 = B + N * W, *Wa = W1 + N * W, *Wb = Wa + R * W, *W3 = Wb + R * W;
   for (int i = tid; i < N; i += T) {
@@ -90,7 +103,7 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
       if (lane == 0) {
         const double2 v = cscale(acc, sc);
         o.dsig[w] = v;
-        if (half) o.dsig[N - 1 - w] = make_double2(v.x, -v.y);
+        if (HALF) o.dsig[N - 1 - w] = make_double2(v.x, -v.y);
       }
     }
     return;
@@ -173,26 +186,27 @@ __device__ __forceinline__ void rhs(const PointDesc &P, const RhsIO &o, double l
     if (on && l == 0) {
       const int at = (k1 * N + k2) * N + k3;
       out[at] = v;
-      if (half) out[N * N * N - 1 - at] = make_double2(v.x, -v.y);
+      if (HALF) out[N * N * N - 1 - at] = make_double2(v.x, -v.y);
     }
   }
 }
 
+template <bool HALF>
 __global__ void __launch_bounds__(T) k_rhs_small(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                                                 int n_below, int mask, int part, int half) {
+                                                 int n_below, int mask, int part) {
   extern __shared__ double2 sm[];
   chain_wait();
   const PointDesc &P = pts[blockIdx.y];
   const RhsIO &o = io[blockIdx.y];
   if (!o.active || P.N >= n_below) return;
-  rhs(P, o, *o.lam, mask, part, half != 0, blockIdx.x, sm);
+  rhs<HALF>(P, o, *o.lam, mask, part, blockIdx.x, sm);
 }
 
 __global__ void __launch_bounds__(T) k_rhs_small_value(const __grid_constant__ PointDesc P,
                                                        const __grid_constant__ RhsIO o, double lam, int mask,
                                                        int part) {
   extern __shared__ double2 sm[];
-  rhs(P, o, lam, mask, part, false, blockIdx.x, sm);
+  rhs<false>(P, o, lam, mask, part, blockIdx.x, sm);
 }
 
 // (a host-side setting of the current device's context: set on every call, as
@@ -215,15 +229,16 @@ int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
     bytes = small::smem(n, half) > bytes ? small::smem(n, half) : bytes;
     blocks = small::blocks(n, half) > blocks ? small::blocks(n, half) : blocks;
   }
-  if (!small::room(small::k_rhs_small, bytes)) return -3;
+  const auto kernel = half ? small::k_rhs_small<true> : small::k_rhs_small<false>;
+  if (!small::room(kernel, bytes)) return -3;
   const int first = sig_in_place ? small::VERTEX : small::ALL;
-  if (launch_chained(small::k_rhs_small, dim3(blocks, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
-                     first, half ? 1 : 0) != cudaSuccess)
+  if (launch_chained(kernel, dim3(blocks, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
+                     first) != cudaSuccess)
     return -3;
   FRG_COUNT(1);
   if (sig_in_place) {
-    if (launch_chained(small::k_rhs_small, dim3(1, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
-                       (int)small::SIGMA, half ? 1 : 0) != cudaSuccess)
+    if (launch_chained(kernel, dim3(1, n_points), small::T, bytes, st, chain, d_pts, d_io, n_below, mask,
+                       (int)small::SIGMA) != cudaSuccess)
       return -3;
     FRG_COUNT(1);
   }

@@ -7,8 +7,9 @@
 namespace frg {
 
 // Smallest grid whose FP64 channel products take the sliced tensor-core path; the
-// ones below take the one-launch rhs (frg_small.cu).  Measured per rhs: N = 24 44
-// (sliced) against 29 us, N = 28 47 us either way, N = 32 48 against 57 us.
+// ones below take the one-launch rhs (frg_small.cu).  Measured per rhs: N = 24 32
+// (sliced) against 25 us, N = 26 39 against 35 us, N = 28 37 against 40 us, N = 32 40
+// against 47 us.
 constexpr int X64_MIN_N = 28;
 
 // Device-side operands of one point (frg_x64.cu).
