@@ -999,8 +999,9 @@ int frg_advance(frg_ctx *ctx, long max_attempts, frg_flow_stats *stats) {
   // attempts per burst between reads of the controller state: up to 16, but
   // no more than the flows seem to need (the slowest point's remaining
   // interval at its current step, which the step sizes usually outgrow), so
-  // that few attempts run after every point is done
-  const long period = ctx->split ? 16 : 2;
+  // that few attempts run after every point is done (in FP64, too: with a read every
+  // two attempts the flow N = 16 takes 6.53 against 6.17 ms, N = 64 25.9 against 25.6)
+  const long period = 16;
   long a = 0, est = period;
   while (a < max_attempts) {
     const long burst = std::min(std::max(1L, std::min(period, est)), max_attempts - a);
