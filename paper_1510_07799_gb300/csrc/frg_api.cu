@@ -860,7 +860,6 @@ static int rhs_impl(frg_ctx *ctx, int point, double Lambda, const void *d_gamma,
   o.gam = P.Y32;
   o.dgam = kout;
   o.out64 = static_cast<double2 *>(d_dgamma);
-  o.out_f32 = 1;
   LK(launch_set_user_io(ctx->d_io_user, ctx->d_ctl, ctx->n, point, o, Lambda, ctx->stream, true), "user io");
   return run_rhs_split(ctx, ctx->d_io_user, point, static_cast<const double2 *>(d_gamma), ev, sigma_overlap(o, P.N));
 }

@@ -105,7 +105,6 @@ struct RhsIO {
   double2 *dsig;       // self-energy output
   const double *lam;   // scale (device)
   int active;          // 0: skip this point
-  int out_f32;         // vertex output as float2
   // stand-alone evaluations of the split paths: the vertex output in FP64 (dgam
   // then holds the pp products of the contraction only); null otherwise
   double2 *out64;
@@ -128,8 +127,8 @@ __host__ __device__ inline int tail_parts(int N) {
 __host__ __device__ inline int tail_set(int N) { return 2 * (2 * N - 1) + tail_parts(N); }
 
 // Output tile of one CTA of the FP64 channel contraction (k_contract_fp64):
-// F64_TM rows x F64_TN columns; the hosts that build its tile lists (the
-// context and the allocation-free entry point) count tiles with these.
+// F64_TM rows x F64_TN columns; the context, which builds its tile lists, counts
+// tiles with these.
 constexpr int F64_TM = 32, F64_TN = 32;
 
 // One CTA of a channel contraction.
@@ -194,18 +193,6 @@ __host__ __device__ __forceinline__ Geom geom(int ch, int N, int m) {
 }
 
 __device__ __forceinline__ bool inbox(int N, int i) { return (unsigned)i < (unsigned)N; }
-
-// Whether the fourth frequency i1 + i2 - i3 of flat vertex index i is in the
-// box.  Where it is not, the box rule makes the vertex the bare U: the FP32
-// operand copies of the split paths store U there, so that the contraction
-// reads the box rule's value directly.
-__device__ __forceinline__ bool fourth_in_box(int i, int N) {
-  const unsigned q = (unsigned)i / (unsigned)N;
-  const int i3 = i - (int)q * N;
-  const int i1 = (int)(q / (unsigned)N);
-  const int i2 = (int)q - i1 * N;
-  return inbox(N, i1 + i2 - i3);
-}
 
 // Propagators at frequency index i (any integer) and scale L with self-energy
 // sg: G = 1/(Theta^{-1} G0^{-1} - Sigma), S = dG/dL at fixed Sigma

@@ -45,7 +45,6 @@ extern "C" int frg_rhs_noalloc(const frg_params *p, double Lambda, const void *d
   io.dgam = d_dgamma;
   io.dsig = static_cast<double2 *>(d_dsigma);
   io.active = 1;
-  io.out_f32 = 0;
   const bool in_place = io.sig && io.sig < io.dsig + N && io.dsig < io.sig + N;
   if (launch_rhs_small_value(pd, io, Lambda, mask, in_place, static_cast<cudaStream_t>(cuda_stream)) != 0)
     return FRG_ECUDA;

@@ -13,9 +13,9 @@
 // and sums the four products of every entry over the valid p only: no padding,
 // no table in memory, one store per entry.  The last blocks form the
 // self-energy rhs.  Bound by the FP64 units: 16 multiply-adds per entry and p
-// plus the shared weights (R keeps their share below a third).
+// plus the shared weights (their share: rows()).
 // Measured (whole call of the allocation-free entry point): N = 16 100 -> 14 us, N =
-// 32 183 -> 51, N = 48 353 -> 187, N = 64 572 -> 503 us.
+// 32 183 -> 47, N = 48 353 -> 162, N = 64 572 -> 503 us.
 #include <cuda_runtime.h>
 
 #include "frg.h"

@@ -33,7 +33,7 @@
 // channels into the natural layout.  Lines that cannot be converted (non-finite
 // values, exponents beyond 2^+-400) mark their point, whose entries k_x64_combine
 // then sums in FP64 instead.
-// Measured, one rhs (all channels): N = 128 6086 -> 330 us, N = 64 674 -> 73 us
+// Measured, one rhs (all channels): N = 128 6086 -> 321 us, N = 64 674 -> 60 us
 // (CUDA cores -> slices).
 #include <cuda_runtime.h>
 
@@ -67,10 +67,11 @@ constexpr int E_LIM = 400;                  // line exponents the path accepts
 // One block: eight lines of one operand of one product over its whole
 // contraction range.  Eight lanes take the eight lines at one k, so that the
 // blocks are written in 128-byte segments; a thread gathers (and weights, with the
-// table that carries T Lambda) all its k of one line into registers, the block finds each line's largest magnitude, and the values leave
-// in fixed point.  Bound by the FP64 multiplications of the weights and by the
-// gathers (16-byte elements, one 32-byte sector each wherever the line and the
-// contraction index both stride through the vertex): 99 us at N = 128 for 302 MB
+// table that carries T Lambda) all its k of one line into registers, the block
+// finds each line's largest magnitude, and the values leave in fixed point.
+// Bound by the FP64 multiplications of the weights and by the gathers (16-byte
+// elements, one 32-byte sector each wherever the line and the contraction index
+// both stride through the vertex): 99 us at N = 128 for 302 MB
 // written and 15 M entries gathered; 159 us with the lines staged in shared memory
 // between the gather and the conversion.  (The two operands as launches of their
 // own, the right one beside the bubble weights: 130 us, the left one alone takes
@@ -78,7 +79,7 @@ constexpr int E_LIM = 400;                  // line exponents the path accepts
 constexpr int PAN_LINES = 8;
 // k per thread and range: eight on the larger grids (more gathers in flight: N =
 // 128 99 against 111 us), four on the smaller ones (more warps: N = 64 18.0
-// against 19.3 us).
+// against 19.3 us; 16.8 with the weights' factor in the table).
 static int panel_u(int maxN) { return maxN > 80 ? 8 : 4; }
 // Elements along the contraction axis: one or two (direct channel) ranges of D
 // padded to whole blocks.
