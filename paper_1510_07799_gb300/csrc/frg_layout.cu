@@ -105,7 +105,7 @@ __global__ void k_fill_z(const PointDesc *__restrict__ pts) {
 }
 
 template <bool REV, bool ERR, bool OUT64>
-__global__ void __launch_bounds__(comb_threads<REV, ERR>(), ERR ? 4 : REV ? LB_MINBLOCKS_WIDE : LB_MINBLOCKS)
+__global__ void __launch_bounds__(comb_threads<REV, ERR>(), ERR ? 4 : REV ? LB_MINBLOCKS_WIDE : OUT64 ? LB_MINBLOCKS_OUT : LB_MINBLOCKS)
     k_combine(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io, int mask, ErrWeights ew) {
   __shared__ __align__(16) float2 sm[LB * LAP];
   chain_wait();

@@ -27,6 +27,12 @@ constexpr int LCP = LC + 2;
 constexpr int LAP = LB * LCP + 2;
 constexpr int LB_THREADS = 256;
 constexpr int LB_MINBLOCKS = 8;       // resident blocks per SM the kernels are compiled for
+// The last combine of a stand-alone evaluation (FP64 out): five, whose registers keep
+// a thread's eight 16-byte loads in flight (one rhs, eight / six / five / four blocks:
+// N = 100 BF16x3 81.8 / 76.6 / 74.7 / 76.1 us, N = 128 3xTF32 108.2 / 106.6 / 106.1 /
+// 107.1, N = 256 901 / 893 / 894 / 900; with the pp values loaded ahead too, 77.6, 110
+// and 911 at five).
+constexpr int LB_MINBLOCKS_OUT = 5;
 // Kernels that also run on the canonical half only (reversal reduction: half
 // as many blocks with work) use blocks of 512 threads, four per SM, so that the
 // SMs stay as full of warps as with the whole vertex.
