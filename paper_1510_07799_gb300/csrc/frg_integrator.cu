@@ -329,15 +329,20 @@ __device__ __forceinline__ void split_pair(const double2 y0, const double2 y1, f
 // reduction has half as many blocks with work); the seventh stage, with the
 // FP64 state update and the partial error sum, narrow blocks at six per SM for
 // its registers (the canonical half's blocks then fit in one wave).
-template <int S>
-__host__ __device__ constexpr int stage_threads() { return S == 6 ? LB_THREADS : LB_THREADS_WIDE; }
-template <int S>
-__host__ __device__ constexpr int stage_minblocks() { return S == 6 ? 6 : LB_MINBLOCKS_WIDE; }
+// WIDE: the blocks fit the SMs in one go (a single point up to N = 128 under the
+// reversal reduction); else blocks of 256 threads at five per SM, whose registers keep
+// more loads in flight: a batch of 16 points 81.0 -> 79.3 ms (flow N = 128 alone 31.5 ->
+// 31.8).
+template <int S, bool WIDE>
+__host__ __device__ constexpr int stage_threads() { return S == 6 || !WIDE ? LB_THREADS : LB_THREADS_WIDE; }
+template <int S, bool WIDE>
+__host__ __device__ constexpr int stage_minblocks() { return !WIDE ? 5 : S == 6 ? 6 : LB_MINBLOCKS_WIDE; }
+static bool stage_wide(int lb_grid, int n_points) { return (long)lb_grid * n_points <= 152l * LB_MINBLOCKS_WIDE; }
 
 // One layout block of split stage S for a point whose flow is not done; sm:
 // the block in shared memory (LB x LAP float2).  VMAX: fold the block's bound of
 // the FP32 stage input into P.vmax (BF16 slicing).
-template <int S, bool VMAX>
+template <int S, bool WIDE, bool VMAX>
 __device__ __forceinline__ void stage_block(const PointDesc &P, const Ctl &c, int want, float2 *__restrict__ sm) {
   const int N = P.N, n3 = P.n3;
   const bool half = P.rev_half != 0;
@@ -348,7 +353,7 @@ __device__ __forceinline__ void stage_block(const PointDesc &P, const Ctl &c, in
   const float h_hi = d2f(h), h_lo = d2f(h - f2d(h_hi));
   const float U = (float)P.U;
   float vm = 0.f;
-  constexpr int TPB = stage_threads<S>();
+  constexpr int TPB = stage_threads<S, WIDE>();
   constexpr int PAIRS = LB * LB * (LC / 2), PER = PAIRS / TPB;
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
@@ -420,13 +425,13 @@ __device__ __forceinline__ void stage_block(const PointDesc &P, const Ctl &c, in
   if (VMAX) block_max_to(vm, P.vmax + (S & 1));
 }
 
-template <int S>
-__global__ void __launch_bounds__(stage_threads<S>(), stage_minblocks<S>())
+template <int S, bool WIDE>
+__global__ void __launch_bounds__(stage_threads<S, WIDE>(), stage_minblocks<S, WIDE>())
     k_stage_split(const PointDesc *__restrict__ pts, const Ctl *__restrict__ ctl, int want) {
   extern __shared__ float4 lsm4[];
   const Ctl &c = ctl[blockIdx.y];
   if (c.done) return;
-  stage_block<S, true>(pts[blockIdx.y], c, want, reinterpret_cast<float2 *>(lsm4));
+  stage_block<S, WIDE, true>(pts[blockIdx.y], c, want, reinterpret_cast<float2 *>(lsm4));
 }
 
 // A split flow's scatter-add of the rhs of stage S - 1 (it forms k_S) fused
@@ -437,8 +442,8 @@ __global__ void __launch_bounds__(stage_threads<S>(), stage_minblocks<S>())
 // k_S = kG[kslot[S-1]], the per-rhs buffers of parity S - 1); the stage sum
 // keeps the vertex bound of parity S (VMAX: BF16x3 flows, whose contraction
 // reads it).
-template <int S, bool REV, bool VMAX>
-__global__ void __launch_bounds__(stage_threads<S>(), stage_minblocks<S>())
+template <int S, bool WIDE, bool REV, bool VMAX>
+__global__ void __launch_bounds__(stage_threads<S, WIDE>(), stage_minblocks<S, WIDE>())
     k_combine_stage(const PointDesc *__restrict__ pts, const Ctl *__restrict__ ctl, int mask, int want) {
   extern __shared__ float4 lsm4[];
   float2 *sm = reinterpret_cast<float2 *>(lsm4);
@@ -450,9 +455,9 @@ __global__ void __launch_bounds__(stage_threads<S>(), stage_minblocks<S>())
   o.dgam = P.kG[c.kslot[S - 1]];
   o.canon = P.rev_half;
   o.par = (S - 1) & 1;
-  combine_block<REV, false, stage_threads<S>(), VMAX>(P, o, mask, ErrWeights{}, sm);
+  combine_block<REV, false, stage_threads<S, WIDE>(), VMAX>(P, o, mask, ErrWeights{}, sm);
   __syncthreads();  // the scatter-add's reads of the shared block are done
-  stage_block<S, VMAX>(P, c, want, sm);
+  stage_block<S, WIDE, VMAX>(P, c, want, sm);
 }
 
 // Self-energy part of split stage s (one block per point), and the stage's rhs
@@ -649,19 +654,22 @@ static bool stage_attrs(K kernel) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LB_SMEM) == cudaSuccess;
 }
 
-template <int S>
+template <int S, bool WIDE>
 static bool combine_stage_attrs() {
-  return stage_attrs(k_combine_stage<S, true, false>) && stage_attrs(k_combine_stage<S, false, false>) &&
-         stage_attrs(k_combine_stage<S, true, true>) && stage_attrs(k_combine_stage<S, false, true>);
+  return stage_attrs(k_combine_stage<S, WIDE, true, false>) && stage_attrs(k_combine_stage<S, WIDE, false, false>) &&
+         stage_attrs(k_combine_stage<S, WIDE, true, true>) && stage_attrs(k_combine_stage<S, WIDE, false, true>);
 }
 
-int stage_split_init() {
-  const bool ok = stage_attrs(k_stage_split<0>) && stage_attrs(k_stage_split<1>) && stage_attrs(k_stage_split<2>) &&
-                  stage_attrs(k_stage_split<3>) && stage_attrs(k_stage_split<4>) && stage_attrs(k_stage_split<5>) &&
-                  stage_attrs(k_stage_split<6>) && combine_stage_attrs<2>() && combine_stage_attrs<3>() &&
-                  combine_stage_attrs<4>() && combine_stage_attrs<5>() && combine_stage_attrs<6>();
-  return ok ? 0 : -3;
+template <bool WIDE>
+static bool stage_split_attrs() {
+  return stage_attrs(k_stage_split<0, WIDE>) && stage_attrs(k_stage_split<1, WIDE>) &&
+         stage_attrs(k_stage_split<2, WIDE>) && stage_attrs(k_stage_split<3, WIDE>) &&
+         stage_attrs(k_stage_split<4, WIDE>) && stage_attrs(k_stage_split<5, WIDE>) &&
+         stage_attrs(k_stage_split<6, WIDE>) && combine_stage_attrs<2, WIDE>() && combine_stage_attrs<3, WIDE>() &&
+         combine_stage_attrs<4, WIDE>() && combine_stage_attrs<5, WIDE>() && combine_stage_attrs<6, WIDE>();
 }
+
+int stage_split_init() { return stage_split_attrs<true>() && stage_split_attrs<false>() ? 0 : -3; }
 
 int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cudaStream_t st, int n_points,
                       int maxN, bool rev) {
@@ -681,31 +689,44 @@ int launch_stage_fp64(const PointDesc *d_pts, Ctl *d_ctl, int s, RhsIO *d_io, cu
   return e == cudaSuccess ? 0 : -3;
 }
 
+template <int S>
+static cudaError_t stage_at(dim3 g, bool wide, cudaStream_t st, int cv, const PointDesc *d_pts, const Ctl *c,
+                            int want) {
+  return launch_with_carveout(wide ? k_stage_split<S, true> : k_stage_split<S, false>, g,
+                              wide ? stage_threads<S, true>() : stage_threads<S, false>(), LB_SMEM, st, cv, d_pts, c,
+                              want);
+}
+
 int launch_stage(const PointDesc *d_pts, Ctl *d_ctl, int s, cudaStream_t st, int lb_grid, int n_points, int want) {
   const dim3 g(lb_grid, n_points);
   const int cv = step_carveout(n_points);
-  const Ctl *c = d_ctl;
+  const bool wide = stage_wide(lb_grid, n_points);
   cudaError_t e;
   switch (s) {
-    case 0: e = launch_with_carveout(k_stage_split<0>, g, stage_threads<0>(), LB_SMEM, st, cv, d_pts, c, want); break;
-    case 1: e = launch_with_carveout(k_stage_split<1>, g, stage_threads<1>(), LB_SMEM, st, cv, d_pts, c, want); break;
-    case 2: e = launch_with_carveout(k_stage_split<2>, g, stage_threads<2>(), LB_SMEM, st, cv, d_pts, c, want); break;
-    case 3: e = launch_with_carveout(k_stage_split<3>, g, stage_threads<3>(), LB_SMEM, st, cv, d_pts, c, want); break;
-    case 4: e = launch_with_carveout(k_stage_split<4>, g, stage_threads<4>(), LB_SMEM, st, cv, d_pts, c, want); break;
-    case 5: e = launch_with_carveout(k_stage_split<5>, g, stage_threads<5>(), LB_SMEM, st, cv, d_pts, c, want); break;
-    default: e = launch_with_carveout(k_stage_split<6>, g, stage_threads<6>(), LB_SMEM, st, cv, d_pts, c, want); break;
+    case 0: e = stage_at<0>(g, wide, st, cv, d_pts, d_ctl, want); break;
+    case 1: e = stage_at<1>(g, wide, st, cv, d_pts, d_ctl, want); break;
+    case 2: e = stage_at<2>(g, wide, st, cv, d_pts, d_ctl, want); break;
+    case 3: e = stage_at<3>(g, wide, st, cv, d_pts, d_ctl, want); break;
+    case 4: e = stage_at<4>(g, wide, st, cv, d_pts, d_ctl, want); break;
+    case 5: e = stage_at<5>(g, wide, st, cv, d_pts, d_ctl, want); break;
+    default: e = stage_at<6>(g, wide, st, cv, d_pts, d_ctl, want); break;
   }
-  if (e != cudaSuccess) return -3;
   FRG_COUNT(1);
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
+template <int S, bool WIDE>
+static cudaError_t combine_stage_wide(bool rev, bool vmax, dim3 g, cudaStream_t st, int cv, const PointDesc *d_pts,
+                                      const Ctl *c, int m, int want) {
+  auto k = rev ? (vmax ? k_combine_stage<S, WIDE, true, true> : k_combine_stage<S, WIDE, true, false>)
+               : (vmax ? k_combine_stage<S, WIDE, false, true> : k_combine_stage<S, WIDE, false, false>);
+  return launch_with_carveout(k, g, stage_threads<S, WIDE>(), LB_SMEM, st, cv, d_pts, c, m, want);
+}
 template <int S>
 static cudaError_t combine_stage_at(bool rev, bool vmax, dim3 g, cudaStream_t st, int cv, const PointDesc *d_pts,
                                     const Ctl *c, int m, int want) {
-  auto k = rev ? (vmax ? k_combine_stage<S, true, true> : k_combine_stage<S, true, false>)
-               : (vmax ? k_combine_stage<S, false, true> : k_combine_stage<S, false, false>);
-  return launch_with_carveout(k, g, stage_threads<S>(), LB_SMEM, st, cv, d_pts, c, m, want);
+  return stage_wide(g.x, g.y) ? combine_stage_wide<S, true>(rev, vmax, g, st, cv, d_pts, c, m, want)
+                              : combine_stage_wide<S, false>(rev, vmax, g, st, cv, d_pts, c, m, want);
 }
 
 int launch_combine_stage(const PointDesc *d_pts, Ctl *d_ctl, int s, bool rev, bool vmax, int mask, cudaStream_t st,
