@@ -756,7 +756,8 @@ namespace {
 // at N = 256): a large batch reuses the workspace group by group, so that the
 // path never takes more than a small part of the device's memory.
 constexpr size_t X64_WS_CAP = (size_t)4 << 30;
-constexpr int X64_GROUP = 512;  // points per group: grid.z stays below 65536
+constexpr int X64_GROUP = 256;  // points per group: the combine's grid.z, N / IW per point, stays below 65536
+static_assert((FRG_MAX_N + x64::IW - 1) / x64::IW * X64_GROUP < 65536 && 3 * X64_GROUP < 65536, "grid.z");
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 }  // namespace
 
