@@ -191,9 +191,14 @@ static bool small_point(const frg_ctx *ctx, int i) {
 // Whether a rhs chains its launches (launch_ex): always, except while a caller
 // records the stream, which keeps ordinary edges.
 static bool chain_launches(frg_ctx *ctx) {
+  if (ctx->capturing) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return ctx->capturing || (cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess &&
-                            cap == cudaStreamCaptureStatusNone);
+  if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
+    // (the legacy stream beside a capture on another one)
+    cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
 }
 
 // FP64 path.  ev (optional, 6 events): start, after the bubble weights and the
@@ -213,7 +218,7 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
   for (int i = p0; i < p1; ++i) (small_point(ctx, i) ? small : large) = true;
   if (large)
     LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 0, ctx->mask, st,
-                           BUBBLE_TABLES | BUBBLE_SIGMA, chain, half),
+                           BUBBLE_TABLES | BUBBLE_SIGMA, chain ? CHAIN_ALL : 0, half),
        "bubble weights and self-energy");
   if (small)
     LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, sig_in_place, st,
@@ -275,7 +280,9 @@ static int run_rhs_split(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, con
     CK(cudaStreamWaitEvent(ss, ctx->ev_fork, 0), "fork");
     if (tails) CK(cudaStreamWaitEvent(ts, ctx->ev_fork, 0), "fork");
   }
-  LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES, chain), "bubble weights");
+  LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES,
+                         chain ? CHAIN_NEXT : 0),
+     "bubble weights");
   if (fork) CK(cudaEventRecord(ctx->ev_join, ss), "join");
   if (tails)
     LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, ts, TAIL_WINDOW), "tail sums");
@@ -438,7 +445,8 @@ static int run_split_stage(frg_ctx *ctx, int s, bool err, bool fused, bool defer
     CK(cudaStreamWaitEvent(ts, ctx->ev_sst, 0), "self-energy stage");
     LK(launch_tail_sums(ctx->d_pts, io, ctx->n, ctx->maxN, ctx->mask, ts, TAIL_WINDOW), "tail sums");
   }
-  LK(launch_bubble_sigma(ctx->d_pts, io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES, true), "bubble weights");
+  LK(launch_bubble_sigma(ctx->d_pts, io, ctx->n, ctx->maxN, 1, ctx->mask, ss, BUBBLE_TABLES, CHAIN_ALL),
+     "bubble weights");
   CK(cudaEventRecord(ctx->ev_join, ss), "join");
   if (fused)
     LK(launch_combine_stage(ctx->d_pts, ctx->d_ctl, s, ctx->rev_on, ctx->precision == FRG_BF16X3,
@@ -539,8 +547,8 @@ struct FlowStream {
 static int build_step_graph(frg_ctx *ctx) {
   cudaGraph_t gr = nullptr;
   const long l0 = g_kernel_launches;
-  ctx->capturing = true;
   CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal), "begin step capture");
+  ctx->capturing = true;
   const int rc = issue_step(ctx);
   ctx->capturing = false;
   const cudaError_t e = cudaStreamEndCapture(ctx->stream, &gr);

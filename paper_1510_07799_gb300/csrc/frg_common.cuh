@@ -360,10 +360,13 @@ int launch_contract_fp64(const PointDesc *d_pts, const RhsIO *d_io, const WorkIt
 // self-energy rhs (BUBBLE_SIGMA: it also reads the vertex input), so that a
 // flow can compute the tables before the vertex stage input exists.  half (FP64):
 // the self-energy rhs for the lower half of the frequencies, the others their
-// mirrors' conjugates (a reversal-symmetric input).
+// mirrors' conjugates (a reversal-symmetric input).  chain (launch_ex): CHAIN_FIRST the
+// first of the launches, which must directly follow another kernel of this library on
+// st, CHAIN_NEXT the one after it.
+constexpr int CHAIN_FIRST = 1, CHAIN_NEXT = 2, CHAIN_ALL = 3;
 constexpr int BUBBLE_TABLES = 1, BUBBLE_SIGMA = 2;
 int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split, int mask,
-                        cudaStream_t st, int parts = BUBBLE_TABLES | BUBBLE_SIGMA, bool chain = false, bool half = false);
+                        cudaStream_t st, int parts = BUBBLE_TABLES | BUBBLE_SIGMA, int chain = 0, bool half = false);
 // Frequency-box tails: the window propagators and the sums over the window
 // (TAIL_WINDOW), then the constants, the self-energy's added to the
 // self-energy rhs (TAIL_FINISH: after launch_bubble_sigma's self-energy

@@ -133,14 +133,14 @@ __global__ void __launch_bounds__(128)
 }
 
 int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int split, int mask,
-                        cudaStream_t st, int parts, bool chain, bool half) {
+                        cudaStream_t st, int parts, int chain, bool half) {
   const int nrow_max = 2 * maxN - 1;
   // split flows run these beside the stage kernel
   const int cv = split ? side_carveout(n_points, mask) : -1;
   cudaError_t e = cudaSuccess;
   if (parts & BUBBLE_TABLES) {
     const dim3 g((maxN + GS_PER_BLOCK - 1) / GS_PER_BLOCK, n_points);
-    e = launch_ex(k_bubble_gs, g, GS_PER_BLOCK, 0, st, cv, chain, d_pts, d_io);
+    e = launch_ex(k_bubble_gs, g, GS_PER_BLOCK, 0, st, cv, (chain & CHAIN_FIRST) != 0, d_pts, d_io);
     FRG_COUNT(1);
   }
   // blocks [0, 2 nrow_max): table rows; [2 nrow_max, 2 nrow_max + maxN): self-energy entries
@@ -149,7 +149,8 @@ int launch_bubble_sigma(const PointDesc *d_pts, const RhsIO *d_io, int n_points,
   if (b1 > b0) {
     const dim3 g(b1 - b0, n_points);
     const int sig = (mask & 8) != 0;
-    const cudaError_t e2 = launch_ex(split ? k_bubble_sigma<true> : k_bubble_sigma<false>, g, 128, 0, st, cv, chain, d_pts,
+    const cudaError_t e2 = launch_ex(split ? k_bubble_sigma<true> : k_bubble_sigma<false>, g, 128, 0, st, cv,
+                                     (chain & (parts & BUBBLE_TABLES ? CHAIN_NEXT : CHAIN_FIRST)) != 0, d_pts,
                                      d_io, maxN, sig, b0, half ? 1 : 0);
     if (e == cudaSuccess) e = e2;
     FRG_COUNT(1);

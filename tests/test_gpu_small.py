@@ -26,7 +26,7 @@ def run(call, V, sig):
 
 
 @pytest.mark.parametrize("mask", [0xF, 0x9, 0x2, 0x4, 0x8])
-@pytest.mark.parametrize("N", [2, 4, 8, 14, 22, 24, 26, 40, 42, 64])
+@pytest.mark.parametrize("N", [2, 4, 8, 12, 14, 16, 18, 20, 22, 24, 26, 28, 30, 32, 34, 36, 38, 40, 42, 48, 50, 64])
 def test_one_launch_rhs_matches_oracle(N, mask):
     p = frg.Params(U=1.3, T=0.64 / N, eps_d=-0.4, N_f=N)
     V = inputs.random_vertex(N, p.U, seed=N + 7 * mask, crossing=False)
