@@ -209,12 +209,16 @@ __global__ void __launch_bounds__(T) k_rhs_small_value(const __grid_constant__ P
   rhs<false>(P, o, lam, mask, part, blockIdx.x, sm);
 }
 
-// (a host-side setting of the current device's context: set on every call, as
-// the context may have changed)
+// (A host-side setting of the current device's context: set on every call, as the
+// context may have changed, and always to the most any size needs, as another thread
+// may be between its setting and its launch.)
 template <typename K>
 bool room(K kernel, size_t bytes) {
-  return bytes <= 48 * 1024 ||
-         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  if (bytes <= 48 * 1024) return true;
+  size_t most = 0;
+  for (int n = 2; n <= SMALL_MAX_N; n += 2) most = smem(n, false) > most ? smem(n, false) : most;
+  return bytes <= most &&
+         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess;
 }
 }  // namespace small
 

@@ -69,3 +69,36 @@ def test_self_energy_rhs_in_place(N):
             call(V, buf, dg2, buf)
             torch.cuda.synchronize()
             assert torch.equal(dg, dg2) and torch.equal(ds, buf)
+
+
+def test_threads_with_different_sizes():
+    """Calls of different sizes from several threads, each on a stream of its own."""
+    import threading
+
+    cases, errors = [], []
+    for N in (36, 48, 56, 64):
+        p = frg.Params(U=1.3, T=0.64 / N, eps_d=-0.4, N_f=N)
+        V = torch.from_numpy(inputs.random_vertex(N, p.U, seed=N)).cuda()
+        sig = torch.from_numpy(inputs.random_sigma(N, seed=N)).cuda()
+        ref = torch.empty_like(V), torch.empty_like(sig)
+        frg.rhs_noalloc(p, 0.25, V, sig, *ref)
+        cases.append((p, V, sig, ref, (torch.empty_like(V), torch.empty_like(sig)), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def work(p, V, sig, ref, out, stream):
+        try:
+            with torch.cuda.stream(stream):
+                for _ in range(200):
+                    frg.rhs_noalloc(p, 0.25, V, sig, *out)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=c) for c in cases]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    for c in cases:
+        assert torch.equal(c[3][0], c[4][0]) and torch.equal(c[3][1], c[4][1])
