@@ -62,7 +62,8 @@ extern "C" {
  * error of one rhs below 1e-6 for FRG_3XTF32 and 5e-5 for FRG_BF16X3 on the
  * test inputs; whole flows within 1e-6 of the FP64 oracle).
  */
-#define FRG_FP64 0    /* FP64 throughout; grids of 28 frequencies on form the channel products from exact tcgen05 slices */
+#define FRG_FP64 0    /* FP64 throughout; grids of 28 frequencies on form the channel products from tcgen05 digit
+                         slices, whose integer sums are exact, to FP64's accuracy for each entry */
 #define FRG_3XTF32 1  /* split-TF32 (hi*hi + hi*lo + lo*hi) on tcgen05, FP32 accumulate */
 #define FRG_BF16X3 2  /* three BF16 slices, six products, on tcgen05, FP32 accumulate */
 

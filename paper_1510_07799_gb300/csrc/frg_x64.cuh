@@ -17,9 +17,8 @@ struct X64Pt {
   const uint4 *prod;   // per ch * (2N - 1) + m: first left and right operand block, first left and right tile of
                        // exponents; null: not on this path
   ulonglong2 *L, *R;   // fixed-point operand blocks (re, im), 16 k x 64 lines each
-  int *eL, *eR;        // line exponents, 64 per tile
+  int *eL, *eR;        // line records (exponent and flags), 64 per tile
   double2 *PX, *PW;    // direct (layout X) and crossed (layout W) channel outputs
-  int *bad;            // [0] set when a line cannot be sliced (non-finite or extreme values); [1] blocks that have seen it
 };
 
 struct X64Plan;
