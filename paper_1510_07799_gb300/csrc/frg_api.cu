@@ -216,6 +216,10 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
   const int p0 = point < 0 ? 0 : point, p1 = point < 0 ? ctx->n : point + 1;
   bool small = false, large = false;
   for (int i = p0; i < p1; ++i) (small_point(ctx, i) ? small : large) = true;
+  // (the window propagators read the self-energy input, which the self-energy rhs may
+  // overwrite)
+  if (tails)
+    LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st, TAIL_WINDOW), "tail sums");
   if (large)
     LK(launch_bubble_sigma(ctx->d_pts, d_io, ctx->n, ctx->maxN, 0, ctx->mask, st,
                            BUBBLE_TABLES | BUBBLE_SIGMA, chain ? CHAIN_ALL : 0, half),
@@ -224,7 +228,8 @@ static int run_rhs_fp64(frg_ctx *ctx, RhsIO *d_io, int point /* -1: all */, cuda
     LK(launch_rhs_small(ctx->d_pts + p0, d_io + p0, p1 - p0, ctx->maxN, X64_MIN_N, ctx->mask, sig_in_place, st,
                         chain, half),
        "small rhs");
-  if (tails) LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st), "tail sums");
+  if (tails)
+    LK(launch_tail_sums(ctx->d_pts, d_io, ctx->n, ctx->maxN, ctx->mask, st, TAIL_FINISH), "tail constants");
   if (ev) CK(cudaEventRecord(ev[1], st), "event");
   if (ev) CK(cudaEventRecord(ev[2], st), "event");
   if (!chmask) {
