@@ -862,8 +862,10 @@ static int rhs_impl(frg_ctx *ctx, int point, double Lambda, const void *d_gamma,
   o.dsig = static_cast<double2 *>(d_dsigma);
   o.active = 1;
   if (!ctx->split) {
+    bool in_place = false;
+    if (small_point(ctx, point)) LK(small_sigma(o, P.N, ctx->stream, &in_place), "self-energy input");
     LK(launch_set_user_io(ctx->d_io_user, ctx->d_ctl, ctx->n, point, o, Lambda, ctx->stream), "user io");
-    return run_rhs_fp64(ctx, ctx->d_io_user, point, ev, sigma_overlap(o, P.N));
+    return run_rhs_fp64(ctx, ctx->d_io_user, point, ev, in_place);
   }
   // split path: the vertex goes into the FP32 operand copies (scratch between
   // the stages of a flow; the contraction's tensor maps point at them), the

@@ -45,8 +45,9 @@ extern "C" int frg_rhs_noalloc(const frg_params *p, double Lambda, const void *d
   io.dgam = d_dgamma;
   io.dsig = static_cast<double2 *>(d_dsigma);
   io.active = 1;
-  const bool in_place = io.sig && io.sig < io.dsig + N && io.dsig < io.sig + N;
-  if (launch_rhs_small_value(pd, io, Lambda, mask, in_place, static_cast<cudaStream_t>(cuda_stream)) != 0)
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  bool in_place;
+  if (small_sigma(io, N, st, &in_place) != 0 || launch_rhs_small_value(pd, io, Lambda, mask, in_place, st) != 0)
     return FRG_ECUDA;
   return FRG_OK;
 }

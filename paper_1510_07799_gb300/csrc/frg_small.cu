@@ -222,6 +222,29 @@ bool room(K kernel, size_t bytes) {
 }
 }  // namespace small
 
+// (in order with an input that overlaps the copy)
+__global__ void k_move_sigma(double2 *dst, const double2 *src, int N) {
+  const int t = threadIdx.x;
+  double2 v;
+  if (t < N) v = src[t];
+  __syncthreads();
+  if (t < N) dst[t] = v;
+}
+
+int small_sigma(RhsIO &o, int N, cudaStream_t st, bool *in_place) {
+  const auto overlap = [&](const void *p, size_t n) {
+    const char *a = reinterpret_cast<const char *>(o.sig), *b = static_cast<const char *>(p);
+    return a && a < b + n * sizeof(double2) && b < a + N * sizeof(double2);
+  };
+  *in_place = overlap(o.dsig, N);
+  if (!overlap(o.dgam, (size_t)N * N * N)) return 0;
+  k_move_sigma<<<1, SMALL_MAX_N, 0, st>>>(o.dsig, o.sig, N);
+  FRG_COUNT(1);
+  o.sig = o.dsig;
+  *in_place = true;
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
 int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, int maxN, int n_below, int mask,
                      bool sig_in_place, cudaStream_t st, bool chain, bool half) {
   // shared memory and blocks for every size below the bound (both drop where the

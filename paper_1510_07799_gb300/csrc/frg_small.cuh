@@ -14,4 +14,7 @@ int launch_rhs_small(const PointDesc *d_pts, const RhsIO *d_io, int n_points, in
 // The same for one point (N <= SMALL_MAX_N) given by value: no device memory.
 int launch_rhs_small_value(const PointDesc &P, const RhsIO &o, double lam, int mask, bool sig_in_place,
                            cudaStream_t st);
+// Before a stand-alone one-launch rhs: whether its self-energy output overlaps the input;
+// an input that the vertex output overlaps is moved into the self-energy output first.
+int small_sigma(RhsIO &o, int N, cudaStream_t st, bool *in_place);
 }  // namespace frg
