@@ -551,14 +551,15 @@ struct FlowStream {
 // Capture issue_step into the step graph (once per context).
 static int build_step_graph(frg_ctx *ctx) {
   cudaGraph_t gr = nullptr;
-  const long l0 = g_kernel_launches;
   CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal), "begin step capture");
   ctx->capturing = true;
+  long launches = 0;  // (counted when the graph runs)
+  record_launches(&launches);
   const int rc = issue_step(ctx);
+  record_launches(nullptr);
   ctx->capturing = false;
   const cudaError_t e = cudaStreamEndCapture(ctx->stream, &gr);
-  ctx->step_launches = g_kernel_launches - l0;
-  g_kernel_launches = l0;  // counted when the graph runs
+  ctx->step_launches = launches;
   if (rc || e != cudaSuccess) {
     if (gr) cudaGraphDestroy(gr);
     cudaGetLastError();
@@ -906,7 +907,7 @@ int frg_rhs_timed(frg_ctx *ctx, int point, double Lambda, const void *d_gamma, c
   return rc;
 }
 
-long frg_kernel_launches(void) { return frg::g_kernel_launches; }
+long frg_kernel_launches(void) { return frg::launches_counted(); }
 
 int frg_rhs_host_async(frg_ctx *ctx, int point, double Lambda, const double *h_gamma, const double *h_sigma,
                        double *h_dgamma, double *h_dsigma) {

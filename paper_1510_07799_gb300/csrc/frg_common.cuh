@@ -14,9 +14,13 @@
 
 namespace frg {
 
-// Process-wide count of kernel launches issued by this library (diagnostics).
-extern long g_kernel_launches;
-#define FRG_COUNT(n) (::frg::g_kernel_launches += (n))
+// Process-wide count of kernel launches issued by this library (diagnostics; any
+// thread).  While `to` is set (record_launches), the calling thread's launches go there
+// instead: those of a graph being recorded count when it runs.
+void count_launches(long n);
+long launches_counted();
+void record_launches(long *to);
+#define FRG_COUNT(n) (::frg::count_launches(n))
 
 enum Channel { CH_PP = 0, CH_DPH = 1, CH_XPH = 2 };
 

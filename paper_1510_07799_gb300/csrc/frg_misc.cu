@@ -1,11 +1,23 @@
 // frg_misc.cu -- small stream-ordered helper kernels of the C ABI.
+#include <atomic>
+
 #include "frg_common.cuh"
 #include "frg_misc.cuh"
 #include "frg_split.cuh"
 
 namespace frg {
 
-long g_kernel_launches = 0;
+static std::atomic<long> g_launches{0};
+static thread_local long *t_recorded = nullptr;
+
+void count_launches(long n) {
+  if (t_recorded)
+    *t_recorded += n;
+  else
+    g_launches.fetch_add(n, std::memory_order_relaxed);
+}
+long launches_counted() { return g_launches.load(std::memory_order_relaxed); }
+void record_launches(long *to) { t_recorded = to; }
 
 // io[point] = o with its scale stored on the device; every other point
 // inactive.  relaid (split paths): the evaluation rewrites every entry of the
