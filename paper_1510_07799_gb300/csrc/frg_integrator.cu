@@ -511,11 +511,25 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned long long *addr, doub
 // partial sum e' of the seventh stage.  The FP64 division of the scaled error is
 // what costs on this part, and only the largest ratio matters: a ratio in FP32
 // finds the entries within 2^-16 of the block's largest, and those alone are
-// divided in FP64 (the maximum is the same, bit for bit).  Measured at N = 64:
-// 15 us, against 36 us for summing all stages and dividing every entry.
+// divided in FP64 (the maximum is the same, bit for bit).  Entries whose FP32 ratio
+// could overflow or lose digits are divided as well, and are no part of that largest one.
+// Measured at N = 64: 15 us, against 36 us for summing all stages and dividing every
+// entry.
 __device__ __forceinline__ double maxabs(double a, double b) {
   const long long x = __double_as_longlong(a) & 0x7fffffffffffffffll, y = __double_as_longlong(b) & 0x7fffffffffffffffll;
   return __longlong_as_double(x > y ? x : y);
+}
+// The ratio |h acc| / (atol + rtol ym) in FP32, at least: exact to 2^-20 where `sure`
+// is the same, else sure = 0.
+__device__ __forceinline__ float ratio32(double acc, double ym, float hf, float at, float rt, float &sure) {
+  constexpr float LO = 0x1p-60f, HI = 0x1p60f;
+  const float f = fabsf(d2f(acc)), den = at + rt * d2f(ym);
+  sure = 0.f;
+  // (false for a NaN)
+  if (!(f <= HI && den >= LO && den <= HI && hf >= LO && hf <= HI)) return CUDART_INF_F;
+  const float r = hf * fmaxf(f, acc == 0.0 ? 0.f : LO) / den;
+  if (f >= LO) sure = r;
+  return r;
 }
 constexpr int ERR_T = 512;
 __global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ pts, Ctl *__restrict__ ctl, int half) {
@@ -533,7 +547,7 @@ __global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ p
   const double h = c.h;
   double2 acc = make_double2(0.0, 0.0), yi = acc, yni = acc;
   int bad = 0;
-  float rx = 0.f, ry = 0.f;
+  float r = 0.f, sure = 0.f;
   const bool on = i < n;
   if (on) {
     const int k2 = c.kslot[1], k7 = c.kslot[6];
@@ -546,23 +560,21 @@ __global__ void __launch_bounds__(ERR_T) k_error(const PointDesc *__restrict__ p
     acc.y += dE[6] * k.y;
     bad = !isfinite(yni.x) || !isfinite(yni.y);
     const float hf = fabsf(d2f(h)), at = d2f(P.atol), rt = d2f(P.rtol);
-    const float fx = fabsf(d2f(acc.x)), fy = fabsf(d2f(acc.y));
-    rx = hf * fx / (at + rt * d2f(maxabs(yi.x, yni.x)));
-    ry = hf * fy / (at + rt * d2f(maxabs(yi.y, yni.y)));
-    // a sum that FP32 flushes to zero has no FP32 ratio
-    if ((fx == 0.f && acc.x != 0.0) || (fy == 0.f && acc.y != 0.0)) rx = CUDART_INF_F;
+    float sx, sy;
+    const float rx = ratio32(acc.x, maxabs(yi.x, yni.x), hf, at, rt, sx);
+    const float ry = ratio32(acc.y, maxabs(yi.y, yni.y), hf, at, rt, sy);
+    r = fmaxf(rx, ry);
+    sure = fmaxf(sx, sy);
   }
-  // (bits of non-negative floats order as integers, a NaN above infinity)
-  const unsigned bx = __float_as_uint(rx) & 0x7fffffffu, by = __float_as_uint(ry) & 0x7fffffffu;
-  unsigned m = __reduce_max_sync(0xffffffffu, max(bx, by));
+  // (bits of non-negative floats order as integers)
+  unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(sure));
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
   __syncthreads();
   m = 0u;
   for (int w = 0; w < ERR_T / 32; ++w) m = max(m, wmax[w]);
-  // 2^-16 below the maximum (a NaN or an infinity in FP32, or ratios near its
-  // smallest: every entry)
-  const unsigned cut = m >= 0x7f800000u || m < 0x01000000u ? 0u : m - 0x80u;
-  if (on && max(bx, by) >= cut) {
+  // 2^-16 below the maximum (ratios near FP32's smallest: every entry)
+  const unsigned cut = m < 0x01000000u ? 0u : m - 0x80u;
+  if (on && __float_as_uint(r) >= cut) {
     const double ex = fabs(h * acc.x) / (P.atol + P.rtol * maxabs(yi.x, yni.x));
     const double ey = fabs(h * acc.y) / (P.atol + P.rtol * maxabs(yi.y, yni.y));
     if (!isfinite(ex) || !isfinite(ey)) bad = 1;
