@@ -63,7 +63,9 @@ extern "C" {
  * test inputs; whole flows within 1e-6 of the FP64 oracle).
  */
 #define FRG_FP64 0    /* FP64 throughout; grids of 28 frequencies on form the channel products from tcgen05 digit
-                         slices, whose integer sums are exact, to FP64's accuracy for each entry */
+                         slices, whose integer sums are exact, to FP64's accuracy for each entry; the slices take
+                         up to 4 GB of device memory per context (2.9 GB for one point of 256 frequencies), and
+                         where there is no room for them the products run on the CUDA cores */
 #define FRG_3XTF32 1  /* split-TF32 (hi*hi + hi*lo + lo*hi) on tcgen05, FP32 accumulate */
 #define FRG_BF16X3 2  /* three BF16 slices, six products, on tcgen05, FP32 accumulate */
 
@@ -349,6 +351,14 @@ int frg_cross_tile(int ch, int N, int nt, int m, int rt, int out[7]);
  * FRG_EINVAL / FRG_ECUDA.  Synchronises.
  */
 int frg_selftest_wait(frg_ctx *ctx, double limit_ms);
+/*
+ * Self-test of FRG_FP64 contexts whose slices (FRG_FP64 above) find no room on the
+ * device: after frg_selftest_slices(0) the contexts that the calling thread creates
+ * form their channel products on the CUDA cores, as they do when the allocation
+ * fails; frg_selftest_slices(1) ends that.  Existing contexts and other threads are
+ * not affected.  No device work.  Returns FRG_OK.
+ */
+int frg_selftest_slices(int on);
 
 /*
  * Contraction autotuning (split precisions).  The paper distributes work over

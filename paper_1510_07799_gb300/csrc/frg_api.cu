@@ -907,6 +907,11 @@ int frg_rhs_timed(frg_ctx *ctx, int point, double Lambda, const void *d_gamma, c
   return rc;
 }
 
+int frg_selftest_slices(int on) {
+  x64_withhold(!on);
+  return FRG_OK;
+}
+
 long frg_kernel_launches(void) { return frg::launches_counted(); }
 
 int frg_rhs_host_async(frg_ctx *ctx, int point, double Lambda, const double *h_gamma, const double *h_sigma,

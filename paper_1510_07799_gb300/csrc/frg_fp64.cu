@@ -356,18 +356,16 @@ __device__ __forceinline__ size_t out_index(int N, const Geom &g, int r, int c) 
   }
 }
 
-struct F64Smem {
-  double2 Ls[F64_TM][F64_TK + 1];
-  double2 Rs[F64_TK][F64_TN + 1];
-};
-
-// One tile of one channel: store(geometry, local row, column, value) for every
-// entry.
-template <int CH, typename Store>
-__device__ __forceinline__ void f64_tile(const PointDesc &P, const RhsIO &o, const WorkItem &w, F64Smem &sm,
-                                         Store store) {
-  auto &Ls = sm.Ls;
-  auto &Rs = sm.Rs;
+template <int CH, bool ACCUM>
+__global__ void __launch_bounds__(F64_THREADS)
+    k_contract_fp64(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
+                    const WorkItem *__restrict__ work) {
+  __shared__ double2 Ls[F64_TM][F64_TK + 1];
+  __shared__ double2 Rs[F64_TK][F64_TN + 1];
+  const WorkItem w = work[blockIdx.x];
+  const RhsIO &o = io[w.point];
+  if (!o.active) return;
+  const PointDesc &P = pts[w.point];
   const int N = P.N;
   const Geom g = geom(CH, N, w.m);
   const int r0 = w.rt * F64_TM, c0 = w.ct * F64_TN;
@@ -407,29 +405,19 @@ __device__ __forceinline__ void f64_tile(const PointDesc &P, const RhsIO &o, con
     __syncthreads();
   }
   const double sc = (CH == CH_DPH ? 1.0 : -1.0) * P.T * (*o.lam);
+  double2 *out = static_cast<double2 *>(o.dgam);
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int r = r0 + ty * 2 + i, c = c0 + tx * 2 + j;
-      if (r < g.D && c < N) store(g, r, c, make_double2(acc[i][j].x * sc, acc[i][j].y * sc));
+      if (r < g.D && c < N) {
+        const size_t at = out_index<CH>(N, g, r, c);
+        double2 v = make_double2(acc[i][j].x * sc, acc[i][j].y * sc);
+        if (ACCUM) v = cadd(out[at], v);
+        out[at] = v;
+      }
     }
-}
-
-template <int CH, bool ACCUM>
-__global__ void __launch_bounds__(F64_THREADS)
-    k_contract_fp64(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                    const WorkItem *__restrict__ work) {
-  __shared__ F64Smem sm;
-  const WorkItem w = work[blockIdx.x];
-  const RhsIO &o = io[w.point];
-  if (!o.active) return;
-  const PointDesc &P = pts[w.point];
-  double2 *out = static_cast<double2 *>(o.dgam);
-  f64_tile<CH>(P, o, w, sm, [&](const Geom &g, int r, int c, double2 v) {
-    const size_t at = out_index<CH>(P.N, g, r, c);
-    out[at] = ACCUM ? cadd(out[at], v) : v;
-  });
 }
 
 // pp stores, dph and xph accumulate: the three channels run in this order so

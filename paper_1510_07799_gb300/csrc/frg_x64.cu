@@ -973,14 +973,17 @@ constexpr size_t X64_WS_CAP = (size_t)4 << 30;
 constexpr int X64_GROUP = 256;  // points per group: the combine's grid.z, N / IW per point, stays below 65536
 static_assert((FRG_MAX_N + x64::IW - 1) / x64::IW * X64_GROUP < 65536 && 3 * X64_GROUP < 65536, "grid.z");
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+thread_local bool t_withheld = false;  // frg_selftest_slices
 }  // namespace
+
+void x64_withhold(bool on) { t_withheld = on; }
 
 int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, unsigned *d_err) {
   *out = nullptr;
   const int n = (int)pts.size();
   bool any = false;
   for (const PointDesc &P : pts) any = any || P.N >= X64_MIN_N;
-  if (!any || !(chmask & 7)) return 0;
+  if (!any || !(chmask & 7) || t_withheld) return 0;
   int dev = 0, sms = 0, maj = 0, min_ = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -1047,12 +1050,8 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
     ws = std::max(ws, sum);
     i = j;
   }
-  if (cudaMalloc(&p->ws, ws) != cudaSuccess) {
-    cudaGetLastError();
-    x64_destroy(p);
-    return 0;
-  }
-  bool ok = cudaMalloc(&p->d_x, sizeof(X64Pt) * n) == cudaSuccess &&
+  bool ok = cudaMalloc(&p->ws, ws) == cudaSuccess &&
+            cudaMalloc(&p->d_x, sizeof(X64Pt) * n) == cudaSuccess &&
             cudaFuncSetAttribute(x64::k_x64_products, cudaFuncAttributeMaxDynamicSharedMemorySize, x64::SMEM) ==
                 cudaSuccess;
   for (int i = 0; i < n && ok; ++i) {
@@ -1090,8 +1089,9 @@ int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, uns
   }
   ok = ok && cudaMemcpy(p->d_x, p->h.data(), sizeof(X64Pt) * n, cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) {
+    const bool room = cudaGetLastError() != cudaErrorMemoryAllocation;
     x64_destroy(p);
-    return -3;
+    return room ? -3 : 0;
   }
   *out = p;
   return 0;

@@ -27,6 +27,8 @@ struct X64Plan;
 // points on the CUDA-core path).  Returns 0, or -3 when a CUDA call failed.
 int x64_create(X64Plan **out, const std::vector<PointDesc> &pts, int chmask, unsigned *d_err);
 void x64_destroy(X64Plan *p);
+// on: plans that the calling thread makes find no room (frg_selftest_slices).
+void x64_withhold(bool on);
 bool x64_has(const X64Plan *p, int point);
 // Channel products of every point of the plan (point < 0) or of one point; chain:
 // see launch_ex; half (every point): the inputs are reversal-symmetric, so the

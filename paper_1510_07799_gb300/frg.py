@@ -30,7 +30,7 @@ ERRNAMES = {EINVAL: "FRG_EINVAL", ENOMEM: "FRG_ENOMEM", ECUDA: "FRG_ECUDA",
 EXPORTED = ("frg_init", "frg_destroy", "frg_last_error", "frg_rhs", "frg_rhs_host", "frg_flow",
             "frg_advance", "frg_observables", "frg_get_state", "frg_set_state", "frg_stats",
             "frg_rhs_timed", "frg_kernel_launches", "frg_rhs_noalloc", "frg_autotune", "frg_selftest_wait", "frg_rhs_host_async", "frg_sync",
-            "frg_cross_tile")
+            "frg_cross_tile", "frg_selftest_slices")
 NOALLOC_MAX_N = 64
 
 
@@ -127,6 +127,7 @@ def load():
     lib.frg_rhs_noalloc.argtypes = [C.POINTER(_Params), C.c_double, vp, vp, vp, vp, vp]
     lib.frg_autotune.argtypes = [vp, C.POINTER(_Tune)]
     lib.frg_selftest_wait.argtypes = [vp, C.c_double]
+    lib.frg_selftest_slices.argtypes = [C.c_int]
     lib.frg_rhs_host_async.argtypes = [vp, C.c_int, C.c_double, dp, dp, dp, dp]
     lib.frg_sync.argtypes = [vp]
     lib.frg_cross_tile.argtypes = [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int)]
