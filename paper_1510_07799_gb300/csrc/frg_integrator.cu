@@ -522,13 +522,13 @@ __device__ __forceinline__ double maxabs(double a, double b) {
 // The ratio |h acc| / (atol + rtol ym) in FP32, at least: exact to 2^-20 where `sure`
 // is the same, else sure = 0.
 __device__ __forceinline__ float ratio32(double acc, double ym, float hf, float at, float rt, float &sure) {
-  constexpr float LO = 0x1p-60f, HI = 0x1p60f;
+  constexpr float LO = 0x1p-60f, HI = 0x1p60f, H_LO = 0x1p-20f, F_LO = 0x1p-100f;
   const float f = fabsf(d2f(acc)), den = at + rt * d2f(ym);
   sure = 0.f;
   // (false for a NaN)
-  if (!(f <= HI && den >= LO && den <= HI && hf >= LO && hf <= HI)) return CUDART_INF_F;
-  const float r = hf * fmaxf(f, acc == 0.0 ? 0.f : LO) / den;
-  if (f >= LO) sure = r;
+  if (!(f <= HI && den >= LO && den <= HI && hf >= H_LO && hf <= HI)) return CUDART_INF_F;
+  const float r = hf * fmaxf(f, acc == 0.0 ? 0.f : F_LO) / den;
+  if (f >= F_LO) sure = r;
   return r;
 }
 constexpr int ERR_T = 512;
