@@ -229,7 +229,7 @@ __device__ __forceinline__ void propagator_at(const PointDesc &P, int i, double 
 // chain: the kernel follows another one of this library on the same stream, and its
 // blocks may become resident while the predecessor's last ones still run, which takes
 // the launch itself off the serial chain of a rhs (five kernels of 5-30 us at N = 64:
-// 72.7 -> 59.8 us).  Such a kernel calls chain_wait() before it touches anything that
+// 72.7 -> 59.8 us with the products at 30 us).  Such a kernel calls chain_wait() before it touches anything that
 // another kernel reads or writes: it returns once the predecessor has completed and
 // its writes are visible.  The trigger comes after the wait, so at most two neighbours
 // of a chain are on the GPU at a time (a kernel that holds TMEM never meets another

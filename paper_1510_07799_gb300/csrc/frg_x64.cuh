@@ -8,7 +8,7 @@ namespace frg {
 
 // Smallest grid whose FP64 channel products take the sliced tensor-core path; the
 // ones below take the one-launch rhs (frg_small.cu).  Measured per rhs: N = 24 32
-// (sliced) against 25 us, N = 26 39 against 35 us, N = 28 37 against 40 us, N = 32 40
+// (sliced) against 25 us, N = 26 39 against 35 us, N = 28 37 against 40 us, N = 32 42
 // against 47 us.
 constexpr int X64_MIN_N = 28;
 
