@@ -621,12 +621,14 @@ __device__ __noinline__ void settle_tile(const PointDesc &P, const RhsIO &o, con
   }
 }
 
-// The unsettled entries of a tile again in FP64 (all epilogue warps; cnt: two counters in
-// shared memory, the next call's one zeroed here): each group of four columns of a row by
-// one warp, or the whole tile at once where that is less work (a group takes the FP64
-// units some 25 K cycles, a tile 2 K for each of its entries: from a third of the groups on).
+// The unsettled entries of a tile again in FP64 (all epilogue warps): each group of four
+// columns of a row by one warp, or the whole tile at once where that is less work (a
+// group takes the FP64 units some 25 K cycles, a tile 2 K for each of its entries: from a
+// third of the groups on).  Call n counts its groups in cnt[n % 3]; before its barrier it
+// zeroes the counter of call n + 1, which every warp has read (as that of call n - 2)
+// before the barrier of call n - 1.
 __device__ __noinline__ void settle(const PointDesc *__restrict__ pts, const RhsIO *__restrict__ io,
-                                    const X64Pt *__restrict__ xp, const Work &w, SettleSmem &sm, int *cnt, int par,
+                                    const X64Pt *__restrict__ xp, const Work &w, SettleSmem &sm, int *cnt, int n,
                                     int t) {
   const PointDesc &P = pts[w.point];
   const RhsIO &o = io[w.point];
@@ -648,10 +650,10 @@ __device__ __noinline__ void settle(const PointDesc *__restrict__ pts, const Rhs
     const unsigned v = __ballot_sync(0xffffffffu, on);
     groups += __popc((v | v >> 1 | v >> 2 | v >> 3) & 0x11111111u);
   }
-  if (lane == 0 && groups) atomicAdd(&cnt[par], groups);
+  if (lane == 0 && groups) atomicAdd(&cnt[n % 3], groups);
+  if (t == 0) cnt[(n + 1) % 3] = 0;
   epi_sync();
-  const int total = cnt[par];
-  if (t == 0) cnt[par ^ 1] = 0;
+  const int total = *const_cast<volatile int *>(cnt + n % 3);
   if (12 * total > min(LINES, g.D - r0) * min(LINES, N - c0)) {
     if (w.ch == CH_PP)
       settle_tile<CH_PP>(P, o, x, w, sm, t);
@@ -683,7 +685,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t *op_full = raw_empty + 2 * NRAW, *op_empty = op_full + NOP, *tfull = op_empty + NOP, *tempty = tfull + 1;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tempty + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  int *again = reinterpret_cast<int *>(tmem_slot + 2);  // a second pass is wanted; a wait gave up; two counters
+  int *again = reinterpret_cast<int *>(tmem_slot + 2);  // a second pass is wanted; a wait gave up; three counters
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int j = 0; j < 2 * NRAW; ++j) {
@@ -697,7 +699,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     mbar_init(tfull, 1);
     mbar_init(tempty, EPI_W);
     *abort_flag = 0;
-    again[0] = again[1] = again[2] = again[3] = 0;
+    for (int j = 0; j < 5; ++j) again[j] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == MMA_W) tmem_alloc(tmem_slot, 512);
@@ -884,7 +886,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       int n = 0;
       for (int wi = w0; wi < w1; ++wi)
         if (io[work[wi].point].active)
-          settle(pts, io, xp, work[wi], *reinterpret_cast<SettleSmem *>(ops), again + 2, n++ & 1, tid);
+          settle(pts, io, xp, work[wi], *reinterpret_cast<SettleSmem *>(ops), again + 2, n++, tid);
     }
   }
   tc_before();
@@ -900,7 +902,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // bytes of each X row) x 8 i3 (128 bytes of each natural row).
 // IW rows i1 per thread: two make a whole sector of the crossed output's layout, and
 // enough blocks (flow N = 64 25.9 ms, against 26.8 with four and 25.7 with one; N = 128
-// 320.8 us per rhs, against 322.5 and 324.4).
+// 320.8 us per rhs, against 322.5 and 324.4; with products of seven digits).
 constexpr int IW = 2;
 template <bool REV>
 __global__ void __launch_bounds__(256, 6) k_x64_combine(const PointDesc *__restrict__ pts,
@@ -1131,7 +1133,8 @@ int x64_run(X64Plan *p, const PointDesc *d_pts, const RhsIO *d_io, int point, in
     // The combine is not chained: blocks that become resident beside the products' find
     // the SM's storage set up as shared memory and next to no L1, and so do the kernels
     // chained to them (N = 128 336 against 322 us per rhs, N = 64 62.0 against 59.8 us
-    // and 37.8 against 35.8 ms per flow; nothing chained 327 and 65.0 us, 36.2 ms).
+    // and 37.8 against 35.8 ms per flow; nothing chained 327 and 65.0 us, 36.2 ms; all with
+    // seven digits).
     if (launch_chained(x64::panel_u(maxN) == 8 ? x64::k_x64_panels<8> : x64::k_x64_panels<4>, pg,
                        x64::panel_threads(maxN), 0, st, chain, d_pts, d_io, p->d_x, p0, chmask, rev) != cudaSuccess ||
         launch_chained(x64::k_x64_products, s->grid, x64::THREADS, x64::SMEM, st, chain, d_pts, d_io, p->d_x, s->work,
