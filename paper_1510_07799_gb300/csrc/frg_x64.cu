@@ -34,8 +34,8 @@
 // operands into blocks of 16 k x 64 lines; k_x64_products multiplies them
 // (persistent CTAs over a longest-first tile schedule); k_x64_combine sums the
 // channels into the natural layout.
-// Measured, one rhs (all channels): N = 128 6086 -> 402 us, N = 64 674 -> 65 us
-// (CUDA cores -> slices).  The eighth digit, the drains and the wider sums are 81 and 5
+// Measured, one rhs (all channels): N = 128 6086 -> 398 us, N = 64 674 -> 64 us
+// (CUDA cores -> slices).  The eighth digit, the drains and the wider sums are 77 and 4
 // us of it, against seven digits drained once per product.
 #include <cuda_runtime.h>
 
@@ -795,13 +795,14 @@ __global__ void __launch_bounds__(THREADS, 1)
             const uint32_t aq = a0 + (q == 0 ? PLANE : 0), bq = b0 + q * B_PL;
 #pragma unroll
             for (int i = 0; i < SL; ++i) {
-              // (digit 0 starts every accumulator of the chunk's first k-step)
-              const int cols = LINES * (NACC - i), n1 = cols > 256 ? cols / 2 : cols;
+              // (digit 0 starts every accumulator of the chunk's first k-step; 256 columns and the
+              // rest, not two halves: 398 against 402 us per rhs at N = 128)
+              const int cols = LINES * (NACC - i), n1 = cols > 256 ? 256 : cols;
               const uint64_t da = desc(aq + i * A_DIG, A_KC, 128);
               const uint32_t d = tmem + LINES * i, acc = (kb % CHUNK | q | i) ? 1u : 0u;
               mma_f16(d, da, desc(bq, B_KC, 128), idesc(n1), acc);
-              if (cols > 256)  // the second half of the columns: n1 / 8 line groups further on
-                mma_f16(d + n1, da, desc(bq + n1 / 8 * 128, B_KC, 128), idesc(n1), acc);
+              if (cols > 256)  // the rest of the columns: 32 line groups further on
+                mma_f16(d + n1, da, desc(bq + n1 / 8 * 128, B_KC, 128), idesc(cols - n1), acc);
             }
           }
           mma_commit(&op_empty[s]);
